@@ -29,13 +29,14 @@ asl_status asl_create(asl_ctx** out, int device) {
   *out = nullptr;
   int count = 0;
   if (cudaGetDeviceCount(&count) != cudaSuccess || device < 0 || device >= count) return ASL_ERR_CUDA;
-  cudaDeviceProp prop;
-  ASL_CUDA(cudaGetDeviceProperties(&prop, device));
-  if (prop.major != 10) return ASL_ERR_ARCH;      // sm_100 only: no fallback path
+  int major = 0, sms = 0;                         // (cudaGetDeviceProperties would take milliseconds)
+  ASL_CUDA(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device));
+  ASL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
+  if (major != 10) return ASL_ERR_ARCH;           // sm_100 only: no fallback path
   asl_ctx* c = new (std::nothrow) asl_ctx();
   if (!c) return ASL_ERR_CUDA;
   c->device = device;
-  c->sm_count = prop.multiProcessorCount;
+  c->sm_count = sms;
   int prev = 0;
   cudaGetDevice(&prev);
   cudaSetDevice(device);
@@ -81,7 +82,7 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
   if (p->cu_seqlens[0] != 0) return ASL_ERR_INVALID;
 
   std::vector<AslReq> req(p->batch);
-  int64_t sum_T = 0, sum_kept = 0, tiles = 0;
+  int64_t sum_T = 0, sum_kept = 0;
   int32_t max_n = 0, max_T = 0, max_kept = 0;
   for (int b = 0; b < p->batch; ++b) {
     const int64_t n = (int64_t)p->cu_seqlens[b + 1] - p->cu_seqlens[b];
@@ -95,10 +96,9 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
     r.tok_off = p->cu_seqlens[b];
     r.t_off = (int32_t)sum_T;
     r.kept_off = (int32_t)sum_kept;
-    r.pad = (int32_t)tiles;                       // first key tile of the request (SIMT scorer partials)
+    r.pad = 0;
     sum_T += r.T;
     sum_kept += r.kept;
-    tiles += (n + ASL_SIMT_KEY_TILE - 1) / ASL_SIMT_KEY_TILE;
     max_n = r.n > max_n ? r.n : max_n;
     max_T = r.T > max_T ? r.T : max_T;
     max_kept = r.kept > max_kept ? r.kept : max_kept;
@@ -135,27 +135,23 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
   c->sum_kept = sum_kept;
   c->max_n = max_n; c->max_T = max_T; c->max_kept = max_kept;
   c->rows_per_kv = (p->n_q_heads / p->n_kv_heads) * p->window;
-  c->n_key_tiles = (int32_t)tiles;
 
   cudaGetDevice(&prev);
   cudaSetDevice(c->device);
   const bool tc = asl_tc_plan(c);
   asl_topk_plan(c);
   cudaSetDevice(prev);
-  if (fp8 && !tc) { free_plan(c); return ASL_ERR_UNSUPPORTED; }     // only the tensor-core scorer reads 8-bit keys
-  const int G = p->n_q_heads / p->n_kv_heads;
-  // the tensor-core scorer writes two partial column sums per chunk (one per half of the chunk's rows);
-  // under max pooling they belong to different query heads unless a chunk is a single head
-  c->u_parts = (tc && p->pool_mode == ASL_POOL_MAX && p->window > c->tc.NC / 2) ? 2 : 1;
-  c->u_rows_per_kv = p->pool_mode == ASL_POOL_MAX ? G * c->u_parts : (tc ? 2 * c->tc.nchunk : 1);
+  if (!tc) { free_plan(c); return fp8 ? ASL_ERR_UNSUPPORTED : ASL_ERR_CUDA; }     // 8-bit keys: not every window
+  // the scorer writes a partial column sum per half of a chunk's rows; under max pooling the halves (and the chunks of
+  // a window of more than 256 rows) belong to one query head only where a head takes more than one of them
+  const int G = p->n_q_heads / p->n_kv_heads, halves = c->tc.wide ? 2 : 1;
+  c->u_parts = p->pool_mode == ASL_POOL_MAX && c->tc.Wp > 128 ? 2 * c->tc.pieces : 1;
+  c->u_rows_per_kv = p->pool_mode == ASL_POOL_MAX ? G * c->u_parts : c->tc.nchunk * halves;
 
   AslWorkspace& w = c->ws;
   size_t off = 0;
-  size_t partial_bytes = (size_t)tiles * p->n_kv_heads * c->rows_per_kv * sizeof(float2);
-  if (tc && asl_tc_partial_bytes(c) > partial_bytes) partial_bytes = asl_tc_partial_bytes(c);
-  w.score_partials = off; off = asl_align256(off + partial_bytes);
-  const size_t rows_padded = tc && c->tc.nchunk * c->tc.NC > c->rows_per_kv ? (size_t)c->tc.nchunk * c->tc.NC : (size_t)c->rows_per_kv;
-  w.score_offsets = off;  off = asl_align256(off + (size_t)p->batch * p->n_kv_heads * rows_padded * sizeof(float));
+  w.score_partials = off; off = asl_align256(off + asl_tc_partial_bytes(c));
+  w.score_offsets = off;  off = asl_align256(off + (size_t)c->tc.nseg * c->tc.NC * sizeof(float));
   const size_t u_rows = (size_t)p->n_kv_heads * c->u_rows_per_kv;
   for (int i = 0; i < 2; ++i) { w.score_u[i] = off; off = asl_align256(off + u_rows * (size_t)sum_T * sizeof(float)); }
   w.score_q8 = off;
@@ -190,17 +186,14 @@ static asl_status score_columns_impl(asl_ctx* c, const void* q_obs, const void* 
   if (!workspace || workspace_bytes < c->ws.total || !aligned16(workspace)) return ASL_ERR_WORKSPACE;
   char* ws = static_cast<char*>(workspace);
   float* u = reinterpret_cast<float*>(ws + c->ws.score_u[slot]);
-  if (c->tc.enabled) {
-    // requests that have finished are not scored any more: a small kernel ahead of the launch reads their
-    // flags once and writes the launch's phase list without their phases, so that every CTA of the
-    // persistent kernel walks the same list
-    if (c->latch_stat && c->cur_layer >= 0 && c->p.batch <= ASL_SKIP_MAX_BATCH) {
-      const asl_status s = asl_launch_live_phases(c, lse == nullptr, static_cast<cudaStream_t>(stream));
-      if (s != ASL_OK) return s;
-    }
-    return asl_launch_score_tc(c, q_obs, k, lse, u, ws, static_cast<cudaStream_t>(stream));
+  // requests that have finished are not scored any more: a small kernel ahead of the launch reads their
+  // flags once and writes the launch's work list without their phases, so that every CTA of the
+  // persistent kernel walks the same list
+  if (c->latch_stat && c->cur_layer >= 0 && c->p.batch <= ASL_SKIP_MAX_BATCH) {
+    const asl_status s = asl_launch_live_phases(c, lse == nullptr, static_cast<cudaStream_t>(stream));
+    if (s != ASL_OK) return s;
   }
-  return asl_launch_score_simt(c, q_obs, k, lse, u, ws, static_cast<cudaStream_t>(stream));
+  return asl_launch_score_tc(c, q_obs, k, lse, u, ws, static_cast<cudaStream_t>(stream));
 }
 
 static asl_status pool_scores_impl(asl_ctx* c, void* workspace, size_t workspace_bytes, int slot, float* scores_kv,

@@ -55,11 +55,10 @@ struct asl_ctx {
   int32_t* d_err = nullptr;           // device error word of bounded waits
   // scorer plan
   int32_t rows_per_kv = 0;            // G*W
-  int32_t n_key_tiles = 0;            // sum over requests of ceil(n_b / tile)
   int32_t u_rows_per_kv = 1;          // rows of un-pooled column sums per kv head (average pooling: all are added;
                                       // max pooling: G * u_parts, u_parts consecutive rows per query head)
   int32_t u_parts = 1;                // partial rows per query head under max pooling
-  AslTcPlan tc;                       // tensor-core scorer plan (enabled when the shape fits)
+  AslTcPlan tc;                       // scorer plan
   bool topk_one_cta = false;          // the per-head top-k runs as one CTA per segment (asl_topk_plan)
   AslWorkspace ws{};
   int64_t launches = 0;
@@ -113,8 +112,6 @@ constexpr int ASL_SKIP_MAX_BATCH = 4096;  // requests the scorer's per-launch ph
 static inline size_t asl_align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // ---- kernels' host launchers (one per translation unit) ----
-asl_status asl_launch_score_simt(asl_ctx* c, const void* q, const void* k, const float* lse, float* u, char* ws,
-                                 cudaStream_t st);
 asl_status asl_launch_window_lse(asl_ctx* c, const char* ws, float* lse_out, cudaStream_t st);
 bool asl_tc_plan(asl_ctx* c);
 void asl_tc_free(asl_ctx* c);
@@ -137,5 +134,4 @@ asl_status asl_launch_compact(asl_ctx* c, const void* k, const void* v, const in
 asl_status asl_launch_compact_rows(asl_ctx* c, const void* x, const int32_t* idx, void* out, int64_t row_bytes,
                                    cudaStream_t st);
 
-constexpr int ASL_SIMT_KEY_TILE = 128;   // keys per block in the SIMT scorer
 constexpr int ASL_RANK_TILE = 2048;      // keys per block in the radix sort

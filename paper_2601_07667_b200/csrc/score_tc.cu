@@ -4,32 +4,44 @@
 // (request, kv head, row chunk) "segment":
 //
 //   pass 1  D[row][key] = Q_chunk . K_tile^T  (query rows in TMEM lanes): each
-//           epilogue thread keeps, for its rows, the sum of 2^(x - ref) over the
-//           keys of the CTA's tiles (ref: the maximum of the first 32 keys the
-//           row met); each epilogue set publishes (ref, sum) per row.  Once every
-//           set has published, two helper warps per CTA fold the partials of
-//           "their" rows (row r belongs to CTA r mod grid), in a fixed order, into
-//           offset[row] = log2 of the row's softmax denominator, off the
-//           epilogue's critical path.
-//   pass 2  D[key][row] = K_tile . Q_chunk^T  (keys in TMEM lanes): each thread
-//           owns one key and sums exp2(x - offset[row]) over the chunk's rows:
-//           the key's column sum U, already summed over the GQA group.
+//           epilogue thread keeps, for its row, the sum of 2^(x - ref) over the
+//           keys it meets (ref: its first logit of the run); at the
+//           end of a CTA's run of tiles each epilogue group publishes (ref, sum) per
+//           row.  Once every group has published, a helper warp per CTA folds the
+//           partials of "their" rows, in a fixed order, into offset[row] = log2 of
+//           the row's softmax denominator, off the epilogue's critical path.
+//   pass 2  D[key][row] = K_tile . Q_chunk^T  (keys in TMEM lanes): exp2(x -
+//           offset[row]) summed over the chunk's rows: the key's column sum U,
+//           already summed over the GQA group.
 //
-// All arithmetic is in the log2 domain x = (q.k) * log2(e)/sqrt(d).  A "chunk"
-// is up to 256 of the G*W query rows that share a kv head; a "phase" is one pass
-// over one segment's 128-key tiles.  Phases are ordered pass1(s0) pass1(s1)
-// pass2(s0) pass2(s1) pass1(s2) ... so that the offsets a pass-2 phase needs were
-// finished one phase earlier, and so that K of a segment is still in L2 when
-// pass 2 reads it again: HBM sees K once.  The tiles of the whole phase list are
-// dealt round-robin to the CTAs.
+// All arithmetic is in the log2 domain x = (q.k) * log2(e)/sqrt(d).  A "chunk" is
+// up to 256 of the G*W query rows that share a kv head.  Work is dealt in "runs": the
+// contiguous tiles that one CTA takes of one segment in one pass.  Segments form groups;
+// a CTA does its runs of pass 1 of group i, then those of pass 2 of group i - 1: it
+// meets one or two segments at a time and keeps a Q chunk for a whole run, the offsets
+// that pass 2 needs were folded while other tiles were worked on, and most of K of two
+// groups (up to 70 MB each) is still in L2 when pass 2 reads it again.  Dealing every segment's tiles round-robin to all
+// CTAs cost 3 us per segment and pass (64 KB of Q reloaded per CTA, a hand-off each):
+// 32K tokens, 8 kv heads 64 -> 48 us, eight ragged requests with W = 32 350 -> 184 us,
+// W = 128 with 64 query heads at 64K 374 -> 288 us, 128K tokens 163 -> 153 us.
 //
-// Inside a CTA: warp 0 streams K tiles through a 3-stage TMA ring (128B-swizzled)
-// and keeps the Q chunks of two phases resident (the next one is prefetched);
-// warp 1 issues tcgen05.mma into two 256-column TMEM accumulators; warps 2-3 fold
-// pass-1 partials; two sets of eight epilogue warps take alternate tiles, one
-// accumulator each (two warps per TMEM lane quarter, half of the columns each).  The
-// exponentials are split between the MUFU unit and a degree-3 polynomial on the
-// FMA pipe (packed f32x2 arithmetic).
+// What bounds it: two exponentials per logit, and power.  Of every 16 column pairs 3
+// take a degree-4 polynomial on the FMA pipe, the others the MUFU unit (16 per clock and
+// SM): a tile of 128 keys x 256 rows is 32768 of them, 1664 clk of MUFU, and the loop
+// takes about 1950 in the kernel.  Kept up for more than some
+// ten milliseconds the kernel runs at the 1000 W limit (1.6 GHz instead of 1.9), where
+// the energy of the MMAs (0.7 us at the limit per 148 tiles) and of streaming K (45 us at
+// the limit for 268 MB from HBM, 16 from L2) counts as much as instructions do.
+//
+// Inside a CTA: warp 0 streams K tiles through a TMA ring (128B-swizzled) and keeps the Q
+// chunks of two runs resident; warp 1 issues tcgen05.mma from a warp-uniform loop (under
+// a one-thread branch an MMA of 128 columns takes 90-110 clk instead of 64-73) into four
+// 128-column accumulators; warp 2 folds, warp 3 fetches offsets; four groups of four
+// epilogue warps own one accumulator each, so that up to three groups compute while one
+// accumulator fills.  The accumulator is read 16 registers at a time, double buffered.
+// Pass 2 reads it in the 16x256b shape, in which a thread meets only every fourth column
+// pair and can keep its rows' offsets in registers: broadcast loads of the offsets from
+// shared memory (131 KB per tile) cost 400 clk.
 //
 // Every wait (mbarrier, counter) is bounded: when the limit is reached the thread
 // records a code in the context's error word and the CTA drains: producers stop,
@@ -37,33 +49,37 @@
 // in-flight copies are waited for with the same bound and tensor memory is freed.
 #include <cuda.h>
 #include <cuda_fp8.h>
+#include <string.h>
 
 #include "asl_internal.cuh"
 
 namespace {
 
 constexpr int KT = ASL_TC_KEY_TILE;          // keys per tile
-constexpr int NSTAGE = 3;
-constexpr int HALF_BYTES = KT * 128;         // one 64-channel block of a K tile: 128 rows x 128 B
-constexpr int STAGE_BYTES = 2 * HALF_BYTES;
-constexpr int MAX_NC = 256;
-constexpr int Q_BLOCK_BYTES = MAX_NC * 128;  // one 64-channel block of a Q chunk
-constexpr int Q_BUF_BYTES = 2 * Q_BLOCK_BYTES;
-constexpr int THREADS = 640;                 // warp 0: TMA, 1: MMA, 2-3: partial folding, 4-11 / 12-19: epilogue sets
+constexpr int MAX_ROWS = 256;                // query rows of a chunk at most
+constexpr int THREADS = 640;                 // warp 0: TMA, 1: MMA, 2-3: partial folding, 4-19: four epilogue groups
+constexpr int GROUPS = 4;
+constexpr int SYNC_STRIDE = 8;               // words from one segment's counter to the next: a sector each
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;   // every wait gives up after 2 s
 
-// shared-memory map (offsets from the 1024-aligned base of dynamic shared memory)
-constexpr int SM_Q = 0;                                      // two Q chunk buffers
-constexpr int SM_K = SM_Q + 2 * Q_BUF_BYTES;
-constexpr int SM_NEGOFF = SM_K + NSTAGE * STAGE_BYTES;       // float[2][256]: -offset per epilogue set
-constexpr int SM_BAR = SM_NEGOFF + 2048;                     // mbarriers
-constexpr int SM_MISC = SM_BAR + 128;                        // tmem base, abort flag
-constexpr int SMEM_BYTES = SM_MISC + 64;
-static_assert(SMEM_BYTES <= 232448, "shared memory budget of one CTA");
-
-enum { BAR_FULL = 0, BAR_EMPTY = NSTAGE, BAR_TFULL = 2 * NSTAGE, BAR_TEMPTY = 2 * NSTAGE + 2,
-       BAR_QFULL = 2 * NSTAGE + 4, BAR_QEMPTY = 2 * NSTAGE + 6, BAR_DRAIN = 2 * NSTAGE + 8, N_BARS = 2 * NSTAGE + 9 };
-static_assert(N_BARS * 8 <= 128, "barrier area");
+// Shared-memory layout of one CTA (offsets from the 1024-aligned base).  WIDE: a chunk of more than 128 rows.
+template <bool FP8, bool WIDE>
+struct Smem {
+  static constexpr int Q_ROWS = WIDE ? 256 : 128;
+  static constexpr int Q_BLOCK = Q_ROWS * 128;              // a 64-channel block (FP8: an E4M3 term) of a Q chunk
+  static constexpr int Q_BUF = 2 * Q_BLOCK;
+  static constexpr int HALF = KT * 128;                     // a 64-channel block of a K tile: 128 rows x 128 B
+  static constexpr int STAGE = FP8 ? HALF : 2 * HALF;
+  static constexpr int NSTAGE = (WIDE ? 98304 : 163840) / STAGE;
+  static constexpr int K = 2 * Q_BUF;                       // two Q chunks, then the ring of K tiles
+  static constexpr int BARS = K + NSTAGE * STAGE;
+  static constexpr int FULL = 0, EMPTY = NSTAGE, TFULL = 2 * NSTAGE, TEMPTY = TFULL + GROUPS, QFULL = TEMPTY + GROUPS,
+                       QEMPTY = QFULL + 2, OFULL = QEMPTY + 2, OEMPTY = OFULL + 2, DRAIN = OEMPTY + 2, N_BARS = DRAIN + 1;
+  static constexpr int MISC = BARS + 384;                   // tmem base, abort flag, launch number and its parity
+  static constexpr int OFFS = MISC + 64;                    // float[2][256]: -offset of the rows of two pass-2 runs
+  static constexpr int BYTES = OFFS + 2048;
+  static_assert(N_BARS * 8 <= 384 && BYTES <= 232448, "shared memory budget of one CTA");
+};
 
 // ---------------------------------------------------------------- PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -92,6 +108,18 @@ __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long now;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
   return now;
+}
+// Looks once, without suspending the thread.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
 }
 // Bounded wait.  `watch_abort`: also give up when another role raised the flag.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int code,
@@ -125,8 +153,10 @@ __device__ __forceinline__ bool word_wait(const uint32_t* p, uint32_t want, vola
         if (t0 == 0) t0 = now;
         else if (now - t0 > limit_ns || *abort_flag) { gave_up = 1; if (!*abort_flag) *abort_flag = code; break; }
       }
-      __nanosleep(nap);
-      if (nap < nap_max) nap <<= 1;
+      if (it >= 16) {                    // the first looks follow one another at once: what is waited for is about to come
+        __nanosleep(nap);
+        if (nap < nap_max) nap <<= 1;
+      }
     }
   }
   return __shfl_sync(0xffffffffu, gave_up, 0) == 0;
@@ -193,31 +223,41 @@ __device__ __forceinline__ void tc_mma_f8(uint32_t d_tmem, uint64_t a_desc, uint
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accum)
       : "memory");
 }
-// 32 consecutive fp32 columns of this thread's TMEM lane: issue only; the
-// registers hold the data after tc_ld_wait on the same array.
-__device__ __forceinline__ void tc_ld32_issue(uint32_t taddr, uint32_t (&r)[32]) {
+// 16 registers of an accumulator: issue only; they hold the data after tc_ld_wait on the same array.
+// Shape 32x32b: 16 consecutive columns of this thread's lane.
+__device__ __forceinline__ void tc_ld_lane(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+// Shape 16x256b: 16 lanes x 32 columns; registers 4i..4i+3 of thread t hold columns 8i + 2(t%4) + {0, 1} of lanes
+// t/4 and t/4 + 8.
+__device__ __forceinline__ void tc_ld_quad(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
 }
 // Waits for every tcgen05.ld this thread has issued.  The array is an in/out
 // operand so that no use of its registers can be scheduled above the wait.
-__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[32]) {
+__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
-                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]),
-                 "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]),
-                 "+r"(r[30]), "+r"(r[31])
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
                :
                : "memory");
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e != 0;
 }
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -248,6 +288,16 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 __device__ __forceinline__ float hsum(f32x2 v) {
   float lo, hi;
   upk(v, lo, hi);
@@ -260,47 +310,30 @@ __device__ __forceinline__ f32x2 ex2_pair_mufu(f32x2 x) {
   return pk(ex2(a), ex2(b));
 }
 // 2^x of a pair on the FMA pipe (any x < 128): clamp at -125, round to the nearest
-// integer n with the 1.5*2^23 trick, degree-3 minimax polynomial of 2^f on
-// f = x - n in [-0.5, 0.5] (relative error 7.5e-5), n added into the exponent field.
-// Additions are written as fma(a, 1, b): the packed fma issues faster than the packed add.
+// integer n with the 1.5*2^23 trick, degree-4 minimax polynomial of 2^f on
+// f = x - n in [-0.5, 0.5] (relative error 2.6e-6), n added into the exponent field.
+// Packed additions are written as such, not as fma(a, 1, b): as fast, and six constant registers fewer.
 __device__ __forceinline__ f32x2 ex2_pair_poly(f32x2 x) {
   float a, b;
   upk(x, a, b);
   const f32x2 xc = pk(fmaxf(a, -125.0f), fmaxf(b, -125.0f));
-  const f32x2 one = pk(1.0f, 1.0f);
-  const f32x2 t = fma2(xc, one, pk(12582912.0f, 12582912.0f));
-  const f32x2 f = fma2(fma2(t, one, pk(-12582912.0f, -12582912.0f)), pk(-1.0f, -1.0f), xc);
-  f32x2 p = fma2(pk(0.0551716685f, 0.0551716685f), f, pk(0.2426111400f, 0.2426111400f));
-  p = fma2(p, f, pk(0.6932609677f, 0.6932609677f));
-  p = fma2(p, f, pk(0.9999280572f, 0.9999280572f));
+  const f32x2 magic = pk(12582912.0f, 12582912.0f);
+  const f32x2 t = add2(xc, magic);
+  const f32x2 f = sub2(xc, sub2(t, magic));
+  f32x2 p = fma2(pk(0.00956967473f, 0.00956967473f), f, pk(0.0559182465f, 0.0559182465f));
+  p = fma2(p, f, pk(0.240247667f, 0.240247667f));
+  p = fma2(p, f, pk(0.693121731f, 0.693121731f));
+  p = fma2(p, f, pk(0.999999225f, 0.999999225f));
   uint32_t tl, th, pl, ph;
   upku(t, tl, th);
   upku(p, pl, ph);
   return pku(pl + (tl << 23), ph + (th << 23));
 }
-// which of a block's 16 column pairs take the polynomial: POLY_PAIRS_OF_8 of every 8, spread out
-#ifndef ASL_POLY_PAIRS_OF_8
-#define ASL_POLY_PAIRS_OF_8 2
-#endif
-constexpr int POLY_PAIRS_OF_8 = ASL_POLY_PAIRS_OF_8;
-__device__ __forceinline__ constexpr bool pair_is_poly(int pi) {
-  return POLY_PAIRS_OF_8 >= 4 ? (pi & 1) == 1
-                              : ((POLY_PAIRS_OF_8 >= 1 && (pi & 7) == 1) || (POLY_PAIRS_OF_8 >= 2 && (pi & 7) == 5) ||
-                                 (POLY_PAIRS_OF_8 >= 3 && (pi & 7) == 3));
-}
-// sum over 32 accumulator columns of 2^(v*scale + c), c one pair per column pair
-template <typename OffsetPair>
-__device__ __forceinline__ float exp_sum32(const uint32_t (&cur)[32], f32x2 scale2, OffsetPair off) {
-  f32x2 acc_m = pk(0.f, 0.f), acc_p = pk(0.f, 0.f);
-  const f32x2 one = pk(1.0f, 1.0f);
-#pragma unroll
-  for (int pi = 0; pi < 16; ++pi) {
-    const f32x2 x = fma2(pku(cur[2 * pi], cur[2 * pi + 1]), scale2, off(pi));
-    if (pair_is_poly(pi)) acc_p = fma2(ex2_pair_poly(x), one, acc_p);
-    else                  acc_m = fma2(ex2_pair_mufu(x), one, acc_m);
-  }
-  return hsum(fma2(acc_m, one, acc_p));
-}
+// Which of every 16 column pairs take the polynomial, spread out.  3: the loop alone is shortest at 5 (clk per tile,
+// pass 1 / pass 2, at 4, 5, 6: 1821 / 1833, 1725 / 1794, 1747 / 1839), but a polynomial costs more energy than the MUFU
+// unit and more registers; in the kernel, at 128K tokens: 155.4, 156.9, 160.9 us at 3, 4, 5.
+constexpr int POLY_OF_16 = 3;
+__device__ __forceinline__ constexpr bool pair_is_poly(int i) { return ((i & 15) * POLY_OF_16) % 16 + POLY_OF_16 >= 16; }
 
 // K-major, 128B-swizzled operand: rows of 128 B, 8-row groups 1024 B apart.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
@@ -316,269 +349,281 @@ __device__ __forceinline__ uint32_t instr_desc_f8(int M, int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+
+struct TcWork {
+  const TcRun* runs;
+  const int32_t* first;    // [grid] first run of every CTA, or -1
+  const TcFold* folds;     // [segments]
+};
 struct TcArgs {
-  const TcPhase* phases;
-  const AslReq* req;
-  float2* partials;        // pass 1: [segment][CTA][set][NC] (reference, sum) of each epilogue set
+  TcWork list, live;       // the plan's list; the one without finished requests, to be taken where live_hdr[0] is set
+  const int32_t* live_hdr; // or null
+  const TcStage* stages;   // groups of segments whose rows are folded together
+  float2* partials;        // pass 1: [run slot][entry][NC] (reference, sum) of every row
   float* offsets;          // [segment][NC], written by the folding warps, read by pass 2
   const float* lse;        // null, or the rows' natural-log softmax denominators [B][H_q][W]: pass 2 alone
   float* u;                // pass 2 out: column sums
-  uint32_t* published;     // [segment] epilogue sets that have published, accumulated over launches
-  uint32_t* folded;        // [segment] rows whose offset is written, accumulated over launches
+  // [2][2][segment * SYNC_STRIDE]: per segment, epilogue groups that have published and rows whose offset is written.
+  // A launch counts in the set that its number's parity names; the last CTA to arrive clears the other set (whose launch
+  // is over), advances the number and resets the ticket.  The number lives on the device so that a launch replayed from
+  // a CUDA graph counts like any other, and is switched at entry so that no CTA has anything to do at its end.
+  uint32_t* counters;
+  uint32_t* launch;        // launch number, then the ticket of arrived CTAs
   int32_t* err;
   int64_t sum_T;
-  uint32_t* epoch_word;    // two-pass launches completed so far (the counters accumulate over launches); then a ticket word
-  uint32_t epoch_limit;    // beyond it the last CTA clears the counters instead of letting them wrap
-  int32_t nseg;
-  const int32_t* live_hdr; // null, or device {phases, work items} of `phases`, written ahead of the launch (the list without
-                           // the phases of finished requests); then n_phases / total_items below are not used
-  int32_t n_phases, total_items, NC, W, G, Hk, Hq, u_rows_per_kv, u_parts;
+  int32_t n_stages, nseg, NC, HR, W, Wp, m, pieces, G, Hq, u_rows_per_kv, u_parts;
   float scale_log2;
 };
 
-// walks the CTA's items (global item g = blockIdx.x + i*gridDim.x) through the phase list.  The
-// current phase record and the one after it stay in registers: the next record is requested when a
-// phase is entered, so its load latency is hidden behind the phase's tiles.
-struct ItemWalk {
-  const TcPhase* phases;
-  int total, n_phases;
-  int g, ph;
-  TcPhase cur, nxt;
-  __device__ __forceinline__ ItemWalk(const TcArgs& a, int n_phases_, int total_) : phases(a.phases), total(total_), n_phases(n_phases_),
-                                                                                g((int)blockIdx.x), ph(0) {
-    cur = phases[0];
-    nxt = phases[n_phases > 1 ? 1 : 0];
-  }
-  __device__ __forceinline__ bool valid() const { return g < total; }
-  __device__ __forceinline__ const TcPhase& phase() {       // phases are sorted by g0 and cover [0, total)
-    while (g >= cur.g0 + cur.ntiles) {
-      cur = nxt;
-      ++ph;
-      nxt = phases[ph + 1 < n_phases ? ph + 1 : ph];
-    }
-    return cur;
-  }
-  __device__ __forceinline__ bool last_in_phase() const { return g + (int)gridDim.x >= cur.g0 + cur.ntiles; }
-  __device__ __forceinline__ void next() { g += (int)gridDim.x; }
-};
+// Row r of chunk ch is row t of query head g of its kv head (under max pooling heads start at multiples of Wp > W and
+// rows t >= W do not exist; a window of more than 256 rows is cut into pieces, one per chunk).
+struct RowPlace { int g, t; };
+__device__ __forceinline__ RowPlace row_place(const TcArgs& a, int ch, int r) {
+  if (a.pieces > 1) return {ch / a.pieces, (ch % a.pieces) * MAX_ROWS + r};
+  return {ch * a.m + r / a.Wp, r % a.Wp};
+}
+
+__device__ __forceinline__ TcRun load_run(const TcRun* runs, int slot) {
+  TcRun r;
+  const int4* s = reinterpret_cast<const int4*>(runs + slot);
+  int4* d = reinterpret_cast<int4*>(&r);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) d[i] = __ldg(s + i);
+  return r;
+}
+__device__ __forceinline__ void prefetch_run(const TcRun* runs, int slot) {
+  if (slot >= 0) asm volatile("prefetch.global.L1 [%0];" ::"l"(runs + slot));
+}
 
 // FP8: K tiles hold E4M3 codes (one 128-byte row per key: a tile is one 16 KB box), the query chunk holds
-// the two E4M3 terms of every query (term t in the t-th 32 KB block of the chunk's buffer, where bf16
+// the two E4M3 terms of every query (term t in the t-th block of the chunk's buffer, where bf16
 // queries keep their t-th 64-channel block), and a tile takes 2 terms x 4 k-steps of 32 channels.
-template <bool PER_Q, bool FP8>
+// A unit = one accumulator: a 128-key tile x one half of the chunk's rows; units are numbered through all of the
+// CTA's runs and group g takes units g, g + 4, ...
+// FULL: halves of 128 rows (the block loop of pass 2 then has no branches: 128K tokens 171 -> 163 us).
+template <bool PER_Q, bool FP8, bool WIDE, bool FULL>
 __global__ void __launch_bounds__(THREADS, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const TcArgs a) {
+  using S = Smem<FP8, WIDE>;
+  constexpr int HV = WIDE ? 2 : 1;
+  constexpr int ENTRIES = GROUPS / HV;          // groups that meet a row; entry e: tiles e, e + ENTRIES, ... of the run
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
   if (sbase & 1023u) {                       // the swizzled operand layout needs a 1024-byte aligned base
     if (threadIdx.x == 0) atomicCAS(a.err, 0, 901);
     return;
   }
-  const uint32_t bars = sbase + SM_BAR;
-  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(smem + SM_MISC);
-  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + SM_MISC + 4);
-  volatile uint32_t* s_epoch = reinterpret_cast<volatile uint32_t*>(smem + SM_MISC + 8);
-  volatile int* s_list = reinterpret_cast<volatile int*>(smem + SM_MISC + 16);       // {phases, work items} of this launch
+  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(smem + S::MISC);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + S::MISC + 4);
+  volatile uint32_t* s_number = reinterpret_cast<volatile uint32_t*>(smem + S::MISC + 8);     // this launch's number
+  volatile uint32_t* s_set = reinterpret_cast<volatile uint32_t*>(smem + S::MISC + 12);     // its parity
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const int HR = FULL ? 128 : a.HR;
+  auto bar = [&](int i) { return sbase + S::BARS + 8u * (uint32_t)i; };
+  const bool dense = a.Wp == a.W || a.pieces > 1;             // one copy brings all rows of a chunk
+  const int copies = dense ? 1 : a.m;
+  const int box_rows = a.pieces > 1 ? MAX_ROWS : (dense ? a.m * a.W : a.W);
 
-  float* s_negoff = reinterpret_cast<float*>(smem + SM_NEGOFF);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int NC = a.NC;
-  auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
-
-  // ---- set-up: zero the Q buffers (rows past NC feed unused MMA rows), barriers, tensor memory ----
-  if (NC & 127)
-    for (int i = threadIdx.x; i < 2 * Q_BUF_BYTES / 16; i += THREADS) reinterpret_cast<uint4*>(smem + SM_Q)[i] = make_uint4(0, 0, 0, 0);
+  // ---- set-up: zero the Q buffers (rows that no copy writes feed unused MMA rows), barriers, tensor memory ----
+  if (copies * box_rows < S::Q_ROWS)
+    for (int i = threadIdx.x; i < 2 * S::Q_BUF / 16; i += THREADS) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
+  const TcWork work = a.live_hdr && __ldg(a.live_hdr) ? a.live : a.list;
+  const int first = __ldg(work.first + blockIdx.x);
+  if (threadIdx.x == 32) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_q) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_k) : "memory");
+  }
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NSTAGE; ++s) { mbar_init(bar(BAR_FULL + s), 1); mbar_init(bar(BAR_EMPTY + s), 1); }
+    for (int s = 0; s < S::NSTAGE; ++s) { mbar_init(bar(S::FULL + s), 1); mbar_init(bar(S::EMPTY + s), 1); }
+    for (int i = 0; i < GROUPS; ++i) { mbar_init(bar(S::TFULL + i), 1); mbar_init(bar(S::TEMPTY + i), 4); }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(bar(BAR_TFULL + i), 1); mbar_init(bar(BAR_TEMPTY + i), 8);
-      mbar_init(bar(BAR_QFULL + i), 1); mbar_init(bar(BAR_QEMPTY + i), 1);
+      mbar_init(bar(S::QFULL + i), 1); mbar_init(bar(S::QEMPTY + i), 1);
+      mbar_init(bar(S::OFULL + i), 1); mbar_init(bar(S::OEMPTY + i), 4 * GROUPS);
     }
-    mbar_init(bar(BAR_DRAIN), 1);
+    mbar_init(bar(S::DRAIN), 1);
     *s_abort = 0;
-    // This launch's number.  It is read on the device, not passed by the host, so that a launch
-    // replayed from a CUDA graph still counts: no CTA of this launch can see the increment below,
-    // which the last CTA to leave makes.
-    uint32_t done = 0;
-    if (!a.lse) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(done) : "l"(a.epoch_word) : "memory");
-    *s_epoch = done + 1u;
-    s_list[0] = a.live_hdr ? __ldcg(a.live_hdr) : a.n_phases;
-    s_list[1] = a.live_hdr ? __ldcg(a.live_hdr + 1) : a.total_items;
+    uint32_t number = 0;
+    if (!a.lse) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(number) : "l"(a.launch) : "memory");
+    *s_set = number & 1u;
+    *s_number = number;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(sbase + SM_MISC) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(sbase + S::MISC) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
-  const uint32_t epoch = *s_epoch;
-  const int n_phases = s_list[0], total_items = s_list[1];
+  uint32_t* const published = a.counters + (size_t)*s_set * 2 * a.nseg * SYNC_STRIDE;
+  uint32_t* const folded = published + (size_t)a.nseg * SYNC_STRIDE;
 
   if (warp == 0) {
     // =============================== TMA producer ===============================
-    // Local phase l (the l-th phase in which this CTA has a tile) uses Q buffer l%2.
-    if (lane == 0) {
-      ItemWalk w(a, n_phases, total_items);
+    // The CTA's l-th run uses Q buffer l%2.
+    if (lane == 0 && first >= 0) {
       const uint64_t pol_keep = l2_policy_keep(), pol_stream = l2_policy_stream();
-      int item = 0, lp = -1, cur_ph = -1;
-      int q_issued = -1;                       // highest local phase whose Q chunk has been requested
+      int s = 0, item = 0;                     // ring stage and number of the next tile
+      uint32_t s_par = 1;
+      int q_issued = -1;                       // last run whose Q chunk has been requested
       int loaded_seg[2] = {-1, -1};
-      int next_ph = -1;                        // the CTA's next phase after the current one (-1: none)
-      int tok_off = 0;                         // first token of the current phase's request
       bool ok = true;
-      // requests the Q chunk of local phase `l` (phase record p); `block`: wait for the buffer, else only try
-      auto issue_q = [&](int l, const TcPhase& p, bool block) -> bool {
+      // requests the Q chunk of run `l` (record p); `block`: wait for the buffer, else only try
+      auto issue_q = [&](int l, const TcRun& p, bool block) -> bool {
         const int b = l & 1, use = l >> 1;
         if (use >= 1) {
           const uint32_t par = (uint32_t)((use - 1) & 1);
-          if (block) { if (!mbar_wait(bar(BAR_QEMPTY + b), par, s_abort, 11, true)) return false; }
-          else if (!mbar_try(bar(BAR_QEMPTY + b), par)) return true;
+          if (block) { if (!mbar_wait(bar(S::QEMPTY + b), par, s_abort, 11, true)) return false; }
+          else if (!mbar_test(bar(S::QEMPTY + b), par)) return true;
         }
         if (loaded_seg[b] == p.seg) {
-          mbar_arrive(bar(BAR_QFULL + b));     // same chunk as the buffer holds: nothing to copy
+          mbar_arrive(bar(S::QFULL + b));      // same chunk as the buffer holds: nothing to copy
         } else {
-          const int r0 = p.chunk * NC;
-          const int head = p.h * a.G + r0 / a.W, t0 = r0 % a.W;
-          const uint32_t dst = sbase + SM_Q + (uint32_t)b * Q_BUF_BYTES;
-          mbar_expect_tx(bar(BAR_QFULL + b), 2u * 128u * (uint32_t)NC);
-          if (FP8) {
-            tma_load_5d(dst, &tm_q, bar(BAR_QFULL + b), 0, t0, head, p.b, 0);
-            tma_load_5d(dst + Q_BLOCK_BYTES, &tm_q, bar(BAR_QFULL + b), 0, t0, head, p.b, 1);
-          } else {
-            tma_load_4d(dst, &tm_q, bar(BAR_QFULL + b), 0, t0, head, p.b);
-            tma_load_4d(dst + Q_BLOCK_BYTES, &tm_q, bar(BAR_QFULL + b), 64, t0, head, p.b);
+          const RowPlace r0 = row_place(a, p.chunk, 0);
+          mbar_expect_tx(bar(S::QFULL + b), 2u * 128u * (uint32_t)(copies * box_rows));
+          for (int i = 0; i < copies; ++i) {
+            const int head = p.h * a.G + r0.g + i;
+            const uint32_t dst = sbase + (uint32_t)(b * S::Q_BUF + i * a.Wp * 128);
+            if (FP8) {
+              tma_load_5d(dst, &tm_q, bar(S::QFULL + b), 0, r0.t, head, p.b, 0);
+              tma_load_5d(dst + S::Q_BLOCK, &tm_q, bar(S::QFULL + b), 0, r0.t, head, p.b, 1);
+            } else {
+              tma_load_4d(dst, &tm_q, bar(S::QFULL + b), 0, r0.t, head, p.b);
+              tma_load_4d(dst + S::Q_BLOCK, &tm_q, bar(S::QFULL + b), 64, r0.t, head, p.b);
+            }
           }
           loaded_seg[b] = p.seg;
         }
         q_issued = l;
         return true;
       };
-      for (; ok && w.valid(); w.next(), ++item) {
-        const TcPhase p = w.phase();
-        if (w.ph != cur_ph) {
-          cur_ph = w.ph;
-          ++lp;
-          tok_off = p.tok_off;
-          if (q_issued < lp && !issue_q(lp, p, true)) { ok = false; break; }
-          // where does this CTA go after this phase?
-          const int end = p.g0 + p.ntiles;
-          const int gn = w.g + ((end - w.g + (int)gridDim.x - 1) / (int)gridDim.x) * (int)gridDim.x;
-          next_ph = -1;
-          if (gn < w.total) {
-            int q = w.ph + 1;
-            while (gn >= a.phases[q].g0 + a.phases[q].ntiles) ++q;
-            next_ph = q;
-          }
-        }
-        if (next_ph >= 0 && q_issued == lp) {    // prefetch the next phase's Q chunk once its buffer is free
-          if (!issue_q(lp + 1, a.phases[next_ph], false)) { ok = false; break; }
-        }
-        const int s = item % NSTAGE;
-        if (!mbar_wait(bar(BAR_EMPTY + s), ((item / NSTAGE) & 1) ^ 1, s_abort, 12, true)) { ok = false; break; }
-        mbar_expect_tx(bar(BAR_FULL + s), FP8 ? HALF_BYTES : STAGE_BYTES);
-        const uint32_t dst = sbase + SM_K + s * STAGE_BYTES;
-        const int tok = tok_off + (w.g - p.g0) * KT;
+      TcRun p = load_run(work.runs, first);
+      for (int l = 0; ok; ++l) {
+        const TcRun nxt = p.next >= 0 ? load_run(work.runs, p.next) : p;
+        if (q_issued < l && !issue_q(l, p, true)) { ok = false; break; }
         const uint64_t pol = p.pass == 1 ? pol_keep : pol_stream;
-        tma_load_3d(dst, &tm_k, bar(BAR_FULL + s), 0, p.h, tok, pol);
-        if (!FP8) tma_load_3d(dst + HALF_BYTES, &tm_k, bar(BAR_FULL + s), 64, p.h, tok, pol);
+        for (int i = 0; i < p.ntiles; ++i) {
+          if (p.next >= 0 && q_issued == l && !issue_q(l + 1, nxt, false)) { ok = false; break; }   // once its buffer is free
+          if (!mbar_wait(bar(S::EMPTY + s), s_par, s_abort, 12, true)) { ok = false; break; }
+          mbar_expect_tx(bar(S::FULL + s), S::STAGE);
+          const uint32_t dst = sbase + S::K + s * S::STAGE;
+          const int tok = p.tok_off + (p.tile0 + i) * KT;
+          tma_load_3d(dst, &tm_k, bar(S::FULL + s), 0, p.h, tok, pol);
+          if (!FP8) tma_load_3d(dst + S::HALF, &tm_k, bar(S::FULL + s), 64, p.h, tok, pol);
+          ++item;
+          if (++s == S::NSTAGE) { s = 0; s_par ^= 1u; }
+        }
+        if (p.next < 0) break;
+        p = nxt;
       }
       if (!ok) {
         // let the copies already issued land before the CTA's shared memory is released
-        const int armed = item < NSTAGE ? item : NSTAGE;
+        const int armed = item < S::NSTAGE ? item : S::NSTAGE;
         for (int i = 0; i < armed; ++i) {
-          const int it = item - 1 - i, s = it % NSTAGE;
-          mbar_wait(bar(BAR_FULL + s), (it / NSTAGE) & 1, s_abort, 13, false);
+          const int it = item - 1 - i;
+          mbar_wait(bar(S::FULL + it % S::NSTAGE), (it / S::NSTAGE) & 1, s_abort, 13, false);
         }
         for (int l = q_issued; l >= 0 && l > q_issued - 2; --l)
-          mbar_wait(bar(BAR_QFULL + (l & 1)), (l >> 1) & 1, s_abort, 14, false);
+          mbar_wait(bar(S::QFULL + (l & 1)), (l >> 1) & 1, s_abort, 14, false);
       }
     }
   } else if (warp == 1) {
     // =============================== MMA issuer =================================
-    if (lane == 0) {
-      ItemWalk w(a, n_phases, total_items);
-      int item = 0, lp = -1, cur_ph = -1;
-      bool ok = true;
-      const uint32_t idesc1 = FP8 ? instr_desc_f8(128, KT) : instr_desc(128, KT);
-      const uint32_t idesc2 = FP8 ? instr_desc_f8(KT, NC) : instr_desc(KT, NC);
-      // byte offset of k-step ks inside a K tile: bf16 tiles are two 64-channel blocks, 8-bit tiles one block
-      auto k_off = [](int ks) { return (uint32_t)(FP8 ? (ks & 3) * 32 : (ks >> 2) * HALF_BYTES + (ks & 3) * 32); };
-      const int nhalf = (NC > 128) ? 2 : 1;
-      uint32_t qbase = 0;
-      for (; ok && w.valid(); w.next(), ++item) {
-        const TcPhase p = w.phase();
-        if (w.ph != cur_ph) {
-          cur_ph = w.ph;
-          ++lp;
-          if (!mbar_wait(bar(BAR_QFULL + (lp & 1)), (lp >> 1) & 1, s_abort, 21, true)) { ok = false; break; }
-          qbase = sbase + SM_Q + (uint32_t)(lp & 1) * Q_BUF_BYTES;
-        }
-        const int s = item % NSTAGE, acc = item & 1;
-        if (!mbar_wait(bar(BAR_TEMPTY + acc), ((item >> 1) & 1) ^ 1, s_abort, 22, true)) { ok = false; break; }
-        if (!mbar_wait(bar(BAR_FULL + s), (item / NSTAGE) & 1, s_abort, 23, true)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t kbase = sbase + SM_K + s * STAGE_BYTES;
-        const uint32_t d0 = tmem + (uint32_t)(acc * 256);
-        if (p.pass == 2) {
+    // The whole warp walks the units; one elected lane issues.
+    int s = 0, slot = first;
+    uint32_t s_par = 0, u = 0;
+    bool ok = true;
+    const uint32_t idesc1 = FP8 ? instr_desc_f8(128, KT) : instr_desc(128, KT);
+    const uint32_t idesc2 = FP8 ? instr_desc_f8(KT, HR) : instr_desc(KT, HR);
+    for (int l = 0; ok && slot >= 0; ++l) {
+      // (shuffled so that the compiler knows them to be the same in all lanes: descriptors stay in uniform registers)
+      const int pass = __shfl_sync(0xffffffffu, __ldg(&work.runs[slot].pass), 0), ntiles = __shfl_sync(0xffffffffu, __ldg(&work.runs[slot].ntiles), 0),
+                next = __shfl_sync(0xffffffffu, __ldg(&work.runs[slot].next), 0);
+      prefetch_run(work.runs, next);
+      ok = __all_sync(0xffffffffu, mbar_wait(bar(S::QFULL + (l & 1)), (l >> 1) & 1, s_abort, 21, true));
+      const uint32_t qbase = sbase + (uint32_t)((l & 1) * S::Q_BUF);
+      for (int i = 0; ok && i < ntiles; ++i) {
+        ok = __all_sync(0xffffffffu, mbar_wait(bar(S::FULL + s), s_par, s_abort, 23, true));
+        const uint64_t kd = smem_desc(sbase + S::K + s * S::STAGE);
 #pragma unroll
-          for (int ks = 0; ks < 8; ++ks) {
-            const uint64_t ad = smem_desc(kbase + k_off(ks));
-            const uint64_t bd = smem_desc(qbase + (ks >> 2) * Q_BLOCK_BYTES + (ks & 3) * 32);
-            if (FP8) tc_mma_f8(d0, ad, bd, idesc2, ks > 0);
-            else     tc_mma(d0, ad, bd, idesc2, ks > 0);
-          }
-        } else {
-          for (int hf = 0; hf < nhalf; ++hf) {
+        for (int hf = 0; hf < HV; ++hf, ++u) {
+          const int acc = (int)(u & 3u);
+          ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(S::TEMPTY + acc), ((u >> 2) & 1u) ^ 1u, s_abort, 22, true));
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t d = tmem + (uint32_t)(acc * 128);
+          const uint64_t qd = smem_desc(qbase + (uint32_t)(hf * HR * 128));
+          if (elect_one()) {
+            // k-step ks: bf16 tiles are two 64-channel blocks, 8-bit tiles one block that both query terms meet
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
-              const uint64_t ad = smem_desc(qbase + (ks >> 2) * Q_BLOCK_BYTES + hf * (128 * 128) + (ks & 3) * 32);
-              const uint64_t bd = smem_desc(kbase + k_off(ks));
-              if (FP8) tc_mma_f8(d0 + (uint32_t)(hf * 128), ad, bd, idesc1, ks > 0);
-              else     tc_mma(d0 + (uint32_t)(hf * 128), ad, bd, idesc1, ks > 0);
+              const uint64_t ko = kd + (FP8 ? (ks & 3) * 2 : (ks >> 2) * (S::HALF >> 4) + (ks & 3) * 2);
+              const uint64_t qo = qd + (ks >> 2) * (S::Q_BLOCK >> 4) + (ks & 3) * 2;
+              const uint64_t ad = pass == 2 ? ko : qo, bd = pass == 2 ? qo : ko;
+              const uint32_t id = pass == 2 ? idesc2 : idesc1;
+              if (FP8) tc_mma_f8(d, ad, bd, id, ks > 0);
+              else     tc_mma(d, ad, bd, id, ks > 0);
+            }
+            tc_commit(bar(S::TFULL + acc));                      // accumulator ready for its group
+            if (hf == HV - 1) {
+              tc_commit(bar(S::EMPTY + s));                      // ring stage free once these MMAs have read it
+              if (i + 1 == ntiles) tc_commit(bar(S::QEMPTY + (l & 1)));
             }
           }
+          __syncwarp();
         }
-        tc_commit(bar(BAR_EMPTY + s));       // smem stage free once these MMAs have read it
-        tc_commit(bar(BAR_TFULL + acc));     // accumulator ready for the epilogue
-        if (w.last_in_phase()) tc_commit(bar(BAR_QEMPTY + (lp & 1)));   // last tile of the phase here
+        if (++s == S::NSTAGE) { s = 0; s_par ^= 1u; }
       }
-      if (!ok) {  // make sure nothing is still writing tensor memory before it is freed
-        tc_commit(bar(BAR_DRAIN));
-        mbar_wait(bar(BAR_DRAIN), 0, s_abort, 24, false);
-      }
+      slot = next;
     }
-  } else if (warp < 4) {
+    if (!ok) {  // make sure nothing is still writing tensor memory before it is freed
+      if (elect_one()) {
+        tc_commit(bar(S::DRAIN));
+        mbar_wait(bar(S::DRAIN), 0, s_abort, 24, false);
+      }
+      __syncwarp();
+    }
+  } else if (warp == 2) {
     // =============================== partial folding ==============================
-    // For every segment, in phase order: wait until all its epilogue sets have
-    // published, then fold the partials of this CTA's rows in a fixed order (the
-    // result does not depend on timing) and count the rows as done.
-    const int hw = warp - 2;
-    const int grid = (int)gridDim.x;
-    const int entries = 2 * grid;                                  // entry e: CTA e/2, set e%2
-    for (int ph = 0; ph < n_phases; ++ph) {
-      const TcPhase p = a.phases[ph];
-      if (p.pass != 1) continue;
-      if ((int)blockIdx.x + hw * grid >= NC) continue;             // no row of this segment is ours
-      if (!word_wait(a.published + p.seg, epoch * 2u * (uint32_t)p.ncontrib, s_abort, 41, lane, 256)) break;
-      const int first = p.g0 % grid;
-      for (int row = blockIdx.x + hw * grid; row < NC; row += 2 * grid) {
-        const float2* src = a.partials + (int64_t)p.seg * entries * NC + row;
-        auto fetch = [&](int e) {
-          int d = (e >> 1) - first;
-          if (d < 0) d += grid;
-          return (e < entries && d < p.ntiles) ? __ldcg(src + (int64_t)e * NC) : make_float2(-INFINITY, 0.f);
-        };
+    // For every pass-1 stage: the rows of its segments are dealt to the CTAs in runs of `per`; wait until a row's
+    // segment has been published by all its epilogue groups, fold the row's partials in a fixed order (the result does
+    // not depend on timing) and count the row as done.  Up to eight rows at a time, four or more lanes each, so that a
+    // stage costs one round trip for the partials and one for the fence (row after row it was 2 us each, 18 us of
+    // waiting in front of pass 2 for a group of four heads).
+    for (int si = 0; si < a.n_stages; ++si) {
+      const int a0 = __ldg(&a.stages[si].seg0), total = __ldg(&a.stages[si].nseg) * a.NC;
+      const int per = (total + (int)gridDim.x - 1) / (int)gridDim.x;
+      const int lo = (int)blockIdx.x * per, hi = min(total, lo + per);
+      int rpi = 1;                                                            // rows at a time
+      while (rpi < 8 && rpi < per) rpi <<= 1;
+      const int lpr = 32 / rpi, sub = lane / rpi;                             // lanes per row
+      bool ok = true;
+      for (int base = lo; ok && base < hi; base += rpi) {
+        const int s0 = base / a.NC, s1 = min(base + rpi, hi) - 1;
+        const int idx = min(base + lane % rpi, hi - 1);
+        const int sg = idx / a.NC, row = idx - sg * a.NC;
+        const int4 fo = __ldg(reinterpret_cast<const int4*>(work.folds + a0 + sg));        // slot0, nruns, rows, request
+        const bool valid = base + lane % rpi < hi && row < fo.z && fo.y > 0;
+        for (int q = s0; ok && q <= s1 / a.NC; ++q) {
+          const int4 fq = __ldg(reinterpret_cast<const int4*>(work.folds + a0 + q));
+          if (fq.y > 0) ok = word_wait(published + (a0 + q) * SYNC_STRIDE, (uint32_t)(GROUPS * fq.y), s_abort, 41, lane, 128);
+        }
+        if (!ok) break;
+        const int n = valid ? fo.y * ENTRIES : 0;
+        const int n_max = __reduce_max_sync(0xffffffffu, n);
+        const float2* src = a.partials + (int64_t)fo.x * ENTRIES * a.NC + row;
         float M = -INFINITY, L = 0.f;
-        for (int e0 = 0; e0 < entries; e0 += 320) {
-          float2 v[10];
+        for (int e0 = 0; e0 < n_max; e0 += 20 * lpr) {
+          float2 v[20];
 #pragma unroll
-          for (int i = 0; i < 10; ++i) v[i] = fetch(e0 + lane + 32 * i);      // all loads in flight
+          for (int i = 0; i < 20; ++i) {                                      // all loads in flight
+            const int e = e0 + sub + lpr * i;
+            v[i] = e < n ? __ldcg(src + (int64_t)e * a.NC) : make_float2(-INFINITY, 0.f);
+          }
 #pragma unroll
-          for (int i = 0; i < 10; ++i) {
+          for (int i = 0; i < 20; ++i) {
             if (v[i].y > 0.f) {
               const float Mn = fmaxf(M, v[i].x);
               L = L * ex2(M - Mn) + v[i].y * ex2(v[i].x - Mn);
@@ -586,8 +631,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             }
           }
         }
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {                         // butterfly: every lane ends with the same (M, L)
+        for (int o = rpi; o < 32; o <<= 1) {                       // butterfly: every lane of a row ends with the same (M, L)
           const float Mo = __shfl_xor_sync(0xffffffffu, M, o), Lo = __shfl_xor_sync(0xffffffffu, L, o);
           const bool lower = (lane & o) == 0;                      // fold in lane order so both partners agree bitwise
           const float Ma = lower ? M : Mo, La = lower ? L : Lo, Mb = lower ? Mo : M, Lb = lower ? Lo : L;
@@ -597,194 +641,255 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           if (Lb > 0.f) Ln += Lb * ex2(Mb - Mn);
           M = Mn; L = Ln;
         }
-        if (lane == 0) {
-          __stcg(a.offsets + (int64_t)p.seg * NC + row, M + log2f(L));
-          __threadfence();
-          atomicAdd(a.folded + p.seg, 1u);
+        if (valid && sub == 0) __stcg(a.offsets + (int64_t)(a0 + sg) * a.NC + row, M + log2f(L));
+        __syncwarp();
+        if (lane == 0) __threadfence();                            // cumulative: the warp's stores above
+        for (int q = s0; q <= s1 / a.NC; ++q) {
+          const int done = __popc(__ballot_sync(0xffffffffu, valid && sub == 0 && sg == q));
+          if (lane == 0 && done) atomicAdd(folded + (a0 + q) * SYNC_STRIDE, (uint32_t)done);
         }
       }
+      if (!ok) break;
+    }
+  } else if (warp == 3) {
+    // =============================== row offsets ==================================
+    // For every pass-2 run of the CTA: wait until the segment's rows have been folded (one poller per CTA: sixteen
+    // epilogue warps polling on 148 SMs keep the counter's L2 slice busy and the folds' own increments waiting), then
+    // hand the negated offsets to the epilogue in shared memory.
+    if (!a.lse) {
+      uint32_t last = 0;
+      if (lane == 0) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(last) : "l"(a.launch + 1) : "memory");
+      if (__shfl_sync(0xffffffffu, last, 0) == gridDim.x - 1u) {       // every CTA has read the number
+        uint32_t* other = a.counters + (size_t)(*s_set ^ 1u) * 2 * a.nseg * SYNC_STRIDE;
+        for (int i = lane; i < 2 * a.nseg; i += 32) other[(size_t)i * SYNC_STRIDE] = 0;
+        if (lane == 0) { a.launch[0] = *s_number + 1u; a.launch[1] = 0; }
+      }
+    }
+    float* s_off = reinterpret_cast<float*>(smem + S::OFFS);
+    int q = 0;
+    for (int slot = first; slot >= 0;) {
+      const TcRun r = load_run(work.runs, slot);
+      prefetch_run(work.runs, r.next);
+      slot = r.next;
+      if (r.pass != 2) continue;
+      const int buf = q & 1;
+      if (q >= 2 && !__all_sync(0xffffffffu, mbar_wait(bar(S::OEMPTY + buf), ((q >> 1) & 1) ^ 1, s_abort, 32, true))) break;
+      if (!a.lse && !word_wait(folded + r.seg * SYNC_STRIDE, (uint32_t)r.rows, s_abort, 33, lane, 128)) break;
+      const RowPlace p0 = row_place(a, r.chunk, 0);
+      const float* src = a.lse ? a.lse + ((int64_t)r.b * a.Hq + r.h * a.G + p0.g) * a.W + p0.t : a.offsets + (int64_t)r.seg * a.NC;
+      const float unit = a.lse ? -1.4426950408889634f : -1.0f;          // supplied: natural log -> log2 domain
+      float o[MAX_ROWS / 32];
+#pragma unroll
+      for (int i = 0; i < MAX_ROWS / 32; ++i) {
+        const int row = lane + 32 * i;
+        int at = row;
+        bool exists = row < r.rows;
+        if (!dense) {                                                   // max pooling, heads padded to Wp rows
+          const int hd = row / a.Wp, t = row - hd * a.Wp;
+          exists = exists && t < a.W;
+          if (a.lse) at = hd * a.W + t;
+        }
+        o[i] = exists ? __ldcg(src + at) * unit : -INFINITY;            // a padding row: 2^(x - inf) = 0
+      }
+#pragma unroll
+      for (int i = 0; i < MAX_ROWS / 32; ++i) s_off[buf * MAX_ROWS + lane + 32 * i] = o[i];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(S::OFULL + buf));
+      ++q;
     }
   } else {
     // =============================== epilogue ===================================
-    // 16 warps: set = which accumulator (tiles item%2 == set); within a set two warps share each
-    // TMEM lane quarter and split the accumulator's columns in halves (`sub`).
-    const int e = warp - 4;
-    const int set = e >> 3, sub = (e >> 2) & 1;
-    const int quarter = warp & 3;       // TMEM lanes 32*quarter .. +31 are this warp's
+    // Group g owns accumulator g (units u with u%4 == g); WIDE: always half g%2 of the chunk's rows.  Its four warps
+    // take a lane quarter each.
+    const int g = (warp - 4) >> 2;
+    const int quarter = warp & 3;                              // TMEM lanes 32*quarter .. +31 are this warp's
     const int lt = quarter * 32 + lane;                        // TMEM lane of this thread, 0..127
-    const int st = (e & 7) * 32 + lane;                        // thread of the set, 0..255
-    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(set * 256);
-    float scale = a.scale_log2;             // log2(e)/sqrt(d) times the phase's accumulator factor (FP8 keys: per kv head)
-    f32x2 scale2 = pk(scale, scale);
-    float* negoff = s_negoff + set * 256;
-    const int nhalf = (NC > 128) ? 2 : 1;
-    ItemWalk w(a, n_phases, total_items);
-    int item = 0, cur_ph = -1, mine = 0;    // `mine`: tiles this set has taken
-    bool dead = false;                      // a wait expired: keep the barrier sequence, skip the work
-    // pass-1 state of row sub*128 + lt: sum of 2^(x - mref) over the keys seen so far.  mref is the
-    // maximum of the first 32 keys the row met; later blocks do not track the maximum (their terms may
-    // exceed 1, fp32 has the range), unless a sum overflows, in which case the tile is redone with it.
-    float mref = -INFINITY, l = 0.f;
-    bool first_tile = true;                 // this set has not yet taken a tile of the current pass-1 phase
-    for (; w.valid(); w.next(), ++item) {
-      const TcPhase p = w.phase();
-      if (w.ph != cur_ph) {
-        cur_ph = w.ph;
-        if (FP8) {
-          scale = a.scale_log2 * p.kscale;
-          scale2 = pk(scale, scale);
-        }
-        if (p.pass == 1) {
-          mref = -INFINITY;
-          l = 0.f;
-          first_tile = true;
-        } else {
-          // the segment's offsets: wait until every row has been folded, then stage -offset for this set
-          if (!dead && !a.lse) dead = !word_wait(a.folded + p.seg, epoch * (uint32_t)NC, s_abort, 33, lane, 256);
-          bar_sync(2 + set, 256);                                 // the set is done with the previous offsets
-          if (st < NC) {
-            float off = INFINITY;                                 // a padding row: 2^(x - inf) = 0
-            if (st >= p.rows) {
-            } else if (a.lse) {                                   // supplied: natural log -> log2 domain
-              const int r = p.chunk * NC + st;                    // row within the kv head: query head r / W, window row r % W
-              off = __ldg(a.lse + ((int64_t)p.b * a.Hq + p.h * a.G + r / a.W) * a.W + r % a.W) * 1.4426950408889634f;
-            } else {
-              off = __ldcg(a.offsets + (int64_t)p.seg * NC + st);
-            }
-            negoff[st] = dead ? 0.f : -off;
-          }
-          bar_sync(2 + set, 256);
-        }
-      }
-      if ((item & 1) == set) {
-        if (!dead) {
-          const bool ok = mbar_wait(bar(BAR_TFULL + set), mine & 1, s_abort, 31, true);
-          dead = !__all_sync(0xffffffffu, ok);
-        }
+    const int half = WIDE ? (g & 1) : 0;
+    const uint32_t acc_addr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(g * 128);
+    const int nblk = HR >> 5;                                  // 32-column blocks of a pass-2 accumulator
+    uint32_t u0 = 0;                                           // unit number at which the current run starts
+    uint32_t mine = 0;                                         // units this group has taken
+    int q = 0;                                                 // pass-2 runs so far
+    // max pooling: after which 32-column blocks of an accumulator a query head ends
+    int head_ends = 1 << (nblk - 1);
+    if (PER_Q && a.Wp <= 128)
+      for (int i = 1; i < nblk; ++i) head_ends |= (32 * i) % a.Wp == 0 ? 1 << (i - 1) : 0;
+    bool dead = false;                                         // a wait expired: keep the barrier sequence, skip the work
+    auto release = [&]() {                                     // this warp has read its part of the accumulator
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(S::TEMPTY + g));
+    };
+    for (int slot = first; slot >= 0;) {
+      const TcRun* rp = work.runs + slot;
+      const int4 ra = __ldg(reinterpret_cast<const int4*>(rp)), rb = __ldg(reinterpret_cast<const int4*>(rp) + 1),
+                 rc = __ldg(reinterpret_cast<const int4*>(rp) + 2);
+      const int run_slot = __ldg(&rp->slot);
+      const int tile0 = ra.x, ntiles = ra.y, pass = ra.z, seg = ra.w, h = rb.y, chunk = rb.z, next = rb.w;
+      const int T = rc.x, t_off = rc.y, rows = rc.w;
+      prefetch_run(work.runs, next);
+      const float scale = FP8 ? a.scale_log2 * __ldg(&rp->kscale) : a.scale_log2;   // log2(e)/sqrt(d) times the accumulator factor
+      const f32x2 scale2 = pk(scale, scale);
+      const int nu = ntiles * HV;
+      int k = (int)((uint32_t)(g - (int)u0) & 3u);             // first unit of the run that is this group's
+      uint32_t bufs[2][16];
+      auto wait_unit = [&]() {
+        if (!dead) dead = !__all_sync(0xffffffffu, mbar_wait(bar(S::TFULL + g), mine & 1u, s_abort, 31, true));
         ++mine;
-        if (!dead) {
-          tc_fence_after();
-          const int tile = w.g - p.g0;
-          uint32_t cur[32];
-          auto release = [&]() {                                   // this warp has read its part of the accumulator
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(BAR_TEMPTY + set));
-          };
-          if (p.pass == 1) {
-            // ---- pass 1: sum of 2^(x - mref) of this thread's row over the tile's 128 keys ----
-            // Fast walk: every key of the tile is visible to every row; it does not track the maximum.
-            // Careful walk (tiles that reach into the window, or after a sum overflowed in the fast
-            // walk): per-row masks, block maxima, MUFU only.
-            if (sub < nhalf) {
-              const uint32_t addr = lane_base + (uint32_t)(sub * 128);
-              const float keep_m = mref, keep_l = l;
-              bool careful = tile * KT + KT - 1 > p.T;
-              if (!careful) {
-#pragma unroll 1
-                for (int blk = 0; blk < 4; ++blk) {
-                  tc_ld32_issue(addr + (uint32_t)(blk * 32), cur);
-                  tc_ld_wait(cur);
-                  if (first_tile && blk == 0) {                    // first block of the row: its maximum is the reference
-                    float c0 = fmaxf(__uint_as_float(cur[0]), __uint_as_float(cur[1]));
-                    float c1 = fmaxf(__uint_as_float(cur[2]), __uint_as_float(cur[3]));
+        if (!dead) tc_fence_after();
+        return !dead;
+      };
+      if (pass == 1) {
+        // ---- pass 1: sum of 2^(x - mref) of row half*HR + lt over the keys of the group's tiles of the run.  mref is
+        // the row's first logit; the maximum is not tracked (terms may exceed 1, fp32 has the range) unless a sum
+        // overflows, in which case the tile is redone with it.  Which tiles are added together follows from the run
+        // alone, so the result does not depend on what else the launch works on.
+        const int row = half * HR + lt;
+        const bool busy = half * HR + quarter * 32 < rows && quarter * 32 < HR;     // the warp has rows of the chunk
+        const int entry = (k / HV) & (ENTRIES - 1);
+        float mref = -INFINITY, l = 0.f;
+        bool begun = false;
+        for (; k < nu; k += GROUPS) {
+          if (!wait_unit()) continue;
+          if (!busy) { release(); continue; }
+          const int j_tile = (tile0 + k / HV) * KT;
+          const float keep_m = mref, keep_l = l;
+          // every key visible to every row: the fast walk.  It stops before the tile's last 16 keys to look for an
+          // overflow while the accumulator is still there.
+          bool careful = j_tile + KT - 1 > T, tail_careful = false;
+          if (!careful) {
+            tc_ld_lane(acc_addr, bufs[0]);
 #pragma unroll
-                    for (int i = 4; i < 32; i += 4) {
-                      c0 = fmaxf(c0, fmaxf(__uint_as_float(cur[i]), __uint_as_float(cur[i + 1])));
-                      c1 = fmaxf(c1, fmaxf(__uint_as_float(cur[i + 2]), __uint_as_float(cur[i + 3])));
-                    }
-                    mref = fmaxf(c0, c1) * scale;
-                  }
-                  const f32x2 nm2 = pk(-mref, -mref);
-                  l += exp_sum32(cur, scale2, [&](int) { return nm2; });
-                }
-                // a term beyond fp32 range (a logit 127 above the reference): redo the tile carefully
-                careful = __any_sync(0xffffffffu, !(l < INFINITY));
-                if (careful) { mref = keep_m; l = keep_l; }
-              }
-              if (careful) {
-                const int row = sub * 128 + lt;
-                const int lastkey = p.T + (p.chunk * NC + row) % a.W;       // last key this row sees
-#pragma unroll 1
-                for (int blk = 0; blk < 4; ++blk) {
-                  tc_ld32_issue(addr + (uint32_t)(blk * 32), cur);
-                  tc_ld_wait(cur);
-                  const int j0 = tile * KT + blk * 32;
-                  if (j0 <= lastkey) {
-                    float c = -INFINITY;
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) c = fmaxf(c, (j0 + i <= lastkey) ? __uint_as_float(cur[i]) : -INFINITY);
-                    const float mn = fmaxf(mref, c * scale);
-                    float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-                    for (int i = 0; i < 32; i += 2) {
-                      s0 += (j0 + i <= lastkey) ? ex2(fmaf(__uint_as_float(cur[i]), scale, -mn)) : 0.f;
-                      s1 += (j0 + i + 1 <= lastkey) ? ex2(fmaf(__uint_as_float(cur[i + 1]), scale, -mn)) : 0.f;
-                    }
-                    l = fmaf(l, ex2(mref - mn), s0 + s1);
-                    mref = mn;
-                  }
-                }
-              }
-              if (l > 0x1p60f) { l *= 0x1p-60f; mref += 60.f; }     // exact: keeps the running sum far from overflow
-            }
-            release();
-            first_tile = false;
-          } else {
-            // ---- pass 2: this thread's key, exp2(x - offset[row]) summed over its half of the chunk's rows ----
-            const int half_cols = NC >> 1, nblk = half_cols >> 5;
-            const uint32_t addr = lane_base + (uint32_t)(sub * half_cols);
-            const float* no_base = negoff + sub * half_cols;
-            float sums[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-            for (int blk = 0; blk < nblk; ++blk) {
-              tc_ld32_issue(addr + (uint32_t)(blk * 32), cur);
+            for (int j = 0; j < 8; ++j) {
+              uint32_t (&cur)[16] = bufs[j & 1];
               tc_ld_wait(cur);
-              if (blk + 1 == nblk) release();
-              const float4* no = reinterpret_cast<const float4*>(no_base + blk * 32);   // two column pairs per load
-              const float bs = exp_sum32(cur, scale2, [&](int pi) {
-                const float4 v = no[pi >> 1];
-                return (pi & 1) ? pk(v.z, v.w) : pk(v.x, v.y);
-              });
-              if (PER_Q) {                                         // W is a multiple of 32: a block never straddles heads
-                const int slot = (blk * 32) / a.W;
+              if (j < 7) tc_ld_lane(acc_addr + (uint32_t)(16 * (j + 1)), bufs[(j + 1) & 1]);
+              if (j == 0 && !begun) mref = __uint_as_float(cur[0]) * scale;
+              if (j == 7) {
+                careful = __any_sync(0xffffffffu, !(l < INFINITY));   // a term beyond fp32 range (a logit 127 above the reference)
+                if (careful) break;
+                release();
+              }
+              const f32x2 nm2 = pk(-mref, -mref);
+              f32x2 am = pk(0.f, 0.f), ap = pk(0.f, 0.f);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) sums[q] += (q == slot) ? bs : 0.f;
-              } else {
-                sums[0] += bs;
+              for (int i = 0; i < 8; ++i) {
+                const f32x2 x = fma2(pku(cur[2 * i], cur[2 * i + 1]), scale2, nm2);
+                if (pair_is_poly(i + 8 * (j & 1))) ap = add2(ex2_pair_poly(x), ap);
+                else                               am = add2(ex2_pair_mufu(x), am);
+              }
+              const float s = hsum(add2(am, ap));
+              if (j == 7 && __any_sync(0xffffffffu, !(l + s < INFINITY))) tail_careful = true;   // redone below from the registers
+              else l += s;
+            }
+            if (careful) { mref = keep_m; l = keep_l; }
+          }
+          begun = true;
+          if (careful || tail_careful) {
+            // running maximum over 16-key blocks, per-row visibility, MUFU only
+            const int lastkey = T + row_place(a, chunk, row).t;       // last key this row sees
+#pragma unroll 1
+            for (int j = careful ? 0 : 7; j < 8; ++j) {
+              uint32_t (&cur)[16] = bufs[1];
+              if (careful) {
+                tc_ld_lane(acc_addr + (uint32_t)(16 * j), cur);
+                tc_ld_wait(cur);
+              }
+              const int j0 = j_tile + 16 * j;
+              if (j0 <= lastkey) {
+                float c[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                  c[i] = fmaxf((j0 + i <= lastkey) ? __uint_as_float(cur[i]) : -INFINITY, (j0 + i + 8 <= lastkey) ? __uint_as_float(cur[i + 8]) : -INFINITY);
+                const float mn = fmaxf(mref, scale * fmaxf(fmaxf(fmaxf(c[0], c[1]), fmaxf(c[2], c[3])), fmaxf(fmaxf(c[4], c[5]), fmaxf(c[6], c[7]))));
+                float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+                for (int i = 0; i < 16; i += 2) {
+                  s0 += (j0 + i <= lastkey) ? ex2(fmaf(__uint_as_float(cur[i]), scale, -mn)) : 0.f;
+                  s1 += (j0 + i + 1 <= lastkey) ? ex2(fmaf(__uint_as_float(cur[i + 1]), scale, -mn)) : 0.f;
+                }
+                l = fmaf(l, ex2(mref - mn), s0 + s1);
+                mref = mn;
               }
             }
-            const int j = tile * KT + lt;
-            if (j < p.T) {
-              if (PER_Q) {
-                // heads of this half: half_cols / W of them, or a part of one head when W > half_cols
-                const int col0 = p.chunk * NC + sub * half_cols;
-                if (a.W > half_cols) {
-                  a.u[(int64_t)((p.h * a.G + col0 / a.W) * 2 + sub) * a.sum_T + p.t_off + j] = sums[0];
-                } else {
-                  const int nslot = half_cols / a.W;
+            if (careful) release();
+          }
+          if (l > 0x1p60f) { l *= 0x1p-60f; mref += 60.f; }     // exact: keeps the running sum far from overflow
+        }
+        // ---- end of the run: the group publishes (reference, sum) per row ----
+        if (lt < HR) __stcg(a.partials + ((int64_t)run_slot * ENTRIES + entry) * a.NC + row, make_float2(mref, dead ? 0.f : l));
+        bar_sync(1 + g, 128);
+        if (quarter == 0 && lane == 0) {   // the barrier orders the group's stores before this thread's fence: the release is cumulative
+          __threadfence();
+          atomicAdd(published + seg * SYNC_STRIDE, 1u);
+        }
+      } else {
+        // ---- pass 2: for every key, exp2(x - offset[row]) summed over the half's rows.  In the 16x256b shape a
+        // thread meets rows 8i + 2(lane%4) + {0, 1}: their offsets stay in registers for the run.
+        if (!dead) dead = !__all_sync(0xffffffffu, mbar_wait(bar(S::OFULL + (q & 1)), (q >> 1) & 1, s_abort, 34, true));
+        f32x2 noff[16];
+        {
+          const float2* src = reinterpret_cast<const float2*>(smem + S::OFFS) + (q & 1) * (MAX_ROWS / 2) + half * (HR >> 1) + (lane & 3);
 #pragma unroll
-                  for (int q = 0; q < 4; ++q)
-                    if (q < nslot) a.u[(int64_t)((p.h * a.G + col0 / a.W + q) * a.u_parts) * a.sum_T + p.t_off + j] = sums[q];
+          for (int i = 0; i < 16; ++i) {                        // rows past the half: read, not used
+            const float2 v = 8 * i < HR ? src[4 * i] : make_float2(0.f, 0.f);
+            noff[i] = pk(v.x, v.y);
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(S::OEMPTY + (q & 1)));
+          ++q;
+        }
+        for (; k < nu; k += GROUPS) {
+          if (!wait_unit()) continue;
+          const int j = (tile0 + k / HV) * KT + quarter * 32 + (lane >> 2) + 8 * (lane & 1) + 16 * ((lane >> 1) & 1);
+          // max pooling: the query head whose rows come first in this accumulator, and which of its partial sums this is
+          int head = chunk * a.m + (a.Wp <= 128 ? half * HR / a.Wp : 0), part = a.Wp <= 128 ? 0 : half;
+          if (PER_Q && a.pieces > 1) { head = chunk / a.pieces; part = (chunk % a.pieces) * 2 + half; }
+          // sums of four keys (lanes lane/4, +8, +16, +24 of the quarter) over the thread's rows
+          f32x2 ac[4] = {pk(0.f, 0.f), pk(0.f, 0.f), pk(0.f, 0.f), pk(0.f, 0.f)};
+          tc_ld_quad(acc_addr, bufs[0]);
+#pragma unroll
+          for (int blk = 0; blk < 4; ++blk) {
+            if (blk < nblk) {
+#pragma unroll
+              for (int up = 0; up < 2; ++up) {                  // lanes 0-15, 16-31 of the quarter
+                uint32_t (&cur)[16] = bufs[up];
+                tc_ld_wait(cur);
+                if (up == 0) tc_ld_quad(acc_addr + (uint32_t)(32 * blk) + (16u << 16), bufs[1]);
+                else if (blk + 1 < nblk) tc_ld_quad(acc_addr + (uint32_t)(32 * (blk + 1)), bufs[0]);
+                else release();
+                f32x2 ap[2] = {pk(0.f, 0.f), pk(0.f, 0.f)};
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                  const f32x2 x = fma2(pku(cur[2 * i], cur[2 * i + 1]), scale2, noff[4 * blk + (i >> 1)]);
+                  if (pair_is_poly(i + 8 * up)) ap[i & 1] = add2(ex2_pair_poly(x), ap[i & 1]);
+                  else ac[2 * up + (i & 1)] = add2(ex2_pair_mufu(x), ac[2 * up + (i & 1)]);
                 }
-              } else {
-                a.u[(int64_t)(p.h * a.u_rows_per_kv + p.chunk * 2 + sub) * a.sum_T + p.t_off + j] = sums[0];
+                ac[2 * up] = add2(ap[0], ac[2 * up]);
+                ac[2 * up + 1] = add2(ap[1], ac[2 * up + 1]);
+              }
+              if (PER_Q ? (head_ends >> blk) & 1 : blk + 1 == nblk) {
+                // reduce over the four lanes that share keys: each ends with one key
+                const float k0 = hsum(ac[0]), k1 = hsum(ac[1]), k2 = hsum(ac[2]), k3 = hsum(ac[3]);
+                const bool odd = lane & 1, upper = lane & 2;
+                const float q0 = (odd ? k1 : k0) + __shfl_xor_sync(0xffffffffu, odd ? k0 : k1, 1);
+                const float q1 = (odd ? k3 : k2) + __shfl_xor_sync(0xffffffffu, odd ? k2 : k3, 1);
+                const float sum = (upper ? q1 : q0) + __shfl_xor_sync(0xffffffffu, upper ? q0 : q1, 2);
+                if (PER_Q) {
+#pragma unroll
+                  for (int q = 0; q < 4; ++q) ac[q] = pk(0.f, 0.f);
+                  if (j < T && head < a.G) a.u[((int64_t)(h * a.G + head) * a.u_parts + part) * a.sum_T + t_off + j] = sum;
+                  ++head;
+                } else {
+                  if (j < T) a.u[(int64_t)(h * a.u_rows_per_kv + chunk * HV + half) * a.sum_T + t_off + j] = sum;
+                }
               }
             }
           }
         }
       }
-      if (w.last_in_phase() && p.pass == 1) {
-        // ---- end of a pass-1 phase in this CTA: each set publishes its own (reference, sum) per row ----
-        float2* out = a.partials + (((int64_t)p.seg * gridDim.x + blockIdx.x) * 2 + set) * NC;
-        const int row = sub * 128 + lt;
-        if (sub < nhalf && row < NC) __stcg(out + row, make_float2(mref, dead ? 0.f : l));
-        bar_sync(2 + set, 256);
-        if (st == 0) {                 // the barrier orders the set's stores before this thread's fence: the release is cumulative
-          __threadfence();
-          atomicAdd(a.published + p.seg, 1u);
-        }
-      }
+      u0 += (uint32_t)nu;
+      slot = next;
     }
   }
 
@@ -796,20 +901,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   }
   if (threadIdx.x == 0 && *s_abort) atomicCAS(a.err, 0, *s_abort);
-  if (threadIdx.x == 0 && !a.lse) {
-    // the last CTA to leave closes the launch: next launch number, or a fresh start before the counters wrap
-    __threadfence();
-    if (atomicAdd(a.epoch_word + 1, 1u) == gridDim.x - 1u) {
-      a.epoch_word[1] = 0;
-      if (epoch >= a.epoch_limit) {
-        for (int i = 0; i < 2 * a.nseg; ++i) a.published[i] = 0;      // published and folded are contiguous
-        a.epoch_word[0] = 0;
-      } else {
-        a.epoch_word[0] = epoch;
-      }
-      __threadfence();
-    }
-  }
 }
 
 // One warp runs one of the kernel's two kinds of bounded wait on something that never happens (a barrier
@@ -833,54 +924,139 @@ __global__ void bounded_wait_selftest_kernel(int which, unsigned long long limit
   if (threadIdx.x == 0 && !ok && *abort_flag) atomicCAS(err, 0, *abort_flag);
 }
 
-// Device-side controller: the phase list of the next launch without the phases of finished requests.
-// One block.  The requests' flags are read once (a record may be changing under a statistic kernel of the
-// previous layer that is still running: whatever is read here holds for the whole launch), the live
-// phases are copied in order with their first work item recomputed, and the header {phases, items} is
-// written.  Segments that are left out of a two-pass launch have their publish counters advanced as if
-// they had been scored, so that a later launch that scores them again (a new prompt) finds them where
-// its launch number expects them.
-__global__ void __launch_bounds__(256) live_phase_list_kernel(const TcPhase* __restrict__ all, int n_all, const asl_stat* __restrict__ latch,
-                                                             int cur, int batch, int two_pass, int NC, TcPhase* __restrict__ live,
-                                                             int32_t* __restrict__ hdr, uint32_t* __restrict__ published,
-                                                             uint32_t* __restrict__ folded) {
+// Device-side controller: the work list of the next launch without the runs of finished requests; hdr[0] = 0 where
+// there are none (the launch then takes the plan's list).  One block.  The requests' flags are read once (a record may be
+// changing under a statistic kernel of the previous layer that is still running: whatever is read here holds for the
+// whole launch).  Runs stay whole, so that the sums of the requests still observed come out bit for bit as in a launch
+// that skips nothing; groups that have shrunk are merged until they hold about `most` tiles, and a merged group's runs
+// are dealt to the CTAs by where their middle lies among its tiles.
+__device__ unsigned long long block_scan_1024(unsigned long long v, unsigned long long* warp_tot, unsigned long long& total) {   // exclusive
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned long long incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  __syncthreads();
+  if (lane == 31) warp_tot[wid] = incl;
+  __syncthreads();
+  unsigned long long before = 0;
+  total = 0;
+  for (int w = 0; w < 32; ++w) { total += warp_tot[w]; if (w < wid) before += warp_tot[w]; }
+  return before + incl - v;
+}
+__global__ void __launch_bounds__(1024) live_list_kernel(const TcRun* __restrict__ all, int n1, int n2, const TcFold* __restrict__ all_folds, int nseg,
+                                                         int n_groups, int most, const asl_stat* __restrict__ latch, int cur, int batch, int grid,
+                                                         int32_t* __restrict__ hdr, TcRun* __restrict__ runs, int32_t* __restrict__ first,
+                                                         TcFold* __restrict__ folds, int32_t* __restrict__ scratch) {
   __shared__ uint32_t fin[ASL_SKIP_MAX_BATCH / 32];
-  __shared__ int w_items[8], w_cnt[8];
-  __shared__ int base_items, base_cnt;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  for (int b0 = 0; b0 < batch; b0 += 256) {
+  __shared__ unsigned long long warp_tot[32];
+  const int tid = threadIdx.x, lane = tid & 31, n = n1 + n2;
+  int any = 0;
+  for (int b0 = 0; b0 < batch; b0 += 1024) {
     const int b = b0 + tid;
     const uint32_t word = __ballot_sync(0xffffffffu, b < batch && asl_finished(latch + b, cur));
     if (lane == 0) fin[b >> 5] = word;
+    any |= word != 0u;
   }
-  if (tid == 0) { base_items = 0; base_cnt = 0; }
+  any = __syncthreads_or(any);
+  if (tid == 0) hdr[0] = any;
+  if (!any) return;
+  auto live = [&](int b) { return ((fin[b >> 5] >> (b & 31)) & 1u) == 0u; };
+  int32_t* pos = scratch;                        // [n] live tiles of the pass before the run
+  int32_t* num = pos + n;                        // [n] the pass's live runs in order, and where they go: merged group * grid + CTA
+  int32_t* key = num + n;
+  int32_t* group_tiles = key + n;                // [groups]
+  int32_t* merged = group_tiles + n_groups;      // [groups]
+  int32_t* tiles = merged + n_groups;            // [2][groups] live tiles of a merged group, and before it
+  int32_t* base = tiles + 2 * n_groups;
+  int32_t* head = base + 2 * n_groups;           // [groups + 1 stages][2 passes][grid] first and last run (-1: none)
+  const int n_lists = 2 * (n_groups + 1) * grid;
+  int32_t* tail = head + n_lists;
+  for (int i = tid; i < n_groups; i += 1024) group_tiles[i] = 0;
+  for (int i = tid; i < 2 * n_groups; i += 1024) { tiles[i] = 0; base[i] = 0x7fffffff; }
+  for (int i = tid; i < 2 * n_lists; i += 1024) head[i] = -1;
+  for (int s = tid; s < nseg; s += 1024) {
+    TcFold f = all_folds[s];
+    if (!live(f.b)) f.nruns = 0;
+    folds[s] = f;
+  }
   __syncthreads();
-  for (int i0 = 0; i0 < n_all; i0 += 256) {
-    const int i = i0 + tid;
-    TcPhase ph{};
-    bool is_live = false;
-    if (i < n_all) {
-      ph = all[i];
-      is_live = ((fin[ph.b >> 5] >> (ph.b & 31)) & 1u) == 0u;
-      if (!is_live && two_pass && ph.pass == 1) { published[ph.seg] += 2u * (uint32_t)ph.ncontrib; folded[ph.seg] += (uint32_t)NC; }
+  for (int i = n1 + tid; i < n; i += 1024)
+    if (live(all[i].b)) atomicAdd(&group_tiles[all[i].group], all[i].ntiles);
+  __syncthreads();
+  if (tid == 0) {
+    int held = 0, id = 0;
+    for (int g = 0; g < n_groups; ++g) {
+      if (held > 0 && held + group_tiles[g] > most) { ++id; held = 0; }
+      held += group_tiles[g];
+      merged[g] = id;
     }
-    int items = is_live ? ph.ntiles : 0, cnt = is_live ? 1 : 0;
-    int inc_items = items, inc_cnt = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int a = __shfl_up_sync(0xffffffffu, inc_items, o), c2 = __shfl_up_sync(0xffffffffu, inc_cnt, o);
-      if (lane >= o) { inc_items += a; inc_cnt += c2; }
-    }
-    if (lane == 31) { w_items[wid] = inc_items; w_cnt[wid] = inc_cnt; }
-    __syncthreads();
-    int off_items = base_items + inc_items - items, off_cnt = base_cnt + inc_cnt - cnt;
-    for (int w2 = 0; w2 < wid; ++w2) { off_items += w_items[w2]; off_cnt += w_cnt[w2]; }
-    if (is_live) { ph.g0 = off_items; live[off_cnt] = ph; }
-    __syncthreads();
-    if (tid == 255) { base_items = off_items + items; base_cnt = off_cnt + cnt; }
-    __syncthreads();
   }
-  if (tid == 0) { hdr[0] = base_cnt; hdr[1] = base_items; }
+  __syncthreads();
+  int n_live[2];
+  for (int p = 0; p < 2; ++p) {
+    const int at = p ? n1 : 0, np = p ? n2 : n1;
+    unsigned long long sum = 0;                  // runs << 32 | tiles so far
+    for (int i0 = 0; i0 < np; i0 += 1024) {
+      const int i = i0 + tid;
+      const bool mine = i < np && live(all[at + i].b);
+      const int nt = mine ? all[at + i].ntiles : 0;
+      unsigned long long total;
+      const unsigned long long here = sum + block_scan_1024(mine ? (1ull << 32) + (unsigned)nt : 0ull, warp_tot, total);
+      if (mine) {
+        const int mg = merged[all[at + i].group];
+        pos[at + i] = (int)(uint32_t)here;
+        num[at + (int)(here >> 32)] = at + i;
+        atomicAdd(&tiles[p * n_groups + mg], nt);
+        atomicMin(&base[p * n_groups + mg], (int)(uint32_t)here);
+      }
+      sum += total;
+    }
+    n_live[p] = (int)(sum >> 32);
+  }
+  __syncthreads();
+  for (int p = 0; p < 2; ++p)
+    for (int r = tid; r < n_live[p]; r += 1024) {
+      const int at = (p ? n1 : 0) + r, i = num[at], mg = merged[all[i].group];
+      const int64_t middle = 2 * (pos[i] - base[p * n_groups + mg]) + all[i].ntiles;
+      key[at] = mg * grid + (int)(middle * grid / (2 * tiles[p * n_groups + mg]));
+    }
+  __syncthreads();
+  for (int p = 0; p < 2; ++p)
+    for (int r = tid; r < n_live[p]; r += 1024) {
+      const int at = (p ? n1 : 0) + r, i = num[at], k = key[at];
+      TcRun run = all[i];
+      const bool last = r + 1 == n_live[p] || key[at + 1] != k;
+      run.next = last ? -1 : num[at + 1];
+      runs[i] = run;
+      const int list = ((k / grid + p) * 2 + p) * grid + k % grid;      // pass 2 of a group comes a stage after its pass 1
+      if (r == 0 || key[at - 1] != k) head[list] = i;
+      if (last) tail[list] = i;
+    }
+  __syncthreads();
+  for (int i = tid; i < n_lists; i += 1024) {                  // chain a CTA's lists
+    int j = i;
+    if (i < grid) {
+      while (j < n_lists && head[j] < 0) j += grid;
+      first[i] = j < n_lists ? head[j] : -1;
+    }
+    if (tail[i] < 0) continue;
+    for (j = i + grid; j < n_lists && head[j] < 0;) j += grid;
+    if (j < n_lists) runs[tail[i]].next = head[j];
+  }
+}
+
+// Row offsets (log2 of the softmax denominators) of the latest two-pass call as natural-log denominators [B][H_q][W]
+__global__ void __launch_bounds__(256) offsets_to_lse_kernel(const float* __restrict__ offsets, float* __restrict__ lse, int n, int W, int G, int m,
+                                                             int Wp, int pieces, int nchunk, int NC) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  const int t = i % W, hq = i / W, g = hq % G, bh = hq / G;                  // bh: request x kv head
+  const int chunk = pieces > 1 ? g * pieces + t / MAX_ROWS : g / m;
+  const int row = pieces > 1 ? t % MAX_ROWS : (g % m) * Wp + t;
+  lse[i] = __ldcg(offsets + ((int64_t)bh * nchunk + chunk) * NC + row) * 0.6931471805599453f;
 }
 
 // FP8 keys: the bf16 window queries, scaled by Q8_SCALE, as two E4M3 terms hi + lo (hi = nearest code,
@@ -930,120 +1106,252 @@ bool make_map(CUtensorMap* tm, CUtensorMapDataType dtype, const void* base, int 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+struct ScoreKernel {
+  void (*fn)(CUtensorMap, CUtensorMap, TcArgs);
+  int smem;
+};
+template <int I>
+constexpr ScoreKernel score_instance() { return {score_tc_kernel<(I & 8) != 0, (I & 4) != 0, (I & 2) != 0, (I & 1) != 0>, Smem<(I & 4) != 0, (I & 2) != 0>::BYTES}; }
+const ScoreKernel& score_kernel(int i) {       // bits: max pooling, FP8 keys, wide, full halves
+  static const ScoreKernel k[16] = {score_instance<0>(), score_instance<1>(), score_instance<2>(), score_instance<3>(),
+                                    score_instance<4>(), score_instance<5>(), score_instance<6>(), score_instance<7>(),
+                                    score_instance<8>(), score_instance<9>(), score_instance<10>(), score_instance<11>(),
+                                    score_instance<12>(), score_instance<13>(), score_instance<14>(), score_instance<15>()};
+  return k[i];
+}
+int score_kernel_of(const asl_params& p, const AslTcPlan& tp) {
+  return (p.pool_mode == ASL_POOL_MAX ? 8 : 0) + (p.k_dtype == ASL_K_FP8_E4M3 ? 4 : 0) + (tp.wide ? 2 : 0) + (tp.HR == 128 ? 1 : 0);
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------- host side
+namespace {
+
+// FP8 keys are taken for the windows that asl.h promises: chunks of whole heads in multiples of 64 rows
+bool fp8_shape(const asl_params& p) {
+  const int W = p.window, R = p.n_q_heads / p.n_kv_heads * W;
+  if (W % 32 || W > MAX_ROWS) return false;
+  for (int m = MAX_ROWS / W; m >= 1; --m) {
+    const int nc = m * W;
+    if (p.pool_mode == ASL_POOL_MAX ? R % nc == 0 : nc % 64 == 0) return nc % 64 == 0;
+  }
+  return false;
+}
+
+int round_up(int x, int to) { return (x + to - 1) / to * to; }
+int div_up(int x, int by) { return (x + by - 1) / by; }
+
+// How the G*W rows of a kv head are cut into chunks of at most 256 buffer rows in halves of HR.  Average pooling adds
+// all rows of a kv head, so heads follow one another without gaps; max pooling keeps column sums per query head, so
+// heads start on 32-row blocks and no head straddles the halves (unless it needs both).  As few chunks as possible
+// (each streams K again), heads spread evenly over them.
+void plan_chunks(const asl_params& p, AslTcPlan& tp) {
+  const int W = p.window, G = p.n_q_heads / p.n_kv_heads;
+  const bool per_q = p.pool_mode == ASL_POOL_MAX;
+  tp.pieces = 1;
+  if (W > MAX_ROWS) {
+    tp.pieces = div_up(W, MAX_ROWS);
+    tp.Wp = MAX_ROWS; tp.m = 1; tp.nchunk = G * tp.pieces; tp.wide = true; tp.HR = 128;
+  } else if (!per_q) {
+    tp.Wp = W;
+    tp.nchunk = div_up(G, MAX_ROWS / W);
+    tp.m = div_up(G, tp.nchunk);
+    tp.wide = tp.m * W > 128;
+    tp.HR = round_up(tp.wide ? div_up(tp.m * W, 2) : tp.m * W, 32);
+  } else if (W > 128) {
+    tp.Wp = round_up(W, 64); tp.m = 1; tp.nchunk = G; tp.wide = true; tp.HR = tp.Wp / 2;
+  } else {
+    tp.Wp = round_up(W, 32);
+    const int in_half = 128 / tp.Wp;
+    tp.wide = G > in_half;
+    tp.nchunk = div_up(G, tp.wide ? 2 * in_half : in_half);
+    tp.m = div_up(G, tp.nchunk);
+    if (tp.wide) tp.m = round_up(tp.m, 2);
+    tp.HR = tp.m * tp.Wp / (tp.wide ? 2 : 1);
+  }
+  tp.NC = tp.HR * (tp.wide ? 2 : 1);
+}
+
+// Tiles [deal_lo(c), deal_lo(c + 1)) of a group's N belong to CTA c of G (G <= N).  The remainder r moves from group to
+// group so that no CTA always has the odd tile.
+int64_t deal_lo(int64_t c, int64_t N, int64_t G, int64_t r) { return (c * N + r) / G; }
+
+// A work list: groups cut[0] .. cut[1] - 1 and so on of segments `segs`; pass 1 of a group (unless one_pass), then pass 2
+// of the group before it.  Every pass of a group is dealt to the CTAs in contiguous runs.
+struct HostList {
+  std::vector<TcRun> runs[2];
+  std::vector<int32_t> first;
+  std::vector<TcStage> stages;
+  std::vector<TcFold> folds;
+  int32_t most = 0;                        // tiles of the largest group in pass 2
+};
+HostList deal(const std::vector<TcRun>& segs, const std::vector<int>& cut, const asl_ctx* c, int grid, bool one_pass) {
+  HostList l;
+  const int ng = (int)cut.size() - 1;
+  l.folds.resize(segs.size());
+  std::vector<int> at[2];                  // first run of each group
+  for (int p = one_pass ? 1 : 0; p < 2; ++p)
+    for (int g = 0; g < ng; ++g) {
+      std::vector<TcRun>& runs = l.runs[p];
+      at[p].push_back((int)runs.size());
+      int64_t N = 0, g0 = 0;
+      auto tiles = [&](int s) { const AslReq& r = c->req[segs[s].b]; return ((p ? r.T : r.n) + KT - 1) / KT; };
+      for (int s = cut[g]; s < cut[g + 1]; ++s) N += tiles(s);
+      const int64_t G = N < grid ? N : grid, r = (int64_t)g * (N % G) % G;
+      for (int s = cut[g]; s < cut[g + 1]; ++s) {
+        const int slot0 = (int)runs.size();
+        for (int64_t t = g0; t < g0 + tiles(s);) {
+          int64_t cta = (t * G - r) / N;
+          while (deal_lo(cta + 1, N, G, r) <= t) ++cta;
+          int64_t end = deal_lo(cta + 1, N, G, r);
+          if (end > g0 + tiles(s)) end = g0 + tiles(s);
+          TcRun run = segs[s];
+          run.tile0 = (int32_t)(t - g0); run.ntiles = (int32_t)(end - t); run.pass = p + 1; run.group = g;
+          run.slot = (int32_t)runs.size(); run.cta = (int32_t)cta; run.next = -1;
+          runs.push_back(run);
+          t = end;
+        }
+        if (p == 0 || one_pass) l.folds[s] = TcFold{slot0, (int32_t)runs.size() - slot0, segs[s].rows, segs[s].b};
+        g0 += tiles(s);
+      }
+      if (p && N > l.most) l.most = (int32_t)N;
+    }
+  for (int p = 0; p < 2; ++p) at[p].push_back((int)l.runs[p].size());
+  l.first.assign(grid, -1);
+  std::vector<int> last(grid, -1);
+  const int n1 = (int)l.runs[0].size();
+  auto chain = [&](int p, int g) {
+    for (int i = at[p][g]; i < at[p][g + 1]; ++i) {
+      const int cta = l.runs[p][i].cta, index = p * n1 + i, before = last[cta];
+      if (before < 0) l.first[cta] = index;
+      else (before < n1 ? l.runs[0][before] : l.runs[1][before - n1]).next = index;
+      last[cta] = index;
+    }
+  };
+  for (int g = 0; g <= ng; ++g) {
+    if (g < ng && !one_pass) chain(0, g);
+    if (g < ng) l.stages.push_back(TcStage{cut[g], cut[g + 1] - cut[g], 0, 0});
+    if (g > 0) chain(1, g - 1);
+  }
+  return l;
+}
+
+}  // namespace
+
 bool asl_tc_plan(asl_ctx* c) {
   const asl_params& p = c->p;
   AslTcPlan& tp = c->tc;
   tp = AslTcPlan();
-  const int W = p.window, G = p.n_q_heads / p.n_kv_heads, R = G * W;
-  if (p.head_dim != 128 || W % 32 || W > MAX_NC) return false;
-  // Chunk of NC query rows (whole heads, a multiple of 64 rows, at most 256).  Max pooling wants the
-  // chunks to tile the G*W rows exactly (its column sums are kept per query head).  Average pooling
-  // sums all rows of a kv head anyway, so the last chunk may be padded: its extra rows are given an
-  // infinite offset in pass 2 and add nothing.  Fewest chunks first, then least padding.
-  int NC = 0;
-  if (p.pool_mode == ASL_POOL_MAX) {
-    for (int m = MAX_NC / W; m >= 1; --m)
-      if (R % (m * W) == 0) { NC = m * W; break; }
-    if (NC < 64 || NC % 64 || R % NC) return false;
-  } else {
-    int best_chunks = 0;
-    for (int m = 1; m * W <= MAX_NC; ++m) {
-      const int nc = m * W;
-      if (nc % 64) continue;
-      const int chunks = (R + nc - 1) / nc;
-      if (!NC || chunks < best_chunks) { NC = nc; best_chunks = chunks; }
-    }
-    if (!NC) return false;
-  }
-  tp.NC = NC;
-  tp.nchunk = (R + NC - 1) / NC;
+  const int W = p.window, G = p.n_q_heads / p.n_kv_heads;
+  if (p.k_dtype == ASL_K_FP8_E4M3 && !fp8_shape(p)) return false;
+  plan_chunks(p, tp);
   tp.grid = (p.score_ctas > 0 && p.score_ctas < c->sm_count) ? p.score_ctas : c->sm_count;
 
-  // segments in (request, head, chunk) order; phases in groups: pass 1 of `group` segments, then their pass 2
-  struct Seg { int b, h, chunk, tiles1, tiles2; };
-  std::vector<Seg> segs;
+  // segments in (request, head, chunk) order
+  std::vector<TcRun> segs;
+  int64_t tiles = 0;
   for (int b = 0; b < p.batch; ++b)
     for (int h = 0; h < p.n_kv_heads; ++h)
-      for (int ch = 0; ch < tp.nchunk; ++ch)
-        segs.push_back({b, h, ch, (c->req[b].n + KT - 1) / KT, (c->req[b].T + KT - 1) / KT});
+      for (int ch = 0; ch < tp.nchunk; ++ch) {
+        TcRun s{};
+        s.seg = (int32_t)segs.size();
+        s.b = b; s.h = h; s.chunk = ch;
+        s.T = c->req[b].T; s.t_off = c->req[b].t_off; s.tok_off = c->req[b].tok_off;
+        const int heads = G - ch * tp.m < tp.m ? G - ch * tp.m : tp.m;
+        const int rest = W - ch % tp.pieces * MAX_ROWS;
+        s.rows = tp.pieces > 1 ? (rest < MAX_ROWS ? rest : MAX_ROWS) : (heads - 1) * tp.Wp + W;
+        s.kscale = p.k_dtype == ASL_K_FP8_E4M3 ? c->k_scale[h] / Q8_SCALE : 1.0f;
+        segs.push_back(s);
+        tiles += (c->req[b].n + KT - 1) / KT;
+      }
   tp.nseg = (int)segs.size();
-  // Segments per group: pass 1 of all of them runs before their pass 2, which hides the fold of the
-  // row denominators; K of a whole group has to stay in L2 between the passes (72 MB of the 126 MB).
-  int group = 0;
+  if (tiles >= (int64_t)1 << 30) return false;
+
+  // Groups of segments: pass 1 of a group, then pass 2 of the one before it, so that the fold of the row denominators is
+  // hidden behind other tiles.  K of two groups should stay in L2: up to 70 MB each (at 128K tokens two kv heads, 67 MB:
+  // pass 2 then reads a quarter of K from HBM again, and the fewer hand-offs gain more: 155.4 -> 152.7 us against groups
+  // of one kv head), at least two groups.
+  std::vector<int> cut{0};
   {
-    const double seg_bytes = (double)c->sum_tokens * p.k_stride[0] * c->k_elem_bytes / p.n_kv_heads / (double)p.batch;   // one kv head of an average request
-    group = (int)(72.0e6 / (seg_bytes > 1.0 ? seg_bytes : 1.0));
-    group = group < 1 ? 1 : (group > 16 ? 16 : group);
+    auto seg_bytes = [&](int s) { return (double)c->req[segs[s].b].n * 128 * c->k_elem_bytes / tp.nchunk; };
+    double total = 0, run = 0;
+    int groups = 1;
+    for (int s = 0; s < tp.nseg; ++s) {
+      total += seg_bytes(s);
+      if (run > 0 && run + seg_bytes(s) > 70.0e6) { ++groups; run = 0; }
+      run += seg_bytes(s);
+    }
+    groups = groups < 2 ? 2 : groups;
+    run = 0;
+    for (int s = 0; s + 1 < tp.nseg; ++s) {                // evenly sized
+      run += seg_bytes(s);
+      if (run + 0.5 * seg_bytes(s + 1) > total / groups * cut.size()) cut.push_back(s + 1);
+    }
+    cut.push_back(tp.nseg);
   }
-  tp.group = group;
-  int64_t g = 0;
-  auto push = [&](int s, int pass) {
-    TcPhase ph{};
-    ph.g0 = (int32_t)g;
-    ph.ntiles = pass == 1 ? segs[s].tiles1 : segs[s].tiles2;
-    ph.pass = pass; ph.seg = s; ph.b = segs[s].b; ph.h = segs[s].h; ph.chunk = segs[s].chunk;
-    ph.ncontrib = segs[s].tiles1 < tp.grid ? segs[s].tiles1 : tp.grid;    // CTAs with a tile in pass 1
-    ph.T = c->req[ph.b].T; ph.t_off = c->req[ph.b].t_off; ph.tok_off = c->req[ph.b].tok_off;
-    ph.rows = R - ph.chunk * NC < NC ? R - ph.chunk * NC : NC;
-    ph.kscale = p.k_dtype == ASL_K_FP8_E4M3 ? c->k_scale[ph.h] / Q8_SCALE : 1.0f;
-    g += ph.ntiles;
-    tp.phases.push_back(ph);
+  const HostList lists[2] = {deal(segs, cut, c, tp.grid, false), deal(segs, {0, tp.nseg}, c, tp.grid, true)};
+
+  // one allocation for everything the kernels read or count in
+  size_t bytes = 0;
+  std::vector<char> host;
+  auto put = [&](const void* data, size_t n) {
+    const size_t at = bytes;
+    bytes = asl_align256(bytes + n);
+    host.resize(bytes, 0);
+    if (n) memcpy(host.data() + at, data, n);
+    return at;
   };
-  for (int s0 = 0; s0 < tp.nseg; s0 += group) {
-    const int s1 = s0 + group < tp.nseg ? s0 + group : tp.nseg;
-    for (int s = s0; s < s1; ++s) push(s, 1);
-    for (int s = s0; s < s1; ++s) push(s, 2);
+  struct ListAt { size_t runs, first, stages, folds; } at[2];
+  TcList* out[2] = {&tp.both, &tp.only2};
+  for (int i = 0; i < 2; ++i) {
+    const HostList& l = lists[i];
+    out[i]->n1 = (int32_t)l.runs[0].size();
+    out[i]->n2 = (int32_t)l.runs[1].size();
+    out[i]->n_groups = (int32_t)l.stages.size();
+    out[i]->most = l.most;
+    std::vector<TcRun> runs(l.runs[0]);
+    runs.insert(runs.end(), l.runs[1].begin(), l.runs[1].end());
+    at[i] = ListAt{put(runs.data(), runs.size() * sizeof(TcRun)), put(l.first.data(), l.first.size() * sizeof(int32_t)),
+                   put(l.stages.data(), l.stages.size() * sizeof(TcStage)), put(l.folds.data(), l.folds.size() * sizeof(TcFold))};
   }
-  if (g >= ((int64_t)1 << 31) - tp.grid) return false;
-  tp.total_items = (int32_t)g;
-
-  std::vector<TcPhase> only2;
-  int64_t g2 = 0;
-  for (const TcPhase& ph : tp.phases)
-    if (ph.pass == 2) { TcPhase q = ph; q.g0 = (int32_t)g2; g2 += q.ntiles; only2.push_back(q); }
-  tp.n_phases2 = (int32_t)only2.size();
-  tp.total_items2 = (int32_t)g2;
-
-  const size_t sync_bytes = (2 * (size_t)tp.nseg + 2) * sizeof(uint32_t);   // counters, launch number, exit ticket
-  cudaError_t e = cudaMalloc(&tp.d_phases, tp.phases.size() * sizeof(TcPhase));
-  if (e == cudaSuccess) e = cudaMalloc(&tp.d_phases2, only2.size() * sizeof(TcPhase));
-  if (e == cudaSuccess) e = cudaMemcpy(tp.d_phases2, only2.data(), only2.size() * sizeof(TcPhase), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&tp.d_sync, sync_bytes);
-  if (e == cudaSuccess) e = cudaMalloc(&tp.d_live, tp.phases.size() * sizeof(TcPhase));
-  if (e == cudaSuccess) e = cudaMalloc(&tp.d_live_hdr, 2 * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMemcpy(tp.d_phases, tp.phases.data(), tp.phases.size() * sizeof(TcPhase), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemset(tp.d_sync, 0, sync_bytes);
-  if (e != cudaSuccess) { asl_tc_free(c); return false; }
-  cudaFuncSetAttribute(score_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-  cudaFuncSetAttribute(score_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-  cudaFuncSetAttribute(score_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-  cudaFuncSetAttribute(score_tc_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-  if (cudaGetLastError() != cudaSuccess) { asl_tc_free(c); return false; }
+  const size_t sync_words = (4 * (size_t)tp.nseg + 1) * SYNC_STRIDE;
+  const std::vector<uint32_t> zeros(sync_words, 0);
+  const size_t sync_at = put(zeros.data(), sync_words * sizeof(uint32_t));
+  const size_t host_bytes = bytes;
+  auto take = [&](size_t n) { const size_t t = bytes; bytes = asl_align256(bytes + n); return t; };
+  const size_t n_runs = (size_t)tp.both.n1 + tp.both.n2;      // the longer list
+  const size_t live_at[5] = {take(n_runs * sizeof(TcRun)), take((size_t)tp.grid * sizeof(int32_t)), take((size_t)tp.nseg * sizeof(TcFold)),
+                             take((3 * n_runs + 6 * (size_t)tp.both.n_groups + 4 * (size_t)(tp.both.n_groups + 1) * tp.grid) * sizeof(int32_t)),
+                             take(sizeof(int32_t))};
+  cudaError_t e = cudaMalloc(&tp.d_blob, bytes);
+  if (e == cudaSuccess) e = cudaMemcpy(tp.d_blob, host.data(), host_bytes, cudaMemcpyHostToDevice);
+  const ScoreKernel& kern = score_kernel(score_kernel_of(p, tp));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kern.smem);
+  if (e != cudaSuccess) { cudaGetLastError(); asl_tc_free(c); return false; }
+  char* d = static_cast<char*>(tp.d_blob);
+  for (int i = 0; i < 2; ++i) {
+    out[i]->d_runs = reinterpret_cast<TcRun*>(d + at[i].runs);
+    out[i]->d_first = reinterpret_cast<int32_t*>(d + at[i].first);
+    out[i]->d_stages = reinterpret_cast<TcStage*>(d + at[i].stages);
+    out[i]->d_folds = reinterpret_cast<TcFold*>(d + at[i].folds);
+  }
+  tp.d_sync = reinterpret_cast<uint32_t*>(d + sync_at);
+  tp.d_live_runs = reinterpret_cast<TcRun*>(d + live_at[0]);
+  tp.d_live_first = reinterpret_cast<int32_t*>(d + live_at[1]);
+  tp.d_live_folds = reinterpret_cast<TcFold*>(d + live_at[2]);
+  tp.d_live_scratch = reinterpret_cast<int32_t*>(d + live_at[3]);
+  tp.d_live_hdr = reinterpret_cast<int32_t*>(d + live_at[4]);
   tp.enabled = encode_fn() != nullptr;
   return tp.enabled;
 }
 
-size_t asl_tc_partial_bytes(const asl_ctx* c) {
-  const AslTcPlan& tp = c->tc;
-  return (size_t)tp.nseg * tp.grid * 2 * tp.NC * sizeof(float2);
-}
+size_t asl_tc_partial_bytes(const asl_ctx* c) { return (size_t)c->tc.both.n1 * (c->tc.wide ? GROUPS / 2 : GROUPS) * c->tc.NC * sizeof(float2); }
 
 void asl_tc_free(asl_ctx* c) {
   AslTcPlan& tp = c->tc;
-  if (tp.d_phases) cudaFree(tp.d_phases);
-  if (tp.d_phases2) cudaFree(tp.d_phases2);
-  if (tp.d_sync) cudaFree(tp.d_sync);
-  if (tp.d_live) cudaFree(tp.d_live);
-  if (tp.d_live_hdr) cudaFree(tp.d_live_hdr);
-  tp.d_live = nullptr;
-  tp.d_live_hdr = nullptr;
-  tp.d_phases = nullptr;
-  tp.d_phases2 = nullptr;
-  tp.d_sync = nullptr;
-  tp.enabled = false;
+  if (tp.d_blob) cudaFree(tp.d_blob);
+  tp = AslTcPlan();
 }
 
 asl_status asl_launch_wait_selftest(asl_ctx* c, int which, unsigned long long limit_ns, cudaStream_t st) {
@@ -1053,22 +1361,31 @@ asl_status asl_launch_wait_selftest(asl_ctx* c, int which, unsigned long long li
   return ASL_OK;
 }
 
-asl_status asl_launch_live_phases(asl_ctx* c, bool two_pass, cudaStream_t st) {
-  AslTcPlan& tp = c->tc;
-  const TcPhase* all = two_pass ? tp.d_phases : tp.d_phases2;
-  const int n_all = two_pass ? (int)tp.phases.size() : tp.n_phases2;
-  live_phase_list_kernel<<<1, 256, 0, st>>>(all, n_all, c->latch_stat, c->cur_layer, c->p.batch, two_pass ? 1 : 0, tp.NC, tp.d_live,
-                                            tp.d_live_hdr, tp.d_sync, tp.d_sync + tp.nseg);
+asl_status asl_launch_window_lse(asl_ctx* c, const char* ws, float* lse_out, cudaStream_t st) {
+  const AslTcPlan& tp = c->tc;
+  const int n = c->p.batch * c->p.n_q_heads * c->p.window;
+  offsets_to_lse_kernel<<<(n + 255) / 256, 256, 0, st>>>(reinterpret_cast<const float*>(ws + c->ws.score_offsets), lse_out, n, c->p.window,
+                                                         c->p.n_q_heads / c->p.n_kv_heads, tp.m, tp.Wp, tp.pieces, tp.nchunk, tp.NC);
   c->launches += 1;
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;
 }
 
-// after a reported device error the publish counters may be inconsistent: start over
+asl_status asl_launch_live_phases(asl_ctx* c, bool two_pass, cudaStream_t st) {
+  AslTcPlan& tp = c->tc;
+  const TcList& l = two_pass ? tp.both : tp.only2;
+  live_list_kernel<<<1, 1024, 0, st>>>(l.d_runs, l.n1, l.n2, l.d_folds, tp.nseg, l.n_groups, l.most + l.most / 4, c->latch_stat, c->cur_layer,
+                                       c->p.batch, tp.grid, tp.d_live_hdr, tp.d_live_runs, tp.d_live_first, tp.d_live_folds, tp.d_live_scratch);
+  c->launches += 1;
+  ASL_CUDA(cudaGetLastError());
+  return ASL_OK;
+}
+
+// after a reported device error the counters may be inconsistent: start over
 asl_status asl_tc_reset_sync(asl_ctx* c, cudaStream_t st) {
   AslTcPlan& tp = c->tc;
   if (!tp.d_sync) return ASL_OK;
-  ASL_CUDA(cudaMemsetAsync(tp.d_sync, 0, (2 * (size_t)tp.nseg + 2) * sizeof(uint32_t), st));
+  ASL_CUDA(cudaMemsetAsync(tp.d_sync, 0, (4 * (size_t)tp.nseg + 1) * SYNC_STRIDE * sizeof(uint32_t), st));
   return ASL_OK;
 }
 
@@ -1076,10 +1393,11 @@ asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const f
                                cudaStream_t st) {
   const asl_params& p = c->p;
   AslTcPlan& tp = c->tc;
-  const int W = p.window, G = p.n_q_heads / p.n_kv_heads, NC = tp.NC;
+  const int W = p.window, G = p.n_q_heads / p.n_kv_heads;
   const bool fp8 = p.k_dtype == ASL_K_FP8_E4M3;
   CUtensorMap tm_q, tm_k;
-  const cuuint32_t bw = (cuuint32_t)(W < NC ? W : NC);
+  // one copy brings all heads of a chunk where they follow one another in the buffer as in the tensor
+  const cuuint32_t box_t = (cuuint32_t)(W < MAX_ROWS ? W : MAX_ROWS), box_h = (cuuint32_t)(tp.pieces == 1 && tp.Wp == W ? tp.m : 1);
   if (fp8) {
     // the queries as two E4M3 terms in the workspace, then 8-bit maps: rows of 128 one-byte channels
     uint8_t* q8 = reinterpret_cast<uint8_t*>(ws + c->ws.score_q8);
@@ -1089,7 +1407,7 @@ asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const f
     c->launches += 1;
     const cuuint64_t qdims[5] = {128, (cuuint64_t)W, (cuuint64_t)p.n_q_heads, (cuuint64_t)p.batch, 2};
     const cuuint64_t qstr[4] = {128, (cuuint64_t)W * 128, (cuuint64_t)p.n_q_heads * W * 128, (cuuint64_t)total};
-    const cuuint32_t qbox[5] = {128, bw, (cuuint32_t)NC / bw, 1, 1};
+    const cuuint32_t qbox[5] = {128, box_t, box_h, 1, 1};
     if (!make_map(&tm_q, CU_TENSOR_MAP_DATA_TYPE_UINT8, q8, 5, qdims, qstr, qbox)) return ASL_ERR_CUDA;
     const cuuint64_t kdims[3] = {128, (cuuint64_t)p.n_kv_heads, (cuuint64_t)c->sum_tokens};
     const cuuint64_t kstr[2] = {(cuuint64_t)p.k_stride[1], (cuuint64_t)p.k_stride[0]};
@@ -1098,7 +1416,7 @@ asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const f
   } else {
     const cuuint64_t dims[4] = {128, (cuuint64_t)W, (cuuint64_t)p.n_q_heads, (cuuint64_t)p.batch};
     const cuuint64_t strides[3] = {(cuuint64_t)p.q_stride[2] * 2, (cuuint64_t)p.q_stride[1] * 2, (cuuint64_t)p.q_stride[0] * 2};
-    const cuuint32_t box[4] = {64, bw, (cuuint32_t)NC / bw, 1};
+    const cuuint32_t box[4] = {64, box_t, box_h, 1};
     if (!make_map(&tm_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, q, 4, dims, strides, box)) return ASL_ERR_CUDA;
     const cuuint64_t kdims[3] = {128, (cuuint64_t)p.n_kv_heads, (cuuint64_t)c->sum_tokens};
     const cuuint64_t kstr[2] = {(cuuint64_t)p.k_stride[1] * 2, (cuuint64_t)p.k_stride[0] * 2};
@@ -1106,37 +1424,30 @@ asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const f
     if (!make_map(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, k, 3, kdims, kstr, kbox)) return ASL_ERR_CUDA;
   }
   TcArgs a{};
-  const bool live_list = c->latch_stat && c->cur_layer >= 0 && p.batch <= ASL_SKIP_MAX_BATCH;   // written by asl_launch_live_phases just before
-  a.phases = live_list ? tp.d_live : (lse ? tp.d_phases2 : tp.d_phases);
-  a.live_hdr = live_list ? tp.d_live_hdr : nullptr;
+  const TcList& list = lse ? tp.only2 : tp.both;
+  a.list = {list.d_runs, list.d_first, list.d_folds};
+  if (c->latch_stat && c->cur_layer >= 0 && p.batch <= ASL_SKIP_MAX_BATCH) {      // written by asl_launch_live_phases just before
+    a.live = {tp.d_live_runs, tp.d_live_first, tp.d_live_folds};
+    a.live_hdr = tp.d_live_hdr;
+  }
+  a.stages = list.d_stages;
+  a.n_stages = lse ? 0 : list.n_groups;
   a.lse = lse;
-  a.req = c->d_req;
   a.partials = reinterpret_cast<float2*>(ws + c->ws.score_partials);
   a.offsets = reinterpret_cast<float*>(ws + c->ws.score_offsets);
   a.u = u;
-  a.published = tp.d_sync;
-  a.folded = tp.d_sync + tp.nseg;
+  a.counters = tp.d_sync;                                            // the one-pass launch touches neither these
+  a.launch = tp.d_sync + 4 * (size_t)tp.nseg * SYNC_STRIDE;         // nor this
   a.err = c->d_err;
   a.sum_T = c->sum_T;
-  a.epoch_word = tp.d_sync + 2 * tp.nseg;         // the one-pass launch touches neither the counters nor this
-  a.epoch_limit = 0xFFFFFFFFu / (uint32_t)(2 * tp.grid > MAX_NC ? 2 * tp.grid : MAX_NC) - 2u;
   a.nseg = tp.nseg;
-  a.n_phases = lse ? tp.n_phases2 : (int32_t)tp.phases.size();
-  a.total_items = lse ? tp.total_items2 : tp.total_items;
-  a.NC = NC; a.W = W; a.G = G; a.Hk = p.n_kv_heads; a.Hq = p.n_q_heads;
+  a.NC = tp.NC; a.HR = tp.HR; a.W = W; a.Wp = tp.Wp; a.m = tp.m; a.pieces = tp.pieces; a.G = G; a.Hq = p.n_q_heads;
   a.u_rows_per_kv = c->u_rows_per_kv;
   a.u_parts = c->u_parts;
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)p.head_dim));
   // every CTA must be resident at once (pass 2 waits for counters other CTAs advance): one CTA per SM at most
-  const int grid = tp.grid;
-  const bool per_q = p.pool_mode == ASL_POOL_MAX;
-  if (fp8) {
-    if (per_q) score_tc_kernel<true, true><<<grid, THREADS, SMEM_BYTES, st>>>(tm_q, tm_k, a);
-    else       score_tc_kernel<false, true><<<grid, THREADS, SMEM_BYTES, st>>>(tm_q, tm_k, a);
-  } else {
-    if (per_q) score_tc_kernel<true, false><<<grid, THREADS, SMEM_BYTES, st>>>(tm_q, tm_k, a);
-    else       score_tc_kernel<false, false><<<grid, THREADS, SMEM_BYTES, st>>>(tm_q, tm_k, a);
-  }
+  const ScoreKernel& kern = score_kernel(score_kernel_of(p, tp));
+  kern.fn<<<tp.grid, THREADS, kern.smem, st>>>(tm_q, tm_k, a);
   c->launches += 1;
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;

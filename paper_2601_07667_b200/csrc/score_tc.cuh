@@ -1,36 +1,58 @@
-// Plan of the tensor-core scorer: the phase list built at plan time.
+// Plan of the tensor-core scorer: how the query rows of a kv head are cut into chunks, and the work lists built at
+// plan time (or ahead of a launch that leaves finished requests out).
 #pragma once
 #include <stdint.h>
 #include <vector>
 
 constexpr int ASL_TC_KEY_TILE = 128;
 
-// one pass over the 128-key tiles of one segment = (request, kv head, row chunk);
-// its tiles are the global work items g0 .. g0 + ntiles - 1
-// (T, t_off, tok_off: the request's past length, score offset and first token, copied here so that
-// one record is all a role needs when it enters the phase)
-// rows: query rows of the chunk that exist (the last chunk of a kv head may be padded up to NC)
-// kscale: factor between the accumulator and q.k (1 for bf16 keys; k_scale[h] / 16 for FP8 keys, whose
-// queries are scaled by 16 before they are split into two E4M3 terms)
-struct TcPhase { int32_t g0, ntiles, pass, seg, b, h, chunk, ncontrib, T, t_off, tok_off, rows; float kscale; };
+#ifdef __CUDACC__
+#define ASL_HD __host__ __device__
+#else
+#define ASL_HD
+#endif
+
+// A run: the tiles of one segment = (request, kv head, row chunk) that one CTA takes in one pass; `next`: the CTA's next
+// run (-1: none).  (T, t_off, tok_off: the request's past length, score offset and first token, copied here so that one
+// record is all a role needs; rows: query rows of the chunk that exist; kscale: factor between the accumulator and q.k,
+// 1 for bf16 keys and k_scale[h] / 16 for FP8 keys, whose queries are scaled by 16 before they are split into two E4M3
+// terms; slot: number of the run among its pass's; group of segments; cta:
+// whom the plan gave it)
+struct __align__(16) TcRun { int32_t tile0, ntiles, pass, seg, b, h, chunk, next, T, t_off, tok_off, rows; float kscale; int32_t slot, group, cta; };
+
+// A group of segments: seg0 .. seg0 + nseg - 1.
+struct __align__(16) TcStage { int32_t seg0, nseg, pad0, pad1; };
+
+// What the fold of a segment's softmax denominators needs: the pass-1 runs that publish, in slot order.
+struct __align__(16) TcFold { int32_t slot0, nruns, rows, b; };
+
+struct TcList {                  // a work list on the device: runs of pass 1, then of pass 2
+  int32_t n1 = 0, n2 = 0, n_groups = 0;
+  int32_t most = 0;              // tiles of the largest group
+  TcRun* d_runs = nullptr;
+  int32_t* d_first = nullptr;    // [grid] first run of every CTA
+  TcStage* d_stages = nullptr;
+  TcFold* d_folds = nullptr;     // [segments]
+};
 
 struct AslTcPlan {
   bool enabled = false;
-  int NC = 0;           // query rows per chunk (MMA N in pass 2)
+  int NC = 0;           // rows of a chunk's buffer (halves of HR)
+  int HR = 0;           // rows of a half: one accumulator of pass 1 (lanes) or pass 2 (columns), a multiple of 32, at most 128
+  bool wide = false;    // two halves
+  int Wp = 0;           // buffer rows from one query head to the next (the window, padded under max pooling; 256 if longer)
+  int m = 0;            // query heads of a chunk
+  int pieces = 0;       // chunks per query head (windows of more than 256 rows), else 1
   int nchunk = 0;       // chunks per kv head
   int nseg = 0;         // segments
   int grid = 0;         // CTAs of the persistent kernel (one per SM)
-  int group = 0;        // segments whose pass 1 runs before their pass 2
-  int32_t total_items = 0;
-  std::vector<TcPhase> phases;   // both passes
-  TcPhase* d_phases = nullptr;
-  int32_t n_phases2 = 0;         // the pass-2 phases alone (scoring with a supplied log-sum-exp)
-  int32_t total_items2 = 0;
-  TcPhase* d_phases2 = nullptr;
-  uint32_t* d_sync = nullptr;   // [nseg] publish counters, [nseg] folded-row counters, launch number, exit ticket
-  // device-side controller: the phase list of the next launch without the finished requests' phases,
-  // written ahead of the launch (capacity: the longer of the two static lists), and its header
-  // {phases, work items}
-  TcPhase* d_live = nullptr;
+  TcList both, only2;   // both passes; the pass-2 phases alone (scoring with a supplied log-sum-exp)
+  void* d_blob = nullptr;       // the device side of the lists below and above, one allocation
+  uint32_t* d_sync = nullptr;   // two sets of publish and folded-row counters, launch number, ticket of arrived CTAs
+  // device-side controller: the next launch's list without the finished requests' phases, written ahead of it
+  TcRun* d_live_runs = nullptr;
+  int32_t* d_live_first = nullptr;
+  TcFold* d_live_folds = nullptr;
   int32_t* d_live_hdr = nullptr;
+  int32_t* d_live_scratch = nullptr;
 };
