@@ -82,9 +82,11 @@ typedef struct {
   int32_t batch;          /* B >= 1 requests                                          */
   int32_t l_min;          /* first layer at which the statistic is evaluated          */
   int32_t l_obs;          /* rank rows kept (ring depth), >= 2                        */
-  int32_t score_ctas;     /* CTAs of the persistent scorer kernel; 0 = one per SM.  A   */
-                          /* smaller number leaves SMs to kernels of other streams    */
-                          /* (the previous layer's statistic, top-k and compaction)   */
+  int32_t score_ctas;     /* CTAs of the persistent scorer kernel; 0 = one per SM, and */
+                          /* for asl_score_columns (whose caller pipelines layers) 16   */
+                          /* or 32 fewer: that leaves SMs to kernels of other streams   */
+                          /* (the previous layer's statistic, top-k and compaction).    */
+                          /* Sums may differ in their last bits between two numbers     */
   double tau;             /* selection fires when relative variance < tau             */
   const int32_t* cu_seqlens; /* host [B+1] token offsets, cu_seqlens[0] = 0           */
   const int32_t* budgets;    /* host [B] KV_budget per request, window included       */
@@ -229,6 +231,34 @@ asl_status asl_select_topk_gated(asl_ctx* ctx, const float* scores, int32_t n_he
  * k_out, v_out: device bf16 dense [H_k][sum_kept][d]. */
 asl_status asl_compact_kv(asl_ctx* ctx, const void* k, const void* v, const int32_t* idx, void* k_out,
                           void* v_out, void* stream);
+
+/* A layer's five steps in one call, for callers that pipeline layers: asl_score_columns on `stream`, then
+ * asl_pool_scores and asl_rank_stat on `side`, asl_select_topk and asl_compact_kv on `side2`, ordered by events that
+ * the context keeps.  The side streams are not waited for: they run under the scoring of the next layer, and a slot's
+ * buffers are written again only when the work of two layers ago has read them.  Use slots 0 and 1 in turn.
+ * asl_run_join makes `stream` wait for everything issued so far.  asl_run_reset forgets what is in flight, without
+ * waiting: call it before and after capturing layers into a CUDA graph (nothing recorded outside a capture may be
+ * waited for inside it, nor the other way round). */
+typedef struct {
+  void* workspace;
+  size_t workspace_bytes;
+  float* scores_kv[2];     /* per slot, as in asl_pool_scores */
+  float* scores_agg[2];
+  int32_t* rank_ring;
+  asl_stat* stat;
+  int32_t* idx;
+  void* k_out;
+  void* v_out;
+  void* stream;            /* cudaStream_t: scoring */
+  void* side;              /* pooling and statistic */
+  void* side2;             /* top-k and compaction */
+  int32_t one_side;        /* 1: `side` also waits for `side2` at the end of the layer */
+  int32_t reserved0;
+} asl_layer;
+asl_status asl_run_layer(asl_ctx* ctx, const asl_layer* layer, const void* q_obs, const void* k, const void* v,
+                         const float* lse, int32_t layer_idx, int32_t n_rows, int32_t slot);
+asl_status asl_run_join(asl_ctx* ctx, void* stream);
+asl_status asl_run_reset(asl_ctx* ctx);
 
 /* Algorithm 2 (one-shot selection), the one-shot selection at the selection layer: once
  * asl_rank_stat reports `selected`, the tokens that go on to the deeper layers

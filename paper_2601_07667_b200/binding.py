@@ -22,7 +22,7 @@ EXPORTS = ("asl_create", "asl_destroy", "asl_plan", "asl_plan_sizes", "asl_score
            "asl_select_topk", "asl_compact_kv", "asl_device_status", "asl_launch_count", "asl_strerror",
            "asl_rank_desc_static", "asl_score_layer_lse", "asl_window_lse", "asl_compact_rows",
            "asl_score_columns", "asl_pool_scores", "asl_set_controller", "asl_select_topk_gated",
-           "asl_selftest_bounded_wait", "asl_set_layer")
+           "asl_selftest_bounded_wait", "asl_set_layer", "asl_run_layer", "asl_run_join", "asl_run_reset")
 ASL_RANK_STATIC_MAX_T = 262144
 
 
@@ -34,6 +34,13 @@ class AslParams(C.Structure):
                 ("cu_seqlens", C.POINTER(C.c_int32)), ("budgets", C.POINTER(C.c_int32)),
                 ("q_stride", C.c_int64 * 3), ("k_stride", C.c_int64 * 2), ("v_stride", C.c_int64 * 2),
                 ("k_dtype", C.c_int32), ("reserved0", C.c_int32), ("k_scale", C.POINTER(C.c_float))]
+
+
+class AslLayer(C.Structure):
+    _fields_ = [("workspace", C.c_void_p), ("workspace_bytes", C.c_size_t), ("scores_kv", C.c_void_p * 2),
+                ("scores_agg", C.c_void_p * 2), ("rank_ring", C.c_void_p), ("stat", C.c_void_p), ("idx", C.c_void_p),
+                ("k_out", C.c_void_p), ("v_out", C.c_void_p), ("stream", C.c_void_p), ("side", C.c_void_p),
+                ("side2", C.c_void_p), ("one_side", C.c_int32), ("reserved0", C.c_int32)]
 
 
 class AslStat(C.Structure):
@@ -80,6 +87,9 @@ def _load() -> C.CDLL:
     lib.asl_device_status.argtypes = [vp, vp, C.POINTER(i32)]
     lib.asl_rank_desc_static.argtypes = [vp, i32, vp, vp]
     lib.asl_selftest_bounded_wait.argtypes = [vp, i32, i64, vp]
+    lib.asl_run_layer.argtypes = [vp, C.POINTER(AslLayer), vp, vp, vp, vp, i32, i32, i32]
+    lib.asl_run_join.argtypes = [vp, vp]
+    lib.asl_run_reset.argtypes = [vp]
     lib.asl_launch_count.argtypes = [vp]
     lib.asl_launch_count.restype = i64
     lib.asl_strerror.argtypes = [C.c_int]
@@ -252,11 +262,11 @@ def asl_rank_desc_static(scores, T: int, rank_out, stream=None) -> None:
 class LayerPath:
     """Owns a context, its plan and the device buffers of one layer's pass
     (scores, indices, compacted cache, rank ring, statistic), all torch tensors.
-    ``run_layer`` issues the five steps: the scoring proper on the current stream, the
-    rest of the layer (pooling first) on a side stream (``tail_streams=2``: pooling and the rank
-    statistic on one, top-k and compaction on another) that is not waited for, so that it overlaps the scoring of the next layer (both
-    score buffers are double buffered for that; give the plan ``score_ctas``
-    below the SM count to leave those kernels somewhere to run).  ``join`` makes
+    ``run_layer`` issues the five steps in one native call: the scoring proper on the current stream, the
+    rest of the layer on side streams (pooling and the rank statistic on ``side``, top-k and compaction on ``side2``;
+    with ``tail_streams=1`` ``side`` waits for both at the end of every layer) that are not waited for, so that it
+    overlaps the scoring of the next layer (both score buffers are double buffered for that; unless the plan is given
+    ``score_ctas`` the scorer leaves those kernels some SMs).  ``join`` makes
     the current stream wait for everything issued so far; ``read_stat`` joins by
     itself.  A device-wide synchronize covers it too."""
 
@@ -289,7 +299,6 @@ class LayerPath:
         self.workspace = torch.empty(max(self.ws_bytes, 256), dtype=torch.uint8, device=dev)
         self._kv = [torch.empty((n_kv_heads, self.sum_T), dtype=torch.float32, device=dev) for _ in range(2)]
         self._agg = [torch.empty((self.sum_T,), dtype=torch.float32, device=dev) for _ in range(2)]
-        self._agg_free = [None, None]       # event after the side-stream work that last read the buffers
         self._cur = 0
         self.idx = torch.empty((n_kv_heads, self.sum_kept), dtype=torch.int32, device=dev)
         self.k_out = torch.empty((n_kv_heads, self.sum_kept, head_dim),
@@ -297,11 +306,13 @@ class LayerPath:
         self.v_out = torch.empty((n_kv_heads, self.sum_kept, head_dim), dtype=torch.bfloat16, device=dev)
         self.rank_ring = torch.zeros((l_obs, self.sum_T), dtype=torch.int32, device=dev)
         self.stat = torch.zeros((self.batch, C.sizeof(AslStat)), dtype=torch.uint8, device=dev)
-        self.side = torch.cuda.Stream(device=dev)       # rank statistic
-        self.side2 = torch.cuda.Stream(device=dev) if tail_streams >= 2 else self.side     # top-k and compaction
-        self._fork = torch.cuda.Event()
-        self._join = torch.cuda.Event()
-        self._join2 = torch.cuda.Event()
+        self.side = torch.cuda.Stream(device=dev)       # pooling and rank statistic
+        self.side2 = torch.cuda.Stream(device=dev)      # top-k and compaction
+        self._layer = AslLayer(_ptr(self.workspace), self.ws_bytes, (C.c_void_p * 2)(*map(_ptr, self._kv)),
+                               (C.c_void_p * 2)(*map(_ptr, self._agg)), _ptr(self.rank_ring), _ptr(self.stat), _ptr(self.idx),
+                               _ptr(self.k_out), _ptr(self.v_out), None, self.side.cuda_stream, self.side2.cuda_stream,
+                               1 if tail_streams < 2 else 0, 0)
+        self._layer_ref = C.byref(self._layer)
         self.first_layer: Optional[int] = None
         self.latch = False
 
@@ -322,9 +333,7 @@ class LayerPath:
         return self._agg[self._cur]
 
     def _fresh_events(self) -> None:
-        torch = self.torch
-        self._agg_free = [None, None]
-        self._fork, self._join, self._join2 = torch.cuda.Event(), torch.cuda.Event(), torch.cuda.Event()
+        _check(_lib.asl_run_reset(self.ctx), "asl_run_reset")
 
     def capture(self, steps):
         """Records ``run_layer`` for every ``(q_obs, k, v, layer_idx)`` (or ``(..., lse)``) of ``steps``,
@@ -348,10 +357,8 @@ class LayerPath:
         return graph
 
     def join(self) -> None:
-        """The current stream waits for the statistic work issued so far."""
-        cur = self.torch.cuda.current_stream()
-        cur.wait_event(self._join)
-        cur.wait_event(self._join2)
+        """The current stream waits for the work issued so far."""
+        _check(_lib.asl_run_join(self.ctx, self.torch.cuda.current_stream().cuda_stream), "asl_run_join")
 
     def close(self) -> None:
         if self.ctx:
@@ -375,46 +382,36 @@ class LayerPath:
         return min(self.l_obs, layer_idx - self.first_layer + 1)
 
     def run_layer(self, q_obs, k, v, layer_idx: int, *, overlap: bool = True, score_marks=None, lse=None) -> None:
-        """Steps a1..a5 for one layer on the current stream; with ``overlap`` the statistic
-        runs on the side stream and is left in flight (see ``join``).  ``score_marks``: a list
+        """Steps a1..a5 for one layer on the current stream; with ``overlap`` everything after the scoring
+        runs on the side streams and is left in flight (see ``join``).  ``score_marks``: a list
         that receives a (start, end) event pair around the scoring call."""
-        torch = self.torch
-        ctx, ws, wsb = self.ctx, self.workspace, self.ws_bytes
+        main = self.torch.cuda.current_stream()
         rows = self.n_rows(layer_idx)
-        main = torch.cuda.current_stream()
         if self.latch:
-            asl_set_layer(ctx, layer_idx)
+            asl_set_layer(self.ctx, layer_idx)
         self._cur ^= 1
-        agg, skv = self._agg[self._cur], self._kv[self._cur]
-        if self._agg_free[self._cur] is not None:
-            for done in self._agg_free[self._cur]:          # the side work of two layers ago has read them
-                main.wait_event(done)
         if score_marks is not None:
-            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0, e1 = (self.torch.cuda.Event(enable_timing=True) for _ in range(2))
             e0.record(main)
-        asl_score_columns(ctx, q_obs, k, lse, ws, wsb, self._cur)      # lse: the window rows' log-sum-exp, or None
-        if score_marks is not None:
+        if overlap:
+            self._layer.stream = main.cuda_stream
+            status = _lib.asl_run_layer(self.ctx, self._layer_ref, q_obs.data_ptr(), k.data_ptr(), v.data_ptr(),
+                                        _ptr(lse), layer_idx, rows, self._cur)
+            if status != ASL_OK:
+                raise AslError(status, "asl_run_layer")
+        else:
+            self.join()
+            asl_score_columns(self.ctx, q_obs, k, lse, self.workspace, self.ws_bytes, self._cur)
+        if score_marks is not None:                 # the call leaves nothing but the scoring on the main stream
             e1.record(main)
             score_marks.append((e0, e1))
         if overlap:
-            self._fork.record(main)
-            self.side.wait_event(self._fork)
-        asl_pool_scores(ctx, ws, wsb, self._cur, skv, agg, self.side if overlap else main)
-        if overlap and self.side2 is not self.side:
-            pooled = torch.cuda.Event()
-            pooled.record(self.side)
-            self.side2.wait_event(pooled)
-        s1, s2 = (self.side, self.side2) if overlap else (main, main)
-        asl_rank_stat(ctx, agg, layer_idx, rows, self.rank_ring, self.stat, ws, wsb, s1)
-        asl_select_topk(ctx, skv, self.H_k, self.idx, ws, wsb, s2)
-        asl_compact_kv(ctx, k, v, self.idx, self.k_out, self.v_out, s2)
-        if overlap:
-            d1, d2 = torch.cuda.Event(), torch.cuda.Event()
-            d1.record(self.side)
-            d2.record(self.side2)
-            self._agg_free[self._cur] = (d1, d2)
-            self._join.record(self.side)
-            self._join2.record(self.side2)
+            return
+        ctx, ws, wsb, agg, skv = self.ctx, self.workspace, self.ws_bytes, self._agg[self._cur], self._kv[self._cur]
+        asl_pool_scores(ctx, ws, wsb, self._cur, skv, agg, main)
+        asl_rank_stat(ctx, agg, layer_idx, rows, self.rank_ring, self.stat, ws, wsb, main)
+        asl_select_topk(ctx, skv, self.H_k, self.idx, ws, wsb, main)
+        asl_compact_kv(ctx, k, v, self.idx, self.k_out, self.v_out, main)
 
     def read_stat(self) -> np.ndarray:
         """Device -> host copy of the [B] statistic records (synchronises)."""

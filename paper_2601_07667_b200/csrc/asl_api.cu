@@ -52,6 +52,8 @@ asl_status asl_destroy(asl_ctx* c) {
   if (!c) return ASL_ERR_INVALID;
   free_plan(c);
   if (c->d_err) cudaFree(c->d_err);
+  for (cudaEvent_t e : {c->ev_scored, c->ev_pooled, c->ev_done[0][0], c->ev_done[0][1], c->ev_done[1][0], c->ev_done[1][1]})
+    if (e) cudaEventDestroy(e);
   delete c;
   return ASL_OK;
 }
@@ -180,7 +182,7 @@ asl_status asl_plan_sizes(const asl_ctx* c, int64_t* sum_tokens, int64_t* sum_T,
 
 // scoring alone: un-pooled column sums into slot `slot` of the workspace
 static asl_status score_columns_impl(asl_ctx* c, const void* q_obs, const void* k, const float* lse, void* workspace,
-                                     size_t workspace_bytes, int slot, void* stream) {
+                                     size_t workspace_bytes, int slot, bool beside, void* stream) {
   if (!c || !c->planned || !q_obs || !k || slot < 0 || slot > 1) return ASL_ERR_INVALID;
   if (!aligned16(q_obs) || !aligned16(k)) return ASL_ERR_INVALID;
   if (!workspace || workspace_bytes < c->ws.total || !aligned16(workspace)) return ASL_ERR_WORKSPACE;
@@ -190,10 +192,10 @@ static asl_status score_columns_impl(asl_ctx* c, const void* q_obs, const void* 
   // flags once and writes the launch's work list without their phases, so that every CTA of the
   // persistent kernel walks the same list
   if (c->latch_stat && c->cur_layer >= 0 && c->p.batch <= ASL_SKIP_MAX_BATCH) {
-    const asl_status s = asl_launch_live_phases(c, lse == nullptr, static_cast<cudaStream_t>(stream));
+    const asl_status s = asl_launch_live_phases(c, lse == nullptr, beside, static_cast<cudaStream_t>(stream));
     if (s != ASL_OK) return s;
   }
-  return asl_launch_score_tc(c, q_obs, k, lse, u, ws, static_cast<cudaStream_t>(stream));
+  return asl_launch_score_tc(c, q_obs, k, lse, u, ws, beside, static_cast<cudaStream_t>(stream));
 }
 
 static asl_status pool_scores_impl(asl_ctx* c, void* workspace, size_t workspace_bytes, int slot, float* scores_kv,
@@ -207,20 +209,20 @@ static asl_status pool_scores_impl(asl_ctx* c, void* workspace, size_t workspace
 asl_status asl_score_layer(asl_ctx* c, const void* q_obs, const void* k, float* scores_kv, float* scores_agg,
                            void* workspace, size_t workspace_bytes, void* stream) {
   if (!scores_kv || !scores_agg) return ASL_ERR_INVALID;
-  const asl_status s = score_columns_impl(c, q_obs, k, nullptr, workspace, workspace_bytes, 0, stream);
+  const asl_status s = score_columns_impl(c, q_obs, k, nullptr, workspace, workspace_bytes, 0, false, stream);
   return s != ASL_OK ? s : pool_scores_impl(c, workspace, workspace_bytes, 0, scores_kv, scores_agg, stream);
 }
 
 asl_status asl_score_layer_lse(asl_ctx* c, const void* q_obs, const void* k, const float* lse, float* scores_kv,
                                float* scores_agg, void* workspace, size_t workspace_bytes, void* stream) {
   if (!lse || !scores_kv || !scores_agg) return ASL_ERR_INVALID;
-  const asl_status s = score_columns_impl(c, q_obs, k, lse, workspace, workspace_bytes, 0, stream);
+  const asl_status s = score_columns_impl(c, q_obs, k, lse, workspace, workspace_bytes, 0, false, stream);
   return s != ASL_OK ? s : pool_scores_impl(c, workspace, workspace_bytes, 0, scores_kv, scores_agg, stream);
 }
 
 asl_status asl_score_columns(asl_ctx* c, const void* q_obs, const void* k, const float* lse, void* workspace,
                              size_t workspace_bytes, int32_t slot, void* stream) {
-  return score_columns_impl(c, q_obs, k, lse, workspace, workspace_bytes, slot, stream);
+  return score_columns_impl(c, q_obs, k, lse, workspace, workspace_bytes, slot, true, stream);
 }
 
 asl_status asl_pool_scores(asl_ctx* c, void* workspace, size_t workspace_bytes, int32_t slot, float* scores_kv,
@@ -270,6 +272,52 @@ asl_status asl_set_controller(asl_ctx* c, int32_t mode) {
 asl_status asl_set_layer(asl_ctx* c, int32_t layer_idx) {
   if (!c || layer_idx < 0) return ASL_ERR_INVALID;
   c->cur_layer = layer_idx;
+  return ASL_OK;
+}
+
+asl_status asl_run_layer(asl_ctx* c, const asl_layer* l, const void* q_obs, const void* k, const void* v, const float* lse,
+                         int32_t layer_idx, int32_t n_rows, int32_t slot) {
+  if (!c || !l || slot < 0 || slot > 1) return ASL_ERR_INVALID;
+  const cudaStream_t main = static_cast<cudaStream_t>(l->stream), s1 = static_cast<cudaStream_t>(l->side), s2 = static_cast<cudaStream_t>(l->side2);
+  if (!c->ev_scored) {
+    for (cudaEvent_t* e : {&c->ev_scored, &c->ev_pooled, &c->ev_done[0][0], &c->ev_done[0][1], &c->ev_done[1][0], &c->ev_done[1][1]})
+      ASL_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+  }
+  if (c->pending[slot])                             // the work of two layers ago has read the slot's buffers
+    for (cudaEvent_t e : c->ev_done[slot]) ASL_CUDA(cudaStreamWaitEvent(main, e, 0));
+  asl_status st = asl_score_columns(c, q_obs, k, lse, l->workspace, l->workspace_bytes, slot, l->stream);
+  if (st != ASL_OK) return st;
+  ASL_CUDA(cudaEventRecord(c->ev_scored, main));
+  ASL_CUDA(cudaStreamWaitEvent(s1, c->ev_scored, 0));
+  st = asl_pool_scores(c, l->workspace, l->workspace_bytes, slot, l->scores_kv[slot], l->scores_agg[slot], l->side);
+  if (st != ASL_OK) return st;
+  ASL_CUDA(cudaEventRecord(c->ev_pooled, s1));
+  ASL_CUDA(cudaStreamWaitEvent(s2, c->ev_pooled, 0));
+  st = asl_rank_stat(c, l->scores_agg[slot], layer_idx, n_rows, l->rank_ring, l->stat, l->workspace, l->workspace_bytes, l->side);
+  if (st != ASL_OK) return st;
+  st = asl_select_topk(c, l->scores_kv[slot], c->p.n_kv_heads, l->idx, l->workspace, l->workspace_bytes, l->side2);
+  if (st != ASL_OK) return st;
+  st = asl_compact_kv(c, k, v, l->idx, l->k_out, l->v_out, l->side2);
+  if (st != ASL_OK) return st;
+  ASL_CUDA(cudaEventRecord(c->ev_done[slot][1], s2));
+  if (l->one_side) ASL_CUDA(cudaStreamWaitEvent(s1, c->ev_done[slot][1], 0));
+  ASL_CUDA(cudaEventRecord(c->ev_done[slot][0], s1));
+  c->pending[slot] = true;
+  c->last_slot = slot;
+  return ASL_OK;
+}
+
+asl_status asl_run_join(asl_ctx* c, void* stream) {
+  if (!c) return ASL_ERR_INVALID;
+  if (c->last_slot < 0 || !c->pending[c->last_slot]) return ASL_OK;
+  for (cudaEvent_t e : c->ev_done[c->last_slot]) ASL_CUDA(cudaStreamWaitEvent(static_cast<cudaStream_t>(stream), e, 0));
+  return ASL_OK;
+}
+
+asl_status asl_run_reset(asl_ctx* c) {
+  if (!c) return ASL_ERR_INVALID;
+  c->pending[0] = c->pending[1] = false;
+  c->last_slot = -1;
   return ASL_OK;
 }
 

@@ -62,6 +62,10 @@ struct asl_ctx {
   bool topk_one_cta = false;          // the per-head top-k runs as one CTA per segment (asl_topk_plan)
   AslWorkspace ws{};
   int64_t launches = 0;
+  // asl_run_layer: order between a layer's streams, and when the buffers of a slot are free again
+  cudaEvent_t ev_scored = nullptr, ev_pooled = nullptr, ev_done[2][2] = {};
+  bool pending[2] = {false, false};   // the slot's ev_done have been recorded since asl_run_reset
+  int last_slot = -1;
 };
 
 // Under ASL_CONTROLLER_LATCH a request is finished at layer `cur` once its record selected at an
@@ -118,10 +122,10 @@ void asl_tc_free(asl_ctx* c);
 size_t asl_tc_partial_bytes(const asl_ctx* c);
 asl_status asl_tc_reset_sync(asl_ctx* c, cudaStream_t st);
 asl_status asl_launch_wait_selftest(asl_ctx* c, int which, unsigned long long limit_ns, cudaStream_t st);
-asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const float* lse, float* u, char* ws,
+asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const float* lse, float* u, char* ws, bool beside,
                                cudaStream_t st);
 asl_status asl_launch_pool(asl_ctx* c, const float* u, float* scores_kv, float* scores_agg, cudaStream_t st);
-asl_status asl_launch_live_phases(asl_ctx* c, bool two_pass, cudaStream_t st);
+asl_status asl_launch_live_phases(asl_ctx* c, bool two_pass, bool beside, cudaStream_t st);
 asl_status asl_launch_rank(asl_ctx* c, const float* agg, int32_t layer_idx, int32_t n_rows, int32_t* ring,
                            asl_stat* stat, char* ws, cudaStream_t st);
 asl_status asl_launch_topk(asl_ctx* c, const float* scores, int32_t n_heads, int32_t* idx_out, const asl_stat* gate,

@@ -1185,10 +1185,18 @@ struct HostList {
   std::vector<TcStage> stages;
   std::vector<TcFold> folds;
   int32_t most = 0;                        // tiles of the largest group in pass 2
+  int grid = 1;                            // CTAs
 };
-HostList deal(const std::vector<TcRun>& segs, const std::vector<int>& cut, const asl_ctx* c, int grid, bool one_pass) {
+HostList deal(const std::vector<TcRun>& segs, const std::vector<int>& cut, const asl_ctx* c, int most_ctas, bool one_pass) {
   HostList l;
   const int ng = (int)cut.size() - 1;
+  // no more CTAs than the largest group has tiles: what has no work leaves its SM to others from the start
+  for (int g = 0; g < ng; ++g) {
+    int64_t N = 0;
+    for (int s = cut[g]; s < cut[g + 1]; ++s) N += (c->req[segs[s].b].n + KT - 1) / KT;
+    if (N > l.grid) l.grid = N < most_ctas ? (int)N : most_ctas;
+  }
+  const int grid = l.grid;
   l.folds.resize(segs.size());
   std::vector<int> at[2];                  // first run of each group
   for (int p = one_pass ? 1 : 0; p < 2; ++p)
@@ -1246,7 +1254,6 @@ bool asl_tc_plan(asl_ctx* c) {
   const int W = p.window, G = p.n_q_heads / p.n_kv_heads;
   if (p.k_dtype == ASL_K_FP8_E4M3 && !fp8_shape(p)) return false;
   plan_chunks(p, tp);
-  tp.grid = (p.score_ctas > 0 && p.score_ctas < c->sm_count) ? p.score_ctas : c->sm_count;
 
   // segments in (request, head, chunk) order
   std::vector<TcRun> segs;
@@ -1290,7 +1297,17 @@ bool asl_tc_plan(asl_ctx* c) {
     }
     cut.push_back(tp.nseg);
   }
-  const HostList lists[2] = {deal(segs, cut, c, tp.grid, false), deal(segs, {0, tp.nseg}, c, tp.grid, true)};
+  // CTAs: as many as the caller says; else one per SM, and where the call is one half of a layer (asl_score_columns) 16
+  // fewer, so that the rest of the layer before runs beside it, 32 fewer for the shorter one-pass call with one chunk
+  // per kv head
+  const int given = p.score_ctas > 0 && p.score_ctas < c->sm_count ? p.score_ctas : 0;
+  const int spare[2] = {16, tp.nchunk == 1 ? 32 : 16};
+  const int n_lists = given || p.score_ctas > 0 ? 2 : 4;
+  HostList lists[4];
+  for (int i = 0; i < n_lists; ++i) {
+    const int ctas = given ? given : (i < 2 || c->sm_count <= 2 * spare[i & 1] ? c->sm_count : c->sm_count - spare[i & 1]);
+    lists[i] = (i & 1) ? deal(segs, {0, tp.nseg}, c, ctas, true) : deal(segs, cut, c, ctas, false);
+  }
 
   // one allocation for everything the kernels read or count in
   size_t bytes = 0;
@@ -1302,27 +1319,32 @@ bool asl_tc_plan(asl_ctx* c) {
     if (n) memcpy(host.data() + at, data, n);
     return at;
   };
-  struct ListAt { size_t runs, first, stages, folds; } at[2];
-  TcList* out[2] = {&tp.both, &tp.only2};
-  for (int i = 0; i < 2; ++i) {
+  struct ListAt { size_t runs, first, stages, folds; } at[4];
+  size_t n_runs = 0, groups = 0, ctas = 0;                    // of the longest lists
+  for (int i = 0; i < n_lists; ++i) {
     const HostList& l = lists[i];
-    out[i]->n1 = (int32_t)l.runs[0].size();
-    out[i]->n2 = (int32_t)l.runs[1].size();
-    out[i]->n_groups = (int32_t)l.stages.size();
-    out[i]->most = l.most;
+    TcList& out = tp.lists[i >> 1][i & 1];
+    out.grid = l.grid;
+    out.n1 = (int32_t)l.runs[0].size();
+    out.n2 = (int32_t)l.runs[1].size();
+    out.n_groups = (int32_t)l.stages.size();
+    out.most = l.most;
     std::vector<TcRun> runs(l.runs[0]);
     runs.insert(runs.end(), l.runs[1].begin(), l.runs[1].end());
     at[i] = ListAt{put(runs.data(), runs.size() * sizeof(TcRun)), put(l.first.data(), l.first.size() * sizeof(int32_t)),
                    put(l.stages.data(), l.stages.size() * sizeof(TcStage)), put(l.folds.data(), l.folds.size() * sizeof(TcFold))};
+    if (runs.size() > n_runs) n_runs = runs.size();
+    if (l.stages.size() > groups) groups = l.stages.size();
+    if ((size_t)l.grid > ctas) ctas = l.grid;
+    if (out.n1 > tp.partial_slots) tp.partial_slots = out.n1;
   }
   const size_t sync_words = (4 * (size_t)tp.nseg + 1) * SYNC_STRIDE;
   const std::vector<uint32_t> zeros(sync_words, 0);
   const size_t sync_at = put(zeros.data(), sync_words * sizeof(uint32_t));
   const size_t host_bytes = bytes;
   auto take = [&](size_t n) { const size_t t = bytes; bytes = asl_align256(bytes + n); return t; };
-  const size_t n_runs = (size_t)tp.both.n1 + tp.both.n2;      // the longer list
-  const size_t live_at[5] = {take(n_runs * sizeof(TcRun)), take((size_t)tp.grid * sizeof(int32_t)), take((size_t)tp.nseg * sizeof(TcFold)),
-                             take((3 * n_runs + 6 * (size_t)tp.both.n_groups + 4 * (size_t)(tp.both.n_groups + 1) * tp.grid) * sizeof(int32_t)),
+  const size_t live_at[5] = {take(n_runs * sizeof(TcRun)), take(ctas * sizeof(int32_t)), take((size_t)tp.nseg * sizeof(TcFold)),
+                             take((3 * n_runs + 6 * groups + 4 * (groups + 1) * ctas) * sizeof(int32_t)),
                              take(sizeof(int32_t))};
   cudaError_t e = cudaMalloc(&tp.d_blob, bytes);
   if (e == cudaSuccess) e = cudaMemcpy(tp.d_blob, host.data(), host_bytes, cudaMemcpyHostToDevice);
@@ -1330,12 +1352,14 @@ bool asl_tc_plan(asl_ctx* c) {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kern.smem);
   if (e != cudaSuccess) { cudaGetLastError(); asl_tc_free(c); return false; }
   char* d = static_cast<char*>(tp.d_blob);
-  for (int i = 0; i < 2; ++i) {
-    out[i]->d_runs = reinterpret_cast<TcRun*>(d + at[i].runs);
-    out[i]->d_first = reinterpret_cast<int32_t*>(d + at[i].first);
-    out[i]->d_stages = reinterpret_cast<TcStage*>(d + at[i].stages);
-    out[i]->d_folds = reinterpret_cast<TcFold*>(d + at[i].folds);
+  for (int i = 0; i < n_lists; ++i) {
+    TcList& out = tp.lists[i >> 1][i & 1];
+    out.d_runs = reinterpret_cast<TcRun*>(d + at[i].runs);
+    out.d_first = reinterpret_cast<int32_t*>(d + at[i].first);
+    out.d_stages = reinterpret_cast<TcStage*>(d + at[i].stages);
+    out.d_folds = reinterpret_cast<TcFold*>(d + at[i].folds);
   }
+  if (n_lists == 2) { tp.lists[1][0] = tp.lists[0][0]; tp.lists[1][1] = tp.lists[0][1]; }
   tp.d_sync = reinterpret_cast<uint32_t*>(d + sync_at);
   tp.d_live_runs = reinterpret_cast<TcRun*>(d + live_at[0]);
   tp.d_live_first = reinterpret_cast<int32_t*>(d + live_at[1]);
@@ -1346,7 +1370,7 @@ bool asl_tc_plan(asl_ctx* c) {
   return tp.enabled;
 }
 
-size_t asl_tc_partial_bytes(const asl_ctx* c) { return (size_t)c->tc.both.n1 * (c->tc.wide ? GROUPS / 2 : GROUPS) * c->tc.NC * sizeof(float2); }
+size_t asl_tc_partial_bytes(const asl_ctx* c) { return (size_t)c->tc.partial_slots * (c->tc.wide ? GROUPS / 2 : GROUPS) * c->tc.NC * sizeof(float2); }
 
 void asl_tc_free(asl_ctx* c) {
   AslTcPlan& tp = c->tc;
@@ -1371,11 +1395,11 @@ asl_status asl_launch_window_lse(asl_ctx* c, const char* ws, float* lse_out, cud
   return ASL_OK;
 }
 
-asl_status asl_launch_live_phases(asl_ctx* c, bool two_pass, cudaStream_t st) {
+asl_status asl_launch_live_phases(asl_ctx* c, bool two_pass, bool beside, cudaStream_t st) {
   AslTcPlan& tp = c->tc;
-  const TcList& l = two_pass ? tp.both : tp.only2;
+  const TcList& l = tp.lists[beside][!two_pass];
   live_list_kernel<<<1, 1024, 0, st>>>(l.d_runs, l.n1, l.n2, l.d_folds, tp.nseg, l.n_groups, l.most + l.most / 4, c->latch_stat, c->cur_layer,
-                                       c->p.batch, tp.grid, tp.d_live_hdr, tp.d_live_runs, tp.d_live_first, tp.d_live_folds, tp.d_live_scratch);
+                                       c->p.batch, l.grid, tp.d_live_hdr, tp.d_live_runs, tp.d_live_first, tp.d_live_folds, tp.d_live_scratch);
   c->launches += 1;
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;
@@ -1389,7 +1413,7 @@ asl_status asl_tc_reset_sync(asl_ctx* c, cudaStream_t st) {
   return ASL_OK;
 }
 
-asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const float* lse, float* u, char* ws,
+asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const float* lse, float* u, char* ws, bool beside,
                                cudaStream_t st) {
   const asl_params& p = c->p;
   AslTcPlan& tp = c->tc;
@@ -1424,7 +1448,7 @@ asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const f
     if (!make_map(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, k, 3, kdims, kstr, kbox)) return ASL_ERR_CUDA;
   }
   TcArgs a{};
-  const TcList& list = lse ? tp.only2 : tp.both;
+  const TcList& list = tp.lists[beside][lse != nullptr];
   a.list = {list.d_runs, list.d_first, list.d_folds};
   if (c->latch_stat && c->cur_layer >= 0 && p.batch <= ASL_SKIP_MAX_BATCH) {      // written by asl_launch_live_phases just before
     a.live = {tp.d_live_runs, tp.d_live_first, tp.d_live_folds};
@@ -1447,7 +1471,7 @@ asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const f
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)p.head_dim));
   // every CTA must be resident at once (pass 2 waits for counters other CTAs advance): one CTA per SM at most
   const ScoreKernel& kern = score_kernel(score_kernel_of(p, tp));
-  kern.fn<<<tp.grid, THREADS, kern.smem, st>>>(tm_q, tm_k, a);
+  kern.fn<<<list.grid, THREADS, kern.smem, st>>>(tm_q, tm_k, a);
   c->launches += 1;
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;

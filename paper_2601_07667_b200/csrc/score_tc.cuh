@@ -27,6 +27,7 @@ struct __align__(16) TcStage { int32_t seg0, nseg, pad0, pad1; };
 struct __align__(16) TcFold { int32_t slot0, nruns, rows, b; };
 
 struct TcList {                  // a work list on the device: runs of pass 1, then of pass 2
+  int32_t grid = 0;              // CTAs it is dealt to
   int32_t n1 = 0, n2 = 0, n_groups = 0;
   int32_t most = 0;              // tiles of the largest group
   TcRun* d_runs = nullptr;
@@ -45,8 +46,9 @@ struct AslTcPlan {
   int pieces = 0;       // chunks per query head (windows of more than 256 rows), else 1
   int nchunk = 0;       // chunks per kv head
   int nseg = 0;         // segments
-  int grid = 0;         // CTAs of the persistent kernel (one per SM)
-  TcList both, only2;   // both passes; the pass-2 phases alone (scoring with a supplied log-sum-exp)
+  // [0]: a call on its own; [1]: a call that other kernels should find room beside (asl_score_columns).  The same where
+  // the caller gives the number of CTAs.  [][0]: both passes; [][1]: pass 2 alone (a supplied log-sum-exp).
+  TcList lists[2][2];
   void* d_blob = nullptr;       // the device side of the lists below and above, one allocation
   uint32_t* d_sync = nullptr;   // two sets of publish and folded-row counters, launch number, ticket of arrived CTAs
   // device-side controller: the next launch's list without the finished requests' phases, written ahead of it
@@ -55,4 +57,5 @@ struct AslTcPlan {
   TcFold* d_live_folds = nullptr;
   int32_t* d_live_hdr = nullptr;
   int32_t* d_live_scratch = nullptr;
+  int64_t partial_slots = 0;    // pass-1 runs of the longest list
 };
