@@ -84,7 +84,7 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
   if (p->cu_seqlens[0] != 0) return ASL_ERR_INVALID;
 
   std::vector<AslReq> req(p->batch);
-  int64_t sum_T = 0, sum_kept = 0;
+  int64_t sum_T = 0, sum_kept = 0, u_stride = 0;
   int32_t max_n = 0, max_T = 0, max_kept = 0;
   for (int b = 0; b < p->batch; ++b) {
     const int64_t n = (int64_t)p->cu_seqlens[b + 1] - p->cu_seqlens[b];
@@ -98,8 +98,9 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
     r.tok_off = p->cu_seqlens[b];
     r.t_off = (int32_t)sum_T;
     r.kept_off = (int32_t)sum_kept;
-    r.pad = 0;
+    r.u_off = (int32_t)u_stride;
     sum_T += r.T;
+    u_stride += (r.T + 3) / 4 * 4;
     sum_kept += r.kept;
     max_n = r.n > max_n ? r.n : max_n;
     max_T = r.T > max_T ? r.T : max_T;
@@ -108,7 +109,7 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
     const double m_max = fmin((double)r.T, (double)(r.k > 0 ? r.k : 1) * p->l_obs);
     if (m_max * p->l_obs * p->l_obs * (double)r.T * (double)r.T / 4.0 >= 9.0e18) return ASL_ERR_UNSUPPORTED;
   }
-  if (sum_T >= (int64_t)1 << 31 || (int64_t)p->cu_seqlens[p->batch] >= (int64_t)1 << 31) return ASL_ERR_UNSUPPORTED;
+  if (u_stride >= (int64_t)1 << 31 || (int64_t)p->cu_seqlens[p->batch] >= (int64_t)1 << 31) return ASL_ERR_UNSUPPORTED;
 
   int prev = 0;
   cudaGetDevice(&prev);
@@ -134,6 +135,7 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
   c->req = req;
   c->sum_tokens = p->cu_seqlens[p->batch];
   c->sum_T = sum_T;
+  c->u_stride = u_stride;
   c->sum_kept = sum_kept;
   c->max_n = max_n; c->max_T = max_T; c->max_kept = max_kept;
   c->rows_per_kv = (p->n_q_heads / p->n_kv_heads) * p->window;
@@ -155,7 +157,7 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
   w.score_partials = off; off = asl_align256(off + asl_tc_partial_bytes(c));
   w.score_offsets = off;  off = asl_align256(off + (size_t)c->tc.nseg * c->tc.NC * sizeof(float));
   const size_t u_rows = (size_t)p->n_kv_heads * c->u_rows_per_kv;
-  for (int i = 0; i < 2; ++i) { w.score_u[i] = off; off = asl_align256(off + u_rows * (size_t)sum_T * sizeof(float)); }
+  for (int i = 0; i < 2; ++i) { w.score_u[i] = off; off = asl_align256(off + u_rows * (size_t)u_stride * sizeof(float)); }
   w.score_q8 = off;
   if (fp8) off = asl_align256(off + (size_t)2 * p->batch * p->n_q_heads * p->window * p->head_dim);
   w.score_end = off;

@@ -17,7 +17,7 @@ struct AslReq {
   int32_t tok_off;   // cu_seqlens[b]
   int32_t t_off;     // offset of the request's past segment in packed score vectors
   int32_t kept_off;  // offset of the request's segment in packed kept lists
-  int32_t pad;
+  int32_t u_off;     // offset of the request in the rows of un-pooled column sums (a multiple of 4)
 };
 
 // Scratch layout inside the caller's workspace (byte offsets, 256-aligned).
@@ -49,6 +49,7 @@ struct asl_ctx {
   int k_elem_bytes = 2;               // bytes per K element
   std::vector<AslReq> req;
   int64_t sum_tokens = 0, sum_T = 0, sum_kept = 0;
+  int64_t u_stride = 0;               // length of a row of un-pooled column sums: every request starts on 16 bytes
   int32_t max_n = 0, max_T = 0, max_kept = 0;
   AslReq* d_req = nullptr;            // device [B]
   unsigned long long* d_acc = nullptr;  // device [B][2] integer accumulators of the statistic + a block counter

@@ -1,67 +1,136 @@
 // 1-D pooling, GQA group sum and all-head aggregate (Algorithm 1 (1-D pooling, SumGroups) and
-// the "scores" sum of Section 4.1).  One thread per past token walks the kv
-// heads, so the aggregate needs no atomics and is bit-reproducible.
-//   average pooling: input is group-summed column sums, `urows` rows per kv head
-//                    (one per row chunk of the scorer) that are added first
-//                    (pooling is linear, so summing the group first is the same
-//                    up to rounding); zero padding, divisor always S.
-//   max pooling:     input is per query head, `parts` consecutive rows of partial
-//                    sums each, u[H_q][parts][sum_T]; each head is pooled over its
-//                    in-range taps, then the group is summed.
+// the "scores" sum of Section 4.1).  A thread walks all heads of its tokens, so the
+// aggregate needs no atomics and is bit-reproducible.  A "unit" is what gets pooled as one
+// row: a kv head's group-summed sums (average pooling) or one query head's sums (max
+// pooling); the scorer stores it as `nrows` consecutive partial rows that are added first.
+//   average pooling: pooling is linear, so summing the group first is the same up to
+//                    rounding; zero padding, divisor always S.
+//   max pooling:     each head is pooled over its in-range taps, then the group is summed.
 // Taps never cross a request's past segment [0, T_b).
 #include "asl_internal.cuh"
 
 namespace {
 
-constexpr int PT = 256;          // tokens per block
-constexpr int MAX_HALO = 16;     // pooling kernels up to 33 taps go through shared memory
+constexpr int PT = 256;          // threads of a block / tokens per block of the general kernel
+constexpr int MAX_HALO = 16;     // pooling kernels up to 33 taps
+constexpr int HB = 8;            // general kernel: staged units per round
+constexpr int PV_ROWS = 16;      // vector kernel: partial rows in flight per lane
 
-constexpr int HB = 8;            // staged rows per round: their loads are all in flight together
+struct PoolArgs {
+  const float* u;                // [rows][u_stride], every request from a 16-byte boundary on
+  const AslReq* req;
+  int64_t u_stride, sum_T;
+  int32_t Hk, G, S, mode, nrows; // nrows: partial rows per unit
+  const asl_stat* latch;
+  int32_t cur_layer, vec_out;    // vec_out: every request starts on 16 bytes in the outputs too
+  float* scores_kv;
+  float* scores_agg;
+};
 
-// One block pools PT consecutive past tokens of one request.  A "unit" is what
-// gets pooled as one row: a kv head's group-summed sums (average pooling) or one
-// query head's sums (max pooling); it is stored as `nrows` consecutive partial
-// rows of u that are added on the way into shared memory.  HB units are staged
-// per round with their halo, pooled from there, and added up per kv head and
-// over all heads in a fixed order: no atomics, bit-reproducible.
-__global__ void __launch_bounds__(PT + 2 * MAX_HALO) pool_group_kernel(const float* __restrict__ u, const AslReq* __restrict__ req,
-                                                        int Hk, int G, int S, int mode, int urows, int parts, int64_t sum_T,
-                                                        const asl_stat* __restrict__ latch, int cur_layer,
-                                                        float* __restrict__ scores_kv, float* __restrict__ scores_agg) {
+// Windows of up to 9 taps, units of 1, 2, 4, 8 or 16 partial rows.  A lane owns 4 consecutive tokens: one 16-byte load per
+// partial row, sixteen in flight, the rows of a unit added in order, the neighbours' sums fetched by warp shuffles; the
+// first and the last lane of a warp only supply the halo, so a warp pools 120 tokens.  No shared memory and no
+// block-wide barrier.  Bound by the round trips for the rows (one per sixteen): max pooling of 64 query
+// heads at 64K tokens 43 -> 10 us, eight ragged requests of 8 heads 25 -> 6.5 us against one thread per token with rows
+// staged in shared memory; 128K tokens of 8 heads, two partial rows each, 6.1 -> 4.4 us.
+template <bool MAX, int R, int NR>
+__global__ void __launch_bounds__(PT) pool_vec4_kernel(PoolArgs a) {
+  const int b = blockIdx.y;
+  if (a.latch && asl_finished(a.latch + b, a.cur_layer)) return;       // the request's scores stay as its selection layer left them
+  const AslReq rq = a.req[b];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int warp_of_segment = blockIdx.x * (PT / 32) + wid;
+  if (warp_of_segment * 120 >= rq.T) return;                           // the whole warp is past the segment
+  const int j0 = 4 * (warp_of_segment * 30 + lane - 1);                // lanes 0 and 31: halo only
+  const bool inside = j0 >= 0 && j0 < rq.T;
+  const bool owner = inside && lane >= 1 && lane <= 30;
+  const int live = rq.T - j0;                                          // tokens from j0 on (4 or more: all of the lane's)
+  const float outside = MAX ? -INFINITY : 0.f;
+  const float inv = 1.0f / (float)a.S;
+  const float* base = a.u + rq.u_off + j0;
+  const int per_head = MAX ? a.G : 1, units = a.Hk * per_head, rows = units * NR;
+  auto store = [&](float* dst, const float (&p)[4]) {
+    if (a.vec_out && live >= 4) *reinterpret_cast<float4*>(dst) = make_float4(p[0], p[1], p[2], p[3]);
+    else
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (t < live) dst[t] = p[t];
+  };
+  float agg[4] = {0.f, 0.f, 0.f, 0.f}, head[4] = {0.f, 0.f, 0.f, 0.f};
+  int in_head = 0, h = 0;
+  for (int r0 = 0; r0 < rows; r0 += PV_ROWS) {
+    float4 x[PV_ROWS];
+#pragma unroll
+    for (int e = 0; e < PV_ROWS; ++e)
+      x[e] = (inside && r0 + e < rows) ? __ldcg(reinterpret_cast<const float4*>(base + (int64_t)(r0 + e) * a.u_stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < PV_ROWS / NR; ++q) {
+      if (r0 + q * NR >= rows) break;
+      float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int e = 0; e < NR; ++e) { sum.x += x[q * NR + e].x; sum.y += x[q * NR + e].y; sum.z += x[q * NR + e].z; sum.w += x[q * NR + e].w; }
+      float v[12];                                                     // tokens j0-4 .. j0+7
+      v[4] = live > 0 && inside ? sum.x : outside; v[5] = live > 1 && inside ? sum.y : outside;
+      v[6] = live > 2 && inside ? sum.z : outside; v[7] = live > 3 && inside ? sum.w : outside;
+#pragma unroll
+      for (int d = 0; d < R; ++d) {
+        v[3 - d] = __shfl_up_sync(0xffffffffu, v[7 - d], 1);
+        v[8 + d] = __shfl_down_sync(0xffffffffu, v[4 + d], 1);
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        float p = MAX ? v[4 + t - R] : 0.f;
+#pragma unroll
+        for (int d = -R; d <= R; ++d) p = MAX ? fmaxf(p, v[4 + t + d]) : p + v[4 + t + d];
+        head[t] = MAX ? head[t] + p : p * inv;
+      }
+      if (++in_head == per_head) {
+        if (owner) store(a.scores_kv + (int64_t)h * a.sum_T + rq.t_off + j0, head);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) { agg[t] += head[t]; head[t] = 0.f; }
+        in_head = 0;
+        ++h;
+      }
+    }
+  }
+  if (owner) store(a.scores_agg + rq.t_off + j0, agg);
+}
+
+// Everything else: one block pools PT consecutive past tokens of one request, one thread per column of the tile (the
+// last 2 * MAX_HALO threads load the halo); HB units are staged per round in shared memory and pooled from there.
+__global__ void __launch_bounds__(PT + 2 * MAX_HALO) pool_group_kernel(PoolArgs a) {
   __shared__ float tile[HB][PT + 2 * MAX_HALO];
   const int b = blockIdx.y;
-  if (latch && asl_finished(latch + b, cur_layer)) return;      // the request's scores stay as its selection layer left them
-  const AslReq rq = req[b];
+  if (a.latch && asl_finished(a.latch + b, a.cur_layer)) return;
+  const AslReq rq = a.req[b];
   const int j0 = blockIdx.x * PT;
   if (j0 >= rq.T) return;
-  const int r = S / 2;
+  const int r = a.S / 2;
   const int j = j0 + threadIdx.x;
-  const bool live = threadIdx.x < PT && j < rq.T;      // the last 2 * MAX_HALO threads only load halo columns
+  const bool live = threadIdx.x < PT && j < rq.T;
   const int lo = max(0, j - r), hi = min(rq.T - 1, j + r);
-  const float inv = 1.0f / (float)S;
-  const bool avg = mode == ASL_POOL_AVG;
-  const int units = avg ? Hk : Hk * G;
-  const int nrows = avg ? urows : parts;
-  const int per_head = avg ? 1 : G;
+  const float inv = 1.0f / (float)a.S;
+  const bool avg = a.mode == ASL_POOL_AVG;
+  const int per_head = avg ? 1 : a.G, units = a.Hk * per_head;
   float agg = 0.f, p = 0.f;
   for (int u0 = 0; u0 < units; u0 += HB) {
     const int nb = min(HB, units - u0);
-    const int tot = nb * nrows;                       // rows u0*nrows .. u0*nrows + tot - 1 of u
+    const int tot = nb * a.nrows;                     // rows u0*nrows .. u0*nrows + tot - 1 of u
     __syncthreads();
     if (threadIdx.x < PT + 2 * r) {                     // one column of the tile per thread, halo included
       const int i = threadIdx.x;
       const int t = j0 - r + i;
       const bool inside = t >= 0 && t < rq.T;
-      const float* src = u + (int64_t)u0 * nrows * sum_T + rq.t_off + t;
+      const float* src = a.u + (int64_t)u0 * a.nrows * a.u_stride + rq.u_off + t;
 #pragma unroll
       for (int q = 0; q < HB; ++q) tile[q][i] = 0.f;
       for (int e0 = 0; e0 < tot; e0 += 16) {            // sixteen loads in flight
         float x[16];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) x[k] = (inside && e0 + k < tot) ? __ldcg(src + (int64_t)(e0 + k) * sum_T) : 0.f;
+        for (int k = 0; k < 16; ++k) x[k] = (inside && e0 + k < tot) ? __ldcg(src + (int64_t)(e0 + k) * a.u_stride) : 0.f;
 #pragma unroll
         for (int k = 0; k < 16; ++k)
-          if (e0 + k < tot) tile[(e0 + k) / nrows][i] += x[k];
+          if (e0 + k < tot) tile[(e0 + k) / a.nrows][i] += x[k];
       }
     }
     __syncthreads();
@@ -79,96 +148,57 @@ __global__ void __launch_bounds__(PT + 2 * MAX_HALO) pool_group_kernel(const flo
       }
       const int unit = u0 + q;
       if ((unit + 1) % per_head == 0) {
-        if (live) scores_kv[(int64_t)(unit / per_head) * sum_T + rq.t_off + j] = p;
+        if (live) a.scores_kv[(int64_t)(unit / per_head) * a.sum_T + rq.t_off + j] = p;
         agg += p;
         p = 0.f;
       }
     }
   }
-  if (live) scores_agg[rq.t_off + j] = agg;
+  if (live) a.scores_agg[rq.t_off + j] = agg;
 }
 
-// Average pooling without shared memory, for plans whose segments all start and end on 16-byte boundaries of the
-// score rows (T_b and the rows' length multiples of 4) and whose pooling window reaches at most 4 tokens to a
-// side.  A lane owns 4 consecutive tokens: one 16-byte load per partial row, all of a batch of rows in flight, the
-// rows of a kv head added in order, the neighbours' sums fetched by warp shuffles; the first and the last lane of
-// a warp only supply the halo, so a warp pools 120 tokens.  One round trip to memory and no block-wide barrier; the
-// sums are formed in the same order as in the kernel above, so the two give identical bits.
-constexpr int PV_ROWS = 16;      // partial rows in flight per lane
-
-__global__ void __launch_bounds__(PT) pool_avg_vec4_kernel(const float* __restrict__ u, const AslReq* __restrict__ req, int Hk, int S,
-                                                           int urows, int64_t sum_T, const asl_stat* __restrict__ latch, int cur_layer,
-                                                           float* __restrict__ scores_kv, float* __restrict__ scores_agg) {
-  const int b = blockIdx.y;
-  if (latch && asl_finished(latch + b, cur_layer)) return;
-  const AslReq rq = req[b];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int warp_of_segment = blockIdx.x * (PT / 32) + wid;
-  if (warp_of_segment * 120 >= rq.T) return;                           // the whole warp is past the segment
-  const int g = warp_of_segment * 30 + lane - 1;                       // group of 4 tokens; lanes 0 and 31: halo only
-  const int j0 = 4 * g;
-  const bool inside = g >= 0 && j0 < rq.T;
-  const bool owner = inside && lane >= 1 && lane <= 30;
-  const int r = S / 2;
-  const float inv = 1.0f / (float)S;
-  const float* base = u + rq.t_off + j0;
-  float agg[4] = {0.f, 0.f, 0.f, 0.f};
-  const int heads_per_batch = PV_ROWS / urows;                         // urows divides PV_ROWS (checked by the launcher)
-  for (int h0 = 0; h0 < Hk; h0 += heads_per_batch) {
-    float4 x[PV_ROWS];
-#pragma unroll
-    for (int e = 0; e < PV_ROWS; ++e) {
-      const int row = h0 * urows + e;
-      x[e] = (inside && row < Hk * urows) ? __ldcg(reinterpret_cast<const float4*>(base + (int64_t)row * sum_T)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    for (int hh = 0; hh < heads_per_batch && h0 + hh < Hk; ++hh) {
-      float v[12];                                                     // sums of tokens j0-4 .. j0+7
-      float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int e = 0; e < PV_ROWS; ++e)
-        if (e / urows == hh) { sum.x += x[e].x; sum.y += x[e].y; sum.z += x[e].z; sum.w += x[e].w; }
-      v[4] = sum.x; v[5] = sum.y; v[6] = sum.z; v[7] = sum.w;
-      v[0] = __shfl_up_sync(0xffffffffu, sum.x, 1); v[1] = __shfl_up_sync(0xffffffffu, sum.y, 1);
-      v[2] = __shfl_up_sync(0xffffffffu, sum.z, 1); v[3] = __shfl_up_sync(0xffffffffu, sum.w, 1);
-      v[8] = __shfl_down_sync(0xffffffffu, sum.x, 1); v[9] = __shfl_down_sync(0xffffffffu, sum.y, 1);
-      v[10] = __shfl_down_sync(0xffffffffu, sum.z, 1); v[11] = __shfl_down_sync(0xffffffffu, sum.w, 1);
-      float p[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        float acc = 0.f;
-#pragma unroll
-        for (int d = -4; d <= 4; ++d)
-          if (d >= -r && d <= r) acc += v[4 + t + d];                  // tokens outside the segment hold 0: zero padding
-        p[t] = acc * inv;
-        agg[t] += p[t];
-      }
-      if (owner) *reinterpret_cast<float4*>(scores_kv + (int64_t)(h0 + hh) * sum_T + rq.t_off + j0) = make_float4(p[0], p[1], p[2], p[3]);
-    }
+using PoolKernel = void (*)(PoolArgs);
+template <bool MAX, int R>
+PoolKernel pool_vec4_rows(int nrows) {
+  switch (nrows) {
+    case 1: return pool_vec4_kernel<MAX, R, 1>;
+    case 2: return pool_vec4_kernel<MAX, R, 2>;
+    case 4: return pool_vec4_kernel<MAX, R, 4>;
+    case 8: return pool_vec4_kernel<MAX, R, 8>;
+    case 16: return pool_vec4_kernel<MAX, R, 16>;
   }
-  if (owner) *reinterpret_cast<float4*>(scores_agg + rq.t_off + j0) = make_float4(agg[0], agg[1], agg[2], agg[3]);
+  return nullptr;
+}
+template <bool MAX>
+PoolKernel pool_vec4_of(int r, int nrows) {
+  switch (r) {
+    case 0: return pool_vec4_rows<MAX, 0>(nrows);
+    case 1: return pool_vec4_rows<MAX, 1>(nrows);
+    case 2: return pool_vec4_rows<MAX, 2>(nrows);
+    case 3: return pool_vec4_rows<MAX, 3>(nrows);
+    case 4: return pool_vec4_rows<MAX, 4>(nrows);
+  }
+  return nullptr;
 }
 
 }  // namespace
 
 asl_status asl_launch_pool(asl_ctx* c, const float* u, float* scores_kv, float* scores_agg, cudaStream_t st) {
   const asl_params& p = c->p;
-  if (p.pool_kernel / 2 > MAX_HALO) return ASL_ERR_UNSUPPORTED;
-  const int urows = c->u_rows_per_kv;
-  bool vec4 = p.pool_mode == ASL_POOL_AVG && p.pool_kernel / 2 <= 4 && urows <= PV_ROWS && PV_ROWS % urows == 0 && c->sum_T % 4 == 0 &&
-              ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(scores_kv) | reinterpret_cast<uintptr_t>(scores_agg)) & 15) == 0;
-  for (const AslReq& r : c->req) vec4 = vec4 && r.T % 4 == 0 && r.t_off % 4 == 0;
-  if (vec4) {
-    const int warps = c->max_T > 0 ? (c->max_T + 119) / 120 : 1;
-    pool_avg_vec4_kernel<<<dim3((warps + PT / 32 - 1) / (PT / 32), p.batch), PT, 0, st>>>(
-        u, c->d_req, p.n_kv_heads, p.pool_kernel, urows, c->sum_T, c->latch_stat, c->cur_layer, scores_kv, scores_agg);
-    c->launches += 1;
-    ASL_CUDA(cudaGetLastError());
-    return ASL_OK;
+  const int r = p.pool_kernel / 2;
+  if (r > MAX_HALO) return ASL_ERR_UNSUPPORTED;
+  const bool max = p.pool_mode == ASL_POOL_MAX;
+  const int nrows = max ? c->u_parts : c->u_rows_per_kv;
+  bool vec_out = c->sum_T % 4 == 0 && ((reinterpret_cast<uintptr_t>(scores_kv) | reinterpret_cast<uintptr_t>(scores_agg)) & 15) == 0;
+  for (const AslReq& q : c->req) vec_out = vec_out && q.t_off % 4 == 0;
+  const PoolArgs a{u, c->d_req, c->u_stride, c->sum_T, p.n_kv_heads, p.n_q_heads / p.n_kv_heads, p.pool_kernel, p.pool_mode, nrows,
+                   c->latch_stat, c->cur_layer, vec_out, scores_kv, scores_agg};
+  if (const PoolKernel vec4 = max ? pool_vec4_of<true>(r, nrows) : pool_vec4_of<false>(r, nrows)) {
+    const int warps = (c->max_T + 119) / 120;
+    vec4<<<dim3((warps + PT / 32 - 1) / (PT / 32), p.batch), PT, 0, st>>>(a);
+  } else {
+    pool_group_kernel<<<dim3((c->max_T + PT - 1) / PT, p.batch), PT + 2 * MAX_HALO, 0, st>>>(a);
   }
-  dim3 grid((c->max_T + PT - 1) / PT, p.batch);
-  pool_group_kernel<<<grid, PT + 2 * MAX_HALO, 0, st>>>(u, c->d_req, p.n_kv_heads, p.n_q_heads / p.n_kv_heads, p.pool_kernel,
-                                          p.pool_mode, c->u_rows_per_kv, c->u_parts, c->sum_T, c->latch_stat, c->cur_layer,
-                                          scores_kv, scores_agg);
   c->launches += 1;
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;

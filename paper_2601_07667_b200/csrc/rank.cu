@@ -507,7 +507,7 @@ static __device__ __align__(256) unsigned char g_rank_static[sizeof(RankStaticSc
 // reads it, so what an earlier call left behind is never seen.
 __global__ void rank_static_begin(RankStaticScratch* s, int T) {
   AslReq r;
-  r.n = T; r.T = T; r.k = 0; r.kept = 0; r.tok_off = 0; r.t_off = 0; r.kept_off = 0; r.pad = 0;
+  r.n = T; r.T = T; r.k = 0; r.kept = 0; r.tok_off = 0; r.t_off = 0; r.kept_off = 0; r.u_off = 0;
   s->req = r;
 }
 

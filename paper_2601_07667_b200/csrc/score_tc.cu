@@ -370,7 +370,7 @@ struct TcArgs {
   uint32_t* counters;
   uint32_t* launch;        // launch number, then the ticket of arrived CTAs
   int32_t* err;
-  int64_t sum_T;
+  int64_t u_stride;
   int32_t n_stages, nseg, NC, HR, W, Wp, m, pieces, G, Hq, u_rows_per_kv, u_parts;
   float scale_log2;
 };
@@ -726,7 +726,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                  rc = __ldg(reinterpret_cast<const int4*>(rp) + 2);
       const int run_slot = __ldg(&rp->slot);
       const int tile0 = ra.x, ntiles = ra.y, pass = ra.z, seg = ra.w, h = rb.y, chunk = rb.z, next = rb.w;
-      const int T = rc.x, t_off = rc.y, rows = rc.w;
+      const int T = rc.x, u_off = rc.y, rows = rc.w;
       prefetch_run(work.runs, next);
       const float scale = FP8 ? a.scale_log2 * __ldg(&rp->kscale) : a.scale_log2;   // log2(e)/sqrt(d) times the accumulator factor
       const f32x2 scale2 = pk(scale, scale);
@@ -878,10 +878,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 if (PER_Q) {
 #pragma unroll
                   for (int q = 0; q < 4; ++q) ac[q] = pk(0.f, 0.f);
-                  if (j < T && head < a.G) a.u[((int64_t)(h * a.G + head) * a.u_parts + part) * a.sum_T + t_off + j] = sum;
+                  if (j < T && head < a.G) a.u[((int64_t)(h * a.G + head) * a.u_parts + part) * a.u_stride + u_off + j] = sum;
                   ++head;
                 } else {
-                  if (j < T) a.u[(int64_t)(h * a.u_rows_per_kv + chunk * HV + half) * a.sum_T + t_off + j] = sum;
+                  if (j < T) a.u[(int64_t)(h * a.u_rows_per_kv + chunk * HV + half) * a.u_stride + u_off + j] = sum;
                 }
               }
             }
@@ -1264,7 +1264,7 @@ bool asl_tc_plan(asl_ctx* c) {
         TcRun s{};
         s.seg = (int32_t)segs.size();
         s.b = b; s.h = h; s.chunk = ch;
-        s.T = c->req[b].T; s.t_off = c->req[b].t_off; s.tok_off = c->req[b].tok_off;
+        s.T = c->req[b].T; s.u_off = c->req[b].u_off; s.tok_off = c->req[b].tok_off;
         const int heads = G - ch * tp.m < tp.m ? G - ch * tp.m : tp.m;
         const int rest = W - ch % tp.pieces * MAX_ROWS;
         s.rows = tp.pieces > 1 ? (rest < MAX_ROWS ? rest : MAX_ROWS) : (heads - 1) * tp.Wp + W;
@@ -1463,7 +1463,7 @@ asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const f
   a.counters = tp.d_sync;                                            // the one-pass launch touches neither these
   a.launch = tp.d_sync + 4 * (size_t)tp.nseg * SYNC_STRIDE;         // nor this
   a.err = c->d_err;
-  a.sum_T = c->sum_T;
+  a.u_stride = c->u_stride;
   a.nseg = tp.nseg;
   a.NC = tp.NC; a.HR = tp.HR; a.W = W; a.Wp = tp.Wp; a.m = tp.m; a.pieces = tp.pieces; a.G = G; a.Hq = p.n_q_heads;
   a.u_rows_per_kv = c->u_rows_per_kv;

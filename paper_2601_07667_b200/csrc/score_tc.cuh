@@ -13,12 +13,12 @@ constexpr int ASL_TC_KEY_TILE = 128;
 #endif
 
 // A run: the tiles of one segment = (request, kv head, row chunk) that one CTA takes in one pass; `next`: the CTA's next
-// run (-1: none).  (T, t_off, tok_off: the request's past length, score offset and first token, copied here so that one
+// run (-1: none).  (T, u_off, tok_off: the request's past length, offset in the rows of column sums and first token, copied here so that one
 // record is all a role needs; rows: query rows of the chunk that exist; kscale: factor between the accumulator and q.k,
 // 1 for bf16 keys and k_scale[h] / 16 for FP8 keys, whose queries are scaled by 16 before they are split into two E4M3
 // terms; slot: number of the run among its pass's; group of segments; cta:
 // whom the plan gave it)
-struct __align__(16) TcRun { int32_t tile0, ntiles, pass, seg, b, h, chunk, next, T, t_off, tok_off, rows; float kscale; int32_t slot, group, cta; };
+struct __align__(16) TcRun { int32_t tile0, ntiles, pass, seg, b, h, chunk, next, T, u_off, tok_off, rows; float kscale; int32_t slot, group, cta; };
 
 // A group of segments: seg0 .. seg0 + nseg - 1.
 struct __align__(16) TcStage { int32_t seg0, nseg, pad0, pad1; };
