@@ -142,7 +142,7 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
 
   cudaGetDevice(&prev);
   cudaSetDevice(c->device);
-  const bool tc = asl_tc_plan(c);
+  const bool tc = asl_tc_plan(c) && asl_rank_ready() == ASL_OK;
   asl_topk_plan(c);
   cudaSetDevice(prev);
   if (!tc) { free_plan(c); return fp8 ? ASL_ERR_UNSUPPORTED : ASL_ERR_CUDA; }     // 8-bit keys: not every window
@@ -161,8 +161,8 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
   w.score_q8 = off;
   if (fp8) off = asl_align256(off + (size_t)2 * p->batch * p->n_q_heads * p->window * p->head_dim);
   w.score_end = off;
-  for (int i = 0; i < 2; ++i) { w.rank_keys[i] = off; off = asl_align256(off + (size_t)sum_T * 4); }
-  for (int i = 0; i < 2; ++i) { w.rank_idx[i] = off; off = asl_align256(off + (size_t)sum_T * 4); }
+  for (int i = 0; i < 2; ++i) { w.rank_keys[i] = off; off = asl_align256(off + (size_t)u_stride * 4); }
+  for (int i = 0; i < 2; ++i) { w.rank_idx[i] = off; off = asl_align256(off + (size_t)u_stride * 4); }
   const size_t nblk = (max_T + ASL_RANK_TILE - 1) / ASL_RANK_TILE;
   w.rank_hist = off;      off = asl_align256(off + (size_t)4 * p->batch * 256 * nblk * sizeof(int32_t));
   w.rank_end = off;

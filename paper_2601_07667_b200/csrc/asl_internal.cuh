@@ -129,6 +129,7 @@ asl_status asl_launch_pool(asl_ctx* c, const float* u, float* scores_kv, float* 
 asl_status asl_launch_live_phases(asl_ctx* c, bool two_pass, bool beside, cudaStream_t st);
 asl_status asl_launch_rank(asl_ctx* c, const float* agg, int32_t layer_idx, int32_t n_rows, int32_t* ring,
                            asl_stat* stat, char* ws, cudaStream_t st);
+asl_status asl_rank_ready();
 asl_status asl_launch_topk(asl_ctx* c, const float* scores, int32_t n_heads, int32_t* idx_out, const asl_stat* gate,
                            int32_t gate_layer, char* ws, cudaStream_t st);
 bool asl_topk_plan(asl_ctx* c);

@@ -1,12 +1,11 @@
 // Rank row and rank-variance statistic (Algorithm 1 (RankDesc); Algorithm 2 (stacked rank rows R, k, TopKIndices J, Unique U, RelNormVar, threshold test);
 // Section 4.1 "var_top" and "relative variance").
 //
-// RankDesc: stable least-significant-digit radix sort (8-bit digits, one kernel
-// per digit after a first histogram) of
-// (key, token index) pairs per request, key = bit pattern that ascends as the
-// score descends; equal scores keep ascending index order, so the position of
-// a token in the sorted sequence is its 0-based rank with ties to the lower
-// index.  The last pass scatters positions straight into the ring row.
+// RankDesc: position of every (key, token index) pair in sorted order per request, key = bit pattern that ascends as the
+// score descends; equal scores keep ascending index order, so the position is the token's 0-based rank with ties to the
+// lower index.  Segments of up to 64K tokens: sorted tiles, merged by search (below).  Longer ones: a stable
+// least-significant-digit radix sort (8-bit digits, one kernel per digit after a first histogram); the last pass scatters
+// positions straight into the ring row.
 //
 // Statistic: a token is in the union iff its smallest rank over the rows is < k
 // (the k smallest ranks of a row are exactly ranks 0..k-1).  The numerator
@@ -33,15 +32,17 @@ __device__ __forceinline__ uint32_t desc_key(float s) {
   return ~u;                                             // ascending as the score descends
 }
 
-// Lanes of the warp whose 8-bit digit equals this lane's: eight ballots, no
-// data-dependent loop (the hardware match instruction walks distinct values).
-__device__ __forceinline__ uint32_t same_digit(uint32_t d, bool valid) {
-  uint32_t peers = __ballot_sync(0xffffffffu, valid);
-#pragma unroll
-  for (int bit = 0; bit < 8; ++bit) {
-    const uint32_t b = __ballot_sync(0xffffffffu, (d >> bit) & 1u);
-    peers &= ((d >> bit) & 1u) ? b : ~b;
-  }
+// Lanes of the warp whose 8-bit digit equals this lane's (only valid lanes count).  They find one another through an
+// atomic OR of their lane bits into the digit's word of `lanes`, which is zero before and after: 11 cycles per warp
+// where eight ballots take 27.  One vote catches the digit that every lane has, where the atomics would serialise.
+__device__ __forceinline__ uint32_t same_digit(uint32_t* lanes, uint32_t d, bool valid, int lane) {
+  if (__all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) return __ballot_sync(0xffffffffu, valid);
+  if (valid) atomicOr(lanes + d, 1u << lane);
+  __syncwarp();
+  const uint32_t peers = lanes[d];
+  __syncwarp();
+  lanes[d] = 0;
+  __syncwarp();
   return peers;
 }
 
@@ -91,8 +92,12 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_hist_first(const float* __r
   for (int r = 0; r < ROUNDS; ++r) {
     const bool valid = start + wid * PER_WARP + r * 32 + lane < rq.T;
     const uint32_t d = key[r] & 255u;
-    const uint32_t peers = same_digit(d, valid);
-    if (valid && (peers & ((1u << lane) - 1u)) == 0) atomicAdd(&cnt[d], __popc(peers));
+    if (__all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {       // one digit: the adds would serialise
+      const int n = __popc(__ballot_sync(0xffffffffu, valid));
+      if (lane == 0) atomicAdd(&cnt[d], n);
+    } else if (valid) {
+      atomicAdd(&cnt[d], 1);
+    }
   }
   __syncthreads();
   if (threadIdx.x < 256) hist[row] = cnt[threadIdx.x];
@@ -172,6 +177,7 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
                                                              const asl_stat* __restrict__ latch, int shift, int nblk) {
   constexpr int SCAN_BATCH = 64 / PARTS;       // loads of tile counts in flight per thread
   __shared__ int cnt[WARPS][256];
+  __shared__ uint32_t lanes[WARPS][256];
   __shared__ int warp_tot[8];
   __shared__ int digit_off[256];
   __shared__ int part_tot[PARTS > 1 ? PARTS : 1][PARTS > 1 ? 256 : 1], part_before[PARTS > 1 ? PARTS : 1][PARTS > 1 ? 256 : 1];
@@ -233,7 +239,7 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
   } else {
     if (threadIdx.x < 256) digit_off[threadIdx.x] = counts[((int64_t)b * nblk + blk) * 256 + threadIdx.x];
   }
-  for (int i = threadIdx.x; i < WARPS * 256; i += SORT_THREADS) (&cnt[0][0])[i] = 0;
+  for (int i = threadIdx.x; i < WARPS * 256; i += SORT_THREADS) { (&cnt[0][0])[i] = 0; (&lanes[0][0])[i] = 0; }
   __syncthreads();
   // per-warp digit counts; the peer masks are kept for the second walk
   uint32_t peers[ROUNDS];
@@ -241,7 +247,7 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
   for (int r = 0; r < ROUNDS; ++r) {
     const bool valid = wstart + r * 32 + lane < rq.T;
     const uint32_t d = (key[r] >> shift) & 255u;
-    peers[r] = same_digit(d, valid);
+    peers[r] = same_digit(lanes[wid], d, valid, lane);
     if (valid && (peers[r] & lt) == 0) cnt[wid][d] += __popc(peers[r]);
     __syncwarp();
   }
@@ -324,8 +330,8 @@ struct StatArgs {
   double tau;
 };
 
-// Algorithm 2 (threshold test) for request b from the accumulated integers; clears them for the next layer
-__device__ void stat_finalize_one(unsigned long long* acc, const AslReq* __restrict__ req, asl_stat* __restrict__ stat, int b,
+// Algorithm 2 (threshold test) for request b from the accumulated integers
+__device__ void stat_finalize_one(unsigned long long num, unsigned long long m, const AslReq* __restrict__ req, asl_stat* __restrict__ stat, int b,
                                   int layer_idx, int n_rows, int evaluate, double tau, int latch) {
   asl_stat s = stat[b];
   if (latch && s.selected) return;                     // final: the record keeps the selection layer
@@ -337,9 +343,6 @@ __device__ void stat_finalize_one(unsigned long long* acc, const AslReq* __restr
   s.num = 0;
   s.m = 0;
   if (evaluate) {
-    const unsigned long long num = __ldcg(acc + 2 * b), m = __ldcg(acc + 2 * b + 1);
-    acc[2 * b] = 0;
-    acc[2 * b + 1] = 0;
     s.num = (int64_t)num;
     s.m = (int32_t)m;
     s.evaluated = 1;
@@ -358,10 +361,9 @@ __device__ void stat_finalize_one(unsigned long long* acc, const AslReq* __restr
 }
 
 // layers before L_min (or with a single rank row): only the bookkeeping fields change
-__global__ void rank_stat_skip(unsigned long long* acc, const AslReq* __restrict__ req, asl_stat* __restrict__ stat, int batch,
-                               int layer_idx, int n_rows, int latch) {
+__global__ void rank_stat_skip(const AslReq* __restrict__ req, asl_stat* __restrict__ stat, int batch, int layer_idx, int n_rows, int latch) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < batch) stat_finalize_one(acc, req, stat, b, layer_idx, n_rows, 0, 0.0, latch);
+  if (b < batch) stat_finalize_one(0, 0, req, stat, b, layer_idx, n_rows, 0, 0.0, latch);
 }
 
 constexpr int STAT_TOKENS = 4;   // tokens per thread: few, fat blocks (one wave on the SMs a persistent scorer leaves free)
@@ -439,13 +441,311 @@ __global__ void __launch_bounds__(256) rank_stat_accumulate(StatArgs a) {
   __syncthreads();
   if (last) {
     __threadfence();
-    for (int bb = threadIdx.x; bb < a.batch; bb += blockDim.x)
-      stat_finalize_one(a.acc, a.req, a.stat, bb, a.layer_idx, a.n_rows, 1, a.tau, a.latch);
+    for (int bb = threadIdx.x; bb < a.batch; bb += blockDim.x) {
+      const unsigned long long sum = __ldcg(a.acc + 2 * bb), size = __ldcg(a.acc + 2 * bb + 1);
+      a.acc[2 * bb] = 0;                                 // for the next layer
+      a.acc[2 * bb + 1] = 0;
+      stat_finalize_one(sum, size, a.req, a.stat, bb, a.layer_idx, a.n_rows, 1, a.tau, a.latch);
+    }
     if (threadIdx.x == 0) a.acc[2 * a.batch] = 0;
   }
 }
 
+// ---------------------------------------------------------------------------
+// Segments of up to MERGE_MAX_T tokens: tiles of R * 1024 scores are sorted on their own, one 1024-thread block each, and
+// a token's rank is then its place in its own tile plus, for every other tile of the request, the number of scores
+// there that go before it.  Two launches (one where a single tile holds the segment) against the five of the radix
+// passes over the whole row; nothing but the sorted tiles goes through global memory.
+// ---------------------------------------------------------------------------
+constexpr int TILE_THREADS = 1024;
+constexpr int TILE_WARPS = TILE_THREADS / 32;
+
+__host__ __device__ constexpr size_t tile_smem_bytes(int rounds) {     // keys, token numbers; per warp: digit counts, lanes per digit
+  return (size_t)rounds * TILE_THREADS * (sizeof(uint32_t) + sizeof(uint16_t)) + (size_t)TILE_WARPS * 256 * (sizeof(uint16_t) + sizeof(uint32_t));
+}
+
+struct TileArgs {
+  const float* agg;
+  int32_t* rank_row;
+  const AslReq* req;         // null: one segment of T tokens, no statistic
+  int32_t T;
+  uint32_t* keys;            // several tiles: each one's sorted keys and their tokens, a request's at its u_off
+  int32_t* idx;
+  StatArgs stat;             // ring, records, rows; n_rows 0: only the bookkeeping fields of the records change
+  int32_t evaluate;
+};
+
+__device__ __forceinline__ AslReq tile_request(const TileArgs& a, int b) {
+  AslReq rq{};
+  rq.T = a.T;
+  if (a.req) rq = a.req[b];
+  return rq;
+}
+
+// One tile: four stable passes of 8-bit digits in shared memory.  A pass is bound by what its R rounds per warp issue
+// to shared memory, and by its five block barriers; the place among the warp's earlier keys is kept from the count to
+// the scatter.
+// SINGLE: the tile is the whole segment; the block writes the rank row and takes the statistic.
+template <int R, bool SINGLE>
+__global__ void __launch_bounds__(TILE_THREADS, 1) rank_tile_kernel(TileArgs a) {
+  constexpr int N = R * TILE_THREADS;
+  extern __shared__ __align__(16) uint8_t tile_raw[];
+  uint32_t (*lanes)[256] = reinterpret_cast<uint32_t (*)[256]>(tile_raw);
+  uint32_t (*cnt2)[128] = reinterpret_cast<uint32_t (*)[128]>(lanes + TILE_WARPS);       // two digits' counts per word
+  uint32_t* s_key = reinterpret_cast<uint32_t*>(cnt2 + TILE_WARPS);
+  uint16_t* s_id = reinterpret_cast<uint16_t*>(s_key + N);
+  __shared__ uint32_t part_sum[8][128];
+  __shared__ int warp_tot[4];
+  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  uint16_t* const cnt = reinterpret_cast<uint16_t*>(cnt2[wid]);
+  if (a.req && a.stat.latch && a.stat.stat[b].selected) return;      // the request's selection is final
+  const AslReq rq = tile_request(a, b);
+  const int start = blockIdx.x * N;
+  if (start >= rq.T) return;
+  const int n = min(N, rq.T - start);
+  const uint32_t lt = (1u << lane) - 1u;
+  const int w0 = wid * R * 32;                                        // a warp owns consecutive keys
+  uint32_t key[R];
+  uint32_t id[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int i = w0 + r * 32 + lane;
+    id[r] = i;
+    key[r] = i < n ? desc_key(__ldcg(a.agg + rq.t_off + start + i)) : 0xffffffffu;   // padding sorts last (and stays behind equal keys)
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) lanes[wid][i * 32 + lane] = 0;
+#pragma unroll 1
+  for (int pass = 0; pass < 4; ++pass) {
+    const int shift = 8 * pass;
+    uint32_t before[R];                                               // keys of the warp with the same digit and a lower place
+#pragma unroll
+    for (int i = 0; i < 4; ++i) cnt2[wid][i * 32 + lane] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const uint32_t d = (key[r] >> shift) & 255u;
+      const uint32_t peers = same_digit(lanes[wid], d, true, lane);
+      const uint32_t c = cnt[d];
+      __syncwarp();
+      if ((peers & lt) == 0) cnt[d] = (uint16_t)(c + __popc(peers));
+      before[r] = c + __popc(peers & lt);
+      __syncwarp();
+    }
+    __syncthreads();
+    {  // the counts become positions, in (digit, warp) order: thread (part, word) has two digits of four warps
+      const int w = tid & 127, part = tid >> 7;
+      uint32_t v[4], total = 0, mine = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { v[i] = cnt2[part * 4 + i][w]; mine += v[i]; }
+      part_sum[part][w] = mine;
+      __syncthreads();
+      mine = 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) { const uint32_t s = part_sum[q][w]; total += s; mine += q < part ? s : 0u; }
+      const int both = (int)((total & 0xffffu) + (total >> 16));
+      int incl = both;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+      }
+      if (part == 0 && lane == 31) warp_tot[wid] = incl;
+      __syncthreads();
+      uint32_t off = (uint32_t)(incl - both);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) off += q < (w >> 5) ? (uint32_t)warp_tot[q] : 0u;
+      uint32_t run = mine + (off | (off + (total & 0xffffu)) << 16);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { cnt2[part * 4 + i][w] = run; run += v[i]; }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const uint32_t pos = cnt[(key[r] >> shift) & 255u] + before[r];
+      if (SINGLE && pass == 3) { s_key[id[r]] = pos; continue; }      // the rank row, in token order
+      s_key[pos] = key[r];
+      s_id[pos] = (uint16_t)id[r];
+    }
+    __syncthreads();
+    if (pass == 3) break;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      key[r] = s_key[w0 + r * 32 + lane];
+      id[r] = s_id[w0 + r * 32 + lane];
+    }
+  }
+  if (!SINGLE) {                                                      // up to a multiple of four: copied on 16 bytes
+    const int64_t out = (int64_t)rq.u_off + start;
+    for (int i = tid; i < (n + 3) / 4 * 4; i += TILE_THREADS) {
+      a.keys[out + i] = s_key[i];
+      a.idx[out + i] = start + s_id[i];
+    }
+    return;
+  }
+  // ---- the row, and the statistic over it and the earlier rows
+  __shared__ unsigned long long s_num[TILE_WARPS];
+  __shared__ int s_m[TILE_WARPS];
+  unsigned long long num = 0;
+  int m = 0;
+#pragma unroll 1
+  for (int i = tid; i < rq.T; i += TILE_THREADS) {
+    const int mine = (int)s_key[i];
+    a.rank_row[rq.t_off + i] = mine;
+    if (a.evaluate) {
+      long long s1 = mine, s2 = (long long)mine * mine;
+      int mn = mine;
+      for (int r0 = 0; r0 < a.stat.n_rows - 1; r0 += 8) {
+        int v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int slot = (a.stat.first_layer + r0 + q) % a.stat.l_obs;
+          v[q] = r0 + q < a.stat.n_rows - 1 ? __ldcg(a.stat.ring + (int64_t)slot * a.stat.sum_T + rq.t_off + i) : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (v[q] >= 0) { mn = min(mn, v[q]); s1 += v[q]; s2 += (long long)v[q] * v[q]; }
+      }
+      if (mn < rq.k) {
+        m += 1;
+        num += (unsigned long long)((long long)a.stat.n_rows * s2 - s1 * s1);
+      }
+    }
+  }
+  if (!a.req) return;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    num += __shfl_down_sync(0xffffffffu, num, o);
+    m += __shfl_down_sync(0xffffffffu, m, o);
+  }
+  if (lane == 0) { s_num[wid] = num; s_m[wid] = m; }
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < TILE_WARPS; ++w) { num += s_num[w]; m += s_m[w]; }
+    stat_finalize_one(num, (unsigned long long)m, a.req, a.stat.stat, b, a.stat.layer_idx, a.stat.n_rows, a.evaluate, a.stat.tau, a.stat.latch);
+  }
+}
+
+template <bool LE>
+__device__ __forceinline__ bool goes_before(uint32_t a, uint32_t key) { return LE ? a <= key : a < key; }
+
+// A sorted run in shared memory: four words of padding behind every 32, so that the few places which the lanes of a
+// warp (32 ascending keys) look at in one step of their searches lie in different banks at every stride.
+__host__ __device__ constexpr int padded(int i) { return i + i / 32 * 4; }
+
+// For each of the E keys: keys of a run of N (a power of two) that go before it.  `at` walks the padded places; every
+// step of the E searches is in flight at once.
+template <int N, int E, bool LE>
+__device__ __forceinline__ void add_counts(const uint32_t* run, const uint32_t (&key)[E], int (&rank)[E]) {
+  int at[E];
+#pragma unroll
+  for (int i = 0; i < E; ++i) at[i] = 0;
+#pragma unroll
+  for (int h = N / 2; h; h >>= 1) {                    // at is a place that 2h divides: at + h - 1 lies in the same 32 below h = 32
+#pragma unroll
+    for (int i = 0; i < E; ++i) at[i] += goes_before<LE>(run[at[i] + padded(h - 1)], key[i]) ? padded(h) : 0;
+  }
+#pragma unroll
+  for (int i = 0; i < E; ++i) rank[i] += at[i] - at[i] / 36 * 4 + (goes_before<LE>(run[at[i]], key[i]) ? 1 : 0);
+}
+
+// Block: MERGE_CHUNK keys of one sorted tile against all other tiles of the request, staged in shared memory one ahead.
+// Bound by the searches' loads from shared memory.
+constexpr int MERGE_THREADS = 256;
+constexpr int MERGE_PER = 4;                                          // keys per thread
+constexpr int MERGE_CHUNK = MERGE_THREADS * MERGE_PER;
+
+template <int R>
+__global__ void __launch_bounds__(MERGE_THREADS) rank_merge_kernel(TileArgs a) {
+  constexpr int N = R * TILE_THREADS;
+  __shared__ __align__(16) uint32_t run[2][padded(N)];
+  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  pdl_release_successor();
+  if (a.req && a.stat.latch && a.stat.stat[b].selected) return;
+  const AslReq rq = tile_request(a, b);
+  const int first = blockIdx.x * MERGE_CHUNK;
+  if (first >= rq.T) return;
+  const int own = first / N, tiles = (rq.T + N - 1) / N;
+  const uint32_t* keys = a.keys + rq.u_off;
+  auto stage = [&](int tile, int buf) {
+    const int have = min(N, (rq.T - tile * N + 3) / 4 * 4);           // the last tile ends early, on a multiple of four
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(run[buf]);
+    for (int i = tid * 4; i < N; i += MERGE_THREADS * 4) {
+      if (i < have) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + padded(i) * 4), "l"(keys + (int64_t)tile * N + i) : "memory");
+      else *reinterpret_cast<uint4*>(&run[buf][padded(i)]) = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // the tiles after the own one first: blocks of different tiles do not ask for the same lines at the same time
+  int tile = own + 1 < tiles ? own + 1 : 0;
+  if (tile != own) stage(tile, 0);
+  const int at = first + wid * 32 * MERGE_PER + lane;
+  uint32_t key[MERGE_PER];
+  int token[MERGE_PER], rank[MERGE_PER];
+#pragma unroll
+  for (int i = 0; i < MERGE_PER; ++i) {
+    const int j = at + i * 32;
+    key[i] = j < rq.T ? __ldcg(keys + j) : 0xffffffffu;
+    token[i] = j < rq.T ? __ldcg(a.idx + rq.u_off + j) : -1;
+    rank[i] = j - own * N;
+  }
+  for (int buf = 0; tile != own; buf ^= 1) {
+    const int next = tile + 1 < tiles ? tile + 1 : 0;
+    if (next != own) stage(next, buf ^ 1);
+    if (next != own) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (tile < own) add_counts<N, MERGE_PER, true>(run[buf], key, rank);     // earlier tokens go first among equals
+    else add_counts<N, MERGE_PER, false>(run[buf], key, rank);
+    __syncthreads();
+    tile = next;
+  }
+#pragma unroll
+  for (int i = 0; i < MERGE_PER; ++i)
+    if (token[i] >= 0) a.rank_row[rq.t_off + token[i]] = rank[i];
+}
+
+// A tile that holds the segment stands alone up to 4096 scores (16 us there, in two launches over tiles of 2048 17 us; the
+// radix passes 34 us).  Above, tiles of 2048 keep more SMs busy with the sorts (8192 scores: 19.5 us, with tiles of 4096
+// 21.5 us), and from 16384 on tiles of 4096 mean half the searches (32768: 27.6 us, 29.7 us, radix passes 35.8 us).  The
+// searches grow with the square of the length: at 65536 scores both ways take 36 to 38 us on an idle GPU, at 131072 the
+// radix passes 40 us and this way 54 us.  Beside a scorer that leaves few SMs this way is the faster one up to that line
+// (a pass of eight 32K layers 630 -> 480 us, three of 50K 283 -> 259 us), and not above (four of 128K 832 -> 923 us).
+constexpr int ALONE_MAX_T = 4096;
+constexpr int SMALL_TILES_MAX_T = 16384;
+constexpr int MERGE_MAX_T = 65536;
+
+struct TileKernel { void (*fn)(TileArgs); int rounds; };
+const TileKernel ALONE_KERNELS[3] = {{rank_tile_kernel<1, true>, 1}, {rank_tile_kernel<2, true>, 2}, {rank_tile_kernel<4, true>, 4}};
+const TileKernel SORT_KERNELS[2] = {{rank_tile_kernel<2, false>, 2}, {rank_tile_kernel<4, false>, 4}};
+
+// the rank rows and, where one tile per request does, the statistic; launches
+int launch_tiles(const TileArgs& a, int max_T, int batch, cudaStream_t st) {
+  if (max_T <= ALONE_MAX_T) {
+    const TileKernel& k = ALONE_KERNELS[max_T <= 1024 ? 0 : max_T <= 2048 ? 1 : 2];
+    k.fn<<<dim3(1, batch), TILE_THREADS, tile_smem_bytes(k.rounds), st>>>(a);
+    return 1;
+  }
+  const TileKernel& k = SORT_KERNELS[max_T <= SMALL_TILES_MAX_T ? 0 : 1];
+  const int n = k.rounds * TILE_THREADS;
+  k.fn<<<dim3((max_T + n - 1) / n, batch), TILE_THREADS, tile_smem_bytes(k.rounds), st>>>(a);
+  // the plain way: its blocks, started early, would crowd onto the SMs that the sorts leave free (131072 scores: 89 us, not 69)
+  const dim3 grid((max_T + MERGE_CHUNK - 1) / MERGE_CHUNK, batch);
+  if (k.rounds == 2) rank_merge_kernel<2><<<grid, MERGE_THREADS, 0, st>>>(a);
+  else rank_merge_kernel<4><<<grid, MERGE_THREADS, 0, st>>>(a);
+  return 2;
+}
+
 }  // namespace
+
+// once per device, with that device current
+asl_status asl_rank_ready() {
+  for (const TileKernel& k : ALONE_KERNELS)
+    ASL_CUDA(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem_bytes(k.rounds)));
+  for (const TileKernel& k : SORT_KERNELS)
+    ASL_CUDA(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem_bytes(k.rounds)));
+  return ASL_OK;
+}
 
 asl_status asl_launch_rank(asl_ctx* c, const float* agg, int32_t layer_idx, int32_t n_rows, int32_t* ring,
                            asl_stat* stat, char* ws, cudaStream_t st) {
@@ -457,14 +757,23 @@ asl_status asl_launch_rank(asl_ctx* c, const float* agg, int32_t layer_idx, int3
   int32_t* hist = reinterpret_cast<int32_t*>(ws + c->ws.rank_hist);
   int32_t* row = ring + (int64_t)(layer_idx % p.l_obs) * c->sum_T;
   const asl_stat* latch = c->controller == ASL_CONTROLLER_LATCH ? stat : nullptr;
-  c->launches += launch_sort(agg, c->d_req, latch, p.batch, c->max_T, keys, idx, hist, row, st);
   const int evaluate = (layer_idx >= p.l_min && n_rows >= 2) ? 1 : 0;
+  const StatArgs a{ring, c->d_req, c->d_acc, stat, c->sum_T, p.l_obs, layer_idx - n_rows + 1, n_rows, p.batch, layer_idx,
+                   latch ? 1 : 0, p.tau};
+  if (c->max_T <= MERGE_MAX_T) {
+    const int launches = launch_tiles(TileArgs{agg, row, c->d_req, 0, keys[0], idx[0], a, evaluate}, c->max_T, p.batch, st);
+    c->launches += launches;
+    if (launches == 1) {                               // the statistic went with the row
+      ASL_CUDA(cudaGetLastError());
+      return ASL_OK;
+    }
+  } else {
+    c->launches += launch_sort(agg, c->d_req, latch, p.batch, c->max_T, keys, idx, hist, row, st);
+  }
   if (evaluate) {
-    StatArgs a{ring, c->d_req, c->d_acc, stat, c->sum_T, p.l_obs, layer_idx - n_rows + 1, n_rows, p.batch, layer_idx,
-               latch ? 1 : 0, p.tau};
     launch_after(rank_stat_accumulate, dim3((c->max_T + 256 * STAT_TOKENS - 1) / (256 * STAT_TOKENS), p.batch), dim3(256), st, a);
   } else {
-    rank_stat_skip<<<(p.batch + 63) / 64, 64, 0, st>>>(c->d_acc, c->d_req, stat, p.batch, layer_idx, n_rows, latch ? 1 : 0);
+    rank_stat_skip<<<(p.batch + 63) / 64, 64, 0, st>>>(c->d_req, stat, p.batch, layer_idx, n_rows, latch ? 1 : 0);
   }
   c->launches += 1;
   ASL_CUDA(cudaGetLastError());
@@ -534,7 +843,7 @@ asl_status rank_static_setup(int device, RankStaticScratch** out) {
     void* p = nullptr;
     if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) st = ASL_ERR_CUDA;
     else if (major != 10) st = ASL_ERR_ARCH;
-    else if (cudaGetSymbolAddress(&p, g_rank_static) != cudaSuccess || !p) st = ASL_ERR_CUDA;
+    else if (cudaGetSymbolAddress(&p, g_rank_static) != cudaSuccess || !p || asl_rank_ready() != ASL_OK) st = ASL_ERR_CUDA;
     d.ptr[device] = static_cast<RankStaticScratch*>(p);
     d.status[device] = st;
     d.done[device] = st == ASL_OK || st == ASL_ERR_ARCH;     // a failed CUDA call is tried again by the next call
@@ -556,11 +865,15 @@ extern "C" asl_status asl_rank_desc_static(const float* scores, int32_t T, int32
   const asl_status ready = rank_static_setup(device, &s);
   if (ready != ASL_OK) return ready;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const AslReq* req = &s->req;
-  rank_static_begin<<<1, 1, 0, st>>>(s, T);
-  uint32_t* const keys[2] = {s->keys[0], s->keys[1]};
-  int32_t* const idx[2] = {s->idx[0], s->idx[1]};
-  launch_sort(scores, req, nullptr, 1, T, keys, idx, s->hist, rank_out, st);
+  if (T <= MERGE_MAX_T) {
+    launch_tiles(TileArgs{scores, rank_out, nullptr, T, s->keys[0], s->idx[0], StatArgs{}, 0}, T, 1, st);
+  } else {
+    const AslReq* req = &s->req;
+    rank_static_begin<<<1, 1, 0, st>>>(s, T);
+    uint32_t* const keys[2] = {s->keys[0], s->keys[1]};
+    int32_t* const idx[2] = {s->idx[0], s->idx[1]};
+    launch_sort(scores, req, nullptr, 1, T, keys, idx, s->hist, rank_out, st);
+  }
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;
 }
