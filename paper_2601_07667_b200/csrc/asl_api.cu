@@ -142,8 +142,7 @@ asl_status asl_plan(asl_ctx* c, const asl_params* p, size_t* workspace_bytes) {
 
   cudaGetDevice(&prev);
   cudaSetDevice(c->device);
-  const bool tc = asl_tc_plan(c) && asl_rank_ready() == ASL_OK;
-  asl_topk_plan(c);
+  const bool tc = asl_tc_plan(c) && asl_topk_plan(c) && asl_rank_ready() == ASL_OK;
   cudaSetDevice(prev);
   if (!tc) { free_plan(c); return fp8 ? ASL_ERR_UNSUPPORTED : ASL_ERR_CUDA; }     // 8-bit keys: not every window
   // the scorer writes a partial column sum per half of a chunk's rows; under max pooling the halves (and the chunks of

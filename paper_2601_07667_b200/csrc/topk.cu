@@ -3,9 +3,9 @@
 // Radix select on an order-preserving 32-bit image of the fp32 score, 11+11+10
 // bits from the top: the exact k-th largest key is found; every token with a
 // larger key is kept, and of the tokens equal to it the lowest-indexed fill the
-// remainder.  Two forms.  Plans whose longest segment has 8 K to 256 K scores
-// and whose k is a small part of it run one CTA per segment in a single launch
-// (second half of this file).  Everything else is cut into tiles of 4096 scores,
+// remainder.  Two forms.  Plans whose longest segment has up to 256 K scores
+// run one CTA per segment in a single launch
+// (second half of this file).  Longer ones are cut into tiles of 4096 scores,
 // one 256-thread CTA per tile with its 16 scores per thread in registers, and
 // into five short kernels that meet only through global memory:
 //
@@ -274,142 +274,78 @@ __global__ void __launch_bounds__(THREADS) topk_emit_kernel(TopkArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// One CTA per segment.
+// One CTA per segment (plans whose longest segment has up to 256 K scores): one launch, no scratch in global memory.
 //
-// For segments of a few thousand to a few hundred thousand scores the whole
-// selection runs in one 1024-thread CTA with no scratch in global memory:
+//   2048 sampled scores -> two keys L <= H that hold the k-th largest key between them with a wide margin (segments of up
+//   to 12288 scores: their smallest and largest key) -> ONE pass over the segment: a bitmap of the keys above H, and a
+//   list in shared memory of the keys in [L, H] -> exact radix select of the remaining rank in the list, digits taken
+//   from the top of the range H - L -> the list's larger keys into the bitmap, the keys equal to the k-th into a second
+//   one, the lowest-indexed of which fill the remainder -> ordered emit from the bitmap.
 //
-//   sample 4096 scores -> a lower bound L that, with a wide margin, at least k
-//   scores reach -> ONE pass over the segment that keeps every (key, index) with
-//   key >= L in shared memory -> exact radix select of the k-th largest key among
-//   them -> two bitmaps over the segment (keys above the k-th, keys equal to it)
-//   -> ordered emit from the bitmaps.
+// The bounds are only a way to look at few keys: the pass counts, and if the k-th key is not between them or the list
+// overflows (long runs of equal scores), the CTA takes the same radix select over the whole segment (four more passes).
+// Both ways end in the exact k-th key and the same tie rule, so the kept list does not depend on which ran.
 //
-// The bound is only a way to look at few keys: the pass counts what it keeps, and
-// if fewer than k scores reached L, or more than the shared-memory list holds
-// (long runs of equal scores, a k that is a large part of T), the CTA takes the
-// same 11+11+10-bit radix select as the tiled kernels over the whole segment
-// (three more passes and one to fill the bitmaps).  Both ways end in the exact
-// k-th key and the same tie rule, so the kept list does not depend on which ran.
+// A lane reads 16-byte vectors, eight in flight; bit p of the bitmaps is score p - mis, mis scores lying between the
+// 16-byte boundary before the row and the row, so that a vector is a nibble of a word.  (One score per lane and a ballot
+// per word takes six times the instructions: 40 us for the pass over 131008 scores instead of 8.)  Bound by what one SM
+// pulls from L2 and by the chain of passes:
+// one segment of 96K scores, k = 3.8K: 24.8 -> 22.0 us; 32 segments of 3 to 24 K scores, k half of them: 29 us (five
+// tiled kernels) -> 15 us.
 // ---------------------------------------------------------------------------
 constexpr int SEG_THREADS = 1024;
 constexpr int SEG_WARPS = SEG_THREADS / 32;
 constexpr int SEG_CAP = 12288;                 // (key, index) pairs the shared-memory list holds
 constexpr int SEG_SAMPLE = 2048;
-constexpr int SEG_MIN_T = 8192;                // shorter segments: the full select at once (a sample would be most of them)
 constexpr int SEG_MAX_T = 262144;              // the bitmaps cover this many scores
-constexpr int SEG_UNROLL = 8;                  // 16-byte loads in flight per thread
+constexpr int SEG_UNROLL = 8;                  // 16-byte loads in flight per lane
 
-struct SegSmem {
+struct __align__(16) SegSmem {
   int hist[BINS];
   uint32_t cand_key[SEG_CAP];
   int32_t cand_idx[SEG_CAP];
-  // behind this struct, sized for the plan's longest segment (seg_smem_bytes): two bitmaps over the segment
-  // and, per bitmap word, the kept scores before it (short-list emit)
-  int warp_a[SEG_WARPS], warp_b[SEG_WARPS];
+  int warp_a[SEG_WARPS];
+  uint32_t lo[SEG_WARPS], hi[SEG_WARPS];
   int found[2][2];
-  int n_cand;
+  int n_cand, n_above;
+  // behind this struct, sized for the plan's longest segment: two bitmaps over the segment
 };
+__host__ __device__ inline int seg_words(int max_T) { return ((max_T + 3 + 31) / 32 + 3) & ~3; }
+inline size_t seg_smem_bytes(int max_T) { return sizeof(SegSmem) + (size_t)seg_words(max_T) * 2 * sizeof(uint32_t); }
 
-// dynamic shared memory of the kernel for segments of up to max_T scores
-__host__ __device__ inline int seg_words(int max_T) { return ((max_T + 31) / 32 + 3) & ~3; }
-inline size_t seg_smem_bytes(int max_T) { return sizeof(SegSmem) + (size_t)seg_words(max_T) * (2 * sizeof(uint32_t) + 2 * sizeof(uint16_t)); }
-
-// The sample rank whose key is taken as the lower bound: the expected number of sampled scores among
-// the k largest, plus four standard deviations and two.
-__host__ __device__ inline int seg_sample_rank(int T, int k) {
-  const float mean = (float)SEG_SAMPLE * (float)k / (float)T;
-  return (int)ceilf(mean + 4.f * sqrtf(mean)) + 2;
-}
-
-// Warp `wid` walks a contiguous run of 16-byte vectors of the segment; the vectors are aligned in
-// memory, so the first and the last may hold fewer than four scores of the segment.
-struct SegWalk {
-  const float* row;
-  const float4* base4;
-  int T, mis, per, v_begin, v_end;
-  __device__ SegWalk(const float* row_, int T_, int wid) : row(row_), T(T_) {
-    mis = (int)((reinterpret_cast<uintptr_t>(row_) >> 2) & 3);
-    base4 = reinterpret_cast<const float4*>(row_ - mis);
-    const int nv = (T + mis + 3) >> 2;
-    per = (((nv + SEG_WARPS - 1) / SEG_WARPS) + 32 * SEG_UNROLL - 1) / (32 * SEG_UNROLL) * (32 * SEG_UNROLL);   // whole load blocks
-    v_begin = min(nv, wid * per);
-    v_end = min(nv, v_begin + per);
-  }
-  __device__ __forceinline__ int first_index(int v) const { return v * 4 - mis; }
-  // keys of vector v; bit c of the result: element c is a score of the segment
-  __device__ __forceinline__ uint32_t load(int v, uint32_t (&key)[4]) const {
-    key[0] = key[1] = key[2] = key[3] = 0u;
-    if (v >= v_end) return 0u;
-    const int e0 = v * 4 - mis;
-    if (e0 >= 0 && e0 + 4 <= T) {
-      const float4 x = __ldcg(base4 + v);
-      key[0] = asc_key(x.x); key[1] = asc_key(x.y); key[2] = asc_key(x.z); key[3] = asc_key(x.w);
-      return 15u;
-    }
-    uint32_t m = 0u;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int e = e0 + c;
-      if (e >= 0 && e < T) { key[c] = asc_key(__ldcg(row + e)); m |= 1u << c; }
-    }
-    return m;
-  }
-  // SEG_UNROLL vectors per lane from vector s0 on (s0 is the same for the whole warp).  Away from the ends of
-  // the warp's run and of the segment every load is a full vector: all of them are issued before the first is used.
-  // all SEG_UNROLL x 32 vectors from s0 on are full vectors of the segment inside this warp's run
-  __device__ __forceinline__ bool interior(int s0) const {
-    return s0 + 32 * SEG_UNROLL <= v_end && s0 * 4 - mis >= 0 && (s0 + 32 * SEG_UNROLL) * 4 - mis <= T;
-  }
-  __device__ __forceinline__ void load_block(int s0, int lane, uint32_t (&key)[SEG_UNROLL][4], uint32_t (&m)[SEG_UNROLL]) const {
-    if (interior(s0)) {
-      float4 x[SEG_UNROLL];
-#pragma unroll
-      for (int u = 0; u < SEG_UNROLL; ++u) x[u] = __ldcg(base4 + s0 + 32 * u + lane);
-#pragma unroll
-      for (int u = 0; u < SEG_UNROLL; ++u) {
-        key[u][0] = asc_key(x[u].x); key[u][1] = asc_key(x[u].y); key[u][2] = asc_key(x[u].z); key[u][3] = asc_key(x[u].w);
-        m[u] = 15u;
-      }
-    } else {
-#pragma unroll
-      for (int u = 0; u < SEG_UNROLL; ++u) m[u] = load(s0 + 32 * u + lane, key[u]);
-    }
-  }
-};
-
-// exclusive prefix, at position `wid`, of the 32 per-warp totals in `tot` (every warp computes it for itself)
-__device__ __forceinline__ int seg_warp_base(const int* tot, int lane, int wid) {
-  const int t = tot[lane];
-  int incl = t;
+// exclusive prefix over the block of v, in thread order
+__device__ __forceinline__ int seg_block_prefix(SegSmem& sm, int v) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int incl = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
+    const int u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
   }
-  return __shfl_sync(0xffffffffu, incl - t, wid);
+  __syncthreads();
+  if (lane == 31) sm.warp_a[wid] = incl;
+  __syncthreads();
+  const int t = sm.warp_a[lane];
+  int w = t;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, w, o);
+    if (lane >= o) w += u;
+  }
+  return incl - v + __shfl_sync(0xffffffffu, w - t, wid);
 }
 
-// pick() for 1024 threads over a table in shared memory (NB = 2048 or 1024 bins); `par` alternates between
-// consecutive calls (the result of a call stays readable while the next one runs)
+// The bin of the shared table (NB bins, counted from the top) that holds the `remaining`-th largest key, and how many
+// keys of that bin are still wanted; `par` alternates between consecutive calls.
 template <int NB>
 __device__ __forceinline__ void seg_pick(SegSmem& sm, int remaining, int par, int& bin, int& rem_out) {
   constexpr int PER = NB / SEG_THREADS;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int top = NB - 1 - PER * tid;
+  const int top = NB - 1 - PER * (int)threadIdx.x;
   int c[PER];
   int sum = 0;
 #pragma unroll
   for (int j = 0; j < PER; ++j) { c[j] = sm.hist[top - j]; sum += c[j]; }
-  int incl = sum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  if (lane == 31) sm.warp_a[wid] = incl;
-  __syncthreads();
-  int above = incl - sum + seg_warp_base(sm.warp_a, lane, wid);
+  int above = seg_block_prefix(sm, sum);
   if (above < remaining && remaining <= above + sum) {
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
@@ -422,106 +358,179 @@ __device__ __forceinline__ void seg_pick(SegSmem& sm, int remaining, int par, in
   rem_out = sm.found[par][1];
 }
 
-__device__ __forceinline__ void seg_clear_hist(SegSmem& sm) {
-  for (int i = threadIdx.x; i < BINS; i += SEG_THREADS) sm.hist[i] = 0;
-  __syncthreads();
-}
-
-// digit histogram of the listed keys whose bits under `mask` equal `prefix`
-__device__ __forceinline__ void seg_list_hist(SegSmem& sm, int n, uint32_t mask, uint32_t prefix, int shift, uint32_t dmask) {
-  seg_clear_hist(sm);
-  for (int i = threadIdx.x; i < n; i += SEG_THREADS) {
-    const uint32_t key = sm.cand_key[i];
-    if ((key & mask) == prefix) atomicAdd(&sm.hist[(key >> shift) & dmask], 1);
-  }
-  __syncthreads();
-}
-
-// the same over the whole segment (one pass over its scores)
-__device__ __forceinline__ void seg_full_hist(SegSmem& sm, const SegWalk& w, uint32_t mask, uint32_t prefix, int shift,
-                                              uint32_t dmask) {
-  seg_clear_hist(sm);
-  const int lane = threadIdx.x & 31;
-  for (int s = w.v_begin; s < w.v_end; s += 32 * SEG_UNROLL) {
-    uint32_t key[SEG_UNROLL][4], m[SEG_UNROLL];
-    w.load_block(s, lane, key, m);
-    int run_bin = -1, run = 0;
-#pragma unroll
-    for (int u = 0; u < SEG_UNROLL; ++u) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const bool in = ((m[u] >> c) & 1u) && ((key[u][c] & mask) == prefix);
-        const int d = (int)((key[u][c] >> shift) & dmask);
-        if (in && d == run_bin) { ++run; continue; }
-        if (run) atomicAdd(&sm.hist[run_bin], run);
-        run_bin = in ? d : -1;
-        run = in ? 1 : 0;
-      }
+// The `rank`-th largest of keys[0..n) in shared memory (all of them in [lo, hi]) and how many equal to it are wanted.
+__device__ __forceinline__ void seg_select(SegSmem& sm, int n, uint32_t lo, uint32_t hi, int rank, uint32_t& thr, int& need) {
+  int shift = 32 - __clz((int)((hi - lo) | 1u));            // bits of the range still open
+  uint32_t base = lo;                                        // keys in [base, base + 2^shift) are still candidates
+  need = rank;
+  for (int par = 0; shift > 0; par ^= 1) {
+    const int bits = shift < 11 ? shift : 11;
+    for (int i = threadIdx.x; i < BINS; i += SEG_THREADS) sm.hist[i] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += SEG_THREADS) {
+      const uint32_t d = sm.cand_key[i] - base;
+      if (shift == 32 || (d >> shift) == 0u) atomicAdd(&sm.hist[d >> (shift - bits)], 1);
     }
-    if (run) atomicAdd(&sm.hist[run_bin], run);
+    __syncthreads();
+    int bin;
+    seg_pick<BINS>(sm, need, par, bin, need);
+    shift -= bits;
+    base += (uint32_t)bin << shift;
   }
-  __syncthreads();
+  thr = base;
 }
 
 __global__ void __launch_bounds__(SEG_THREADS, 1) topk_segment_kernel(TopkArgs a) {
   extern __shared__ __align__(16) uint8_t seg_smem_raw[];
   SegSmem& sm = *reinterpret_cast<SegSmem*>(seg_smem_raw);
-  const int cap_words = seg_words(a.max_T);
   uint32_t* const bm_gt = reinterpret_cast<uint32_t*>(seg_smem_raw + sizeof(SegSmem));
-  uint32_t* const bm_eq = bm_gt + cap_words;
-  uint16_t* const pre_gt = reinterpret_cast<uint16_t*>(bm_eq + cap_words);
-  uint16_t* const pre_eq = pre_gt + cap_words;
+  uint32_t* const bm_eq = bm_gt + seg_words(a.max_T);
   const Segment s = segment_of(a);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (!s.open) return;
   for (int t = tid; t < s.kept - s.k; t += SEG_THREADS) s.out[s.k + t] = s.T + t;   // the window
   if (s.k == 0) return;
-  const SegWalk w(s.row, s.T, wid);
+  const int mis = (int)((reinterpret_cast<uintptr_t>(s.row) >> 2) & 3);
+  const float4* const row4 = reinterpret_cast<const float4*>(s.row - mis);
+  const int nv = (s.T + mis + 3) >> 2, words = (nv + 7) >> 3;      // vectors; bitmap words
+  // A warp takes blocks of SEG_UNROLL x 32 vectors.  bits of vector v (score bits); m: which of its elements are scores.
+  auto load_block = [&](int v0, uint4 (&x)[SEG_UNROLL], uint32_t (&m)[SEG_UNROLL]) {
+#pragma unroll
+    for (int u = 0; u < SEG_UNROLL; ++u) {
+      const int v = v0 + 32 * u + lane;
+      m[u] = v < nv ? 15u : 0u;
+      if (v == 0) m[u] &= 15u << mis;
+      if (v == nv - 1) m[u] &= 15u >> (4 * nv - mis - s.T);
+      x[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (m[u] == 15u) x[u] = __ldcg(reinterpret_cast<const uint4*>(row4) + v);
+    }
+#pragma unroll
+    for (int u = 0; u < SEG_UNROLL; ++u) {
+      if (m[u] != 15u && m[u] != 0u) {                       // the ends of a row off a 16-byte boundary
+        const uint32_t* e = reinterpret_cast<const uint32_t*>(row4 + v0 + 32 * u + lane);
+        if (m[u] & 1u) x[u].x = __ldcg(e);
+        if (m[u] & 2u) x[u].y = __ldcg(e + 1);
+        if (m[u] & 4u) x[u].z = __ldcg(e + 2);
+        if (m[u] & 8u) x[u].w = __ldcg(e + 3);
+      }
+    }
+  };
+  // a nibble per lane -> the bitmap word of eight lanes, stored by one of them
+  auto put_word = [&](uint32_t* bm, int v, uint32_t nibble) {
+    uint32_t w = nibble << (4 * (lane & 7));
+    w |= __shfl_xor_sync(0xffffffffu, w, 1);
+    w |= __shfl_xor_sync(0xffffffffu, w, 2);
+    w |= __shfl_xor_sync(0xffffffffu, w, 4);
+    if ((lane & 7) == 0 && (v >> 3) < words) bm[v >> 3] = w;
+  };
+  auto nibble_of = [](const uint4& x, auto test) {
+    return (test(x.x) ? 1u : 0u) | (test(x.y) ? 2u : 0u) | (test(x.z) ? 4u : 0u) | (test(x.w) ? 8u : 0u);
+  };
 
-  // ---- the short list: every score that reaches a sampled lower bound
-  bool listed = false;
-  int n = 0;
-  if (s.T >= SEG_MIN_T) {
-    if (tid == 0) sm.n_cand = 0;
-    {
-      float x[SEG_SAMPLE / SEG_THREADS];
+  // ---- bounds on the k-th largest key
+  uint32_t L = 0u, H = 0xffffffffu;
+  const bool whole = s.T <= SEG_CAP;                        // the list takes every key
+  if (tid == 0) { sm.n_cand = 0; sm.n_above = 0; }
+  if (!whole) {
+    float x[SEG_SAMPLE / SEG_THREADS];
+    uint32_t mn = 0xffffffffu, mx = 0u;
 #pragma unroll
-      for (int j = 0; j < SEG_SAMPLE / SEG_THREADS; ++j) x[j] = __ldcg(s.row + (int)(((long long)(tid + j * SEG_THREADS) * s.T) / SEG_SAMPLE));
+    for (int j = 0; j < SEG_SAMPLE / SEG_THREADS; ++j) x[j] = __ldcg(s.row + (int)(((long long)(tid + j * SEG_THREADS) * s.T) / SEG_SAMPLE));
 #pragma unroll
-      for (int j = 0; j < SEG_SAMPLE / SEG_THREADS; ++j) sm.cand_key[tid + j * SEG_THREADS] = asc_key(x[j]);
+    for (int j = 0; j < SEG_SAMPLE / SEG_THREADS; ++j) {
+      const uint32_t key = asc_key(x[j]);
+      sm.cand_key[tid + j * SEG_THREADS] = key;
+      mn = min(mn, key);
+      mx = max(mx, key);
+    }
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) { sm.lo[wid] = mn; sm.hi[wid] = mx; }
+    __syncthreads();
+    mn = __reduce_min_sync(0xffffffffu, sm.lo[lane]);
+    mx = __reduce_max_sync(0xffffffffu, sm.hi[lane]);
+    // sample ranks four standard deviations and two to either side of the expected one; their bins in a histogram of the
+    // sample's range are bound enough
+    const float mean = (float)SEG_SAMPLE * (float)s.k / (float)s.T;
+    const float dev = 4.f * sqrtf(mean * (1.f - (float)s.k / (float)s.T)) + 2.f;
+    const int r_lo = (int)ceilf(mean + dev), r_hi = (int)floorf(mean - dev);
+    const int open = 32 - __clz((int)((mx - mn) | 1u)), shift = open > 11 ? open - 11 : 0;
+    for (int i = tid; i < BINS; i += SEG_THREADS) sm.hist[i] = 0;
+    __syncthreads();
+    for (int i = tid; i < SEG_SAMPLE; i += SEG_THREADS) atomicAdd(&sm.hist[(sm.cand_key[i] - mn) >> shift], 1);
+    __syncthreads();
+    int bin, rest;
+    if (r_lo <= SEG_SAMPLE) { seg_pick<BINS>(sm, r_lo, 0, bin, rest); L = mn + ((uint32_t)bin << shift); }
+    // an upper bound costs the pass as much as the lower one: only where the keys above L would not fit the list
+    if (r_hi >= 1 && 1.2f * (float)s.T * (float)min(r_lo, SEG_SAMPLE) > (float)SEG_CAP * (float)SEG_SAMPLE) {
+      seg_pick<BINS>(sm, r_hi, 1, bin, rest);
+      const uint32_t top = mn + ((uint32_t)bin << shift) + ((1u << shift) - 1u);
+      H = top < mn ? 0xffffffffu : top;
     }
     __syncthreads();
-    int b1, b2, rem1, rem2;
-    seg_list_hist(sm, SEG_SAMPLE, 0u, 0u, 21, 2047u);
-    seg_pick<2048>(sm, min(SEG_SAMPLE, seg_sample_rank(s.T, s.k)), 0, b1, rem1);
-    seg_list_hist(sm, SEG_SAMPLE, 2047u << 21, (uint32_t)b1 << 21, 10, 2047u);
-    seg_pick<2048>(sm, rem1, 1, b2, rem2);
-    const uint32_t bound = ((uint32_t)b1 << 21) | ((uint32_t)b2 << 10);
-    // A strictly positive bound is compared on the raw bits: key >= bound <=> bits - lo < 2^31 - lo (unsigned).
-    const bool raw = bound > 0x80000000u;
-    const uint32_t lo = bound & 0x7fffffffu, span = 0x80000000u - lo;
-    for (int s0 = w.v_begin; s0 < w.v_end; s0 += 32 * SEG_UNROLL) {
-      uint32_t hit = 0u;                                  // bit 4u+c: element c of the lane's u-th vector is listed
-      if (raw && w.interior(s0)) {
-        float4 x[SEG_UNROLL];
+  }
+
+  // ---- one pass: the bitmap of keys above H, the list of keys in [L, H]
+  uint32_t mn = 0xffffffffu, mx = 0u;                       // of the listed keys
+  for (int i = tid; i < words; i += SEG_THREADS) { bm_eq[i] = 0u; bm_gt[i] = 0u; }
+  if (!whole) __syncthreads();
+  if (whole) {
+    for (int i0 = tid; i0 < s.T; i0 += 4 * SEG_THREADS) {
+      float x[4];
 #pragma unroll
-        for (int u = 0; u < SEG_UNROLL; ++u) x[u] = __ldcg(w.base4 + s0 + 32 * u + lane);
+      for (int u = 0; u < 4; ++u) x[u] = i0 + u * SEG_THREADS < s.T ? __ldcg(s.row + i0 + u * SEG_THREADS) : 0.f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * SEG_THREADS;
+        if (i >= s.T) break;
+        const uint32_t key = asc_key(x[u]);
+        sm.cand_key[i] = key;
+        mn = min(mn, key);
+        mx = max(mx, key);
+      }
+    }
+  } else {
+    // Bounds above zero are compared on the raw bits: a score reaches L unless its sign bit or that of bits - lo is set; the
+    // sign is shifted into a mask, three instructions per score.
+    const bool raw = L > 0x80000000u;
+    const uint32_t lo = L & 0x7fffffffu, hi = H == 0xffffffffu ? 0x7fffffffu : (H & 0x7fffffffu) + 1u;
+    const bool none_above = H == 0xffffffffu;
+    auto below = [](uint32_t bits, uint32_t bound, uint32_t mask) { return __funnelshift_l(bits | (bits - bound), mask, 1); };
+    int above = 0;
+    for (int v0 = wid * 32 * SEG_UNROLL; v0 < nv; v0 += SEG_WARPS * 32 * SEG_UNROLL) {
+      uint32_t hit, gt;                                     // bit 4u + c: element c of the lane's u-th vector reaches L / is above H
+      if (raw && v0 > 0 && v0 + 32 * SEG_UNROLL < nv) {     // (not the first or the last vector of the row)
+        uint4 x[SEG_UNROLL];
+#pragma unroll
+        for (int u = 0; u < SEG_UNROLL; ++u) x[u] = __ldcg(reinterpret_cast<const uint4*>(row4) + v0 + 32 * u + lane);
+        uint32_t not_hit = 0u, not_gt = 0u;
+#pragma unroll
+        for (int u = SEG_UNROLL - 1; u >= 0; --u)
+          not_hit = below(x[u].x, lo, below(x[u].y, lo, below(x[u].z, lo, below(x[u].w, lo, not_hit))));
+        if (!none_above) {
+#pragma unroll
+          for (int u = SEG_UNROLL - 1; u >= 0; --u)
+            not_gt = below(x[u].x, hi, below(x[u].y, hi, below(x[u].z, hi, below(x[u].w, hi, not_gt))));
+        }
+        hit = ~not_hit;
+        gt = none_above ? 0u : ~not_gt;
+      } else {
+        uint4 x[SEG_UNROLL];
+        uint32_t m[SEG_UNROLL];
+        load_block(v0, x, m);
+        hit = gt = 0u;
 #pragma unroll
         for (int u = 0; u < SEG_UNROLL; ++u) {
-          hit |= (__float_as_uint(x[u].x) - lo < span ? 1u : 0u) << (4 * u);
-          hit |= (__float_as_uint(x[u].y) - lo < span ? 2u : 0u) << (4 * u);
-          hit |= (__float_as_uint(x[u].z) - lo < span ? 4u : 0u) << (4 * u);
-          hit |= (__float_as_uint(x[u].w) - lo < span ? 8u : 0u) << (4 * u);
+          hit |= (nibble_of(x[u], [&](uint32_t b) { return asc_key(__uint_as_float(b)) >= L; }) & m[u]) << (4 * u);
+          gt |= (nibble_of(x[u], [&](uint32_t b) { return asc_key(__uint_as_float(b)) > H; }) & m[u]) << (4 * u);
         }
-      } else {
-        uint32_t key[SEG_UNROLL][4], m[SEG_UNROLL];
-        w.load_block(s0, lane, key, m);
-#pragma unroll
-        for (int u = 0; u < SEG_UNROLL; ++u)
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            if (((m[u] >> c) & 1u) && key[u][c] >= bound) hit |= 1u << (4 * u + c);
       }
+      if (__any_sync(0xffffffffu, gt != 0u)) {
+        above += __popc(gt);
+#pragma unroll
+        for (int u = 0; u < SEG_UNROLL; ++u) put_word(bm_gt, v0 + 32 * u + lane, (gt >> (4 * u)) & 15u);
+      }
+      hit &= ~gt;
       const int cnt = __popc(hit);
       int incl = cnt;
 #pragma unroll
@@ -530,152 +539,134 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) topk_segment_kernel(TopkArgs a
         if (lane >= o) incl += v;
       }
       const int total = __shfl_sync(0xffffffffu, incl, 31);
-      if (total == 0) continue;                         // the same for the whole warp
-      int base = 0;
-      if (lane == 31) base = atomicAdd(&sm.n_cand, total);
-      base = __shfl_sync(0xffffffffu, base, 31);
-      int slot = base + incl - cnt;
+      if (total == 0) continue;                             // the same for the whole warp
+      int at = 0;
+      if (lane == 31) at = atomicAdd(&sm.n_cand, total);
+      int slot = __shfl_sync(0xffffffffu, at, 31) + incl - cnt;
       while (hit) {
         const int bpos = __ffs(hit) - 1;
         hit &= hit - 1;
-        if (slot < SEG_CAP) sm.cand_idx[slot] = w.first_index(s0 + 32 * (bpos >> 2) + lane) + (bpos & 3);
+        if (slot < SEG_CAP) sm.cand_idx[slot] = 4 * (v0 + 32 * (bpos >> 2) + lane) + (bpos & 3) - mis;
         ++slot;
       }
     }
+    above = __reduce_add_sync(0xffffffffu, above);
+    if (lane == 0 && above) atomicAdd(&sm.n_above, above);
     __syncthreads();
-    n = sm.n_cand;
-    listed = n >= s.k && n <= SEG_CAP;
-    if (listed) {
-      for (int i0 = 0; i0 < n; i0 += 4 * SEG_THREADS) {
-        float x[4];
+    const int listed = min(sm.n_cand, SEG_CAP);
+    for (int i0 = tid; i0 < listed; i0 += 4 * SEG_THREADS) {         // their keys
+      float x[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int i = i0 + j * SEG_THREADS + tid;
-          x[j] = i < n ? __ldcg(s.row + sm.cand_idx[i]) : 0.f;
-        }
+      for (int u = 0; u < 4; ++u) x[u] = i0 + u * SEG_THREADS < listed ? __ldcg(s.row + sm.cand_idx[i0 + u * SEG_THREADS]) : 0.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int i = i0 + j * SEG_THREADS + tid;
-          if (i < n) sm.cand_key[i] = asc_key(x[j]);
-        }
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * SEG_THREADS;
+        if (i >= listed) break;
+        const uint32_t key = asc_key(x[u]);
+        sm.cand_key[i] = key;
+        mn = min(mn, key);
+        mx = max(mx, key);
       }
-      __syncthreads();
     }
   }
-
-  // ---- the exact k-th largest key and how many keys equal to it are kept
-  int bin1, bin2, bin3, rem1, rem2, need;
-  if (listed) {
-    seg_list_hist(sm, n, 0u, 0u, 21, 2047u);
-    seg_pick<2048>(sm, s.k, 0, bin1, rem1);
-    seg_list_hist(sm, n, 2047u << 21, (uint32_t)bin1 << 21, 10, 2047u);
-    seg_pick<2048>(sm, rem1, 1, bin2, rem2);
-    seg_list_hist(sm, n, 0xfffffc00u, ((uint32_t)bin1 << 21) | ((uint32_t)bin2 << 10), 0, 1023u);
-    seg_pick<1024>(sm, rem2, 0, bin3, need);
-  } else {
-    seg_full_hist(sm, w, 0u, 0u, 21, 2047u);
-    seg_pick<2048>(sm, s.k, 0, bin1, rem1);
-    seg_full_hist(sm, w, 2047u << 21, (uint32_t)bin1 << 21, 10, 2047u);
-    seg_pick<2048>(sm, rem1, 1, bin2, rem2);
-    seg_full_hist(sm, w, 0xfffffc00u, ((uint32_t)bin1 << 21) | ((uint32_t)bin2 << 10), 0, 1023u);
-    seg_pick<1024>(sm, rem2, 0, bin3, need);
-  }
-  const uint32_t thr = ((uint32_t)bin1 << 21) | ((uint32_t)bin2 << 10) | (uint32_t)bin3;
-
-  // ---- bitmaps over the segment: keys above the k-th, keys equal to it
-  const int words = (s.T + 31) >> 5;
-  for (int i = tid; i < words; i += SEG_THREADS) { bm_gt[i] = 0u; bm_eq[i] = 0u; }
+  mn = __reduce_min_sync(0xffffffffu, mn);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0) { sm.lo[wid] = mn; sm.hi[wid] = mx; }
   __syncthreads();
+  mn = __reduce_min_sync(0xffffffffu, sm.lo[lane]);
+  mx = __reduce_max_sync(0xffffffffu, sm.hi[lane]);
+  const int n = whole ? s.T : sm.n_cand, n_above = sm.n_above;
+  const bool listed = n <= SEG_CAP && n_above < s.k && s.k <= n_above + n;
+
+  // ---- the exact k-th largest key, how many keys equal to it are kept, and the two bitmaps
+  uint32_t thr;
+  int need;
   if (listed) {
+    seg_select(sm, n, mn, mx, s.k - n_above, thr, need);
     for (int i = tid; i < n; i += SEG_THREADS) {
       const uint32_t key = sm.cand_key[i];
-      const int e = sm.cand_idx[i];
+      const int e = (whole ? i : sm.cand_idx[i]) + mis;
       if (key > thr) atomicOr(&bm_gt[e >> 5], 1u << (e & 31));
       else if (key == thr) atomicOr(&bm_eq[e >> 5], 1u << (e & 31));
     }
   } else {
-    for (int s0 = w.v_begin; s0 < w.v_end; s0 += 32 * SEG_UNROLL) {
-      uint32_t key[SEG_UNROLL][4], m[SEG_UNROLL];
-      w.load_block(s0, lane, key, m);
+    uint32_t base = 0u;
+    int shift = 32;
+    need = s.k;
+    for (int par = 0; shift > 0; par ^= 1) {
+      const int bits = shift < 11 ? shift : 11;
+      for (int i = tid; i < BINS; i += SEG_THREADS) sm.hist[i] = 0;
+      __syncthreads();
+      for (int v0 = wid * 32 * SEG_UNROLL; v0 < nv; v0 += SEG_WARPS * 32 * SEG_UNROLL) {
+        uint4 x[SEG_UNROLL];
+        uint32_t m[SEG_UNROLL];
+        load_block(v0, x, m);
+        int run_bin = -1, run = 0;                           // neighbouring scores often share a digit: one atomic per run
 #pragma unroll
-      for (int u = 0; u < SEG_UNROLL; ++u)
+        for (int u = 0; u < SEG_UNROLL; ++u)
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if ((m[u] >> c) & 1u) {
-            const int e = w.first_index(s0 + 32 * u + lane) + c;
-            if (key[u][c] > thr) atomicOr(&bm_gt[e >> 5], 1u << (e & 31));
-            else if (key[u][c] == thr) atomicOr(&bm_eq[e >> 5], 1u << (e & 31));
+          for (int c = 0; c < 4; ++c) {
+            const uint32_t b = c == 0 ? x[u].x : (c == 1 ? x[u].y : (c == 2 ? x[u].z : x[u].w));
+            const uint32_t d = asc_key(__uint_as_float(b)) - base;
+            const bool in = ((m[u] >> c) & 1u) && (shift == 32 || (d >> shift) == 0u);
+            const int bin = in ? (int)(d >> (shift - bits)) : -1;
+            if (in && bin == run_bin) { ++run; continue; }
+            if (run) atomicAdd(&sm.hist[run_bin], run);
+            run_bin = bin;
+            run = in ? 1 : 0;
           }
+        if (run) atomicAdd(&sm.hist[run_bin], run);
+      }
+      __syncthreads();
+      int bin;
+      seg_pick<BINS>(sm, need, par, bin, need);
+      shift -= bits;
+      base += (uint32_t)bin << shift;
+    }
+    thr = base;
+    for (int v0 = wid * 32 * SEG_UNROLL; v0 < nv; v0 += SEG_WARPS * 32 * SEG_UNROLL) {
+      uint4 x[SEG_UNROLL];
+      uint32_t m[SEG_UNROLL];
+      load_block(v0, x, m);
+#pragma unroll
+      for (int u = 0; u < SEG_UNROLL; ++u) {
+        put_word(bm_gt, v0 + 32 * u + lane, nibble_of(x[u], [&](uint32_t b) { return asc_key(__uint_as_float(b)) > thr; }) & m[u]);
+        put_word(bm_eq, v0 + 32 * u + lane, nibble_of(x[u], [&](uint32_t b) { return asc_key(__uint_as_float(b)) == thr; }) & m[u]);
+      }
     }
   }
   __syncthreads();
 
-  // ---- ordered emit (Algorithm 1 (TopK and window append)): thread t owns a run of bitmap words
+  // ---- of the equal keys the first `need`; thread t owns a run of words
   const int wpt = (words + SEG_THREADS - 1) / SEG_THREADS;
   const int w0 = min(words, tid * wpt), w1 = min(words, w0 + wpt);
-  int cg = 0, ce = 0;
-  for (int i = w0; i < w1; ++i) { cg += __popc(bm_gt[i]); ce += __popc(bm_eq[i]); }
-  int ig = cg, ie = ce;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int vg = __shfl_up_sync(0xffffffffu, ig, o), ve = __shfl_up_sync(0xffffffffu, ie, o);
-    if (lane >= o) { ig += vg; ie += ve; }
+  int eq = 0;
+  for (int i = w0; i < w1; ++i) eq += __popc(bm_eq[i]);
+  int left = need - seg_block_prefix(sm, eq);
+  int kept = 0;
+  for (int i = w0; i < w1; ++i) {
+    uint32_t q = bm_eq[i];
+    const int cnt = __popc(q);
+    if (left < cnt) {                                        // keep the lowest `left` of them
+      uint32_t some = 0u;
+      for (int c = 0; c < left; ++c) { some |= q & (0u - q); q &= q - 1; }
+      q = some;
+    }
+    left -= cnt;
+    const uint32_t word = bm_gt[i] | q;
+    bm_gt[i] = word;
+    kept += __popc(word);
   }
-  if (lane == 31) { sm.warp_a[wid] = ig; sm.warp_b[wid] = ie; }
-  __syncthreads();
-  int gt_before = ig - cg + seg_warp_base(sm.warp_a, lane, wid), eq_before = ie - ce + seg_warp_base(sm.warp_b, lane, wid);
-  if (listed) {
-    // every listed score finds its own place: kept scores before its word (at most SEG_CAP: 16 bits) plus those
-    // before it in its word; the work is spread evenly however the kept tokens cluster
-    for (int i = w0; i < w1; ++i) {
-      pre_gt[i] = (uint16_t)gt_before;
-      pre_eq[i] = (uint16_t)eq_before;
-      gt_before += __popc(bm_gt[i]);
-      eq_before += __popc(bm_eq[i]);
-    }
-    __syncthreads();
-    // places first (they read the listed keys), then the kept indices into the keys' storage in output order,
-    // then one coalesced copy: a scattered store to global memory costs a cache-line access each
-    int place[SEG_CAP / SEG_THREADS];
-#pragma unroll
-    for (int j = 0; j < SEG_CAP / SEG_THREADS; ++j) {
-      const int i = tid + j * SEG_THREADS;
-      place[j] = -1;
-      if (i < n) {
-        const uint32_t key = sm.cand_key[i];
-        if (key >= thr) {
-          const int e = sm.cand_idx[i], wd = e >> 5;
-          const uint32_t below = (1u << (e & 31)) - 1u;
-          const int g = pre_gt[wd] + __popc(bm_gt[wd] & below), q = pre_eq[wd] + __popc(bm_eq[wd] & below);
-          if (key > thr) place[j] = g + min(q, need);
-          else if (q < need) place[j] = g + q;
-        }
-      }
-    }
-    __syncthreads();
-    int32_t* ordered = reinterpret_cast<int32_t*>(sm.cand_key);
-#pragma unroll
-    for (int j = 0; j < SEG_CAP / SEG_THREADS; ++j)
-      if (place[j] >= 0) ordered[place[j]] = sm.cand_idx[tid + j * SEG_THREADS];
+  // ---- ordered emit (Algorithm 1 (TopK and window append)): in shared memory first where the kept indices fit there (the
+  // list is done with), so that the copy out is coalesced
+  int32_t* const ordered = reinterpret_cast<int32_t*>(sm.cand_key);
+  const bool staged = s.k <= 2 * SEG_CAP;
+  int32_t* to = (staged ? ordered : s.out) + seg_block_prefix(sm, kept);
+  for (int i = w0; i < w1; ++i)
+    for (uint32_t bits = bm_gt[i]; bits; bits &= bits - 1) *to++ = i * 32 + __ffs(bits) - 1 - mis;
+  if (staged) {
     __syncthreads();
     for (int i = tid; i < s.k; i += SEG_THREADS) s.out[i] = ordered[i];
-    return;
-  }
-  for (int i = w0; i < w1; ++i) {
-    const uint32_t g = bm_gt[i], q = bm_eq[i];
-    uint32_t bits = g | q;
-    while (bits) {
-      const int bpos = __ffs(bits) - 1;
-      bits &= bits - 1;
-      const int idx = i * 32 + bpos;
-      if ((g >> bpos) & 1u) {
-        s.out[gt_before + min(eq_before, need)] = idx;
-        ++gt_before;
-      } else {
-        if (eq_before < need) s.out[gt_before + eq_before] = idx;
-        ++eq_before;
-      }
-    }
   }
 }
 
@@ -686,23 +677,14 @@ size_t asl_topk_scratch_bytes(int64_t segments, int64_t max_T) {
   return (size_t)(segments * SEG_INTS + segments * tiles * 2) * sizeof(int32_t);
 }
 
-// Whether the plan's segments go to the one-CTA kernel: the longest fits its bitmaps, is long enough for a
-// sample to be a small part of it, and for every long segment the scores expected above the sampled bound
-// (sample rank / sample size of the segment, with a fifth on top) fit the shared-memory list.  Called with the
-// context's device current.
+// Whether the plan's segments go to the one-CTA kernel: the longest fits its bitmaps.  Called with the context's device
+// current.
 bool asl_topk_plan(asl_ctx* c) {
-  c->topk_one_cta = false;
-  if (c->max_T < SEG_MIN_T || c->max_T > SEG_MAX_T) return false;
-  for (const AslReq& r : c->req) {
-    if (r.T < SEG_MIN_T || r.k == 0) continue;
-    const int rank = seg_sample_rank(r.T, r.k) < SEG_SAMPLE ? seg_sample_rank(r.T, r.k) : SEG_SAMPLE;
-    if (1.2 * (double)r.T * rank / SEG_SAMPLE > (double)SEG_CAP) return false;
-  }
+  c->topk_one_cta = c->max_T <= SEG_MAX_T;
   if (cudaFuncSetAttribute(topk_segment_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)seg_smem_bytes(SEG_MAX_T)) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  c->topk_one_cta = true;
   return true;
 }
 
