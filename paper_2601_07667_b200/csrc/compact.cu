@@ -1,8 +1,13 @@
 // K/V compaction (Algorithm 1 (K[I], V[I])): out[h][r][:] = x[tok_off + idx[h][r]][h][:].
-// 16 threads move one row (256 bytes of bf16, 128 bytes of FP8 codes) as 16-byte vectors; K and V in one launch.
+// 16 threads move one row (256 bytes of bf16, 128 bytes of FP8 codes) as 16-byte vectors; K and V in one launch, four
+// rows per thread with all eight loads in flight.  Bound by HBM's rate for scattered 256-byte rows: half of four 24K-token
+// prompts' rows (223 MB moved) 50.5 us one row per thread -> 44.6 us (5.0 TB/s).
 #include "asl_internal.cuh"
 
 namespace {
+
+constexpr int ROWS = 4;                   // rows per thread
+constexpr int BLOCK_ROWS = 16 * ROWS;     // rows per 256-thread block
 
 __global__ void __launch_bounds__(256) compact_kv_kernel(const uint8_t* __restrict__ k, const uint8_t* __restrict__ v,
                                                          const int32_t* __restrict__ idx, const AslReq* __restrict__ req,
@@ -14,18 +19,23 @@ __global__ void __launch_bounds__(256) compact_kv_kernel(const uint8_t* __restri
   const int b = blockIdx.z, h = blockIdx.y;
   if (latch && asl_finished(latch + b, cur_layer)) return;       // finished request: its compacted cache is final
   const AslReq rq = req[b];
-  const int r = blockIdx.x * (blockDim.x / 16) + threadIdx.x / 16;
+  const int r0 = blockIdx.x * BLOCK_ROWS + threadIdx.x / 16;
   const int c = threadIdx.x % 16;
-  if (r >= rq.kept) return;
-  const int64_t orow = (int64_t)h * sum_kept + rq.kept_off + r;
-  const int64_t tok = (int64_t)rq.tok_off + idx[orow];
-  if (c < k_vec) {
-    const uint4 kv = __ldcs(reinterpret_cast<const uint4*>(k + tok * ks_t + (int64_t)h * ks_h + c * 16));
-    __stcs(reinterpret_cast<uint4*>(k_out + (orow * k_vec + c) * 16), kv);
+  if (blockIdx.x * BLOCK_ROWS >= rq.kept) return;
+  const int64_t orow = (int64_t)h * sum_kept + rq.kept_off + r0;
+  int64_t tok[ROWS];
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i) tok[i] = r0 + 16 * i < rq.kept ? (int64_t)rq.tok_off + __ldg(idx + orow + 16 * i) : -1;
+  uint4 kv[ROWS], vv[ROWS];
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i) {
+    if (tok[i] >= 0 && c < k_vec) kv[i] = __ldcs(reinterpret_cast<const uint4*>(k + tok[i] * ks_t + (int64_t)h * ks_h + c * 16));
+    if (tok[i] >= 0 && c < v_vec) vv[i] = __ldcs(reinterpret_cast<const uint4*>(v + tok[i] * vs_t + (int64_t)h * vs_h + c * 16));
   }
-  if (c < v_vec) {
-    const uint4 vv = __ldcs(reinterpret_cast<const uint4*>(v + tok * vs_t + (int64_t)h * vs_h + c * 16));
-    __stcs(reinterpret_cast<uint4*>(v_out + (orow * v_vec + c) * 16), vv);
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i) {
+    if (tok[i] >= 0 && c < k_vec) __stcs(reinterpret_cast<uint4*>(k_out + ((orow + 16 * i) * k_vec + c) * 16), kv[i]);
+    if (tok[i] >= 0 && c < v_vec) __stcs(reinterpret_cast<uint4*>(v_out + ((orow + 16 * i) * v_vec + c) * 16), vv[i]);
   }
 }
 
@@ -60,7 +70,7 @@ asl_status asl_launch_compact(asl_ctx* c, const void* k, const void* v, const in
   const asl_params& p = c->p;
   const int kb = c->k_elem_bytes;                          // K elements are 2 bytes (bf16) or 1 (FP8 codes), V is bf16
   const int k_vec = p.head_dim * kb / 16, v_vec = p.head_dim * 2 / 16;
-  dim3 grid((c->max_kept + 15) / 16, p.n_kv_heads, p.batch);
+  dim3 grid((c->max_kept + BLOCK_ROWS - 1) / BLOCK_ROWS, p.n_kv_heads, p.batch);
   compact_kv_kernel<<<grid, 256, 0, st>>>(static_cast<const uint8_t*>(k), static_cast<const uint8_t*>(v), idx, c->d_req,
                                           p.k_stride[0] * kb, p.k_stride[1] * kb, p.v_stride[0] * 2, p.v_stride[1] * 2,
                                           c->sum_kept, k_vec, v_vec, c->latch_stat, c->cur_layer,

@@ -1,0 +1,37 @@
+"""GPU parity of K/V compaction at row counts around a block's 64, bf16 and FP8 keys."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_07667_b200 import binding as B
+from paper_2601_07667_b200 import inputs as I
+
+from asl_check import bits_of, make_path, to_dev, with_fp8_keys
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("fp8", [False, True])
+def test_compaction_of_any_number_of_rows(fp8):
+    w = 64
+    seqlens, kept = (65, 80, 200, 200, 200, 300, 500), (64, 65, 127, 128, 129, 193, 500)
+    wl = I.workload("C3", n_q_heads=32, n_kv_heads=8, window=w, seqlens=seqlens, budgets=kept, layers=1, l_min=1, l_obs=2)
+    x = I.layer_inputs(wl, 0, seed=3)
+    launch = {}
+    if fp8:
+        x = with_fp8_keys(x)
+        launch = dict(k_dtype=B.ASL_K_FP8_E4M3, k_scale=[float(s) for s in x["k_scale"]])
+    path = make_path(wl, **launch)
+    rng, cu = np.random.default_rng(4), wl.cu_seqlens()
+    idx = np.stack([np.concatenate([np.sort(rng.choice(n, m, replace=False)) for n, m in zip(seqlens, kept)]) for _ in range(wl.n_kv_heads)])
+    idx_dev = torch.from_numpy(idx.astype(np.int32)).cuda()
+    path.k_out.zero_(), path.v_out.zero_()
+    B.asl_compact_kv(path.ctx, to_dev(x["k"]), to_dev(x["v"]), idx_dev, path.k_out, path.v_out)
+    torch.cuda.synchronize()
+    k_out, v_out, at = bits_of(path.k_out), bits_of(path.v_out), 0
+    for b, m in enumerate(kept):
+        for h in range(wl.n_kv_heads):
+            rows = cu[b] + idx[h, at:at + m]
+            assert (k_out[h, at:at + m] == x["k"][rows, h]).all() and (v_out[h, at:at + m] == x["v"][rows, h]).all(), (b, h)
+        at += m
+    path.close()
