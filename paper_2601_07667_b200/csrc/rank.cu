@@ -633,20 +633,28 @@ __device__ __forceinline__ bool goes_before(uint32_t a, uint32_t key) { return L
 // warp (32 ascending keys) look at in one step of their searches lie in different banks at every stride.
 __host__ __device__ constexpr int padded(int i) { return i + i / 32 * 4; }
 
-// For each of the E keys: keys of a run of N (a power of two) that go before it.  `at` walks the padded places; every
-// step of the E searches is in flight at once.
+// For each of the E keys: keys of a run of N (a power of two) that go before it.  `at` walks the padded places as byte
+// addresses, so that a step is a load, a compare and an add (65536 scores: 37.9 us with indices -> 31.7 us); a step of
+// all E searches is in flight at once.
 template <int N, int E, bool LE>
-__device__ __forceinline__ void add_counts(const uint32_t* run, const uint32_t (&key)[E], int (&rank)[E]) {
-  int at[E];
+__device__ __forceinline__ void add_counts(uint32_t run, const uint32_t (&key)[E], int (&rank)[E]) {
+  uint32_t at[E], x[E];
 #pragma unroll
-  for (int i = 0; i < E; ++i) at[i] = 0;
+  for (int i = 0; i < E; ++i) at[i] = run;
 #pragma unroll
-  for (int h = N / 2; h; h >>= 1) {                    // at is a place that 2h divides: at + h - 1 lies in the same 32 below h = 32
+  for (int h = N / 2; h; h >>= 1) {                    // at is a place that 2h divides: the one h - 1 further is padded(h - 1) further
 #pragma unroll
-    for (int i = 0; i < E; ++i) at[i] += goes_before<LE>(run[at[i] + padded(h - 1)], key[i]) ? padded(h) : 0;
+    for (int i = 0; i < E; ++i) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x[i]) : "r"(at[i] + padded(h - 1) * 4) : "memory");
+#pragma unroll
+    for (int i = 0; i < E; ++i)
+      if (goes_before<LE>(x[i], key[i])) at[i] += padded(h) * 4;
   }
 #pragma unroll
-  for (int i = 0; i < E; ++i) rank[i] += at[i] - at[i] / 36 * 4 + (goes_before<LE>(run[at[i]], key[i]) ? 1 : 0);
+  for (int i = 0; i < E; ++i) {
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x[i]) : "r"(at[i]) : "memory");
+    const int p = (int)(at[i] - run) / 4;
+    rank[i] += p - p / 36 * 4 + (goes_before<LE>(x[i], key[i]) ? 1 : 0);
+  }
 }
 
 // Block: MERGE_CHUNK keys of one sorted tile against all other tiles of the request, staged in shared memory one ahead.
@@ -679,12 +687,12 @@ __global__ void __launch_bounds__(MERGE_THREADS) rank_merge_kernel(TileArgs a) {
   // the tiles after the own one first: blocks of different tiles do not ask for the same lines at the same time
   int tile = own + 1 < tiles ? own + 1 : 0;
   if (tile != own) stage(tile, 0);
-  const int at = first + wid * 32 * MERGE_PER + lane;
+  const int mine = first + wid * 32 * MERGE_PER + lane;
   uint32_t key[MERGE_PER];
   int token[MERGE_PER], rank[MERGE_PER];
 #pragma unroll
   for (int i = 0; i < MERGE_PER; ++i) {
-    const int j = at + i * 32;
+    const int j = mine + i * 32;
     key[i] = j < rq.T ? __ldcg(keys + j) : 0xffffffffu;
     token[i] = j < rq.T ? __ldcg(a.idx + rq.u_off + j) : -1;
     rank[i] = j - own * N;
@@ -695,8 +703,9 @@ __global__ void __launch_bounds__(MERGE_THREADS) rank_merge_kernel(TileArgs a) {
     if (next != own) asm volatile("cp.async.wait_group 1;" ::: "memory");
     else asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    if (tile < own) add_counts<N, MERGE_PER, true>(run[buf], key, rank);     // earlier tokens go first among equals
-    else add_counts<N, MERGE_PER, false>(run[buf], key, rank);
+    const uint32_t at = (uint32_t)__cvta_generic_to_shared(run[buf]);
+    if (tile < own) add_counts<N, MERGE_PER, true>(at, key, rank);     // earlier tokens go first among equals
+    else add_counts<N, MERGE_PER, false>(at, key, rank);
     __syncthreads();
     tile = next;
   }
@@ -707,10 +716,10 @@ __global__ void __launch_bounds__(MERGE_THREADS) rank_merge_kernel(TileArgs a) {
 
 // A tile that holds the segment stands alone up to 4096 scores (16 us there, in two launches over tiles of 2048 17 us; the
 // radix passes 34 us).  Above, tiles of 2048 keep more SMs busy with the sorts (8192 scores: 19.5 us, with tiles of 4096
-// 21.5 us), and from 16384 on tiles of 4096 mean half the searches (32768: 27.6 us, 29.7 us, radix passes 35.8 us).  The
-// searches grow with the square of the length: at 65536 scores both ways take 36 to 38 us on an idle GPU, at 131072 the
-// radix passes 40 us and this way 54 us.  Beside a scorer that leaves few SMs this way is the faster one up to that line
-// (a pass of eight 32K layers 630 -> 480 us, three of 50K 283 -> 259 us), and not above (four of 128K 832 -> 923 us).
+// 21.5 us), and from 16384 on tiles of 4096 mean half the searches (32768: 25.6 us, radix passes 35.8 us; 65536: 31.7 us
+// and 36 us).  The searches grow with the square of the length, and beside a scorer that leaves few SMs their work counts:
+// this way is the faster one up to that line (a pass of eight 32K layers 630 -> 480 us, three of 50K 283 -> 259 us), and
+// not above (four of 128K 832 -> 923 us).
 constexpr int ALONE_MAX_T = 4096;
 constexpr int SMALL_TILES_MAX_T = 16384;
 constexpr int MERGE_MAX_T = 65536;
