@@ -1277,8 +1277,8 @@ bool asl_tc_plan(asl_ctx* c) {
 
   // Groups of segments: pass 1 of a group, then pass 2 of the one before it, so that the fold of the row denominators is
   // hidden behind other tiles.  K of two groups should stay in L2: up to 70 MB each (at 128K tokens two kv heads, 67 MB:
-  // pass 2 then reads a quarter of K from HBM again, and the fewer hand-offs gain more: 155.4 -> 152.7 us against groups
-  // of one kv head), at least two groups.
+  // pass 2 then reads 60 % of K from HBM again, and the fewer hand-offs gain more: four layers 810 -> 802 us, eight ragged
+  // requests 598 -> 575 us against groups of up to 36 MB), at least two groups.
   std::vector<int> cut{0};
   {
     auto seg_bytes = [&](int s) { return (double)c->req[segs[s].b].n * 128 * c->k_elem_bytes / tp.nchunk; };
