@@ -17,6 +17,8 @@
 // needs a neighbour on a particular SM: the kernels run on whatever SMs a
 // concurrently running persistent kernel leaves free.  The emit writes the kept
 // indices in ascending order, followed by T .. n-1.
+#include <math.h>
+
 #include "asl_internal.cuh"
 
 namespace {
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(THREADS) topk_emit_kernel(TopkArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// One CTA per segment (plans whose longest segment has up to 256 K scores): one launch, no scratch in global memory.
+// One CTA per segment (up to 256 K scores; which calls take it: one_cta_is_faster): one launch, no scratch in global memory.
 //
 //   2048 sampled scores -> two keys L <= H that hold the k-th largest key between them with a wide margin (segments of up
 //   to 12288 scores: their smallest and largest key) -> ONE pass over the segment: a bitmap of the keys above H, and a
@@ -677,15 +679,35 @@ size_t asl_topk_scratch_bytes(int64_t segments, int64_t max_T) {
   return (size_t)(segments * SEG_INTS + segments * tiles * 2) * sizeof(int32_t);
 }
 
-// Whether the plan's segments go to the one-CTA kernel: the longest fits its bitmaps.  Called with the context's device
-// current.
+// Whether the one-CTA kernel can take the plan's segments: the longest fits its bitmaps, and the keys expected between the
+// two sampled bounds (above the lower one where that is all the list needs) fit the list with a quarter to spare (bins are coarse); where they
+// do not, the kernel would select over whole segments: 130 us and more.  Called with the context's device current.
 bool asl_topk_plan(asl_ctx* c) {
   c->topk_one_cta = c->max_T <= SEG_MAX_T;
+  for (const AslReq& r : c->req) {
+    if (r.T <= SEG_CAP) continue;
+    const double mean = (double)SEG_SAMPLE * r.k / r.T, dev = 4.0 * sqrt(mean * (1.0 - (double)r.k / r.T)) + 2.0;
+    const double above = (double)r.T * fmin(mean + dev, SEG_SAMPLE) / SEG_SAMPLE;
+    if (1.25 * fmin(above, 2.0 * dev * r.T / SEG_SAMPLE) > SEG_CAP) c->topk_one_cta = false;
+  }
   if (cudaFuncSetAttribute(topk_segment_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)seg_smem_bytes(SEG_MAX_T)) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
   return true;
+}
+
+// The faster form, in us measured back to back on an idle GPU (1, 8, 32 and 64 segments of 16K to 256K scores, k of 2 to 60 %
+// of them; within 2 us of most measurements): one CTA takes as long as the longest segment and the largest k say,
+// whatever the number of segments, and 6 us more where k is too large for the ordered copy; the tiled kernels take as long
+// as the scores of all segments say.  One segment of 96K, k = 4K: 20.8 and 21.6 us; 8 of 128K, k = 13K: 31 and 27 us;
+// 64 of 64K, k = 23K: 26 and 55 us.
+static bool one_cta_is_faster(const asl_ctx* c, int n_heads) {
+  const double k = c->max_kept - c->p.window;
+  const double one = 10.0 + 0.08e-3 * c->max_T + 0.75e-3 * fmin(k, 6500.0) + 0.3e-3 * c->max_T / 65536.0 * fmax(0.0, k - 6500.0) +
+                     (k > 2 * SEG_CAP ? 6.0 : 0.0);
+  const double tiled = 20.5 + 7.3e-6 * (double)n_heads * (double)c->sum_T;
+  return one <= tiled;
 }
 
 asl_status asl_launch_topk(asl_ctx* c, const float* scores, int32_t n_heads, int32_t* idx_out, const asl_stat* gate,
@@ -708,7 +730,7 @@ asl_status asl_launch_topk(asl_ctx* c, const float* scores, int32_t n_heads, int
   a.gate_layer = gate_layer;
   a.latch = gate ? nullptr : c->latch_stat;      // the gated call has its own rule
   a.cur_layer = c->cur_layer;
-  if (c->topk_one_cta) {
+  if (c->topk_one_cta && one_cta_is_faster(c, n_heads)) {
     topk_segment_kernel<<<dim3(1, n_heads, c->p.batch), SEG_THREADS, seg_smem_bytes(c->max_T), st>>>(a);
     c->launches += 1;
     ASL_CUDA(cudaGetLastError());

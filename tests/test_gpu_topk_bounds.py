@@ -11,13 +11,14 @@ CAP = 12288                                              # scores the kernel lis
 
 
 @pytest.mark.parametrize("kind", ["smooth", "signed", "ties", "steps"])
-@pytest.mark.parametrize("T,k", [
-    (1, 1), (31, 30), (1025, 1), (CAP - 1, 700), (CAP, CAP - 1), (CAP + 1, 12), (24577, 24576), (30001, 15000),
-    (70003, 24576), (70003, 24577), (70003, 69999), (131071, 2 * CAP + 5), (262144, 131072), (262145, 4000),
+@pytest.mark.parametrize("T,k,heads", [                  # many heads: one CTA per segment whatever k; few: large k is tiled
+    (1, 1, 2), (31, 30, 2), (1025, 1, 2), (CAP - 1, 700, 2), (CAP, CAP - 1, 2), (CAP + 1, 12, 2), (24577, 24576, 32),
+    (30001, 15000, 2), (30001, 15000, 16), (70003, 24576, 32), (70003, 24577, 32), (70003, 69999, 2), (131071, 2 * CAP + 5, 32),
+    (131071, 2 * CAP + 5, 2), (262144, 5000, 16), (262144, 131072, 2), (262145, 4000, 2),
 ])
-def test_topk(T, k, kind):
+def test_topk(T, k, heads, kind):
     w = 32
-    wl = I.workload("C1", seqlens=(T + w, 77 + w), budgets=(k + w, 20 + w))     # the second head's row starts off 16 bytes
+    wl = I.workload("C1", n_q_heads=heads, n_kv_heads=heads, seqlens=(T + w, 77 + w), budgets=(k + w, 20 + w))     # odd heads start off 16 bytes
     rng = np.random.default_rng(T + k)
     s = rng.normal(-9.0, 1.5, size=(wl.n_kv_heads, T + 77))
     if kind == "smooth":
