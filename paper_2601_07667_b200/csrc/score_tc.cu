@@ -309,13 +309,21 @@ __device__ __forceinline__ f32x2 ex2_pair_mufu(f32x2 x) {
   upk(x, a, b);
   return pk(ex2(a), ex2(b));
 }
-// 2^x of a pair on the FMA pipe (any x < 128): clamp at -125, round to the nearest
+// 2^x of a pair on the FMA pipe: clamp at -125, round to the nearest
 // integer n with the 1.5*2^23 trick, degree-4 minimax polynomial of 2^f on
 // f = x - n in [-0.5, 0.5] (relative error 2.6e-6), n added into the exponent field.
 // Packed additions are written as such, not as fma(a, 1, b): as fast, and six constant registers fewer.
+// ABOVE: x may lie above the fp32 range, and then comes out as infinity or NaN, as a sum that looks for an overflow
+// needs it: n = 129 fills the exponent field.  Without the upper clamp n runs into the sign bit there (2^130 as
+// -1.2e-38, 2^300 as -1.8e13).  Pass 2 has no such x: a logit is not above the log2 of its row's softmax denominator.
+// (The two more instructions a pair: eight layers of 32K tokens 466 -> 470 us, 0.9 to 1.3 % over the runs, four of 128K
+// 820 -> 821, 0.2 to 0.7 %.  Tried: the largest x kept by one three-way maximum a pair, 1.3 to 1.5 and 0.7 to 1.9 %; 2 or 1
+// of 16 pairs polynomial in pass 1, 1.8 and 1.5 to 2.5 %.)
+template <bool ABOVE>
 __device__ __forceinline__ f32x2 ex2_pair_poly(f32x2 x) {
   float a, b;
   upk(x, a, b);
+  if (ABOVE) { a = fminf(a, 129.0f); b = fminf(b, 129.0f); }
   const f32x2 xc = pk(fmaxf(a, -125.0f), fmaxf(b, -125.0f));
   const f32x2 magic = pk(12582912.0f, 12582912.0f);
   const f32x2 t = add2(xc, magic);
@@ -724,7 +732,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       const TcRun* rp = work.runs + slot;
       const int4 ra = __ldg(reinterpret_cast<const int4*>(rp)), rb = __ldg(reinterpret_cast<const int4*>(rp) + 1),
                  rc = __ldg(reinterpret_cast<const int4*>(rp) + 2);
-      const int run_slot = __ldg(&rp->slot);
       const int tile0 = ra.x, ntiles = ra.y, pass = ra.z, seg = ra.w, h = rb.y, chunk = rb.z, next = rb.w;
       const int T = rc.x, u_off = rc.y, rows = rc.w;
       prefetch_run(work.runs, next);
@@ -775,7 +782,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 #pragma unroll
               for (int i = 0; i < 8; ++i) {
                 const f32x2 x = fma2(pku(cur[2 * i], cur[2 * i + 1]), scale2, nm2);
-                if (pair_is_poly(i + 8 * (j & 1))) ap = add2(ex2_pair_poly(x), ap);
+                if (pair_is_poly(i + 8 * (j & 1))) ap = add2(ex2_pair_poly<true>(x), ap);
                 else                               am = add2(ex2_pair_mufu(x), am);
               }
               const float s = hsum(add2(am, ap));
@@ -817,11 +824,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           if (l > 0x1p60f) { l *= 0x1p-60f; mref += 60.f; }     // exact: keeps the running sum far from overflow
         }
         // ---- end of the run: the group publishes (reference, sum) per row ----
-        if (lt < HR) __stcg(a.partials + ((int64_t)run_slot * ENTRIES + entry) * a.NC + row, make_float2(mref, dead ? 0.f : l));
+        if (lt < HR) __stcg(a.partials + ((int64_t)__ldg(&work.runs[slot].slot) * ENTRIES + entry) * a.NC + row, make_float2(mref, dead ? 0.f : l));
         bar_sync(1 + g, 128);
         if (quarter == 0 && lane == 0) {   // the barrier orders the group's stores before this thread's fence: the release is cumulative
           __threadfence();
-          atomicAdd(published + seg * SYNC_STRIDE, 1u);
+          atomicAdd(published + __ldg(&work.runs[slot].seg) * SYNC_STRIDE, 1u);       // (read again: a register less through the tiles)
         }
       } else {
         // ---- pass 2: for every key, exp2(x - offset[row]) summed over the half's rows.  In the 16x256b shape a
@@ -862,7 +869,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                   const f32x2 x = fma2(pku(cur[2 * i], cur[2 * i + 1]), scale2, noff[4 * blk + (i >> 1)]);
-                  if (pair_is_poly(i + 8 * up)) ap[i & 1] = add2(ex2_pair_poly(x), ap[i & 1]);
+                  if (pair_is_poly(i + 8 * up)) ap[i & 1] = add2(ex2_pair_poly<false>(x), ap[i & 1]);
                   else ac[2 * up + (i & 1)] = add2(ex2_pair_mufu(x), ac[2 * up + (i & 1)]);
                 }
                 ac[2 * up] = add2(ap[0], ac[2 * up]);
