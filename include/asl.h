@@ -18,7 +18,10 @@
  *     every buffer it passes; the library keeps no reference after the call's
  *     work has finished on the stream.
  *   - Calls are asynchronous on `stream` (a cudaStream_t passed as void*);
- *     no entry point synchronises with the host.
+ *     only asl_create, asl_plan, asl_destroy and asl_device_status synchronise
+ *     with the host.  Calls that launch kernels launch them on the calling
+ *     thread's current device, which has to be the context's; asl_create and
+ *     asl_plan switch to it by themselves and back.
  *   - The library allocates device memory only inside asl_create/asl_plan
  *     (a few KB of per-request tables); scratch comes from the caller's
  *     workspace, whose size asl_plan reports.  The workspace is split into

@@ -1,11 +1,16 @@
 // C-ABI entry points: argument checks, planning, workspace layout, dispatch.
 #include <math.h>
 #include <stdlib.h>
+#include <array>
 #include <new>
 
 #include "asl_internal.cuh"
 
 namespace {
+
+std::array<cudaEvent_t*, 6> layer_events(asl_ctx* c) {
+  return {&c->ev_scored, &c->ev_pooled, &c->ev_done[0][0], &c->ev_done[0][1], &c->ev_done[1][0], &c->ev_done[1][1]};
+}
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -42,8 +47,10 @@ asl_status asl_create(asl_ctx** out, int device) {
   cudaSetDevice(device);
   cudaError_t e = cudaMalloc(&c->d_err, sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, sizeof(int32_t));
+  for (cudaEvent_t* ev : layer_events(c))           // here and not at the first layer: they belong to the device current now
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   cudaSetDevice(prev);
-  if (e != cudaSuccess) { delete c; return ASL_ERR_CUDA; }
+  if (e != cudaSuccess) { asl_destroy(c); return ASL_ERR_CUDA; }
   *out = c;
   return ASL_OK;
 }
@@ -52,8 +59,8 @@ asl_status asl_destroy(asl_ctx* c) {
   if (!c) return ASL_ERR_INVALID;
   free_plan(c);
   if (c->d_err) cudaFree(c->d_err);
-  for (cudaEvent_t e : {c->ev_scored, c->ev_pooled, c->ev_done[0][0], c->ev_done[0][1], c->ev_done[1][0], c->ev_done[1][1]})
-    if (e) cudaEventDestroy(e);
+  for (cudaEvent_t* e : layer_events(c))
+    if (*e) cudaEventDestroy(*e);
   delete c;
   return ASL_OK;
 }
@@ -280,10 +287,6 @@ asl_status asl_run_layer(asl_ctx* c, const asl_layer* l, const void* q_obs, cons
                          int32_t layer_idx, int32_t n_rows, int32_t slot) {
   if (!c || !l || slot < 0 || slot > 1) return ASL_ERR_INVALID;
   const cudaStream_t main = static_cast<cudaStream_t>(l->stream), s1 = static_cast<cudaStream_t>(l->side), s2 = static_cast<cudaStream_t>(l->side2);
-  if (!c->ev_scored) {
-    for (cudaEvent_t* e : {&c->ev_scored, &c->ev_pooled, &c->ev_done[0][0], &c->ev_done[0][1], &c->ev_done[1][0], &c->ev_done[1][1]})
-      ASL_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
-  }
   if (c->pending[slot])                             // the work of two layers ago has read the slot's buffers
     for (cudaEvent_t e : c->ev_done[slot]) ASL_CUDA(cudaStreamWaitEvent(main, e, 0));
   asl_status st = asl_score_columns(c, q_obs, k, lse, l->workspace, l->workspace_bytes, slot, l->stream);
