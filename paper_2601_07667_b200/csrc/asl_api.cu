@@ -283,6 +283,20 @@ asl_status asl_set_layer(asl_ctx* c, int32_t layer_idx) {
   return ASL_OK;
 }
 
+// what follows the scoring of a layer, on its side streams
+static asl_status issue_tail(asl_ctx* c, const asl_layer* l, const void* k, const void* v, int32_t layer_idx, int32_t n_rows, int32_t slot) {
+  const cudaStream_t s1 = static_cast<cudaStream_t>(l->side), s2 = static_cast<cudaStream_t>(l->side2);
+  asl_status st = asl_pool_scores(c, l->workspace, l->workspace_bytes, slot, l->scores_kv[slot], l->scores_agg[slot], l->side);
+  if (st != ASL_OK) return st;
+  ASL_CUDA(cudaEventRecord(c->ev_pooled, s1));
+  ASL_CUDA(cudaStreamWaitEvent(s2, c->ev_pooled, 0));
+  st = asl_rank_stat(c, l->scores_agg[slot], layer_idx, n_rows, l->rank_ring, l->stat, l->workspace, l->workspace_bytes, l->side);
+  if (st != ASL_OK) return st;
+  st = asl_select_topk(c, l->scores_kv[slot], c->p.n_kv_heads, l->idx, l->workspace, l->workspace_bytes, l->side2);
+  if (st != ASL_OK) return st;
+  return asl_compact_kv(c, k, v, l->idx, l->k_out, l->v_out, l->side2);
+}
+
 asl_status asl_run_layer(asl_ctx* c, const asl_layer* l, const void* q_obs, const void* k, const void* v, const float* lse,
                          int32_t layer_idx, int32_t n_rows, int32_t slot) {
   if (!c || !l || slot < 0 || slot > 1) return ASL_ERR_INVALID;
@@ -293,22 +307,15 @@ asl_status asl_run_layer(asl_ctx* c, const asl_layer* l, const void* q_obs, cons
   if (st != ASL_OK) return st;
   ASL_CUDA(cudaEventRecord(c->ev_scored, main));
   ASL_CUDA(cudaStreamWaitEvent(s1, c->ev_scored, 0));
-  st = asl_pool_scores(c, l->workspace, l->workspace_bytes, slot, l->scores_kv[slot], l->scores_agg[slot], l->side);
-  if (st != ASL_OK) return st;
-  ASL_CUDA(cudaEventRecord(c->ev_pooled, s1));
-  ASL_CUDA(cudaStreamWaitEvent(s2, c->ev_pooled, 0));
-  st = asl_rank_stat(c, l->scores_agg[slot], layer_idx, n_rows, l->rank_ring, l->stat, l->workspace, l->workspace_bytes, l->side);
-  if (st != ASL_OK) return st;
-  st = asl_select_topk(c, l->scores_kv[slot], c->p.n_kv_heads, l->idx, l->workspace, l->workspace_bytes, l->side2);
-  if (st != ASL_OK) return st;
-  st = asl_compact_kv(c, k, v, l->idx, l->k_out, l->v_out, l->side2);
-  if (st != ASL_OK) return st;
+  st = issue_tail(c, l, k, v, layer_idx, n_rows, slot);
+  // a step that fails leaves those before it queued: the slot's next use and a join wait for them as for a whole layer
+  if (st != ASL_OK) ASL_CUDA(cudaStreamWaitEvent(s2, c->ev_scored, 0));        // (a capture may not have reached s2 yet)
   ASL_CUDA(cudaEventRecord(c->ev_done[slot][1], s2));
   if (l->one_side) ASL_CUDA(cudaStreamWaitEvent(s1, c->ev_done[slot][1], 0));
   ASL_CUDA(cudaEventRecord(c->ev_done[slot][0], s1));
   c->pending[slot] = true;
   c->last_slot = slot;
-  return ASL_OK;
+  return st;
 }
 
 asl_status asl_run_join(asl_ctx* c, void* stream) {

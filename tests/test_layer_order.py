@@ -68,6 +68,36 @@ class Layers:
         assert self.lib.asl_destroy(self.ctx) == B.ASL_OK
 
 
+@pytest.mark.parametrize("one_side", [0, 1])
+@pytest.mark.parametrize("fail,issued", [
+    ("pool", ["score"]), ("rank", ["score", "pool"]), ("topk", ["score", "pool", "rank"]),
+    ("compact", ["score", "pool", "rank", "topk"]),
+    (dict(n_rows=3), ["score", "pool"]), (dict(idx=None), ["score", "pool", "rank"]),      # refused by a step's own checks
+])
+def test_a_slot_waits_for_what_a_failed_layer_left_in_flight(lib, fail, issued, one_side):
+    """A step of a layer fails when the steps before it are already queued: the slot's next scoring, and whoever joins,
+    must still wait for them (the pooling reads the slot's sums on another stream)."""
+    p = Layers(lib)
+    assert p.run(1, one_side) == B.ASL_OK and p.run(0, one_side) == B.ASL_OK
+    at = len(p.order()[0])
+    if isinstance(fail, str):
+        lib.fake_fail(fail.encode(), 1)
+        assert p.run(1, one_side) == B.ASL_ERR_CUDA
+    else:
+        assert p.run(1, one_side, **fail) == B.ASL_ERR_INVALID
+    names, _, _ = p.order()
+    left = set(range(at, len(names)))
+    assert names[at:] == issued
+    assert p.lib.asl_run_join(p.ctx, 109) == B.ASL_OK
+    assert left <= p.order()[2][109]
+    nxt = len(names)
+    assert p.run(1, one_side) == B.ASL_OK
+    names, before, _ = p.order()
+    assert names[nxt:] == ["score", "pool", "rank", "topk", "compact"]
+    assert left <= before[nxt]
+    p.close()
+
+
 def test_layers_in_order(lib):
     """Three good layers: a step follows what it reads, and a slot's scoring what read the slot two layers ago."""
     p = Layers(lib)
