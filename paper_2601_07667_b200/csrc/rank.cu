@@ -22,8 +22,7 @@ constexpr int SORT_THREADS = 256;
 constexpr int WARPS = SORT_THREADS / 32;
 constexpr int PER_WARP = TILE / WARPS;   // consecutive keys of one warp
 constexpr int ROUNDS = PER_WARP / 32;    // walked 32 at a time, all loads issued up front
-constexpr int PARTS = SORT_THREADS / 256;  // threads per digit where a thread walks a digit's column of tile counts
-static_assert(SORT_THREADS % 256 == 0 && SORT_THREADS <= 1024 && TILE % SORT_THREADS == 0, "a thread per digit; whole rounds");
+static_assert(SORT_THREADS == 256 && TILE % SORT_THREADS == 0, "a thread per digit; whole rounds");
 
 __device__ __forceinline__ uint32_t desc_key(float s) {
   uint32_t u = __float_as_uint(s);
@@ -175,12 +174,11 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
                                                              int32_t* __restrict__ next_counts,
                                                              const AslReq* __restrict__ req,
                                                              const asl_stat* __restrict__ latch, int shift, int nblk) {
-  constexpr int SCAN_BATCH = 64 / PARTS;       // loads of tile counts in flight per thread
+  constexpr int SCAN_BATCH = 64;               // loads of tile counts in flight per thread
   __shared__ int cnt[WARPS][256];
   __shared__ uint32_t lanes[WARPS][256];
   __shared__ int warp_tot[8];
   __shared__ int digit_off[256];
-  __shared__ int part_tot[PARTS > 1 ? PARTS : 1][PARTS > 1 ? 256 : 1], part_before[PARTS > 1 ? PARTS : 1][PARTS > 1 ? 256 : 1];
   pdl_release_successor();
   const int b = blockIdx.y, blk = blockIdx.x;
   if (latch && latch[b].selected) return;
@@ -198,30 +196,16 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
   load_tile<FIRST>(agg, keys_in, idx_in, rq, wstart, lane, key, id);
   if (FIRST) pdl_wait_predecessor();
   if (SCAN) {
-    // PARTS threads per digit, each over a run of the tiles' counts with all of its loads in flight
-    const int d = threadIdx.x & 255, part = threadIdx.x >> 8;
+    // a thread per digit, with all of its loads in flight
     const int used = (rq.T + TILE - 1) / TILE;
-    const int per = (used + PARTS - 1) / PARTS;
-    const int b0 = part * per, b1 = min(used, b0 + per);
-    const int32_t* col = counts + (int64_t)b * nblk * 256 + d;
+    const int32_t* col = counts + (int64_t)b * nblk * 256 + threadIdx.x;
     int before = 0, total = 0;
-    for (int i0 = b0; i0 < b1; i0 += SCAN_BATCH) {
+    for (int i0 = 0; i0 < used; i0 += SCAN_BATCH) {
       int v[SCAN_BATCH];
 #pragma unroll
-      for (int k = 0; k < SCAN_BATCH; ++k) v[k] = (i0 + k < b1) ? __ldcg(col + (int64_t)(i0 + k) * 256) : 0;
+      for (int k = 0; k < SCAN_BATCH; ++k) v[k] = (i0 + k < used) ? __ldcg(col + (int64_t)(i0 + k) * 256) : 0;
 #pragma unroll
       for (int k = 0; k < SCAN_BATCH; ++k) { total += v[k]; if (i0 + k < blk) before += v[k]; }
-    }
-    if (PARTS > 1) {
-      part_tot[part][d] = total;
-      part_before[part][d] = before;
-      __syncthreads();
-      total = 0;
-      before = 0;
-      if (threadIdx.x < 256) {
-#pragma unroll
-        for (int q = 0; q < PARTS; ++q) { total += part_tot[q][d]; before += part_before[q][d]; }
-      }
     }
     int incl = total;                       // exclusive scan of the digit totals over the 256 digits
 #pragma unroll
@@ -229,15 +213,13 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
       const int v = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += v;
     }
-    if (threadIdx.x < 256 && lane == 31) warp_tot[wid] = incl;
+    if (lane == 31) warp_tot[wid] = incl;
     __syncthreads();
-    if (threadIdx.x < 256) {
-      int off = incl - total + before;
-      for (int w2 = 0; w2 < wid; ++w2) off += warp_tot[w2];
-      digit_off[threadIdx.x] = off;
-    }
+    int off = incl - total + before;
+    for (int w2 = 0; w2 < wid; ++w2) off += warp_tot[w2];
+    digit_off[threadIdx.x] = off;
   } else {
-    if (threadIdx.x < 256) digit_off[threadIdx.x] = counts[((int64_t)b * nblk + blk) * 256 + threadIdx.x];
+    digit_off[threadIdx.x] = counts[((int64_t)b * nblk + blk) * 256 + threadIdx.x];
   }
   for (int i = threadIdx.x; i < WARPS * 256; i += SORT_THREADS) { (&cnt[0][0])[i] = 0; (&lanes[0][0])[i] = 0; }
   __syncthreads();

@@ -1373,8 +1373,7 @@ bool asl_tc_plan(asl_ctx* c) {
   tp.d_live_folds = reinterpret_cast<TcFold*>(d + live_at[2]);
   tp.d_live_scratch = reinterpret_cast<int32_t*>(d + live_at[3]);
   tp.d_live_hdr = reinterpret_cast<int32_t*>(d + live_at[4]);
-  tp.enabled = encode_fn() != nullptr;
-  return tp.enabled;
+  return encode_fn() != nullptr;
 }
 
 size_t asl_tc_partial_bytes(const asl_ctx* c) { return (size_t)c->tc.partial_slots * (c->tc.wide ? GROUPS / 2 : GROUPS) * c->tc.NC * sizeof(float2); }

@@ -37,7 +37,6 @@ struct TcList {                  // a work list on the device: runs of pass 1, t
 };
 
 struct AslTcPlan {
-  bool enabled = false;
   int NC = 0;           // rows of a chunk's buffer (halves of HR)
   int HR = 0;           // rows of a half: one accumulator of pass 1 (lanes) or pass 2 (columns), a multiple of 32, at most 128
   bool wide = false;    // two halves
