@@ -104,8 +104,11 @@ typedef struct {
                           /* [H_k][sum_kept][d] bytes), V stays bf16.  The queries stay   */
                           /* bf16: the scorer splits each into two E4M3 terms (exact for  */
                           /* 1/64 <= |q| <= 28, else to 2^-13 / saturated) and runs the   */
-                          /* contraction on the 8-bit tensor-core path.  Shapes the       */
-                          /* tensor-core scorer does not take are ASL_ERR_UNSUPPORTED.    */
+                          /* contraction on the 8-bit tensor-core path.  Windows: with    */
+                          /* average pooling 32, 64, 96, 128, 192 and 256; with max       */
+                          /* pooling multiples of 32 up to 256 for which m * window is a  */
+                          /* multiple of 64, m being the largest divisor of H_q / H_k     */
+                          /* with m * window <= 256; all others are ASL_ERR_UNSUPPORTED.  */
   int32_t reserved0;
   const float* k_scale;   /* host [H_k], finite and > 0; read only for ASL_K_FP8_E4M3     */
 } asl_params;
@@ -167,7 +170,13 @@ asl_status asl_score_layer_lse(asl_ctx* ctx, const void* q_obs, const void* k, c
  * its un-pooled sums in slot 0 or 1 of the workspace; the second half is the
  * pooling, SumGroups and the aggregate.  The second half of layer l may run on
  * another stream while the first half of layer l+1 fills the other slot.
- * asl_score_layer = both halves on slot 0. */
+ * asl_score_layer computes the same as both halves on slot 0, but where the plan
+ * leaves the number of CTAs to the library (score_ctas = 0) the first half takes
+ * 16 or 32 fewer than asl_score_layer: sums that then fall to other CTAs are added
+ * in another order and may differ in their last bits, and with them rank rows and
+ * kept lists, which are discontinuous in the scores.  With score_ctas or lse given,
+ * or where no group of segments has more tiles than the smaller number of CTAs, the
+ * two agree bit for bit. */
 asl_status asl_score_columns(asl_ctx* ctx, const void* q_obs, const void* k, const float* lse, void* workspace,
                              size_t workspace_bytes, int32_t slot, void* stream);
 asl_status asl_pool_scores(asl_ctx* ctx, void* workspace, size_t workspace_bytes, int32_t slot, float* scores_kv,
@@ -239,6 +248,9 @@ asl_status asl_compact_kv(asl_ctx* ctx, const void* k, const void* v, const int3
  * asl_pool_scores and asl_rank_stat on `side`, asl_select_topk and asl_compact_kv on `side2`, ordered by events that
  * the context keeps.  The side streams are not waited for: they run under the scoring of the next layer, and a slot's
  * buffers are written again only when the work of two layers ago has read them.  Use slots 0 and 1 in turn.
+ * k and v are read on `side2` after `stream` has gone on: they stay as they are until a join (a caching allocator that
+ * knows them by `stream` alone has to be told, or must not get them back before).  Where a step fails its status is
+ * returned, what was issued before it stays in flight, and the slot's next use and a join wait for that too.
  * asl_run_join makes `stream` wait for everything issued so far.  asl_run_reset forgets what is in flight, without
  * waiting: call it before and after capturing layers into a CUDA graph (nothing recorded outside a capture may be
  * waited for inside it, nor the other way round). */

@@ -383,7 +383,8 @@ class LayerPath:
 
     def run_layer(self, q_obs, k, v, layer_idx: int, *, overlap: bool = True, score_marks=None, lse=None) -> None:
         """Steps a1..a5 for one layer on the current stream; with ``overlap`` everything after the scoring
-        runs on the side streams and is left in flight (see ``join``).  ``score_marks``: a list
+        runs on the side streams and is left in flight (see ``join``): ``k`` and ``v`` are read there, so keep them (or
+        ``record_stream(path.side2)``) until a join.  ``score_marks``: a list
         that receives a (start, end) event pair around the scoring call."""
         main = self.torch.cuda.current_stream()
         rows = self.n_rows(layer_idx)

@@ -18,10 +18,11 @@
 // up to 256 of the G*W query rows that share a kv head.  Work is dealt in "runs": the
 // contiguous tiles that one CTA takes of one segment in one pass.  Segments form groups;
 // a CTA does its runs of pass 1 of group i, then those of pass 2 of group i - 1: it
-// meets one or two segments at a time and keeps a Q chunk for a whole run, the offsets
-// that pass 2 needs were folded while other tiles were worked on, and most of K of two
-// groups (up to 70 MB each) is still in L2 when pass 2 reads it again.  Dealing every segment's tiles round-robin to all
-// CTAs cost 3 us per segment and pass (64 KB of Q reloaded per CTA, a hand-off each):
+// meets one or two segments at a time and keeps a Q chunk for a whole run, and the
+// offsets that pass 2 needs were folded while other tiles were worked on.  Between the two
+// reads of a tile lie up to two groups (up to 70 MB each): of 134 MB of K (64K tokens, 8 kv
+// heads) pass 2 finds 60 % in L2, of 268 MB 40 %.  Dealing every segment's tiles round-robin
+// to all CTAs cost 3 us per segment and pass (64 KB of Q reloaded per CTA, a hand-off each):
 // 32K tokens, 8 kv heads 64 -> 48 us, eight ragged requests with W = 32 350 -> 184 us,
 // W = 128 with 64 query heads at 64K 374 -> 288 us, 128K tokens 163 -> 153 us.
 //
@@ -29,9 +30,9 @@
 // take a degree-4 polynomial on the FMA pipe, the others the MUFU unit (16 per clock and
 // SM): a tile of 128 keys x 256 rows is 32768 of them, 1664 clk of MUFU, and the loop
 // takes about 1950 in the kernel.  Kept up for more than some
-// ten milliseconds the kernel runs at the 1000 W limit (1.6 GHz instead of 1.9), where
-// the energy of the MMAs (0.7 us at the limit per 148 tiles) and of streaming K (45 us at
-// the limit for 268 MB from HBM, 16 from L2) counts as much as instructions do.
+// ten milliseconds the kernel runs at the 1000 W limit: at 128K tokens a layer takes 204 us
+// at 1.55 GHz and 988 W, 201 mJ (one pass over K: 113 us, 112 mJ), and 167 us in a burst at
+// 1.97 GHz.
 //
 // Inside a CTA: warp 0 streams K tiles through a TMA ring (128B-swizzled) and keeps the Q
 // chunks of two runs resident; warp 1 issues tcgen05.mma from a warp-uniform loop (under
@@ -338,8 +339,8 @@ __device__ __forceinline__ f32x2 ex2_pair_poly(f32x2 x) {
   return pku(pl + (tl << 23), ph + (th << 23));
 }
 // Which of every 16 column pairs take the polynomial, spread out.  3: the loop alone is shortest at 5 (clk per tile,
-// pass 1 / pass 2, at 4, 5, 6: 1821 / 1833, 1725 / 1794, 1747 / 1839), but a polynomial costs more energy than the MUFU
-// unit and more registers; in the kernel, at 128K tokens: 155.4, 156.9, 160.9 us at 3, 4, 5.
+// pass 1 / pass 2, at 4, 5, 6: 1821 / 1833, 1725 / 1794, 1747 / 1839), but a polynomial takes more
+// registers; in the kernel, at 128K tokens: 155.4, 156.9, 160.9 us at 3, 4, 5.
 constexpr int POLY_OF_16 = 3;
 __device__ __forceinline__ constexpr bool pair_is_poly(int i) { return ((i & 15) * POLY_OF_16) % 16 + POLY_OF_16 >= 16; }
 
@@ -1135,7 +1136,8 @@ int score_kernel_of(const asl_params& p, const AslTcPlan& tp) {
 // ---------------------------------------------------------------- host side
 namespace {
 
-// FP8 keys are taken for the windows that asl.h promises: chunks of whole heads in multiples of 64 rows
+// The FP8 windows that asl.h names.  (plan_chunks cuts any window; the scorer before this one took chunks of whole heads
+// in multiples of 64 rows only, and what it refused is refused still: no other window is tested with FP8 keys.)
 bool fp8_shape(const asl_params& p) {
   const int W = p.window, R = p.n_q_heads / p.n_kv_heads * W;
   if (W % 32 || W > MAX_ROWS) return false;
@@ -1283,9 +1285,12 @@ bool asl_tc_plan(asl_ctx* c) {
   if (tiles >= (int64_t)1 << 30) return false;
 
   // Groups of segments: pass 1 of a group, then pass 2 of the one before it, so that the fold of the row denominators is
-  // hidden behind other tiles.  K of two groups should stay in L2: up to 70 MB each (at 128K tokens two kv heads, 67 MB:
-  // pass 2 then reads 60 % of K from HBM again, and the fewer hand-offs gain more: four layers 810 -> 802 us, eight ragged
-  // requests 598 -> 575 us against groups of up to 36 MB), at least two groups.
+  // hidden behind other tiles; at least two of them, of up to 70 MB of K each.  Small groups leave more of K in L2 for pass 2
+  // (above), large ones need fewer hand-offs, and the hand-offs count for more.  In us at 36, 50, 70, 100, 140 and 270 MB:
+  // four layers of 100K tokens 668, 670, 642, 645, 640, 640; of 128K 843, 843, 841, 843, 845, 834; of 192K 1236, 1240, 1241,
+  // 1243, 1232, 1218; two layers of eight ragged requests 616, 599, 602, 602, 592, 582; two with W = 128 and 64 query heads
+  // at 64K 761, 758, 760, 768, 760, 762.  So the limit is above the step at 100K tokens (25.6 MB a kv head: two in a group),
+  // but not where batches are fastest.
   std::vector<int> cut{0};
   {
     auto seg_bytes = [&](int s) { return (double)c->req[segs[s].b].n * 128 * c->k_elem_bytes / tp.nchunk; };

@@ -3,9 +3,9 @@
 // Radix select on an order-preserving 32-bit image of the fp32 score, 11+11+10
 // bits from the top: the exact k-th largest key is found; every token with a
 // larger key is kept, and of the tokens equal to it the lowest-indexed fill the
-// remainder.  Two forms.  Plans whose longest segment has up to 256 K scores
-// run one CTA per segment in a single launch
-// (second half of this file).  Longer ones are cut into tiles of 4096 scores,
+// remainder.  Two forms.  Segments of up to 256 K scores go to one CTA each in a
+// single launch (second half of this file) wherever an estimate of both forms' times
+// says so (one_cta_is_faster).  The others are cut into tiles of 4096 scores,
 // one 256-thread CTA per tile with its 16 scores per thread in registers, and
 // into five short kernels that meet only through global memory:
 //
@@ -698,9 +698,11 @@ bool asl_topk_plan(asl_ctx* c) {
 }
 
 // The faster form, in us measured back to back on an idle GPU (1, 8, 32 and 64 segments of 16K to 256K scores, k of 2 to 60 %
-// of them; within 2 us of most measurements): one CTA takes as long as the longest segment and the largest k say,
-// whatever the number of segments, and 6 us more where k is too large for the ordered copy; the tiled kernels take as long
-// as the scores of all segments say.  One segment of 96K, k = 4K: 20.8 and 21.6 us; 8 of 128K, k = 13K: 31 and 27 us;
+// of them; within 2 us of most measurements): one CTA takes as long as the longest segment and the largest k say, for any
+// number of segments up to the SM count (172 KB of shared memory a CTA at 256K scores: one to an SM), and 6 us more where k
+// is too large for the ordered copy; the tiled kernels take as long as the scores of all segments say.  An estimate, no
+// bound: it takes the longest segment and the largest k for one request's where they are two, and a layer issues the call
+// beside a scorer that leaves 16 SMs, where neither form has been measured against the other.  One segment of 96K, k = 4K: 20.8 and 21.6 us; 8 of 128K, k = 13K: 31 and 27 us;
 // 64 of 64K, k = 23K: 26 and 55 us.
 static bool one_cta_is_faster(const asl_ctx* c, int n_heads) {
   const double k = c->max_kept - c->p.window;

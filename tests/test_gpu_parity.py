@@ -79,7 +79,7 @@ def test_edge_shapes(seqlens, budgets, w, S):
 @pytest.mark.parametrize("seqlens,w,S", [
     ((152, 156, 2032 + 32, 36), 32, 9),      # segments of 120, 124, 2032 and 4 past tokens (a warp pools 120): widest window of the kernel
     ((152, 156, 2032 + 32, 36), 32, 1),      # no neighbours at all
-    ((1000 + 24, 484 + 24), 24, 3),          # one partial row per kv head (the CUDA-core scorer's layout)
+    ((1000 + 24, 484 + 24), 24, 3),          # a window off the multiples of 32: one partial row per kv head
     ((3000 + 64, 1200 + 64), 64, 11),        # a window beyond the kernel's reach: the general kernel on the same layout
     ((3000 + 64, 1201 + 64), 64, 7),         # second segment off a 16-byte boundary: the general kernel
 ])
@@ -100,7 +100,7 @@ def test_average_pooling_on_aligned_segments(seqlens, w, S):
     (4, 2, 256, 1, 1500),     # window as large as a chunk
     (4, 4, 64, 0, 1111),      # no grouping: 64-row chunk
     (6, 2, 32, 0, 1000),      # 96-row chunk
-    (28, 4, 64, 0, 2500),     # seven query heads per kv head: 448 rows in seven 64-row chunks
+    (28, 4, 64, 0, 2500),     # seven query heads per kv head: 448 rows in chunks of 256 and 192
 ])
 def test_scorer_shapes(Hq, Hk, w, mode, n):
     wl = I.workload("C3", n_q_heads=Hq, n_kv_heads=Hk, window=w, pool_mode=mode, seqlens=(n,), budgets=(w + 100,),
@@ -142,6 +142,7 @@ def test_strided_inputs_on_the_tensor_core_scorer():
 
 
 def test_strided_inputs_on_the_cuda_core_scorer():
+    """(Named when such windows had a scorer on the CUDA cores; a window off the multiples of 32, ragged.)"""
     _strided_case(I.workload("C1", seqlens=(1500, 700), budgets=(200, 100), window=24, layers=2, l_min=1, l_obs=2), 6)
 
 
@@ -199,7 +200,7 @@ def test_fp8_keys_are_refused_where_no_tensor_core_path_exists():
                 cu_seqlens=[0, 500], budgets=[64], l_min=1, l_obs=2, tau=0.3,
                 q_stride=(8 * 24 * 128, 24 * 128, 128), k_stride=(256, 128), v_stride=(256, 128))
     with pytest.raises(B.AslError) as e:
-        B.asl_plan(ctx, **base, k_dtype=B.ASL_K_FP8_E4M3, k_scale=[1.0, 1.0])       # W = 24: CUDA-core scorer only
+        B.asl_plan(ctx, **base, k_dtype=B.ASL_K_FP8_E4M3, k_scale=[1.0, 1.0])       # W = 24 is none of the FP8 windows
     assert e.value.status == B.ASL_ERR_UNSUPPORTED
     ok = {**base, "window": 32, "q_stride": (8 * 32 * 128, 32 * 128, 128)}
     for bad in (dict(k_scale=None), dict(k_scale=[1.0, 0.0]), dict(k_scale=[1.0, float("inf")]), dict(k_stride=(264, 128))):
@@ -211,9 +212,10 @@ def test_fp8_keys_are_refused_where_no_tensor_core_path_exists():
 
 
 def test_logits_far_above_the_first_keys_of_a_row():
-    """Keys whose logit exceeds the row's reference (the maximum over its first 32 keys) by more than
-    fp32's exponent range, so that the plain pass-1 sums overflow: in the last 32 keys of a tile (redone
-    from registers), in the middle of a tile (the tile is redone with running maxima), twice in a row."""
+    """Several keys whose logit exceeds the row's reference (its first logit of the run) by more than fp32's
+    exponent range, some of them in neighbouring columns and tiles, so that pass-1 sums overflow, the tile is redone
+    with running maxima, and a still larger key follows.  What a row's largest key hides here, a single heavy key
+    in each column of a tile, its last 16 keys among them, is test_gpu_scorer_overflow.py."""
     from paper_2601_07667_b200 import binding as B
     from asl_check import assert_scores_close, oracle_layer
     Hq, Hk, w, n = 32, 8, 64, 3000
@@ -602,7 +604,7 @@ def test_layers_replayed_from_a_cuda_graph_match_the_calls():
                                             (28, 4, 64, 0, 1500), (6, 2, 32, 0, 700)])     # the last two: padded chunks
 def test_one_pass_scoring_with_supplied_lse(Hq, Hk, w, mode, n):
     """asl_score_layer_lse fed the oracle's log-sum-exp gives the oracle's scores; asl_window_lse
-    returns the denominators the two-pass call found (tensor-core shapes and the CUDA-core fallback)."""
+    returns the denominators the two-pass call found."""
     from paper_2601_07667_b200 import binding as B
     from asl_check import assert_scores_close, oracle_layer
     wl = I.workload("C3", n_q_heads=Hq, n_kv_heads=Hk, window=w, pool_mode=mode, seqlens=(n,), budgets=(w + 50,),
@@ -628,8 +630,9 @@ def test_one_pass_scoring_with_supplied_lse(Hq, Hk, w, mode, n):
 
 @pytest.mark.parametrize("Hq,Hk,w,mode,n", [(32, 8, 64, 0, 3000), (8, 2, 32, 1, 2000), (6, 2, 40, 0, 900)])
 def test_scoring_in_two_halves_matches_the_single_call_and_the_oracle(Hq, Hk, w, mode, n):
-    """asl_score_columns + asl_pool_scores on either workspace slot give the oracle's scores and,
-    bit for bit, what asl_score_layer gives; the two slots do not disturb each other."""
+    """asl_score_columns + asl_pool_scores on either workspace slot give the oracle's scores and, at these sizes
+    (no group of segments has more tiles than either takes CTAs), bit for bit what asl_score_layer gives; the two
+    slots do not disturb each other."""
     from paper_2601_07667_b200 import binding as B
     from asl_check import assert_scores_close, oracle_layer
     wl = I.workload("C3", n_q_heads=Hq, n_kv_heads=Hk, window=w, pool_mode=mode, seqlens=(n,), budgets=(w + 50,),
