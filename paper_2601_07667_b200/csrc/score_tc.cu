@@ -30,9 +30,9 @@
 // take a degree-4 polynomial on the FMA pipe, the others the MUFU unit (16 per clock and
 // SM): a tile of 128 keys x 256 rows is 32768 of them, 1664 clk of MUFU, and the loop
 // takes about 1950 in the kernel.  Kept up for more than some
-// ten milliseconds the kernel runs at the 1000 W limit: at 128K tokens a layer takes 204 us
-// at 1.55 GHz and 988 W, 201 mJ (one pass over K: 113 us, 112 mJ), and 167 us in a burst at
-// 1.97 GHz.
+// ten milliseconds the kernel runs at the 1000 W limit: at 128K tokens a layer takes 193 to
+// 204 us (two boards, at 1.62 and 1.55 GHz, 990 W: 191 to 201 mJ; one pass over K 108 to 113
+// us), and 166 us in a burst at 1.97 GHz.
 //
 // Inside a CTA: warp 0 streams K tiles through a TMA ring (128B-swizzled) and keeps the Q
 // chunks of two runs resident; warp 1 issues tcgen05.mma from a warp-uniform loop (under
@@ -317,8 +317,8 @@ __device__ __forceinline__ f32x2 ex2_pair_mufu(f32x2 x) {
 // ABOVE: x may lie above the fp32 range, and then comes out as infinity or NaN, as a sum that looks for an overflow
 // needs it: n = 129 fills the exponent field.  Without the upper clamp n runs into the sign bit there (2^130 as
 // -1.2e-38, 2^300 as -1.8e13).  Pass 2 has no such x: a logit is not above the log2 of its row's softmax denominator.
-// (The two more instructions a pair: eight layers of 32K tokens 466 -> 470 us, 0.9 to 1.3 % over the runs, four of 128K
-// 820 -> 821, 0.2 to 0.7 %.  Tried: the largest x kept by one three-way maximum a pair, 1.3 to 1.5 and 0.7 to 1.9 %; 2 or 1
+// (The two more instructions a pair: eight layers of 32K tokens 466 -> 470 us, 0.9 to 1.5 % over the runs, four of 128K
+// 820 -> 821, 0.2 to 0.7 %, two prompts with W = 24 31.2 -> 31.7.  Tried: the largest x kept by one three-way maximum a pair, 1.3 to 1.5 and 0.7 to 1.9 %; 2 or 1
 // of 16 pairs polynomial in pass 1, 1.8 and 1.5 to 2.5 %.)
 template <bool ABOVE>
 __device__ __forceinline__ f32x2 ex2_pair_poly(f32x2 x) {

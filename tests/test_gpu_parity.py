@@ -194,6 +194,7 @@ def test_fp8_key_cache(Hq, Hk, w, mode, n):
 
 
 def test_fp8_keys_are_refused_where_no_tensor_core_path_exists():
+    """FP8 keys with a window that asl.h does not name, or with scales or strides that cannot be, are refused."""
     from paper_2601_07667_b200 import binding as B
     ctx = B.asl_create(0)
     base = dict(n_q_heads=8, n_kv_heads=2, head_dim=128, window=24, pool_kernel=7, pool_mode=0,
