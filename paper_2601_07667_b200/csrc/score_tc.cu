@@ -32,7 +32,7 @@
 // takes about 1950 in the kernel.  Kept up for more than some
 // ten milliseconds the kernel runs at the 1000 W limit: at 128K tokens a layer takes 193 to
 // 204 us (two boards, at 1.62 and 1.55 GHz, 990 W: 191 to 201 mJ; one pass over K 108 to 113
-// us), and 166 us in a burst at 1.97 GHz.
+// us), and 166 to 170 us in a burst at 1.97 GHz.
 //
 // Inside a CTA: warp 0 streams K tiles through a TMA ring (128B-swizzled) and keeps the Q
 // chunks of two runs resident; warp 1 issues tcgen05.mma from a warp-uniform loop (under
