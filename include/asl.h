@@ -298,7 +298,7 @@ asl_status asl_compact_rows(asl_ctx* ctx, const void* x, const int32_t* idx, voi
  * Such a caller can use neither asl_create/asl_plan (both allocate small device
  * tables) nor a workspace it has nowhere to take from.  This call needs no
  * context and no workspace: its sort scratch is a fixed array compiled into
- * the library (about 4.5 MiB of device memory on every GPU that loads the
+ * the library (about 4.1 MiB of device memory on every GPU that loads the
  * library, held until the process exits).
  *
  *   scores    device fp32 [T]   one request's aggregate scores

@@ -3,9 +3,9 @@
 //
 // RankDesc: position of every (key, token index) pair in sorted order per request, key = bit pattern that ascends as the
 // score descends; equal scores keep ascending index order, so the position is the token's 0-based rank with ties to the
-// lower index.  Segments of up to 64K tokens: sorted tiles, merged by search (below).  Longer ones: a stable
-// least-significant-digit radix sort (8-bit digits, one kernel per digit after a first histogram); the last pass scatters
-// positions straight into the ring row.
+// lower index.  Single segments of up to 4096 tokens: every token counts those before it.  Up to 256K tokens: split at
+// sampled pairs, then placed bucket by bucket (below).  Longer ones: a stable least-significant-digit radix sort (8-bit
+// digits, one kernel per digit after a first histogram); the last pass scatters positions straight into the ring row.
 //
 // Statistic: a token is in the union iff its smallest rank over the rows is < k
 // (the k smallest ranks of a row are exactly ranks 0..k-1).  The numerator
@@ -159,13 +159,10 @@ __global__ void __launch_bounds__(1024) rank_scan(int32_t* __restrict__ hist, co
   }
 }
 
-// Stable scatter of one tile; the last pass writes rank[token] = position.
-// SCAN: `counts` holds raw tile counts and the tile's first output positions are
-// summed here (thread = digit walks the tiles' rows; used while the request has few
-// tiles); otherwise `counts` was turned into positions by rank_scan.  A pass that is
-// not the last counts, per destination tile, the next digit of every pair it writes
-// (integer atomics: the table does not depend on the order of arrival).
-template <bool FIRST, bool SCAN>
+// Stable scatter of one tile; the last pass writes rank[token] = position.  A pass that is not the last counts, per
+// destination tile, the next digit of every pair it writes (integer atomics: the table does not depend on the order of
+// arrival).
+template <bool FIRST>
 __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __restrict__ agg,
                                                              const uint32_t* __restrict__ keys_in,
                                                              const int32_t* __restrict__ idx_in,
@@ -174,10 +171,8 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
                                                              int32_t* __restrict__ next_counts,
                                                              const AslReq* __restrict__ req,
                                                              const asl_stat* __restrict__ latch, int shift, int nblk) {
-  constexpr int SCAN_BATCH = 64;               // loads of tile counts in flight per thread
   __shared__ int cnt[WARPS][256];
   __shared__ uint32_t lanes[WARPS][256];
-  __shared__ int warp_tot[8];
   __shared__ int digit_off[256];
   pdl_release_successor();
   const int b = blockIdx.y, blk = blockIdx.x;
@@ -195,32 +190,7 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
   if (!FIRST) pdl_wait_predecessor();
   load_tile<FIRST>(agg, keys_in, idx_in, rq, wstart, lane, key, id);
   if (FIRST) pdl_wait_predecessor();
-  if (SCAN) {
-    // a thread per digit, with all of its loads in flight
-    const int used = (rq.T + TILE - 1) / TILE;
-    const int32_t* col = counts + (int64_t)b * nblk * 256 + threadIdx.x;
-    int before = 0, total = 0;
-    for (int i0 = 0; i0 < used; i0 += SCAN_BATCH) {
-      int v[SCAN_BATCH];
-#pragma unroll
-      for (int k = 0; k < SCAN_BATCH; ++k) v[k] = (i0 + k < used) ? __ldcg(col + (int64_t)(i0 + k) * 256) : 0;
-#pragma unroll
-      for (int k = 0; k < SCAN_BATCH; ++k) { total += v[k]; if (i0 + k < blk) before += v[k]; }
-    }
-    int incl = total;                       // exclusive scan of the digit totals over the 256 digits
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    if (lane == 31) warp_tot[wid] = incl;
-    __syncthreads();
-    int off = incl - total + before;
-    for (int w2 = 0; w2 < wid; ++w2) off += warp_tot[w2];
-    digit_off[threadIdx.x] = off;
-  } else {
-    digit_off[threadIdx.x] = counts[((int64_t)b * nblk + blk) * 256 + threadIdx.x];
-  }
+  digit_off[threadIdx.x] = counts[((int64_t)b * nblk + blk) * 256 + threadIdx.x];
   for (int i = threadIdx.x; i < WARPS * 256; i += SORT_THREADS) { (&cnt[0][0])[i] = 0; (&lanes[0][0])[i] = 0; }
   __syncthreads();
   // per-warp digit counts; the peer masks are kept for the second walk
@@ -272,15 +242,11 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
 }
 
 // the four passes of one rank row; scratch: two key and two index arrays, four tables of tile histograms
-constexpr int SCAN_IN_SCATTER_MAX_TILES = 128;
-
 int launch_sort(const float* agg, const AslReq* req, const asl_stat* latch, int batch, int max_T, uint32_t* const keys[2],
                 int32_t* const idx[2], int32_t* hist, int32_t* rank_row, cudaStream_t st) {
   const int nblk = (max_T + TILE - 1) / TILE;
   const dim3 grid(nblk, batch);
   const int64_t table = (int64_t)batch * nblk * 256;
-  const bool fused_scan = nblk <= SCAN_IN_SCATTER_MAX_TILES;
-  int launches = 1;
   rank_hist_first<<<grid, SORT_THREADS, 0, st>>>(agg, req, latch, nblk, table, hist);
   for (int pass = 0; pass < 4; ++pass) {
     const int in = (pass + 1) & 1, out = in ^ 1;           // pass 0 reads the scores, writes buffer 0
@@ -288,17 +254,11 @@ int launch_sort(const float* agg, const AslReq* req, const asl_stat* latch, int 
     int32_t* row = pass == 3 ? rank_row : nullptr;
     int32_t* cur = hist + pass * table;
     int32_t* nxt = pass == 3 ? nullptr : hist + (pass + 1) * table;
-    if (!fused_scan) { launch_after(rank_scan, dim3(batch), dim3(1024), st, cur, req, latch, nblk); ++launches; }
-    ++launches;
-    if (pass == 0) {
-      if (fused_scan) launch_after(rank_scatter<true, true>, grid, dim3(SORT_THREADS), st, agg, nullptr, nullptr, keys[out], idx[out], row, cur, nxt, req, latch, shift, nblk);
-      else launch_after(rank_scatter<true, false>, grid, dim3(SORT_THREADS), st, agg, nullptr, nullptr, keys[out], idx[out], row, cur, nxt, req, latch, shift, nblk);
-    } else {
-      if (fused_scan) launch_after(rank_scatter<false, true>, grid, dim3(SORT_THREADS), st, nullptr, keys[in], idx[in], keys[out], idx[out], row, cur, nxt, req, latch, shift, nblk);
-      else launch_after(rank_scatter<false, false>, grid, dim3(SORT_THREADS), st, nullptr, keys[in], idx[in], keys[out], idx[out], row, cur, nxt, req, latch, shift, nblk);
-    }
+    launch_after(rank_scan, dim3(batch), dim3(1024), st, cur, req, latch, nblk);
+    if (pass == 0) launch_after(rank_scatter<true>, grid, dim3(SORT_THREADS), st, agg, nullptr, nullptr, keys[out], idx[out], row, cur, nxt, req, latch, shift, nblk);
+    else launch_after(rank_scatter<false>, grid, dim3(SORT_THREADS), st, nullptr, keys[in], idx[in], keys[out], idx[out], row, cur, nxt, req, latch, shift, nblk);
   }
-  return launches;
+  return 9;
 }
 
 
@@ -346,6 +306,31 @@ __device__ void stat_finalize_one(unsigned long long num, unsigned long long m, 
 __global__ void rank_stat_skip(const AslReq* __restrict__ req, asl_stat* __restrict__ stat, int batch, int layer_idx, int n_rows, int latch) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < batch) stat_finalize_one(0, 0, req, stat, b, layer_idx, n_rows, 0, 0.0, latch);
+}
+
+// Thread 0 adds its block's share of request b; the block that finishes last sees every block's and closes the statistic.
+__device__ void stat_close(const StatArgs& a, int b, unsigned long long num, int m, int evaluate) {
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    if (m) {
+      atomicAdd(&a.acc[2 * b], num);
+      atomicAdd(&a.acc[2 * b + 1], (unsigned long long)m);
+    }
+    __threadfence();
+    const unsigned long long blocks = (unsigned long long)gridDim.x * gridDim.y;
+    last = atomicAdd(&a.acc[2 * a.batch], 1ull) + 1 == blocks;
+  }
+  __syncthreads();
+  if (last) {
+    __threadfence();
+    for (int bb = threadIdx.x; bb < a.batch; bb += blockDim.x) {
+      const unsigned long long sum = __ldcg(a.acc + 2 * bb), size = __ldcg(a.acc + 2 * bb + 1);
+      a.acc[2 * bb] = 0;                                 // for the next layer
+      a.acc[2 * bb + 1] = 0;
+      stat_finalize_one(sum, size, a.req, a.stat, bb, a.layer_idx, a.n_rows, evaluate, a.tau, a.latch);
+    }
+    if (threadIdx.x == 0) a.acc[2 * a.batch] = 0;
+  }
 }
 
 constexpr int STAT_TOKENS = 4;   // tokens per thread: few, fat blocks (one wave on the SMs a persistent scorer leaves free)
@@ -408,322 +393,415 @@ __global__ void __launch_bounds__(256) rank_stat_accumulate(StatArgs a) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (lane == 0) { s_num[wid] = num; s_m[wid] = m; }
   __syncthreads();
-  __shared__ bool last;
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0)
     for (int w2 = 1; w2 < 8; ++w2) { num += s_num[w2]; m += s_m[w2]; }
-    if (m) {
-      atomicAdd(&a.acc[2 * b], num);
-      atomicAdd(&a.acc[2 * b + 1], (unsigned long long)m);
-    }
-    // the block that finishes last sees every block's sums and closes the statistic
-    __threadfence();
-    const unsigned long long blocks = (unsigned long long)gridDim.x * gridDim.y;
-    last = atomicAdd(&a.acc[2 * a.batch], 1ull) + 1 == blocks;
-  }
-  __syncthreads();
-  if (last) {
-    __threadfence();
-    for (int bb = threadIdx.x; bb < a.batch; bb += blockDim.x) {
-      const unsigned long long sum = __ldcg(a.acc + 2 * bb), size = __ldcg(a.acc + 2 * bb + 1);
-      a.acc[2 * bb] = 0;                                 // for the next layer
-      a.acc[2 * bb + 1] = 0;
-      stat_finalize_one(sum, size, a.req, a.stat, bb, a.layer_idx, a.n_rows, 1, a.tau, a.latch);
-    }
-    if (threadIdx.x == 0) a.acc[2 * a.batch] = 0;
-  }
+  stat_close(a, b, num, m, 1);
 }
 
-// ---------------------------------------------------------------------------
-// Segments of up to MERGE_MAX_T tokens: tiles of R * 1024 scores are sorted on their own, one 1024-thread block each, and
-// a token's rank is then its place in its own tile plus, for every other tile of the request, the number of scores
-// there that go before it.  Two launches (one where a single tile holds the segment) against the five of the radix
-// passes over the whole row; nothing but the sorted tiles goes through global memory.
-// ---------------------------------------------------------------------------
-constexpr int TILE_THREADS = 1024;
-constexpr int TILE_WARPS = TILE_THREADS / 32;
-
-__host__ __device__ constexpr size_t tile_smem_bytes(int rounds) {     // keys, token numbers; per warp: digit counts, lanes per digit
-  return (size_t)rounds * TILE_THREADS * (sizeof(uint32_t) + sizeof(uint16_t)) + (size_t)TILE_WARPS * 256 * (sizeof(uint16_t) + sizeof(uint32_t));
-}
-
-struct TileArgs {
+struct RowArgs {
   const float* agg;
   int32_t* rank_row;
-  const AslReq* req;         // null: one segment of T tokens, no statistic
+  const AslReq* req;           // null: one segment of T tokens, no statistic
   int32_t T;
-  uint32_t* keys;            // several tiles: each one's sorted keys and their tokens, a request's at its u_off
-  int32_t* idx;
-  StatArgs stat;             // ring, records, rows; n_rows 0: only the bookkeeping fields of the records change
+  unsigned long long* pairs;   // the tiles' pairs, bucket after bucket; a request's at its u_off
+  unsigned long long* list;    // room of the same size for buckets that do not fit a block
+  unsigned long long* splitters;   // [request][S], the first of them unused
+  uint16_t* table;             // [request][tile][split_pitch] first place of every bucket in the tile
+  int32_t max_tiles;
+  StatArgs stat;               // ring, records, rows
   int32_t evaluate;
 };
 
-__device__ __forceinline__ AslReq tile_request(const TileArgs& a, int b) {
+__device__ __forceinline__ AslReq row_request(const RowArgs& a, int b) {
   AslReq rq{};
   rq.T = a.T;
   if (a.req) rq = a.req[b];
   return rq;
 }
+__device__ __forceinline__ bool row_is_final(const RowArgs& a, int b) { return a.req && a.stat.latch && a.stat.stat[b].selected; }
 
-// One tile: four stable passes of 8-bit digits in shared memory.  A pass is bound by what its R rounds per warp issue
-// to shared memory, and by its five block barriers; the place among the warp's earlier keys is kept from the count to
-// the scatter.
-// SINGLE: the tile is the whole segment; the block writes the rank row and takes the statistic.
-template <int R, bool SINGLE>
-__global__ void __launch_bounds__(TILE_THREADS, 1) rank_tile_kernel(TileArgs a) {
-  constexpr int N = R * TILE_THREADS;
-  extern __shared__ __align__(16) uint8_t tile_raw[];
-  uint32_t (*lanes)[256] = reinterpret_cast<uint32_t (*)[256]>(tile_raw);
-  uint32_t (*cnt2)[128] = reinterpret_cast<uint32_t (*)[128]>(lanes + TILE_WARPS);       // two digits' counts per word
-  uint32_t* s_key = reinterpret_cast<uint32_t*>(cnt2 + TILE_WARPS);
-  uint16_t* s_id = reinterpret_cast<uint16_t*>(s_key + N);
-  __shared__ uint32_t part_sum[8][128];
-  __shared__ int warp_tot[4];
-  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  uint16_t* const cnt = reinterpret_cast<uint16_t*>(cnt2[wid]);
-  if (a.req && a.stat.latch && a.stat.stat[b].selected) return;      // the request's selection is final
-  const AslReq rq = tile_request(a, b);
-  const int start = blockIdx.x * N;
-  if (start >= rq.T) return;
-  const int n = min(N, rq.T - start);
-  const uint32_t lt = (1u << lane) - 1u;
-  const int w0 = wid * R * 32;                                        // a warp owns consecutive keys
-  uint32_t key[R];
-  uint32_t id[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int i = w0 + r * 32 + lane;
-    id[r] = i;
-    key[r] = i < n ? desc_key(__ldcg(a.agg + rq.t_off + start + i)) : 0xffffffffu;   // padding sorts last (and stays behind equal keys)
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) lanes[wid][i * 32 + lane] = 0;
-#pragma unroll 1
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = 8 * pass;
-    uint32_t before[R];                                               // keys of the warp with the same digit and a lower place
-#pragma unroll
-    for (int i = 0; i < 4; ++i) cnt2[wid][i * 32 + lane] = 0;
-    __syncwarp();
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const uint32_t d = (key[r] >> shift) & 255u;
-      const uint32_t peers = same_digit(lanes[wid], d, true, lane);
-      const uint32_t c = cnt[d];
-      __syncwarp();
-      if ((peers & lt) == 0) cnt[d] = (uint16_t)(c + __popc(peers));
-      before[r] = c + __popc(peers & lt);
-      __syncwarp();
-    }
-    __syncthreads();
-    {  // the counts become positions, in (digit, warp) order: thread (part, word) has two digits of four warps
-      const int w = tid & 127, part = tid >> 7;
-      uint32_t v[4], total = 0, mine = 0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { v[i] = cnt2[part * 4 + i][w]; mine += v[i]; }
-      part_sum[part][w] = mine;
-      __syncthreads();
-      mine = 0;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) { const uint32_t s = part_sum[q][w]; total += s; mine += q < part ? s : 0u; }
-      const int both = (int)((total & 0xffffu) + (total >> 16));
-      int incl = both;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += u;
-      }
-      if (part == 0 && lane == 31) warp_tot[wid] = incl;
-      __syncthreads();
-      uint32_t off = (uint32_t)(incl - both);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) off += q < (w >> 5) ? (uint32_t)warp_tot[q] : 0u;
-      uint32_t run = mine + (off | (off + (total & 0xffffu)) << 16);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { cnt2[part * 4 + i][w] = run; run += v[i]; }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const uint32_t pos = cnt[(key[r] >> shift) & 255u] + before[r];
-      if (SINGLE && pass == 3) { s_key[id[r]] = pos; continue; }      // the rank row, in token order
-      s_key[pos] = key[r];
-      s_id[pos] = (uint16_t)id[r];
-    }
-    __syncthreads();
-    if (pass == 3) break;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      key[r] = s_key[w0 + r * 32 + lane];
-      id[r] = s_id[w0 + r * 32 + lane];
-    }
-  }
-  if (!SINGLE) {                                                      // up to a multiple of four: copied on 16 bytes
-    const int64_t out = (int64_t)rq.u_off + start;
-    for (int i = tid; i < (n + 3) / 4 * 4; i += TILE_THREADS) {
-      a.keys[out + i] = s_key[i];
-      a.idx[out + i] = start + s_id[i];
-    }
-    return;
-  }
-  // ---- the row, and the statistic over it and the earlier rows
-  __shared__ unsigned long long s_num[TILE_WARPS];
-  __shared__ int s_m[TILE_WARPS];
+// ---------------------------------------------------------------------------
+// One segment of up to COUNT_MAX_T tokens: a token's rank is the number of tokens that go before it, counted outright.
+// A block takes 32 tokens, one per lane; its warps share the others, which lie in shared memory (a broadcast load per
+// four).  The statistic of the block's tokens goes with them: one launch.  T^2 compares are 2 us of the whole GPU at 4096
+// tokens; bound by the launch and three round trips.  4096 scores: 14.3 us by one block's radix sort, a chain of shared-
+// memory passes, -> 7.4 us.  Not for batches, whose compares add up, and not above: at 8192 tokens the compares alone are
+// 8 us, and eight times that beside a scorer.
+// ---------------------------------------------------------------------------
+constexpr int COUNT_MAX_T = 4096;
+constexpr int COUNT_THREADS = 1024;
+constexpr int COUNT_WARPS = COUNT_THREADS / 32;
+
+__global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
+  __shared__ __align__(16) uint32_t keys[COUNT_MAX_T];
+  __shared__ int part[COUNT_WARPS][32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const bool open = !row_is_final(a, 0);
+  const AslReq rq = row_request(a, 0);
+  const int T = rq.T, padded = (T + 127) & ~127;                     // padding goes before nothing
   unsigned long long num = 0;
   int m = 0;
-#pragma unroll 1
-  for (int i = tid; i < rq.T; i += TILE_THREADS) {
-    const int mine = (int)s_key[i];
-    a.rank_row[rq.t_off + i] = mine;
-    if (a.evaluate) {
-      long long s1 = mine, s2 = (long long)mine * mine;
-      int mn = mine;
+  if (open) {
+    const int i0 = blockIdx.x * 32, i = i0 + lane;
+    // the earlier rows' ranks of the block's tokens, on their way while it counts
+    long long s1 = 0, s2 = 0;
+    int mn = 0x7fffffff;
+    if (wid == 0 && a.evaluate) {
       for (int r0 = 0; r0 < a.stat.n_rows - 1; r0 += 8) {
         int v[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           const int slot = (a.stat.first_layer + r0 + q) % a.stat.l_obs;
-          v[q] = r0 + q < a.stat.n_rows - 1 ? __ldcg(a.stat.ring + (int64_t)slot * a.stat.sum_T + rq.t_off + i) : -1;
+          v[q] = i < T && r0 + q < a.stat.n_rows - 1 ? __ldcg(a.stat.ring + (int64_t)slot * a.stat.sum_T + rq.t_off + i) : -1;
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
           if (v[q] >= 0) { mn = min(mn, v[q]); s1 += v[q]; s2 += (long long)v[q] * v[q]; }
       }
-      if (mn < rq.k) {
-        m += 1;
-        num += (unsigned long long)((long long)a.stat.n_rows * s2 - s1 * s1);
+    }
+#pragma unroll
+    for (int q = 0; q < COUNT_MAX_T / COUNT_THREADS; ++q) {
+      const int j = tid + q * COUNT_THREADS;
+      if (j < padded) keys[j] = j < T ? desc_key(__ldcg(a.agg + rq.t_off + j)) : 0xffffffffu;
+    }
+    __syncthreads();
+    const uint32_t key = keys[min(i, padded - 1)];
+    const int per = padded / COUNT_WARPS, j0 = wid * per, j1 = j0 + per;        // (a multiple of four)
+    int before = 0;
+    for (int j = j0; j < min(j1, i0); j += 4) {                       // earlier tokens go first among equals
+      const uint4 k = *reinterpret_cast<const uint4*>(keys + j);
+      before += (k.x <= key) + (k.y <= key) + (k.z <= key) + (k.w <= key);
+    }
+    for (int j = max(j0, i0); j < min(j1, i0 + 32); ++j) before += keys[j] < key || (keys[j] == key && j < i);
+    for (int j = max(j0, i0 + 32); j < j1; j += 4) {
+      const uint4 k = *reinterpret_cast<const uint4*>(keys + j);
+      before += (k.x < key) + (k.y < key) + (k.z < key) + (k.w < key);
+    }
+    part[wid][lane] = before;
+    __syncthreads();
+    if (wid == 0) {
+      int rank = 0;
+#pragma unroll
+      for (int w = 0; w < COUNT_WARPS; ++w) rank += part[w][lane];
+      if (i < T) {
+        a.rank_row[rq.t_off + i] = rank;
+        mn = min(mn, rank);
+        s1 += rank;
+        s2 += (long long)rank * rank;
+        if (a.evaluate && mn < rq.k) {
+          m = 1;
+          num = (unsigned long long)((long long)a.stat.n_rows * s2 - s1 * s1);
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        num += __shfl_down_sync(0xffffffffu, num, o);
+        m += __shfl_down_sync(0xffffffffu, m, o);
       }
     }
   }
-  if (!a.req) return;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    num += __shfl_down_sync(0xffffffffu, num, o);
-    m += __shfl_down_sync(0xffffffffu, m, o);
-  }
-  if (lane == 0) { s_num[wid] = num; s_m[wid] = m; }
-  __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < TILE_WARPS; ++w) { num += s_num[w]; m += s_m[w]; }
-    stat_finalize_one(num, (unsigned long long)m, a.req, a.stat.stat, b, a.stat.layer_idx, a.stat.n_rows, a.evaluate, a.stat.tau, a.stat.latch);
-  }
+  if (a.req) stat_close(a.stat, 0, num, m, a.evaluate);
 }
 
-template <bool LE>
-__device__ __forceinline__ bool goes_before(uint32_t a, uint32_t key) { return LE ? a <= key : a < key; }
+// ---------------------------------------------------------------------------
+// Segments of up to SPLIT_MAX_T tokens: (key, token) pairs are all different, so S pairs sampled across the segment, once
+// sorted, cut it into S buckets of about the same size whatever the scores are, long runs of equal ones included.
+//
+//   rank_split_kernel   a block takes a tile of 4 S scores: sorts the sample (all blocks the same one), finds each score's
+//                       bucket in the sorted sample, writes the tile's pairs bucket after bucket, and where each begins
+//   rank_place_kernel   a block takes four buckets: the pairs that go before them are the sum of their first places over
+//                       the tiles; its own are dealt to bins (two of them a pair on average) by where they lie between
+//                       their bucket's splitters, and a pair is compared with those of its bin only
+//
+// Neither waits for another block, and the row does not depend on the order in which pairs arrive.  Bound by latency: the
+// first takes 4 to 6 us (the sample's round trip, its sort, 8 to 10 steps of search), the second 7 (three round trips).
+// 100003 tokens with the statistic: five radix passes 34.6 us -> 20.8.  32768 tokens beside a scorer that leaves 16 SMs:
+// sorted tiles of 4096 and their merge, whose searches grow with the square of the length, 35 us -> 23; eight layers
+// 471 -> 460 us.  Longer segments would need a larger sample, whose sort every block repeats.
+// ---------------------------------------------------------------------------
+constexpr int SPLIT_MAX_T = 262144;
+constexpr int SPLIT_MAX_TILES = 64;
+__host__ __device__ constexpr int split_pitch(int S) { return S + 8; }
+__host__ __device__ constexpr int split_max_T(int S) { return S == 256 ? 32768 : (S == 512 ? 131072 : SPLIT_MAX_T); }
+static_assert(split_max_T(256) <= 4 * 256 * SPLIT_MAX_TILES && split_max_T(512) <= 4 * 512 * SPLIT_MAX_TILES && SPLIT_MAX_T <= 4 * 1024 * SPLIT_MAX_TILES, "tiles of a segment");
 
-// A sorted run in shared memory: four words of padding behind every 32, so that the few places which the lanes of a
-// warp (32 ascending keys) look at in one step of their searches lie in different banks at every stride.
-__host__ __device__ constexpr int padded(int i) { return i + i / 32 * 4; }
+__device__ __forceinline__ unsigned long long pair_of(uint32_t key, int token) { return (unsigned long long)key << 32 | (uint32_t)token; }
 
-// For each of the E keys: keys of a run of N (a power of two) that go before it.  `at` walks the padded places as byte
-// addresses, so that a step is a load, a compare and an add (65536 scores: 37.9 us with indices -> 31.7 us); a step of
-// all E searches is in flight at once.
-template <int N, int E, bool LE>
-__device__ __forceinline__ void add_counts(uint32_t run, const uint32_t (&key)[E], int (&rank)[E]) {
-  uint32_t at[E], x[E];
-#pragma unroll
-  for (int i = 0; i < E; ++i) at[i] = run;
-#pragma unroll
-  for (int h = N / 2; h; h >>= 1) {                    // at is a place that 2h divides: the one h - 1 further is padded(h - 1) further
-#pragma unroll
-    for (int i = 0; i < E; ++i) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x[i]) : "r"(at[i] + padded(h - 1) * 4) : "memory");
-#pragma unroll
-    for (int i = 0; i < E; ++i)
-      if (goes_before<LE>(x[i], key[i])) at[i] += padded(h) * 4;
-  }
-#pragma unroll
-  for (int i = 0; i < E; ++i) {
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x[i]) : "r"(at[i]) : "memory");
-    const int p = (int)(at[i] - run) / 4;
-    rank[i] += p - p / 36 * 4 + (goes_before<LE>(x[i], key[i]) ? 1 : 0);
-  }
-}
-
-// Block: MERGE_CHUNK keys of one sorted tile against all other tiles of the request, staged in shared memory one ahead.
-// Bound by the searches' loads from shared memory.
-constexpr int MERGE_THREADS = 256;
-constexpr int MERGE_PER = 4;                                          // keys per thread
-constexpr int MERGE_CHUNK = MERGE_THREADS * MERGE_PER;
-
-template <int R>
-__global__ void __launch_bounds__(MERGE_THREADS) rank_merge_kernel(TileArgs a) {
-  constexpr int N = R * TILE_THREADS;
-  __shared__ __align__(16) uint32_t run[2][padded(N)];
+template <int S>
+__global__ void __launch_bounds__(S) rank_split_kernel(RowArgs a) {
+  constexpr int PER = 4, TILE_N = PER * S, LEVELS = S == 256 ? 8 : (S == 512 ? 9 : 10);
+  static_assert(1 << LEVELS == S, "a thread per sampled pair");
+  extern __shared__ __align__(16) uint8_t split_raw[];
+  unsigned long long* const stage = reinterpret_cast<unsigned long long*>(split_raw);     // [TILE_N]; the sample's sort uses it first
+  unsigned long long* const tree = stage + TILE_N;                                        // [S] the splitters in the order of a search, from 1 on
+  int* const count = reinterpret_cast<int*>(tree + S);                                    // [S]
+  __shared__ int warp_tot[S / 32];
   const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  pdl_release_successor();
-  if (a.req && a.stat.latch && a.stat.stat[b].selected) return;
-  const AslReq rq = tile_request(a, b);
-  const int first = blockIdx.x * MERGE_CHUNK;
-  if (first >= rq.T) return;
-  const int own = first / N, tiles = (rq.T + N - 1) / N;
-  const uint32_t* keys = a.keys + rq.u_off;
-  auto stage = [&](int tile, int buf) {
-    const int have = min(N, (rq.T - tile * N + 3) / 4 * 4);           // the last tile ends early, on a multiple of four
-    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(run[buf]);
-    for (int i = tid * 4; i < N; i += MERGE_THREADS * 4) {
-      if (i < have) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + padded(i) * 4), "l"(keys + (int64_t)tile * N + i) : "memory");
-      else *reinterpret_cast<uint4*>(&run[buf][padded(i)]) = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+  if (row_is_final(a, b)) return;
+  const AslReq rq = row_request(a, b);
+  const int start = blockIdx.x * TILE_N;
+  if (start >= rq.T) return;
+  const int n = min(TILE_N, rq.T - start);
+  // a sampled token lies somewhere in its S-th of the segment, so that no period of the scores can meet the sample's
+  const int s_lo = (int)((long long)tid * rq.T / S), s_hi = (int)((long long)(tid + 1) * rq.T / S);
+  const int s_at = min(rq.T - 1, s_lo + (int)(((uint32_t)tid * 2654435761u >> 8) % (uint32_t)max(1, s_hi - s_lo)));
+  const float s_score = __ldcg(a.agg + rq.t_off + s_at);
+  float score[PER];
+#pragma unroll
+  for (int r = 0; r < PER; ++r) score[r] = r * S + tid < n ? __ldcg(a.agg + rq.t_off + start + r * S + tid) : 0.f;
+  count[tid] = 0;
+  // bitonic sort, a pair per thread: exchanges within a warp by shuffles, across warps through two buffers in turn
+  unsigned long long v = pair_of(desc_key(s_score), s_at);
+  int flip = 0;
+#pragma unroll
+  for (int k = 2; k <= S; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      unsigned long long o;
+      if (j >= 32) {
+        stage[flip * S + tid] = v;
+        __syncthreads();
+        o = stage[flip * S + (tid ^ j)];
+        flip ^= 1;
+      } else {
+        o = __shfl_xor_sync(0xffffffffu, v, j);
+      }
+      v = (((tid & k) == 0) == ((tid & j) == 0)) == (o < v) ? o : v;
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  // the tiles after the own one first: blocks of different tiles do not ask for the same lines at the same time
-  int tile = own + 1 < tiles ? own + 1 : 0;
-  if (tile != own) stage(tile, 0);
-  const int mine = first + wid * 32 * MERGE_PER + lane;
-  uint32_t key[MERGE_PER];
-  int token[MERGE_PER], rank[MERGE_PER];
-#pragma unroll
-  for (int i = 0; i < MERGE_PER; ++i) {
-    const int j = mine + i * 32;
-    key[i] = j < rq.T ? __ldcg(keys + j) : 0xffffffffu;
-    token[i] = j < rq.T ? __ldcg(a.idx + rq.u_off + j) : -1;
-    rank[i] = j - own * N;
   }
-  for (int buf = 0; tile != own; buf ^= 1) {
-    const int next = tile + 1 < tiles ? tile + 1 : 0;
-    if (next != own) stage(next, buf ^ 1);
-    if (next != own) asm volatile("cp.async.wait_group 1;" ::: "memory");
-    else asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();
-    const uint32_t at = (uint32_t)__cvta_generic_to_shared(run[buf]);
-    if (tile < own) add_counts<N, MERGE_PER, true>(at, key, rank);     // earlier tokens go first among equals
-    else add_counts<N, MERGE_PER, false>(at, key, rank);
-    __syncthreads();
-    tile = next;
+  __syncthreads();
+  stage[tid] = v;
+  __syncthreads();
+  if (tid) {                                           // node `tid` of the search tree: the middle of what its path leaves
+    const int level = 31 - __clz(tid);
+    tree[tid] = stage[(2 * (tid - (1 << level)) + 1) * (S >> (level + 1))];
   }
+  __syncthreads();
+  unsigned long long pair[PER];
+  int node[PER];
 #pragma unroll
-  for (int i = 0; i < MERGE_PER; ++i)
-    if (token[i] >= 0) a.rank_row[rq.t_off + token[i]] = rank[i];
+  for (int r = 0; r < PER; ++r) { pair[r] = pair_of(desc_key(score[r]), start + r * S + tid); node[r] = 1; }
+#pragma unroll
+  for (int l = 0; l < LEVELS; ++l)
+#pragma unroll
+    for (int r = 0; r < PER; ++r) node[r] = 2 * node[r] + (pair[r] >= tree[node[r]] ? 1 : 0);
+  int place[PER];
+#pragma unroll
+  for (int r = 0; r < PER; ++r) place[r] = r * S + tid < n ? atomicAdd(&count[node[r] - S], 1) : 0;
+  __syncthreads();
+  int mine = count[tid], incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  if (lane == 31) warp_tot[wid] = incl;
+  __syncthreads();
+  int before = incl - mine;
+  {
+    int t = lane < S / 32 && lane < wid ? warp_tot[lane] : 0;
+    before += __reduce_add_sync(0xffffffffu, t);
+  }
+  count[tid] = before;
+  if (blockIdx.x == 0) a.splitters[b * S + tid] = v;
+  uint16_t* const row = a.table + ((int64_t)b * a.max_tiles + blockIdx.x) * split_pitch(S);
+  row[tid] = (uint16_t)before;
+  if (tid == 0) row[S] = (uint16_t)n;
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < PER; ++r)
+    if (r * S + tid < n) stage[count[node[r] - S] + place[r]] = pair[r];
+  __syncthreads();
+  unsigned long long* const out = a.pairs + rq.u_off + start;
+#pragma unroll
+  for (int r = 0; r < PER; ++r)
+    if (r * S + tid < n) out[r * S + tid] = stage[r * S + tid];
 }
 
-// A tile that holds the segment stands alone up to 4096 scores (16 us there, in two launches over tiles of 2048 17 us; the
-// radix passes 34 us).  Above, tiles of 2048 keep more SMs busy with the sorts (8192 scores: 19.5 us, with tiles of 4096
-// 21.5 us), and from 16384 on tiles of 4096 mean half the searches (32768: 25.6 us, radix passes 35.8 us; 65536: 31.7 us
-// and 36 us).  The searches grow with the square of the length, and beside a scorer that leaves few SMs their work counts:
-// this way is the faster one up to that line (a pass of eight 32K layers 630 -> 480 us, three of 50K 283 -> 259 us), and
-// not above (four of 128K 832 -> 923 us).
-constexpr int ALONE_MAX_T = 4096;
-constexpr int SMALL_TILES_MAX_T = 16384;
-constexpr int MERGE_MAX_T = 65536;
+constexpr int PLACE_GROUP = 4;                         // buckets of a block
+constexpr int PLACE_THREADS = 512;
+template <int S>
+struct PlaceSmem {
+  static constexpr int PER = S == 256 ? 6 : 12;        // pairs of a thread that stay on the SM: six times the average
+  static constexpr int HELD = PER * PLACE_THREADS, BINS = 4 * PLACE_THREADS;
+  unsigned long long held[HELD];
+  unsigned long long split[PLACE_GROUP], least[PLACE_GROUP], most[PLACE_GROUP];
+  float scale[PLACE_GROUP];
+  int bin[BINS + 4];
+  int first_of[SPLIT_MAX_TILES + 1], from[SPLIT_MAX_TILES];       // the tiles' parts in the buckets, and in their tiles
+  int warp_tot[PLACE_THREADS / 32], base;
+};
 
-struct TileKernel { void (*fn)(TileArgs); int rounds; };
-const TileKernel ALONE_KERNELS[3] = {{rank_tile_kernel<1, true>, 1}, {rank_tile_kernel<2, true>, 2}, {rank_tile_kernel<4, true>, 4}};
-const TileKernel SORT_KERNELS[2] = {{rank_tile_kernel<2, false>, 2}, {rank_tile_kernel<4, false>, 4}};
-
-// the rank rows and, where one tile per request does, the statistic; launches
-int launch_tiles(const TileArgs& a, int max_T, int batch, cudaStream_t st) {
-  if (max_T <= ALONE_MAX_T) {
-    const TileKernel& k = ALONE_KERNELS[max_T <= 1024 ? 0 : max_T <= 2048 ? 1 : 2];
-    k.fn<<<dim3(1, batch), TILE_THREADS, tile_smem_bytes(k.rounds), st>>>(a);
-    return 1;
+template <int S>
+__global__ void __launch_bounds__(PLACE_THREADS, S == 256 ? 3 : 2) rank_place_kernel(RowArgs a) {
+  using M = PlaceSmem<S>;
+  constexpr int TILE_N = 4 * S, THREADS = PLACE_THREADS, PER = M::PER, HELD = M::HELD, BINS = M::BINS, OWN = BINS / PLACE_GROUP;
+  extern __shared__ __align__(16) uint8_t place_raw[];
+  M& sm = *reinterpret_cast<M*>(place_raw);
+  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, b0 = blockIdx.x * PLACE_GROUP;
+  pdl_release_successor();
+  if (row_is_final(a, b)) return;
+  const AslReq rq = row_request(a, b);
+  const int tiles = (rq.T + TILE_N - 1) / TILE_N;
+  *reinterpret_cast<int4*>(sm.bin + 4 * tid) = make_int4(0, 0, 0, 0);
+  if (wid == 0) {
+    int lo[2] = {0, 0}, n[2] = {0, 0};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int t = 2 * lane + q;
+      if (t < tiles) {
+        const uint16_t* row = a.table + ((int64_t)b * a.max_tiles + t) * split_pitch(S) + b0;
+        lo[q] = __ldcg(row);
+        n[q] = __ldcg(row + PLACE_GROUP) - lo[q];
+      }
+    }
+    int incl = n[0] + n[1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    sm.first_of[2 * lane] = incl - n[1] - n[0];
+    sm.first_of[2 * lane + 1] = incl - n[1];
+    sm.from[2 * lane] = 2 * lane * TILE_N + lo[0];
+    sm.from[2 * lane + 1] = (2 * lane + 1) * TILE_N + lo[1];
+    if (lane == 31) sm.first_of[SPLIT_MAX_TILES] = incl;
+    const int base = __reduce_add_sync(0xffffffffu, lo[0] + lo[1]);
+    if (lane == 0) sm.base = base;
+  } else if (tid >= 32 && tid < 32 + PLACE_GROUP) {
+    // a bucket's bins lie between its two splitters; the first and the last bucket have one only, and take four times
+    // their neighbour's width
+    const int g = tid - 32, q = b0 + g;
+    const unsigned long long* split = a.splitters + b * S;
+    const unsigned long long x0 = __ldcg(split + max(q, 1)), x1 = __ldcg(split + min(q + 1, S - 1));
+    const unsigned long long y = q == 0 ? __ldcg(split + 2) - x0 : (q == S - 1 ? x0 - __ldcg(split + S - 2) : x1 - x0);
+    const unsigned long long width = q == 0 || q == S - 1 ? min(y, ~0ull >> 3) * 4 : y;
+    sm.split[g] = x0;
+    sm.least[g] = q == 0 ? x0 - min(x0, width) : x0;
+    sm.scale[g] = (float)OWN / __ull2float_rz(max(1ull, width));
   }
-  const TileKernel& k = SORT_KERNELS[max_T <= SMALL_TILES_MAX_T ? 0 : 1];
-  const int n = k.rounds * TILE_THREADS;
-  k.fn<<<dim3((max_T + n - 1) / n, batch), TILE_THREADS, tile_smem_bytes(k.rounds), st>>>(a);
-  // the plain way: its blocks, started early, would crowd onto the SMs that the sorts leave free (131072 scores: 89 us, not 69)
-  const dim3 grid((max_T + MERGE_CHUNK - 1) / MERGE_CHUNK, batch);
-  if (k.rounds == 2) rank_merge_kernel<2><<<grid, MERGE_THREADS, 0, st>>>(a);
-  else rank_merge_kernel<4><<<grid, MERGE_THREADS, 0, st>>>(a);
+  __syncthreads();
+  const int m = sm.first_of[SPLIT_MAX_TILES], base = sm.base;
+  if (m == 0) return;
+  const unsigned long long* const pairs = a.pairs + rq.u_off;
+  auto pair_at = [&](int e) {                          // the block's e-th pair, tile after tile
+    int t = 0;
+#pragma unroll
+    for (int h = SPLIT_MAX_TILES / 2; h; h >>= 1) t += sm.first_of[t + h] <= e ? h : 0;
+    return __ldcg(pairs + sm.from[t] + (e - sm.first_of[t]));
+  };
+  auto bucket_of = [&](unsigned long long pair) {
+    int g = 0;
+#pragma unroll
+    for (int q = 1; q < PLACE_GROUP; ++q) g += pair >= sm.split[q] ? 1 : 0;
+    return g;
+  };
+  auto bin_of = [&](unsigned long long pair) {         // no pair gets a lower one than a smaller pair
+    const int g = bucket_of(pair);
+    const unsigned long long least = sm.least[g];
+    return g * OWN + (pair > least ? min(OWN - 1, (int)(__ull2float_rz(pair - least) * sm.scale[g])) : 0);
+  };
+  auto put = [&](unsigned long long pair, int rank) { a.rank_row[rq.t_off + (int)(uint32_t)pair] = rank; };
+  const bool fits = m <= HELD;
+  unsigned long long pair[PER];
+  // a pair's place among those of its bin, in the order of arrival; then where the bins begin
+  uint32_t at[PER];                              // bin << 16 | place
+  if (fits) {
+#pragma unroll
+    for (int r = 0; r < PER; ++r)
+      if (r * THREADS < m) pair[r] = pair_at(min(r * THREADS + tid, m - 1));
+#pragma unroll
+    for (int r = 0; r < PER; ++r)
+      if (r * THREADS + tid < m) {
+        const int q = bin_of(pair[r]);
+        at[r] = (uint32_t)q << 16 | (uint32_t)atomicAdd(&sm.bin[q], 1);
+      }
+  } else {
+    // buckets that do not fit (some row in ten thousand has such, or one whose sampled scores are unlike the others): the
+    // same through global memory, the bins between the smallest and the largest pair that each bucket really has
+    __syncthreads();
+    if (tid < PLACE_GROUP) { sm.least[tid] = ~0ull; sm.most[tid] = 0ull; }
+    __syncthreads();
+    for (int e = tid; e < m; e += THREADS) {
+      const unsigned long long p = pair_at(e);
+      const int g = bucket_of(p);
+      if (p < *(volatile unsigned long long*)&sm.least[g]) atomicMin(&sm.least[g], p);
+      if (p > *(volatile unsigned long long*)&sm.most[g]) atomicMax(&sm.most[g], p);
+    }
+    __syncthreads();
+    if (tid < PLACE_GROUP) sm.scale[tid] = (float)OWN / __ull2float_rz(max(1ull, sm.most[tid] - sm.least[tid]));     // (an empty bucket's is not used)
+    __syncthreads();
+    for (int e = tid; e < m; e += THREADS) atomicAdd(&sm.bin[bin_of(pair_at(e))], 1);
+  }
+  __syncthreads();
+  {
+    const int4 c = *reinterpret_cast<int4*>(sm.bin + 4 * tid);
+    const int mine = c.x + c.y + c.z + c.w;
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) sm.warp_tot[wid] = incl;
+    __syncthreads();
+    int run = incl - mine + __reduce_add_sync(0xffffffffu, lane < wid ? sm.warp_tot[lane] : 0);
+    int4 s;
+    s.x = run; s.y = s.x + c.x; s.z = s.y + c.y; s.w = s.z + c.z;
+    *reinterpret_cast<int4*>(sm.bin + 4 * tid) = s;
+    if (tid == THREADS - 1) sm.bin[BINS] = m;
+  }
+  __syncthreads();
+  if (fits) {
+#pragma unroll
+    for (int r = 0; r < PER; ++r)
+      if (r * THREADS + tid < m) sm.held[sm.bin[at[r] >> 16] + (int)(at[r] & 0xffffu)] = pair[r];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < PER; ++r)
+      if (r * THREADS + tid < m) {
+        const int q = (int)(at[r] >> 16), begin = sm.bin[q], end = sm.bin[q + 1];
+        int rank = base + begin;
+        for (int i = begin; i < end; ++i) rank += sm.held[i] < pair[r] ? 1 : 0;
+        put(pair[r], rank);
+      }
+  } else {
+    // `bin` becomes the bins' ends as the pairs arrive
+    unsigned long long* const list = a.list + rq.u_off + base;
+    for (int e = tid; e < m; e += THREADS) {
+      const unsigned long long p = pair_at(e);
+      list[atomicAdd(&sm.bin[bin_of(p)], 1)] = p;
+    }
+    __syncthreads();
+    for (int e = tid; e < m; e += THREADS) {
+      const unsigned long long p = list[e];
+      const int q = bin_of(p), begin = q ? sm.bin[q - 1] : 0, end = sm.bin[q];
+      int rank = base + begin;
+      for (int i = begin; i < end; ++i) rank += list[i] < p ? 1 : 0;
+      put(p, rank);
+    }
+  }
+}
+
+template <int S>
+constexpr int split_smem_bytes() { return (int)(5 * S * sizeof(unsigned long long) + S * sizeof(int)); }
+
+void launch_count(const RowArgs& r, int T, cudaStream_t st) { rank_count_kernel<<<(T + 31) / 32, COUNT_THREADS, 0, st>>>(r); }
+
+template <int S>
+void launch_split_of(RowArgs r, int max_T, int batch, cudaStream_t st) {
+  r.max_tiles = (max_T + 4 * S - 1) / (4 * S);
+  r.table = reinterpret_cast<uint16_t*>(r.splitters + (size_t)batch * S);
+  rank_split_kernel<S><<<dim3(r.max_tiles, batch), S, split_smem_bytes<S>(), st>>>(r);
+  rank_place_kernel<S><<<dim3(S / PLACE_GROUP, batch), PLACE_THREADS, sizeof(PlaceSmem<S>), st>>>(r);
+}
+
+// Buckets of up to 128 pairs on average to 32K tokens, 256 above.  (A block of one bucket each, bins between its smallest and
+// its largest pair: 100003 tokens 25.8 us, and eight layers of 32K no faster than by merging; the blocks' fixed costs count.)
+int launch_split(const RowArgs& r, int max_T, int batch, cudaStream_t st) {
+  if (max_T <= split_max_T(256)) launch_split_of<256>(r, max_T, batch, st);
+  else if (max_T <= split_max_T(512)) launch_split_of<512>(r, max_T, batch, st);
+  else launch_split_of<1024>(r, max_T, batch, st);
   return 2;
 }
 
@@ -731,10 +809,9 @@ int launch_tiles(const TileArgs& a, int max_T, int batch, cudaStream_t st) {
 
 // once per device, with that device current
 asl_status asl_rank_ready() {
-  for (const TileKernel& k : ALONE_KERNELS)
-    ASL_CUDA(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem_bytes(k.rounds)));
-  for (const TileKernel& k : SORT_KERNELS)
-    ASL_CUDA(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem_bytes(k.rounds)));
+  ASL_CUDA(cudaFuncSetAttribute(rank_split_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, split_smem_bytes<1024>()));
+  ASL_CUDA(cudaFuncSetAttribute(rank_place_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlaceSmem<512>)));
+  ASL_CUDA(cudaFuncSetAttribute(rank_place_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlaceSmem<1024>)));
   return ASL_OK;
 }
 
@@ -751,16 +828,16 @@ asl_status asl_launch_rank(asl_ctx* c, const float* agg, int32_t layer_idx, int3
   const int evaluate = (layer_idx >= p.l_min && n_rows >= 2) ? 1 : 0;
   const StatArgs a{ring, c->d_req, c->d_acc, stat, c->sum_T, p.l_obs, layer_idx - n_rows + 1, n_rows, p.batch, layer_idx,
                    latch ? 1 : 0, p.tau};
-  if (c->max_T <= MERGE_MAX_T) {
-    const int launches = launch_tiles(TileArgs{agg, row, c->d_req, 0, keys[0], idx[0], a, evaluate}, c->max_T, p.batch, st);
-    c->launches += launches;
-    if (launches == 1) {                               // the statistic went with the row
-      ASL_CUDA(cudaGetLastError());
-      return ASL_OK;
-    }
-  } else {
-    c->launches += launch_sort(agg, c->d_req, latch, p.batch, c->max_T, keys, idx, hist, row, st);
+  RowArgs r{agg, row, c->d_req, 0, reinterpret_cast<unsigned long long*>(keys[0]), reinterpret_cast<unsigned long long*>(idx[0]),
+            reinterpret_cast<unsigned long long*>(hist), nullptr, 0, a, evaluate};
+  if (p.batch == 1 && c->max_T <= COUNT_MAX_T) {         // the statistic goes with the row
+    launch_count(r, c->max_T, st);
+    c->launches += 1;
+    ASL_CUDA(cudaGetLastError());
+    return ASL_OK;
   }
+  if (c->max_T <= SPLIT_MAX_T) c->launches += launch_split(r, c->max_T, p.batch, st);
+  else c->launches += launch_sort(agg, c->d_req, latch, p.batch, c->max_T, keys, idx, hist, row, st);
   if (evaluate) {
     launch_after(rank_stat_accumulate, dim3((c->max_T + 256 * STAT_TOKENS - 1) / (256 * STAT_TOKENS), p.batch), dim3(256), st, a);
   } else {
@@ -778,9 +855,9 @@ asl_status asl_launch_rank(asl_ctx* c, const float* agg, int32_t layer_idx, int3
 // they run: a serving engine that hands its whole memory pool to its own
 // allocator at start-up, a plugin called from inside another runtime's
 // execution callback, code running under a "no cudaMalloc after init" rule.
-// For them the sort's scratch (two ping-pong key arrays, two payload arrays,
-// the per-tile digit histograms and a one-entry request table) lives in this
-// file-scope device array.  Every device that loads the library carries these
+// For them the scratch (two arrays of pairs and the table of bucket starts)
+// lives in this file-scope device array; nothing in it has to start from a known
+// value: every call writes what it reads.  Every device that loads the library carries these
 // bytes until the process exits, which is why the segment length is capped.
 //
 // In host code `g_rank_static` is only a handle: the device address is asked
@@ -790,26 +867,15 @@ asl_status asl_launch_rank(asl_ctx* c, const float* agg, int32_t layer_idx, int3
 namespace {
 
 constexpr int STATIC_MAX_T = ASL_RANK_STATIC_MAX_T;
-constexpr int STATIC_NBLK = (STATIC_MAX_T + TILE - 1) / TILE;
 constexpr int STATIC_MAX_DEVICES = 64;
+static_assert(STATIC_MAX_T <= SPLIT_MAX_T, "the radix passes need a request table");
 
 struct RankStaticScratch {
-  AslReq req;                       // the one request the kernels index with blockIdx.y = 0
-  uint32_t keys[2][STATIC_MAX_T];
-  int32_t idx[2][STATIC_MAX_T];
-  int32_t hist[4 * 256 * STATIC_NBLK];
+  unsigned long long pairs[STATIC_MAX_T], list[STATIC_MAX_T];
+  unsigned long long table[1024 + SPLIT_MAX_TILES * split_pitch(1024) / 4];       // splitters, then the tiles' bucket starts
 };
 
 static __device__ __align__(256) unsigned char g_rank_static[sizeof(RankStaticScratch)];
-
-// Writes the request record.  Nothing else in the scratch has to start from a
-// known value: the sort writes every key, payload and histogram entry before it
-// reads it, so what an earlier call left behind is never seen.
-__global__ void rank_static_begin(RankStaticScratch* s, int T) {
-  AslReq r;
-  r.n = T; r.T = T; r.k = 0; r.kept = 0; r.tok_off = 0; r.t_off = 0; r.kept_off = 0; r.u_off = 0;
-  s->req = r;
-}
 
 struct RankStaticDevices {
   RankStaticScratch* ptr[STATIC_MAX_DEVICES] = {};
@@ -856,15 +922,9 @@ extern "C" asl_status asl_rank_desc_static(const float* scores, int32_t T, int32
   const asl_status ready = rank_static_setup(device, &s);
   if (ready != ASL_OK) return ready;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (T <= MERGE_MAX_T) {
-    launch_tiles(TileArgs{scores, rank_out, nullptr, T, s->keys[0], s->idx[0], StatArgs{}, 0}, T, 1, st);
-  } else {
-    const AslReq* req = &s->req;
-    rank_static_begin<<<1, 1, 0, st>>>(s, T);
-    uint32_t* const keys[2] = {s->keys[0], s->keys[1]};
-    int32_t* const idx[2] = {s->idx[0], s->idx[1]};
-    launch_sort(scores, req, nullptr, 1, T, keys, idx, s->hist, rank_out, st);
-  }
+  const RowArgs r{scores, rank_out, nullptr, T, s->pairs, s->list, s->table, nullptr, 0, StatArgs{}, 0};
+  if (T <= COUNT_MAX_T) launch_count(r, T, st);
+  else launch_split(r, T, 1, st);
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;
 }

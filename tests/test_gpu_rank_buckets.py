@@ -1,0 +1,71 @@
+"""GPU parity of rank rows where their kernels begin and end: the counted segments' last length and the first split one,
+every change of the sample's size, the last split length and the first of the radix passes.  Scores: smooth, heavy tailed,
+ties in runs, equal only, and a row that puts all but the sampled tokens into one bucket, too large for a block."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import asl_oracle as O
+from paper_2601_07667_b200 import binding as B
+from paper_2601_07667_b200 import inputs as I
+
+from asl_check import make_path
+
+pytestmark = pytest.mark.gpu
+
+
+def _sampled(T):
+    """The tokens at which the split samples a segment of T tokens."""
+    S = 256 if T <= 32768 else 512 if T <= 131072 else 1024
+    s = np.arange(S, dtype=np.int64)
+    lo, hi = s * T // S, (s + 1) * T // S
+    return np.minimum(T - 1, lo + ((s * 2654435761) % 2**32 >> 8) % np.maximum(1, hi - lo))
+
+
+def _scores(T, kind, rng):
+    if kind == "normal":
+        return rng.standard_normal(T).astype(np.float32)
+    if kind == "tail":
+        return np.exp(rng.normal(-9, 4, T)).astype(np.float32)
+    if kind == "ties":
+        return np.repeat(np.round(rng.standard_normal(T // 7 + 1) * 2) / 2, 7)[:T].astype(np.float32)
+    if kind == "equal":
+        return np.full(T, 0.25, np.float32)
+    s = rng.random(T) if kind == "one bucket" else np.full(T, 0.5)      # "one bucket, equal"
+    s[_sampled(T)] = 2.0 + rng.random(_sampled(T).size)
+    return s.astype(np.float32)
+
+
+KINDS = ("normal", "tail", "ties", "equal", "one bucket", "one bucket, equal")
+
+
+@pytest.mark.parametrize("T", [1, 31, 33, 127, 129, 4095, 4096, 4097, 5119, 32768, 32769, 131072, 131073, 262144])
+def test_rank_row_at_the_edges_of_its_kernels(T):
+    rng = np.random.default_rng(T)
+    for kind in KINDS:
+        s = _scores(T, kind, rng)
+        out = torch.full((T,), -1, dtype=torch.int32, device="cuda")
+        B.asl_rank_desc_static(torch.from_numpy(s).cuda(), T, out)
+        assert (out.cpu().numpy() == O.rank_desc(s.astype(np.float64))).all(), kind
+
+
+@pytest.mark.parametrize("lengths", [(33,), (4096,), (4097,), (70001, 40000, 3), (131073, 200), (262144,), (262145, 5000)])
+def test_row_and_statistic_of_a_plan(lengths):
+    w, rows, ranks = 32, 4, []
+    wl = I.workload("C1", seqlens=tuple(T + w for T in lengths), budgets=tuple(w + T // 9 for T in lengths), l_min=1, l_obs=rows)
+    path = make_path(wl)
+    rng = np.random.default_rng(sum(lengths))
+    for layer in range(rows + 1):
+        per = [_scores(T, KINDS[layer % 6], rng) for T in lengths]
+        path.scores_agg.copy_(torch.from_numpy(np.concatenate(per)))
+        B.asl_rank_stat(path.ctx, path.scores_agg, layer, min(layer + 1, rows), path.rank_ring, path.stat, path.workspace, path.ws_bytes)
+        ranks.append([O.rank_desc(s.astype(np.float64)) for s in per])
+        got, at, stat = path.rank_ring[layer % rows].cpu().numpy(), 0, path.read_stat()
+        for b, T in enumerate(lengths):
+            assert (got[at:at + T] == ranks[-1][b]).all(), (layer, b)
+            at += T
+            assert stat[b]["evaluated"] == (layer >= 1) and stat[b]["layer_idx"] == layer
+            if layer >= 1:
+                num, m, _ = O.rank_statistic(np.stack([r[b] for r in ranks[-min(layer + 1, rows):]]), T // 9)
+                assert (stat[b]["num"], stat[b]["m"]) == (num, m)
+    path.close()
