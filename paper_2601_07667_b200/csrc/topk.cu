@@ -301,6 +301,8 @@ constexpr int SEG_CAP = 12288;                 // (key, index) pairs the shared-
 constexpr int SEG_SAMPLE = 2048;
 constexpr int SEG_MAX_T = 262144;              // the bitmaps cover this many scores
 constexpr int SEG_UNROLL = 8;                  // 16-byte loads in flight per lane
+constexpr int SEG_DENSE = 16, SEG_DENSE_WORDS = 8;  // bits of a word that the whole warp writes; such words of 32 at most
+constexpr int SEG_FEW = 512;                   // keys of one bin that are ranked by comparing each with all
 
 struct __align__(16) SegSmem {
   int hist[BINS];
@@ -308,8 +310,9 @@ struct __align__(16) SegSmem {
   int32_t cand_idx[SEG_CAP];
   int warp_a[SEG_WARPS];
   uint32_t lo[SEG_WARPS], hi[SEG_WARPS];
-  int found[2][2];
-  int n_cand, n_above;
+  int found[2][3];
+  int n_cand, n_above, n_few;
+  uint32_t few[SEG_FEW];
   // behind this struct, sized for the plan's longest segment: two bitmaps over the segment
 };
 __host__ __device__ inline int seg_words(int max_T) { return ((max_T + 3 + 31) / 32 + 3) & ~3; }
@@ -337,12 +340,11 @@ __device__ __forceinline__ int seg_block_prefix(SegSmem& sm, int v) {
   return incl - v + __shfl_sync(0xffffffffu, w - t, wid);
 }
 
-// The bin of the shared table (NB bins, counted from the top) that holds the `remaining`-th largest key, and how many
-// keys of that bin are still wanted; `par` alternates between consecutive calls.
-template <int NB>
-__device__ __forceinline__ void seg_pick(SegSmem& sm, int remaining, int par, int& bin, int& rem_out) {
-  constexpr int PER = NB / SEG_THREADS;
-  const int top = NB - 1 - PER * (int)threadIdx.x;
+// The bin of the shared table (counted from the top) that holds the `remaining`-th largest key, how many keys of that
+// bin are still wanted and how many it has; `par` alternates between consecutive calls.
+__device__ __forceinline__ void seg_pick(SegSmem& sm, int remaining, int par, uint32_t& bin, int& rem_out, int& in_bin) {
+  constexpr int PER = BINS / SEG_THREADS;
+  const int top = BINS - 1 - PER * (int)threadIdx.x;
   int c[PER];
   int sum = 0;
 #pragma unroll
@@ -351,35 +353,57 @@ __device__ __forceinline__ void seg_pick(SegSmem& sm, int remaining, int par, in
   if (above < remaining && remaining <= above + sum) {
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-      if (above < remaining && remaining <= above + c[j]) { sm.found[par][0] = top - j; sm.found[par][1] = remaining - above; }
+      if (above < remaining && remaining <= above + c[j]) { sm.found[par][0] = top - j; sm.found[par][1] = remaining - above; sm.found[par][2] = c[j]; }
       above += c[j];
     }
   }
   __syncthreads();
   bin = sm.found[par][0];
   rem_out = sm.found[par][1];
+  in_bin = sm.found[par][2];
 }
 
-// The `rank`-th largest of keys[0..n) in shared memory (all of them in [lo, hi]) and how many equal to it are wanted.
-__device__ __forceinline__ void seg_select(SegSmem& sm, int n, uint32_t lo, uint32_t hi, int rank, uint32_t& thr, int& need) {
+// The `rank`-th largest of keys[0..n) in shared memory (all of them in [lo, hi]), how many equal to it are wanted and how
+// many there are.  Digits from the top of the range, until the bin that counts holds few keys: after one digit of 2048 bins
+// as a rule.
+__device__ __forceinline__ void seg_select(SegSmem& sm, int n, uint32_t lo, uint32_t hi, int rank, uint32_t& thr, int& need, int& equal) {
   int shift = 32 - __clz((int)((hi - lo) | 1u));            // bits of the range still open
   uint32_t base = lo;                                        // keys in [base, base + 2^shift) are still candidates
   need = rank;
-  for (int par = 0; shift > 0; par ^= 1) {
+  for (int par = 0;; par ^= 1) {
     const int bits = shift < 11 ? shift : 11;
     for (int i = threadIdx.x; i < BINS; i += SEG_THREADS) sm.hist[i] = 0;
+    if (threadIdx.x == 0) sm.n_few = 0;
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += SEG_THREADS) {
       const uint32_t d = sm.cand_key[i] - base;
       if (shift == 32 || (d >> shift) == 0u) atomicAdd(&sm.hist[d >> (shift - bits)], 1);
     }
     __syncthreads();
-    int bin;
-    seg_pick<BINS>(sm, need, par, bin, need);
+    seg_pick(sm, need, par, lo, need, equal);
     shift -= bits;
-    base += (uint32_t)bin << shift;
+    base += lo << shift;
+    if (shift == 0) { thr = base; return; }
+    if (equal > SEG_FEW) continue;
+    for (int i = threadIdx.x; i < n; i += SEG_THREADS) {
+      const uint32_t key = sm.cand_key[i];
+      if (((key - base) >> shift) == 0u) sm.few[atomicAdd(&sm.n_few, 1)] = key;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < equal) {
+      const uint32_t key = sm.few[threadIdx.x];
+      int larger = 0, same = 0;
+      for (int i = 0; i < equal; ++i) { larger += sm.few[i] > key; same += sm.few[i] == key; }
+      if (larger < need && need <= larger + same) {          // the same by every equal key
+        sm.found[par ^ 1][0] = (int)key; sm.found[par ^ 1][1] = need - larger; sm.found[par ^ 1][2] = same;
+      }
+    }
+    __syncthreads();
+    thr = (uint32_t)sm.found[par ^ 1][0];
+    need = sm.found[par ^ 1][1];
+    equal = sm.found[par ^ 1][2];
+    return;
   }
-  thr = base;
 }
 
 __global__ void __launch_bounds__(SEG_THREADS, 1) topk_segment_kernel(TopkArgs a) {
@@ -461,12 +485,13 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) topk_segment_kernel(TopkArgs a
     __syncthreads();
     for (int i = tid; i < SEG_SAMPLE; i += SEG_THREADS) atomicAdd(&sm.hist[(sm.cand_key[i] - mn) >> shift], 1);
     __syncthreads();
-    int bin, rest;
-    if (r_lo <= SEG_SAMPLE) { seg_pick<BINS>(sm, r_lo, 0, bin, rest); L = mn + ((uint32_t)bin << shift); }
+    uint32_t bin;
+    int rest, count;
+    if (r_lo <= SEG_SAMPLE) { seg_pick(sm, r_lo, 0, bin, rest, count); L = mn + (bin << shift); }
     // an upper bound costs the pass as much as the lower one: only where the keys above L would not fit the list
     if (r_hi >= 1 && 1.2f * (float)s.T * (float)min(r_lo, SEG_SAMPLE) > (float)SEG_CAP * (float)SEG_SAMPLE) {
-      seg_pick<BINS>(sm, r_hi, 1, bin, rest);
-      const uint32_t top = mn + ((uint32_t)bin << shift) + ((1u << shift) - 1u);
+      seg_pick(sm, r_hi, 1, bin, rest, count);
+      const uint32_t top = mn + (bin << shift) + ((1u << shift) - 1u);
       H = top < mn ? 0xffffffffu : top;
     }
     __syncthreads();
@@ -582,13 +607,13 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) topk_segment_kernel(TopkArgs a
 
   // ---- the exact k-th largest key, how many keys equal to it are kept, and the two bitmaps
   uint32_t thr;
-  int need;
+  int need, equal;                                          // keys equal to it: kept, and in all
   if (listed) {
-    seg_select(sm, n, mn, mx, s.k - n_above, thr, need);
+    seg_select(sm, n, mn, mx, s.k - n_above, thr, need, equal);
     for (int i = tid; i < n; i += SEG_THREADS) {
       const uint32_t key = sm.cand_key[i];
       const int e = (whole ? i : sm.cand_idx[i]) + mis;
-      if (key > thr) atomicOr(&bm_gt[e >> 5], 1u << (e & 31));
+      if (key > thr || (key == thr && need == equal)) atomicOr(&bm_gt[e >> 5], 1u << (e & 31));
       else if (key == thr) atomicOr(&bm_eq[e >> 5], 1u << (e & 31));
     }
   } else {
@@ -620,10 +645,10 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) topk_segment_kernel(TopkArgs a
         if (run) atomicAdd(&sm.hist[run_bin], run);
       }
       __syncthreads();
-      int bin;
-      seg_pick<BINS>(sm, need, par, bin, need);
+      uint32_t bin;
+      seg_pick(sm, need, par, bin, need, equal);
       shift -= bits;
-      base += (uint32_t)bin << shift;
+      base += bin << shift;
     }
     thr = base;
     for (int v0 = wid * 32 * SEG_UNROLL; v0 < nv; v0 += SEG_WARPS * 32 * SEG_UNROLL) {
@@ -642,30 +667,50 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) topk_segment_kernel(TopkArgs a
   // ---- of the equal keys the first `need`; thread t owns a run of words
   const int wpt = (words + SEG_THREADS - 1) / SEG_THREADS;
   const int w0 = min(words, tid * wpt), w1 = min(words, w0 + wpt);
-  int eq = 0;
-  for (int i = w0; i < w1; ++i) eq += __popc(bm_eq[i]);
-  int left = need - seg_block_prefix(sm, eq);
   int kept = 0;
-  for (int i = w0; i < w1; ++i) {
-    uint32_t q = bm_eq[i];
-    const int cnt = __popc(q);
-    if (left < cnt) {                                        // keep the lowest `left` of them
-      uint32_t some = 0u;
-      for (int c = 0; c < left; ++c) { some |= q & (0u - q); q &= q - 1; }
-      q = some;
+  if (listed && need == equal) {                             // no tie to cut: they are all in the bitmap
+    for (int i = w0; i < w1; ++i) kept += __popc(bm_gt[i]);
+  } else {
+    int eq = 0;
+    for (int i = w0; i < w1; ++i) eq += __popc(bm_eq[i]);
+    int left = need - seg_block_prefix(sm, eq);
+    for (int i = w0; i < w1; ++i) {
+      uint32_t q = bm_eq[i];
+      const int cnt = __popc(q);
+      if (left < cnt) {                                      // keep the lowest `left` of them
+        uint32_t some = 0u;
+        for (int c = 0; c < left; ++c) { some |= q & (0u - q); q &= q - 1; }
+        q = some;
+      }
+      left -= cnt;
+      const uint32_t word = bm_gt[i] | q;
+      bm_gt[i] = word;
+      kept += __popc(word);
     }
-    left -= cnt;
-    const uint32_t word = bm_gt[i] | q;
-    bm_gt[i] = word;
-    kept += __popc(word);
   }
   // ---- ordered emit (Algorithm 1 (TopK and window append)): in shared memory first where the kept indices fit there (the
   // list is done with), so that the copy out is coalesced
   int32_t* const ordered = reinterpret_cast<int32_t*>(sm.cand_key);
   const bool staged = s.k <= 2 * SEG_CAP;
-  int32_t* to = (staged ? ordered : s.out) + seg_block_prefix(sm, kept);
-  for (int i = w0; i < w1; ++i)
-    for (uint32_t bits = bm_gt[i]; bits; bits &= bits - 1) *to++ = i * 32 + __ffs(bits) - 1 - mis;
+  int32_t* const to = staged ? ordered : s.out;
+  int at = seg_block_prefix(sm, kept);
+  for (int j = 0; j < wpt; ++j) {                            // a word with many bits (kept tokens come in passages): by the whole warp
+    const int i = tid * wpt + j;
+    const uint32_t word = i < words ? bm_gt[i] : 0u;
+    uint32_t dense = __ballot_sync(0xffffffffu, __popc(word) >= SEG_DENSE);
+    if (__popc(dense) > SEG_DENSE_WORDS) dense = 0u;         // (nearly all words are: each lane its own takes no longer)
+    if (!((dense >> lane) & 1u)) {
+      int32_t* p = to + at;
+      for (uint32_t bits = word; bits; bits &= bits - 1) *p++ = i * 32 + __ffs(bits) - 1 - mis;
+    }
+    for (; dense; dense &= dense - 1) {
+      const int from = __ffs(dense) - 1;
+      const uint32_t w = __shfl_sync(0xffffffffu, word, from);
+      const int p = __shfl_sync(0xffffffffu, at, from);
+      if ((w >> lane) & 1u) to[p + __popc(w & ((1u << lane) - 1u))] = (i + (from - lane) * wpt) * 32 + lane - mis;
+    }
+    at += __popc(word);
+  }
   if (staged) {
     __syncthreads();
     for (int i = tid; i < s.k; i += SEG_THREADS) s.out[i] = ordered[i];
