@@ -509,9 +509,9 @@ __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
 //
 //   rank_split_kernel   a block takes a tile of 4 S scores: sorts the sample (all blocks the same one), finds each score's
 //                       bucket in the sorted sample, writes the tile's pairs bucket after bucket, and where each begins
-//   rank_place_kernel   a block takes four buckets: the pairs that go before them are the sum of their first places over
-//                       the tiles; its own are dealt to bins (two of them a pair on average) by where they lie between
-//                       their bucket's splitters, and a pair is compared with those of its bin only
+//   rank_place_kernel   a block takes a few buckets: the pairs that go before them are the sum of their first places over
+//                       the tiles; its own are dealt to bins (two to four of them a pair on average) by where they lie
+//                       between their bucket's splitters, and a pair is compared with those of its bin only
 //
 // Neither waits for another block, and the row does not depend on the order in which pairs arrive.  Bound by latency: the
 // first takes 4 to 6 us (the sample's round trip, its sort, 8 to 10 steps of search), the second 7 (three round trips).
@@ -537,8 +537,8 @@ __global__ void __launch_bounds__(S) rank_split_kernel(RowArgs a) {
   int* const count = reinterpret_cast<int*>(tree + S);                                    // [S]
   __shared__ int warp_tot[S / 32];
   const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (row_is_final(a, b)) return;
   const AslReq rq = row_request(a, b);
+  if (row_is_final(a, b)) return;
   const int start = blockIdx.x * TILE_N;
   if (start >= rq.T) return;
   const int n = min(TILE_N, rq.T - start);
@@ -618,31 +618,37 @@ __global__ void __launch_bounds__(S) rank_split_kernel(RowArgs a) {
     if (r * S + tid < n) out[r * S + tid] = stage[r * S + tid];
 }
 
-constexpr int PLACE_GROUP = 4;                         // buckets of a block
 constexpr int PLACE_THREADS = 512;
 template <int S>
 struct PlaceSmem {
-  static constexpr int PER = S == 256 ? 6 : 12;        // pairs of a thread that stay on the SM: six times the average
+  static constexpr int PER = S == 256 ? 6 : (S == 512 ? 8 : 12);        // pairs of a thread that stay on the SM
   static constexpr int HELD = PER * PLACE_THREADS, BINS = 4 * PLACE_THREADS;
+  static constexpr int MIN_GROUP = S == 512 ? 2 : 4, MAX_GROUP = 64;  // buckets of a block
   unsigned long long held[HELD];
-  unsigned long long split[PLACE_GROUP], least[PLACE_GROUP], most[PLACE_GROUP];
-  float scale[PLACE_GROUP];
+  unsigned long long split[MAX_GROUP], least[MAX_GROUP], most[MAX_GROUP];
+  float scale[MAX_GROUP];
   int bin[BINS + 4];
   int first_of[SPLIT_MAX_TILES + 1], from[SPLIT_MAX_TILES];       // the tiles' parts in the buckets, and in their tiles
   int warp_tot[PLACE_THREADS / 32], base;
 };
 
 template <int S>
-__global__ void __launch_bounds__(PLACE_THREADS, S == 256 ? 3 : 2) rank_place_kernel(RowArgs a) {
+__global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_kernel(RowArgs a) {
   using M = PlaceSmem<S>;
-  constexpr int TILE_N = 4 * S, THREADS = PLACE_THREADS, PER = M::PER, HELD = M::HELD, BINS = M::BINS, OWN = BINS / PLACE_GROUP;
+  constexpr int TILE_N = 4 * S, THREADS = PLACE_THREADS, PER = M::PER, HELD = M::HELD, BINS = M::BINS;
   extern __shared__ __align__(16) uint8_t place_raw[];
   M& sm = *reinterpret_cast<M*>(place_raw);
-  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, b0 = blockIdx.x * PLACE_GROUP;
+  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   pdl_release_successor();
-  if (row_is_final(a, b)) return;
   const AslReq rq = row_request(a, b);
+  if (row_is_final(a, b)) return;
   const int tiles = (rq.T + TILE_N - 1) / TILE_N;
+  // buckets of a block: as many (a power of two) as give a block a sixth of the pairs that it can hold, so that nearly every
+  // block has room for its own (eight ragged requests, blocks of four buckets whatever their lengths: 39 us, not 31)
+  int group = M::MIN_GROUP;
+  while (group < M::MAX_GROUP && (long long)rq.T * group * 2 <= (long long)S * (HELD / 6)) group *= 2;
+  const int b0 = blockIdx.x * group, own = BINS / group;
+  if (b0 >= S) return;
   *reinterpret_cast<int4*>(sm.bin + 4 * tid) = make_int4(0, 0, 0, 0);
   if (wid == 0) {
     int lo[2] = {0, 0}, n[2] = {0, 0};
@@ -652,7 +658,7 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 256 ? 3 : 2) rank_place_ke
       if (t < tiles) {
         const uint16_t* row = a.table + ((int64_t)b * a.max_tiles + t) * split_pitch(S) + b0;
         lo[q] = __ldcg(row);
-        n[q] = __ldcg(row + PLACE_GROUP) - lo[q];
+        n[q] = __ldcg(row + group) - lo[q];
       }
     }
     int incl = n[0] + n[1];
@@ -668,17 +674,13 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 256 ? 3 : 2) rank_place_ke
     if (lane == 31) sm.first_of[SPLIT_MAX_TILES] = incl;
     const int base = __reduce_add_sync(0xffffffffu, lo[0] + lo[1]);
     if (lane == 0) sm.base = base;
-  } else if (tid >= 32 && tid < 32 + PLACE_GROUP) {
-    // a bucket's bins lie between its two splitters; the first and the last bucket have one only, and take four times
-    // their neighbour's width
+  } else if (tid < 32 + group) {
+    // a bucket's bins lie between its two splitters; the first and the last bucket have one only (below)
     const int g = tid - 32, q = b0 + g;
     const unsigned long long* split = a.splitters + b * S;
     const unsigned long long x0 = __ldcg(split + max(q, 1)), x1 = __ldcg(split + min(q + 1, S - 1));
-    const unsigned long long y = q == 0 ? __ldcg(split + 2) - x0 : (q == S - 1 ? x0 - __ldcg(split + S - 2) : x1 - x0);
-    const unsigned long long width = q == 0 || q == S - 1 ? min(y, ~0ull >> 3) * 4 : y;
-    sm.split[g] = x0;
-    sm.least[g] = q == 0 ? x0 - min(x0, width) : x0;
-    sm.scale[g] = (float)OWN / __ull2float_rz(max(1ull, width));
+    sm.split[g] = sm.least[g] = x0;
+    sm.scale[g] = (float)own / __ull2float_rz(max(1ull, x1 - x0));
   }
   __syncthreads();
   const int m = sm.first_of[SPLIT_MAX_TILES], base = sm.base;
@@ -692,14 +694,13 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 256 ? 3 : 2) rank_place_ke
   };
   auto bucket_of = [&](unsigned long long pair) {
     int g = 0;
-#pragma unroll
-    for (int q = 1; q < PLACE_GROUP; ++q) g += pair >= sm.split[q] ? 1 : 0;
+    for (int h = group / 2; h; h >>= 1) g += pair >= sm.split[g + h] ? h : 0;
     return g;
   };
   auto bin_of = [&](unsigned long long pair) {         // no pair gets a lower one than a smaller pair
     const int g = bucket_of(pair);
     const unsigned long long least = sm.least[g];
-    return g * OWN + (pair > least ? min(OWN - 1, (int)(__ull2float_rz(pair - least) * sm.scale[g])) : 0);
+    return g * own + (pair > least ? min(own - 1, (int)(__ull2float_rz(pair - least) * sm.scale[g])) : 0);
   };
   auto put = [&](unsigned long long pair, int rank) { a.rank_row[rq.t_off + (int)(uint32_t)pair] = rank; };
   const bool fits = m <= HELD;
@@ -710,6 +711,27 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 256 ? 3 : 2) rank_place_ke
 #pragma unroll
     for (int r = 0; r < PER; ++r)
       if (r * THREADS < m) pair[r] = pair_at(min(r * THREADS + tid, m - 1));
+    if (b0 == 0 || b0 + group == S) {                  // the segment's first pair, or its last one, is the bound that lacks
+      unsigned long long end = pair[0];
+#pragma unroll
+      for (int r = 1; r < PER; ++r)
+        if (r * THREADS < m) end = b0 == 0 ? min(end, pair[r]) : max(end, pair[r]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(0xffffffffu, end, o);
+        end = b0 == 0 ? min(end, other) : max(end, other);
+      }
+      if (lane == 0) sm.most[wid] = end;
+      __syncthreads();
+      if (tid == 0) {
+        for (int w = 1; w < THREADS / 32; ++w) end = b0 == 0 ? min(end, sm.most[w]) : max(end, sm.most[w]);
+        const int g = b0 == 0 ? 0 : group - 1;
+        const unsigned long long low = b0 == 0 ? end : sm.least[g], high = b0 == 0 ? sm.least[0] : end;
+        sm.least[g] = min(low, high);                  // (an empty bucket's is not used)
+        sm.scale[g] = (float)own / __ull2float_rz(max(1ull, high - min(low, high)));
+      }
+      __syncthreads();
+    }
 #pragma unroll
     for (int r = 0; r < PER; ++r)
       if (r * THREADS + tid < m) {
@@ -720,7 +742,7 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 256 ? 3 : 2) rank_place_ke
     // buckets that do not fit (some row in ten thousand has such, or one whose sampled scores are unlike the others): the
     // same through global memory, the bins between the smallest and the largest pair that each bucket really has
     __syncthreads();
-    if (tid < PLACE_GROUP) { sm.least[tid] = ~0ull; sm.most[tid] = 0ull; }
+    if (tid < group) { sm.least[tid] = ~0ull; sm.most[tid] = 0ull; }
     __syncthreads();
     for (int e = tid; e < m; e += THREADS) {
       const unsigned long long p = pair_at(e);
@@ -729,7 +751,7 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 256 ? 3 : 2) rank_place_ke
       if (p > *(volatile unsigned long long*)&sm.most[g]) atomicMax(&sm.most[g], p);
     }
     __syncthreads();
-    if (tid < PLACE_GROUP) sm.scale[tid] = (float)OWN / __ull2float_rz(max(1ull, sm.most[tid] - sm.least[tid]));     // (an empty bucket's is not used)
+    if (tid < group) sm.scale[tid] = (float)own / __ull2float_rz(max(1ull, sm.most[tid] - sm.least[tid]));     // (an empty bucket's is not used)
     __syncthreads();
     for (int e = tid; e < m; e += THREADS) atomicAdd(&sm.bin[bin_of(pair_at(e))], 1);
   }
@@ -762,6 +784,7 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 256 ? 3 : 2) rank_place_ke
       if (r * THREADS + tid < m) {
         const int q = (int)(at[r] >> 16), begin = sm.bin[q], end = sm.bin[q + 1];
         int rank = base + begin;
+#pragma unroll 4
         for (int i = begin; i < end; ++i) rank += sm.held[i] < pair[r] ? 1 : 0;
         put(pair[r], rank);
       }
@@ -777,6 +800,7 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 256 ? 3 : 2) rank_place_ke
       const unsigned long long p = list[e];
       const int q = bin_of(p), begin = q ? sm.bin[q - 1] : 0, end = sm.bin[q];
       int rank = base + begin;
+#pragma unroll 4
       for (int i = begin; i < end; ++i) rank += list[i] < p ? 1 : 0;
       put(p, rank);
     }
@@ -793,7 +817,7 @@ void launch_split_of(RowArgs r, int max_T, int batch, cudaStream_t st) {
   r.max_tiles = (max_T + 4 * S - 1) / (4 * S);
   r.table = reinterpret_cast<uint16_t*>(r.splitters + (size_t)batch * S);
   rank_split_kernel<S><<<dim3(r.max_tiles, batch), S, split_smem_bytes<S>(), st>>>(r);
-  rank_place_kernel<S><<<dim3(S / PLACE_GROUP, batch), PLACE_THREADS, sizeof(PlaceSmem<S>), st>>>(r);
+  rank_place_kernel<S><<<dim3(S / PlaceSmem<S>::MIN_GROUP, batch), PLACE_THREADS, sizeof(PlaceSmem<S>), st>>>(r);
 }
 
 // Buckets of up to 128 pairs on average to 32K tokens, 256 above.  (A block of one bucket each, bins between its smallest and
