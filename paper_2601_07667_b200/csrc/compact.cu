@@ -16,6 +16,7 @@ __global__ void __launch_bounds__(256) compact_kv_kernel(const uint8_t* __restri
                                                          int cur_layer, uint8_t* __restrict__ k_out,
                                                          uint8_t* __restrict__ v_out) {
   // strides in bytes; a row is k_vec (v_vec) 16-byte vectors; 16 threads per kept row
+  pdl_wait_predecessor();
   const int b = blockIdx.z, h = blockIdx.y;
   if (latch && asl_finished(latch + b, cur_layer)) return;       // finished request: its compacted cache is final
   const AslReq rq = req[b];
@@ -25,7 +26,7 @@ __global__ void __launch_bounds__(256) compact_kv_kernel(const uint8_t* __restri
   const int64_t orow = (int64_t)h * sum_kept + rq.kept_off + r0;
   int64_t tok[ROWS];
 #pragma unroll
-  for (int i = 0; i < ROWS; ++i) tok[i] = r0 + 16 * i < rq.kept ? (int64_t)rq.tok_off + __ldg(idx + orow + 16 * i) : -1;
+  for (int i = 0; i < ROWS; ++i) tok[i] = r0 + 16 * i < rq.kept ? (int64_t)rq.tok_off + __ldcg(idx + orow + 16 * i) : -1;
   uint4 kv[ROWS], vv[ROWS];
 #pragma unroll
   for (int i = 0; i < ROWS; ++i) {
@@ -44,13 +45,14 @@ __global__ void __launch_bounds__(256) compact_kv_kernel(const uint8_t* __restri
 __global__ void __launch_bounds__(256) compact_rows_kernel(const uint4* __restrict__ x, const int32_t* __restrict__ idx,
                                                            const AslReq* __restrict__ req, int vec_per_row,
                                                            uint4* __restrict__ out) {
+  pdl_wait_predecessor();
   const int b = blockIdx.y;
   const AslReq rq = req[b];
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= rq.kept) return;
-  const int64_t src = ((int64_t)rq.tok_off + idx[rq.kept_off + r]) * vec_per_row;
+  const int64_t src = ((int64_t)rq.tok_off + __ldcg(idx + rq.kept_off + r)) * vec_per_row;
   const int64_t dst = ((int64_t)rq.kept_off + r) * vec_per_row;
-  for (int c = lane; c < vec_per_row; c += 32) out[dst + c] = x[src + c];
+  for (int c = lane; c < vec_per_row; c += 32) out[dst + c] = __ldcs(x + src + c);
 }
 
 }  // namespace
@@ -58,7 +60,7 @@ __global__ void __launch_bounds__(256) compact_rows_kernel(const uint4* __restri
 asl_status asl_launch_compact_rows(asl_ctx* c, const void* x, const int32_t* idx, void* out, int64_t row_bytes,
                                    cudaStream_t st) {
   dim3 grid((c->max_kept + 7) / 8, c->p.batch);
-  compact_rows_kernel<<<grid, 256, 0, st>>>(static_cast<const uint4*>(x), idx, c->d_req, (int)(row_bytes / 16),
+  launch_after(compact_rows_kernel, grid, dim3(256), st, static_cast<const uint4*>(x), idx, c->d_req, (int)(row_bytes / 16),
                                             static_cast<uint4*>(out));
   c->launches += 1;
   ASL_CUDA(cudaGetLastError());
@@ -71,7 +73,7 @@ asl_status asl_launch_compact(asl_ctx* c, const void* k, const void* v, const in
   const int kb = c->k_elem_bytes;                          // K elements are 2 bytes (bf16) or 1 (FP8 codes), V is bf16
   const int k_vec = p.head_dim * kb / 16, v_vec = p.head_dim * 2 / 16;
   dim3 grid((c->max_kept + BLOCK_ROWS - 1) / BLOCK_ROWS, p.n_kv_heads, p.batch);
-  compact_kv_kernel<<<grid, 256, 0, st>>>(static_cast<const uint8_t*>(k), static_cast<const uint8_t*>(v), idx, c->d_req,
+  launch_after(compact_kv_kernel, grid, dim3(256), st, static_cast<const uint8_t*>(k), static_cast<const uint8_t*>(v), idx, c->d_req,
                                           p.k_stride[0] * kb, p.k_stride[1] * kb, p.v_stride[0] * 2, p.v_stride[1] * 2,
                                           c->sum_kept, k_vec, v_vec, c->latch_stat, c->cur_layer,
                                           static_cast<uint8_t*>(k_out), static_cast<uint8_t*>(v_out));

@@ -35,6 +35,7 @@ struct PoolArgs {
 // staged in shared memory; 128K tokens of 8 heads, two partial rows each, 6.1 -> 4.4 us.
 template <bool MAX, int R, int NR>
 __global__ void __launch_bounds__(PT) pool_vec4_kernel(PoolArgs a) {
+  pdl_wait_predecessor();
   const int b = blockIdx.y;
   if (a.latch && asl_finished(a.latch + b, a.cur_layer)) return;       // the request's scores stay as its selection layer left them
   const AslReq rq = a.req[b];
@@ -100,6 +101,7 @@ __global__ void __launch_bounds__(PT) pool_vec4_kernel(PoolArgs a) {
 // last 2 * MAX_HALO threads load the halo); HB units are staged per round in shared memory and pooled from there.
 __global__ void __launch_bounds__(PT + 2 * MAX_HALO) pool_group_kernel(PoolArgs a) {
   __shared__ float tile[HB][PT + 2 * MAX_HALO];
+  pdl_wait_predecessor();
   const int b = blockIdx.y;
   if (a.latch && asl_finished(a.latch + b, a.cur_layer)) return;
   const AslReq rq = a.req[b];
@@ -195,9 +197,9 @@ asl_status asl_launch_pool(asl_ctx* c, const float* u, float* scores_kv, float* 
                    c->latch_stat, c->cur_layer, vec_out, scores_kv, scores_agg};
   if (const PoolKernel vec4 = max ? pool_vec4_of<true>(r, nrows) : pool_vec4_of<false>(r, nrows)) {
     const int warps = (c->max_T + 119) / 120;
-    vec4<<<dim3((warps + PT / 32 - 1) / (PT / 32), p.batch), PT, 0, st>>>(a);
+    launch_after(vec4, dim3((warps + PT / 32 - 1) / (PT / 32), p.batch), dim3(PT), st, a);
   } else {
-    pool_group_kernel<<<dim3((c->max_T + PT - 1) / PT, p.batch), PT + 2 * MAX_HALO, 0, st>>>(a);
+    launch_after(pool_group_kernel, dim3((c->max_T + PT - 1) / PT, p.batch), dim3(PT + 2 * MAX_HALO), st, a);
   }
   c->launches += 1;
   ASL_CUDA(cudaGetLastError());

@@ -436,6 +436,7 @@ __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
   __shared__ __align__(16) uint32_t keys[COUNT_MAX_T];
   __shared__ int part[COUNT_WARPS][32];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  pdl_wait_predecessor();
   const bool open = !row_is_final(a, 0);
   const AslReq rq = row_request(a, 0);
   const int T = rq.T, padded = (T + 127) & ~127;                     // padding goes before nothing
@@ -538,6 +539,7 @@ __global__ void __launch_bounds__(S) rank_split_kernel(RowArgs a) {
   __shared__ int warp_tot[S / 32];
   const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const AslReq rq = row_request(a, b);
+  pdl_wait_predecessor();
   if (row_is_final(a, b)) return;
   const int start = blockIdx.x * TILE_N;
   if (start >= rq.T) return;
@@ -641,6 +643,7 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_k
   const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   pdl_release_successor();
   const AslReq rq = row_request(a, b);
+  pdl_wait_predecessor();
   if (row_is_final(a, b)) return;
   const int tiles = (rq.T + TILE_N - 1) / TILE_N;
   // buckets of a block: as many (a power of two) as give a block a sixth of the pairs that it can hold, so that nearly every
@@ -810,14 +813,14 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_k
 template <int S>
 constexpr int split_smem_bytes() { return (int)(5 * S * sizeof(unsigned long long) + S * sizeof(int)); }
 
-void launch_count(const RowArgs& r, int T, cudaStream_t st) { rank_count_kernel<<<(T + 31) / 32, COUNT_THREADS, 0, st>>>(r); }
+void launch_count(const RowArgs& r, int T, cudaStream_t st) { launch_after(rank_count_kernel, dim3((T + 31) / 32), dim3(COUNT_THREADS), st, r); }
 
 template <int S>
 void launch_split_of(RowArgs r, int max_T, int batch, cudaStream_t st) {
   r.max_tiles = (max_T + 4 * S - 1) / (4 * S);
   r.table = reinterpret_cast<uint16_t*>(r.splitters + (size_t)batch * S);
-  rank_split_kernel<S><<<dim3(r.max_tiles, batch), S, split_smem_bytes<S>(), st>>>(r);
-  rank_place_kernel<S><<<dim3(S / PlaceSmem<S>::MIN_GROUP, batch), PLACE_THREADS, sizeof(PlaceSmem<S>), st>>>(r);
+  launch_after_smem(rank_split_kernel<S>, dim3(r.max_tiles, batch), dim3(S), split_smem_bytes<S>(), st, r);
+  launch_after_smem(rank_place_kernel<S>, dim3(S / PlaceSmem<S>::MIN_GROUP, batch), dim3(PLACE_THREADS), sizeof(PlaceSmem<S>), st, r);
 }
 
 // Buckets of up to 128 pairs on average to 32K tokens, 256 above.  (A block of one bucket each, bins between its smallest and

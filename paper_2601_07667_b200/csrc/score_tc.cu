@@ -436,8 +436,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   // ---- set-up: zero the Q buffers (rows that no copy writes feed unused MMA rows), barriers, tensor memory ----
   if (copies * box_rows < S::Q_ROWS)
     for (int i = threadIdx.x; i < 2 * S::Q_BUF / 16; i += THREADS) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
-  const TcWork work = a.live_hdr && __ldg(a.live_hdr) ? a.live : a.list;
-  const int first = __ldg(work.first + blockIdx.x);
   if (threadIdx.x == 32) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_q) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_k) : "memory");
@@ -451,6 +449,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
     mbar_init(bar(S::DRAIN), 1);
     *s_abort = 0;
+    pdl_wait_predecessor();                  // (the number may be another launch's to advance)
     uint32_t number = 0;
     if (!a.lse) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(number) : "l"(a.launch) : "memory");
     *s_set = number & 1u;
@@ -466,6 +465,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
+  pdl_wait_predecessor();                    // all above is the CTA's own; operands, lists and counters may be the work of kernels before
+  const TcWork work = a.live_hdr && __ldg(a.live_hdr) ? a.live : a.list;
+  const int first = __ldg(work.first + blockIdx.x);
   uint32_t* const published = a.counters + (size_t)*s_set * 2 * a.nseg * SYNC_STRIDE;
   uint32_t* const folded = published + (size_t)a.nseg * SYNC_STRIDE;
 
@@ -1482,7 +1484,8 @@ asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const f
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)p.head_dim));
   // every CTA must be resident at once (pass 2 waits for counters other CTAs advance): one CTA per SM at most
   const ScoreKernel& kern = score_kernel(score_kernel_of(p, tp));
-  kern.fn<<<list.grid, THREADS, kern.smem, st>>>(tm_q, tm_k, a);
+  if (a.live_hdr) kern.fn<<<list.grid, THREADS, kern.smem, st>>>(tm_q, tm_k, a);     // (the kernel before writes the list, which is read as constant)
+  else launch_after_smem(kern.fn, dim3(list.grid), dim3(THREADS), kern.smem, st, tm_q, tm_k, a);
   c->launches += 1;
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;

@@ -220,7 +220,6 @@ __global__ void __launch_bounds__(THREADS) topk_emit_kernel(TopkArgs a) {
   const Segment s = segment_of(a);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int tiles = max(1, (s.T + TILE - 1) / TILE);
-  pdl_release_successor();
   if (!s.open || s.tile >= tiles) return;
   uint32_t key[PER_THREAD];
   if (s.k) load_keys(s, key);
@@ -411,6 +410,7 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) topk_segment_kernel(TopkArgs a
   SegSmem& sm = *reinterpret_cast<SegSmem*>(seg_smem_raw);
   uint32_t* const bm_gt = reinterpret_cast<uint32_t*>(seg_smem_raw + sizeof(SegSmem));
   uint32_t* const bm_eq = bm_gt + seg_words(a.max_T);
+  pdl_wait_predecessor();
   const Segment s = segment_of(a);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (!s.open) return;
@@ -778,7 +778,7 @@ asl_status asl_launch_topk(asl_ctx* c, const float* scores, int32_t n_heads, int
   a.latch = gate ? nullptr : c->latch_stat;      // the gated call has its own rule
   a.cur_layer = c->cur_layer;
   if (c->topk_one_cta && one_cta_is_faster(c, n_heads)) {
-    topk_segment_kernel<<<dim3(1, n_heads, c->p.batch), SEG_THREADS, seg_smem_bytes(c->max_T), st>>>(a);
+    launch_after_smem(topk_segment_kernel, dim3(1, n_heads, c->p.batch), dim3(SEG_THREADS), seg_smem_bytes(c->max_T), st, a);
     c->launches += 1;
     ASL_CUDA(cudaGetLastError());
     return ASL_OK;

@@ -1,0 +1,81 @@
+"""Calls issued back to back, each on the results of the one before it, while inputs are overwritten in between: kernels
+that become resident before their predecessor has ended must still see all of its work, on one stream, behind an event of
+another stream, and in a captured graph."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import asl_oracle as O
+from paper_2601_07667_b200 import binding as B
+from paper_2601_07667_b200 import inputs as I
+
+from asl_check import make_path
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("how", ["one stream", "events", "graph"])
+@pytest.mark.parametrize("T", [3000, 40000])
+def test_select_compact_and_rank_chains(T, how):
+    w, rounds = 32, 6
+    wl = I.workload("C1", seqlens=(T + w,), budgets=(w + T // 5,), l_min=0, l_obs=rounds)
+    path = make_path(wl)
+    H, d = wl.n_kv_heads, 128
+    g = torch.Generator(device="cuda").manual_seed(T)
+    scores = torch.rand((rounds, H, T), generator=g, device="cuda")
+    keys = torch.randint(-30000, 30000, (rounds, T + w, H, d), generator=g, device="cuda", dtype=torch.int16)
+    kv, agg = torch.empty((H, T), device="cuda"), torch.empty(T, device="cuda")
+    k, v = torch.empty_like(keys[0]), torch.empty_like(keys[0])
+    outs = [(torch.empty_like(path.idx), torch.empty_like(path.k_out), torch.empty_like(path.v_out), torch.empty_like(path.rank_ring[0]))
+            for _ in range(rounds)]
+    side = torch.cuda.Stream()
+
+    def chain():
+        main = torch.cuda.current_stream()
+        for r, (idx, k_out, v_out, row) in enumerate(outs):
+            kv.copy_(scores[r])
+            agg.copy_(scores[r, 0])
+            if how == "one stream":
+                k.copy_(keys[r])
+                v.copy_(keys[r])
+            else:                                             # the keys come from another stream
+                side.wait_stream(main)
+                with torch.cuda.stream(side):
+                    k.copy_(keys[r])
+                    v.copy_(keys[r])
+            B.asl_select_topk(path.ctx, kv, H, path.idx, path.workspace, path.ws_bytes)
+            if how != "one stream":
+                main.wait_stream(side)
+            B.asl_compact_kv(path.ctx, k, v, path.idx, path.k_out, path.v_out)
+            idx.copy_(path.idx)
+            k_out.copy_(path.k_out)
+            v_out.copy_(path.v_out)
+            B.asl_rank_stat(path.ctx, agg, r, r + 1, path.rank_ring, path.stat, path.workspace, path.ws_bytes)
+            row.copy_(path.rank_ring[r])
+
+    chain()                                                   # (once before a capture)
+    if how == "graph":
+        torch.cuda.synchronize()
+        for o in outs:
+            for t in o:
+                t.zero_()
+        path.stat.zero_()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            chain()
+        graph.replay()
+    torch.cuda.synchronize()
+    s, kk, ranks = scores.cpu().numpy(), keys.cpu().numpy(), []
+    for r, (idx, k_out, v_out, row) in enumerate(outs):
+        got_k = k_out.view(torch.int16).cpu().numpy()
+        for h in range(H):
+            ref = O.select_topk(s[r, h].astype(np.float64), T // 5, T + w, w)
+            assert (idx[h].cpu().numpy() == ref).all(), (r, h)
+            assert (got_k[h] == kk[r, ref, h]).all(), (r, h)
+        assert torch.equal(k_out, v_out)
+        ranks.append(O.rank_desc(s[r, 0].astype(np.float64)))
+        assert (row.cpu().numpy() == ranks[-1]).all(), r
+    num, m, _ = O.rank_statistic(np.stack(ranks), T // 5)
+    stat = path.read_stat()[0]
+    assert (stat["num"], stat["m"]) == (num, m)
+    path.close()
