@@ -60,6 +60,7 @@ constexpr int KT = ASL_TC_KEY_TILE;          // keys per tile
 constexpr int MAX_ROWS = 256;                // query rows of a chunk at most
 constexpr int THREADS = 640;                 // warp 0: TMA, 1: MMA, 2-3: partial folding, 4-19: four epilogue groups
 constexpr int GROUPS = 4;
+constexpr unsigned long long OFFSET_READY = 1ull << 32;
 constexpr int SYNC_STRIDE = 8;               // words from one segment's counter to the next: a sector each
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;   // every wait gives up after 2 s
 
@@ -137,6 +138,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
   *abort_flag = code;
   return false;
+}
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
 }
 // Bounded wait until the 32-bit word at p equals `want` (acquire).  Lane 0 polls.
 __device__ __forceinline__ bool word_wait(const uint32_t* p, uint32_t want, volatile int* abort_flag, int code, int lane,
@@ -372,11 +378,17 @@ struct TcArgs {
   float* offsets;          // [segment][NC], written by the folding warps, read by pass 2
   const float* lse;        // null, or the rows' natural-log softmax denominators [B][H_q][W]: pass 2 alone
   float* u;                // pass 2 out: column sums
-  // [2][2][segment * SYNC_STRIDE]: per segment, epilogue groups that have published and rows whose offset is written.
+  // [2][segment * SYNC_STRIDE]: epilogue groups of the segment that have published.
   // A launch counts in the set that its number's parity names; the last CTA to arrive clears the other set (whose launch
   // is over), advances the number and resets the ticket.  The number lives on the device so that a launch replayed from
   // a CUDA graph counts like any other, and is switched at entry so that no CTA has anything to do at its end.
   uint32_t* counters;
+  // [2][segment][NC], sets as above: a row's offset with OFFSET_READY above it, or zero.  The folding warps write the value
+  // and the flag in one word, so that who waits for it has it with the look that finds it there, and nothing is fenced; they
+  // clear the same rows of the other set.  (A counter of folded rows behind a fence, then a load of the offsets, were two
+  // round trips more in front of pass 2: 4096 tokens 18.3 -> 14.2 us, two prompts with W = 24 23 -> 20, 32K 46.2 -> 45.7,
+  // 128K 163.7 -> 164.1.)
+  unsigned long long* ready;
   uint32_t* launch;        // launch number, then the ticket of arrived CTAs
   int32_t* err;
   int64_t u_stride;
@@ -468,8 +480,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   pdl_wait_predecessor();                    // all above is the CTA's own; operands, lists and counters may be the work of kernels before
   const TcWork work = a.live_hdr && __ldg(a.live_hdr) ? a.live : a.list;
   const int first = __ldg(work.first + blockIdx.x);
-  uint32_t* const published = a.counters + (size_t)*s_set * 2 * a.nseg * SYNC_STRIDE;
-  uint32_t* const folded = published + (size_t)a.nseg * SYNC_STRIDE;
+  uint32_t* const published = a.counters + (size_t)*s_set * a.nseg * SYNC_STRIDE;
 
   if (warp == 0) {
     // =============================== TMA producer ===============================
@@ -600,9 +611,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // =============================== partial folding ==============================
     // For every pass-1 stage: the rows of its segments are dealt to the CTAs in runs of `per`; wait until a row's
     // segment has been published by all its epilogue groups, fold the row's partials in a fixed order (the result does
-    // not depend on timing) and count the row as done.  Up to eight rows at a time, four or more lanes each, so that a
-    // stage costs one round trip for the partials and one for the fence (row after row it was 2 us each, 18 us of
-    // waiting in front of pass 2 for a group of four heads).
+    // not depend on timing) and write its offset.  Up to eight rows at a time, four or more lanes each, so that a
+    // stage costs one round trip for the partials (row after row it was 2 us each, 18 us of waiting in front of pass 2 for
+    // a group of four heads).
+    unsigned long long* const ready = a.ready + (size_t)*s_set * a.nseg * a.NC;
     for (int si = 0; si < a.n_stages; ++si) {
       const int a0 = __ldg(&a.stages[si].seg0), total = __ldg(&a.stages[si].nseg) * a.NC;
       const int per = (total + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -617,6 +629,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const int sg = idx / a.NC, row = idx - sg * a.NC;
         const int4 fo = __ldg(reinterpret_cast<const int4*>(work.folds + a0 + sg));        // slot0, nruns, rows, request
         const bool valid = base + lane % rpi < hi && row < fo.z && fo.y > 0;
+        if (sub == 0) __stcg(a.ready + ((size_t)(*s_set ^ 1u) * a.nseg + a0 + sg) * a.NC + row, 0ull);
         for (int q = s0; ok && q <= s1 / a.NC; ++q) {
           const int4 fq = __ldg(reinterpret_cast<const int4*>(work.folds + a0 + q));
           if (fq.y > 0) ok = word_wait(published + (a0 + q) * SYNC_STRIDE, (uint32_t)(GROUPS * fq.y), s_abort, 41, lane, 128);
@@ -652,32 +665,31 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           if (Lb > 0.f) Ln += Lb * ex2(Mb - Mn);
           M = Mn; L = Ln;
         }
-        if (valid && sub == 0) __stcg(a.offsets + (int64_t)(a0 + sg) * a.NC + row, M + log2f(L));
-        __syncwarp();
-        if (lane == 0) __threadfence();                            // cumulative: the warp's stores above
-        for (int q = s0; q <= s1 / a.NC; ++q) {
-          const int done = __popc(__ballot_sync(0xffffffffu, valid && sub == 0 && sg == q));
-          if (lane == 0 && done) atomicAdd(folded + (a0 + q) * SYNC_STRIDE, (uint32_t)done);
+        if (valid && sub == 0) {
+          const float offset = M + log2f(L);
+          const int64_t at = (int64_t)(a0 + sg) * a.NC + row;
+          asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(ready + at), "l"(OFFSET_READY | __float_as_uint(offset)) : "memory");
+          __stcg(a.offsets + at, offset);                          // for asl_window_lse
         }
       }
       if (!ok) break;
     }
   } else if (warp == 3) {
     // =============================== row offsets ==================================
-    // For every pass-2 run of the CTA: wait until the segment's rows have been folded (one poller per CTA: sixteen
-    // epilogue warps polling on 148 SMs keep the counter's L2 slice busy and the folds' own increments waiting), then
-    // hand the negated offsets to the epilogue in shared memory.
+    // For every pass-2 run of the CTA: look for the segment's offsets until all are there (one warp per CTA: sixteen on 148
+    // SMs would keep the L2 slices busy), then hand them, negated, to the epilogue in shared memory.
     if (!a.lse) {
       uint32_t last = 0;
       if (lane == 0) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(last) : "l"(a.launch + 1) : "memory");
       if (__shfl_sync(0xffffffffu, last, 0) == gridDim.x - 1u) {       // every CTA has read the number
-        uint32_t* other = a.counters + (size_t)(*s_set ^ 1u) * 2 * a.nseg * SYNC_STRIDE;
-        for (int i = lane; i < 2 * a.nseg; i += 32) other[(size_t)i * SYNC_STRIDE] = 0;
+        uint32_t* other = a.counters + (size_t)(*s_set ^ 1u) * a.nseg * SYNC_STRIDE;
+        for (int i = lane; i < a.nseg; i += 32) other[(size_t)i * SYNC_STRIDE] = 0;
         if (lane == 0) { a.launch[0] = *s_number + 1u; a.launch[1] = 0; }
       }
     }
     float* s_off = reinterpret_cast<float*>(smem + S::OFFS);
     int q = 0;
+    bool ok = true;
     for (int slot = first; slot >= 0;) {
       const TcRun r = load_run(work.runs, slot);
       prefetch_run(work.runs, r.next);
@@ -685,11 +697,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       if (r.pass != 2) continue;
       const int buf = q & 1;
       if (q >= 2 && !__all_sync(0xffffffffu, mbar_wait(bar(S::OEMPTY + buf), ((q >> 1) & 1) ^ 1, s_abort, 32, true))) break;
-      if (!a.lse && !word_wait(folded + r.seg * SYNC_STRIDE, (uint32_t)r.rows, s_abort, 33, lane, 128)) break;
       const RowPlace p0 = row_place(a, r.chunk, 0);
-      const float* src = a.lse ? a.lse + ((int64_t)r.b * a.Hq + r.h * a.G + p0.g) * a.W + p0.t : a.offsets + (int64_t)r.seg * a.NC;
-      const float unit = a.lse ? -1.4426950408889634f : -1.0f;          // supplied: natural log -> log2 domain
+      const float* lse = a.lse + ((int64_t)r.b * a.Hq + r.h * a.G + p0.g) * a.W + p0.t;
+      const unsigned long long* src = a.ready + ((size_t)*s_set * a.nseg + r.seg) * a.NC;
       float o[MAX_ROWS / 32];
+      uint32_t left = 0;                                                // rows of this lane that are not there yet
 #pragma unroll
       for (int i = 0; i < MAX_ROWS / 32; ++i) {
         const int row = lane + 32 * i;
@@ -698,10 +710,38 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (!dense) {                                                   // max pooling, heads padded to Wp rows
           const int hd = row / a.Wp, t = row - hd * a.Wp;
           exists = exists && t < a.W;
-          if (a.lse) at = hd * a.W + t;
+          at = hd * a.W + t;
         }
-        o[i] = exists ? __ldcg(src + at) * unit : -INFINITY;            // a padding row: 2^(x - inf) = 0
+        o[i] = -INFINITY;                                               // a padding row: 2^(x - inf) = 0
+        if (exists && a.lse) o[i] = __ldcg(lse + at) * -1.4426950408889634f;      // natural log -> log2 domain
+        if (exists && !a.lse) left |= 1u << i;
       }
+      unsigned long long t0 = 0;
+      uint32_t nap = 32;
+      for (uint32_t it = 0; __any_sync(0xffffffffu, left != 0u); ++it) {
+        unsigned long long v[MAX_ROWS / 32];
+        // (a wait that lasts looks at the first rows only until they are there)
+        const uint32_t look = it >= 8 && __any_sync(0xffffffffu, left & 1u) ? left & 1u : left;
+#pragma unroll
+        for (int i = 0; i < MAX_ROWS / 32; ++i) v[i] = (look >> i) & 1u ? ld_relaxed(src + lane + 32 * i) : 0ull;
+#pragma unroll
+        for (int i = 0; i < MAX_ROWS / 32; ++i)
+          if (v[i]) { o[i] = -__uint_as_float((uint32_t)v[i]); left &= ~(1u << i); }
+        if ((it & 7u) == 7u) {
+          int gave_up = 0;
+          if (lane == 0) {
+            const unsigned long long now = global_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > WAIT_LIMIT_NS || *s_abort) { gave_up = 1; if (!*s_abort) *s_abort = 33; }
+          }
+          if (__shfl_sync(0xffffffffu, gave_up, 0)) { ok = false; break; }
+        }
+        if (it >= 8) {                       // the first looks follow one another at once: what is waited for is about to come
+          __nanosleep(nap);
+          if (nap < 256) nap <<= 1;
+        }
+      }
+      if (!ok) break;
 #pragma unroll
       for (int i = 0; i < MAX_ROWS / 32; ++i) s_off[buf * MAX_ROWS + lane + 32 * i] = o[i];
       __syncwarp();
@@ -1150,6 +1190,11 @@ bool fp8_shape(const asl_params& p) {
   return false;
 }
 
+// counters, launch number and ticket, offsets
+size_t sync_bytes(const AslTcPlan& tp) {
+  return (2 * (size_t)tp.nseg + 1) * SYNC_STRIDE * sizeof(uint32_t) + 2 * (size_t)tp.nseg * tp.NC * sizeof(unsigned long long);
+}
+
 int round_up(int x, int to) { return (x + to - 1) / to * to; }
 int div_up(int x, int by) { return (x + by - 1) / by; }
 
@@ -1287,12 +1332,17 @@ bool asl_tc_plan(asl_ctx* c) {
   if (tiles >= (int64_t)1 << 30) return false;
 
   // Groups of segments: pass 1 of a group, then pass 2 of the one before it, so that the fold of the row denominators is
-  // hidden behind other tiles; at least two of them, of up to 70 MB of K each.  Small groups leave more of K in L2 for pass 2
+  // hidden behind other tiles; at least two of them, of up to 70 MB of K each.  (One, where no CTA of
+  // any call has more than one tile of a pass: there is then nothing to hide the fold behind, and it is waited for once
+  // instead of twice.  In us with two groups and one: 1500 tokens of 8 kv heads 21.2, 15.8, 4096 of 2 heads 13.9, 11.6.  It
+  // would pay up to 1.3 tiles a CTA, 3000 tokens 19.6, 16.7, but asl_score_layer and its halves then add in different
+  // orders; at 2.5 tiles not, 6000 tokens 19.0, 21.4.)  Small groups leave more of K in L2 for pass 2
   // (above), large ones need fewer hand-offs, and the hand-offs count for more.  In us at 36, 50, 70, 100, 140 and 270 MB:
   // four layers of 100K tokens 668, 670, 642, 645, 640, 640; of 128K 843, 843, 841, 843, 845, 834; of 192K 1236, 1240, 1241,
   // 1243, 1232, 1218; two layers of eight ragged requests 616, 599, 602, 602, 592, 582; two with W = 128 and 64 query heads
   // at 64K 761, 758, 760, 768, 760, 762.  So the limit is above the step at 100K tokens (25.6 MB a kv head: two in a group),
   // but not where batches are fastest.
+  const int given = p.score_ctas > 0 && p.score_ctas < c->sm_count ? p.score_ctas : 0;
   std::vector<int> cut{0};
   {
     auto seg_bytes = [&](int s) { return (double)c->req[segs[s].b].n * 128 * c->k_elem_bytes / tp.nchunk; };
@@ -1303,7 +1353,7 @@ bool asl_tc_plan(asl_ctx* c) {
       if (run > 0 && run + seg_bytes(s) > 70.0e6) { ++groups; run = 0; }
       run += seg_bytes(s);
     }
-    groups = groups < 2 ? 2 : groups;
+    if (groups < 2 && tiles > (given ? given : c->sm_count - 32)) groups = 2;
     run = 0;
     for (int s = 0; s + 1 < tp.nseg; ++s) {                // evenly sized
       run += seg_bytes(s);
@@ -1314,7 +1364,6 @@ bool asl_tc_plan(asl_ctx* c) {
   // CTAs: as many as the caller says; else one per SM, and where the call is one half of a layer (asl_score_columns) 16
   // fewer, so that the rest of the layer before runs beside it, 32 fewer for the shorter one-pass call with one chunk
   // per kv head
-  const int given = p.score_ctas > 0 && p.score_ctas < c->sm_count ? p.score_ctas : 0;
   const int spare[2] = {16, tp.nchunk == 1 ? 32 : 16};
   const int n_lists = given || p.score_ctas > 0 ? 2 : 4;
   HostList lists[4];
@@ -1352,9 +1401,8 @@ bool asl_tc_plan(asl_ctx* c) {
     if ((size_t)l.grid > ctas) ctas = l.grid;
     if (out.n1 > tp.partial_slots) tp.partial_slots = out.n1;
   }
-  const size_t sync_words = (4 * (size_t)tp.nseg + 1) * SYNC_STRIDE;
-  const std::vector<uint32_t> zeros(sync_words, 0);
-  const size_t sync_at = put(zeros.data(), sync_words * sizeof(uint32_t));
+  const std::vector<char> zeros(sync_bytes(tp), 0);
+  const size_t sync_at = put(zeros.data(), zeros.size());
   const size_t host_bytes = bytes;
   auto take = [&](size_t n) { const size_t t = bytes; bytes = asl_align256(bytes + n); return t; };
   const size_t live_at[5] = {take(n_runs * sizeof(TcRun)), take(ctas * sizeof(int32_t)), take((size_t)tp.nseg * sizeof(TcFold)),
@@ -1422,7 +1470,7 @@ asl_status asl_launch_live_phases(asl_ctx* c, bool two_pass, bool beside, cudaSt
 asl_status asl_tc_reset_sync(asl_ctx* c, cudaStream_t st) {
   AslTcPlan& tp = c->tc;
   if (!tp.d_sync) return ASL_OK;
-  ASL_CUDA(cudaMemsetAsync(tp.d_sync, 0, (4 * (size_t)tp.nseg + 1) * SYNC_STRIDE * sizeof(uint32_t), st));
+  ASL_CUDA(cudaMemsetAsync(tp.d_sync, 0, sync_bytes(tp), st));
   return ASL_OK;
 }
 
@@ -1474,7 +1522,8 @@ asl_status asl_launch_score_tc(asl_ctx* c, const void* q, const void* k, const f
   a.offsets = reinterpret_cast<float*>(ws + c->ws.score_offsets);
   a.u = u;
   a.counters = tp.d_sync;                                            // the one-pass launch touches neither these
-  a.launch = tp.d_sync + 4 * (size_t)tp.nseg * SYNC_STRIDE;         // nor this
+  a.launch = tp.d_sync + 2 * (size_t)tp.nseg * SYNC_STRIDE;         // nor these
+  a.ready = reinterpret_cast<unsigned long long*>(a.launch + SYNC_STRIDE);
   a.err = c->d_err;
   a.u_stride = c->u_stride;
   a.nseg = tp.nseg;

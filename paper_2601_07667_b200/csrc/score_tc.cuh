@@ -49,7 +49,7 @@ struct AslTcPlan {
   // the caller gives the number of CTAs.  [][0]: both passes; [][1]: pass 2 alone (a supplied log-sum-exp).
   TcList lists[2][2];
   void* d_blob = nullptr;       // the device side of the lists below and above, one allocation
-  uint32_t* d_sync = nullptr;   // two sets of publish and folded-row counters, launch number, ticket of arrived CTAs
+  uint32_t* d_sync = nullptr;   // two sets of publish counters, launch number, ticket of arrived CTAs, two sets of offsets
   // device-side controller: the next launch's list without the finished requests' phases, written ahead of it
   TcRun* d_live_runs = nullptr;
   int32_t* d_live_first = nullptr;
