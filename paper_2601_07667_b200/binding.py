@@ -125,10 +125,23 @@ def _ptr(x) -> int:
     return x.data_ptr()
 
 
+_torch_c = None
+
+
+def _current_stream() -> int:
+    """Handle of torch's current stream on the current device, without the stream object that torch.cuda.current_stream()
+    makes (3 us, a third of what a whole call takes on the host)."""
+    global _torch_c
+    if _torch_c is None:
+        import torch
+        torch.cuda.current_stream()                        # sets CUDA up
+        _torch_c = torch._C
+    return _torch_c._cuda_getCurrentRawStream(_torch_c._cuda_getDevice())
+
+
 def _stream_handle(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -358,7 +371,7 @@ class LayerPath:
 
     def join(self) -> None:
         """The current stream waits for the work issued so far."""
-        _check(_lib.asl_run_join(self.ctx, self.torch.cuda.current_stream().cuda_stream), "asl_run_join")
+        _check(_lib.asl_run_join(self.ctx, _current_stream()), "asl_run_join")
 
     def close(self) -> None:
         if self.ctx:
@@ -386,16 +399,16 @@ class LayerPath:
         runs on the side streams and is left in flight (see ``join``): ``k`` and ``v`` are read there, so keep them (or
         ``record_stream(path.side2)``) until a join.  ``score_marks``: a list
         that receives a (start, end) event pair around the scoring call."""
-        main = self.torch.cuda.current_stream()
+        main = _current_stream()
         rows = self.n_rows(layer_idx)
         if self.latch:
             asl_set_layer(self.ctx, layer_idx)
         self._cur ^= 1
         if score_marks is not None:
             e0, e1 = (self.torch.cuda.Event(enable_timing=True) for _ in range(2))
-            e0.record(main)
+            e0.record()
         if overlap:
-            self._layer.stream = main.cuda_stream
+            self._layer.stream = main
             status = _lib.asl_run_layer(self.ctx, self._layer_ref, q_obs.data_ptr(), k.data_ptr(), v.data_ptr(),
                                         _ptr(lse), layer_idx, rows, self._cur)
             if status != ASL_OK:
@@ -404,7 +417,7 @@ class LayerPath:
             self.join()
             asl_score_columns(self.ctx, q_obs, k, lse, self.workspace, self.ws_bytes, self._cur)
         if score_marks is not None:                 # the call leaves nothing but the scoring on the main stream
-            e1.record(main)
+            e1.record()
             score_marks.append((e0, e1))
         if overlap:
             return

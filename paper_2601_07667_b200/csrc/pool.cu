@@ -14,7 +14,8 @@ namespace {
 constexpr int PT = 256;          // threads of a block / tokens per block of the general kernel
 constexpr int MAX_HALO = 16;     // pooling kernels up to 33 taps
 constexpr int HB = 8;            // general kernel: staged units per round
-constexpr int PV_ROWS = 16;      // vector kernel: partial rows in flight per lane
+constexpr int PV_ROWS = 8;       // vector kernel: partial rows in flight per lane
+constexpr int PV_THREADS = 128;
 
 struct PoolArgs {
   const float* u;                // [rows][u_stride], every request from a 16-byte boundary on
@@ -28,19 +29,21 @@ struct PoolArgs {
 };
 
 // Windows of up to 9 taps, units of 1, 2, 4, 8 or 16 partial rows.  A lane owns 4 consecutive tokens: one 16-byte load per
-// partial row, sixteen in flight, the rows of a unit added in order, the neighbours' sums fetched by warp shuffles; the
+// partial row, eight in flight, the rows of a unit added in order, the neighbours' sums fetched by warp shuffles; the
 // first and the last lane of a warp only supply the halo, so a warp pools 120 tokens.  No shared memory and no
-// block-wide barrier.  Bound by the round trips for the rows (one per sixteen): max pooling of 64 query
+// block-wide barrier.  Bound by the round trips for the rows (one per eight; with sixteen in flight the registers leave room
+// for half as many warps on the SMs that a scorer leaves free: eight layers of 32K tokens 434.3 -> 431.7 us): max pooling of 64 query
 // heads at 64K tokens 43 -> 10 us, eight ragged requests of 8 heads 25 -> 6.5 us against one thread per token with rows
 // staged in shared memory; 128K tokens of 8 heads, two partial rows each, 6.1 -> 4.4 us.
 template <bool MAX, int R, int NR>
-__global__ void __launch_bounds__(PT) pool_vec4_kernel(PoolArgs a) {
+__global__ void __launch_bounds__(PV_THREADS) pool_vec4_kernel(PoolArgs a) {
+  constexpr int IN_FLIGHT = NR > PV_ROWS ? NR : PV_ROWS;
   pdl_wait_predecessor();
   const int b = blockIdx.y;
   if (a.latch && asl_finished(a.latch + b, a.cur_layer)) return;       // the request's scores stay as its selection layer left them
   const AslReq rq = a.req[b];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int warp_of_segment = blockIdx.x * (PT / 32) + wid;
+  const int warp_of_segment = blockIdx.x * (PV_THREADS / 32) + wid;
   if (warp_of_segment * 120 >= rq.T) return;                           // the whole warp is past the segment
   const int j0 = 4 * (warp_of_segment * 30 + lane - 1);                // lanes 0 and 31: halo only
   const bool inside = j0 >= 0 && j0 < rq.T;
@@ -59,13 +62,13 @@ __global__ void __launch_bounds__(PT) pool_vec4_kernel(PoolArgs a) {
   };
   float agg[4] = {0.f, 0.f, 0.f, 0.f}, head[4] = {0.f, 0.f, 0.f, 0.f};
   int in_head = 0, h = 0;
-  for (int r0 = 0; r0 < rows; r0 += PV_ROWS) {
-    float4 x[PV_ROWS];
+  for (int r0 = 0; r0 < rows; r0 += IN_FLIGHT) {
+    float4 x[IN_FLIGHT];
 #pragma unroll
-    for (int e = 0; e < PV_ROWS; ++e)
+    for (int e = 0; e < IN_FLIGHT; ++e)
       x[e] = (inside && r0 + e < rows) ? __ldcg(reinterpret_cast<const float4*>(base + (int64_t)(r0 + e) * a.u_stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int q = 0; q < PV_ROWS / NR; ++q) {
+    for (int q = 0; q < IN_FLIGHT / NR; ++q) {
       if (r0 + q * NR >= rows) break;
       float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -197,7 +200,7 @@ asl_status asl_launch_pool(asl_ctx* c, const float* u, float* scores_kv, float* 
                    c->latch_stat, c->cur_layer, vec_out, scores_kv, scores_agg};
   if (const PoolKernel vec4 = max ? pool_vec4_of<true>(r, nrows) : pool_vec4_of<false>(r, nrows)) {
     const int warps = (c->max_T + 119) / 120;
-    launch_after(vec4, dim3((warps + PT / 32 - 1) / (PT / 32), p.batch), dim3(PT), st, a);
+    launch_after(vec4, dim3((warps + PV_THREADS / 32 - 1) / (PV_THREADS / 32), p.batch), dim3(PV_THREADS), st, a);
   } else {
     launch_after(pool_group_kernel, dim3((c->max_T + PT - 1) / PT, p.batch), dim3(PT + 2 * MAX_HALO), st, a);
   }
