@@ -20,8 +20,8 @@
 // a CTA does its runs of pass 1 of group i, then those of pass 2 of group i - 1: it
 // meets one or two segments at a time and keeps a Q chunk for a whole run, and the
 // offsets that pass 2 needs were folded while other tiles were worked on.  Between the two
-// reads of a tile lie up to two groups (up to 70 MB each): of 134 MB of K (64K tokens, 8 kv
-// heads) pass 2 finds 60 % in L2, of 268 MB 40 %.  Dealing every segment's tiles round-robin
+// reads of a tile lie up to two groups (up to 140 MB each), so that of more than 134 MB of K (64K
+// tokens, 8 kv heads) pass 2 finds less than half in L2.  Dealing every segment's tiles round-robin
 // to all CTAs cost 3 us per segment and pass (64 KB of Q reloaded per CTA, a hand-off each):
 // 32K tokens, 8 kv heads 64 -> 48 us, eight ragged requests with W = 32 350 -> 184 us,
 // W = 128 with 64 query heads at 64K 374 -> 288 us, 128K tokens 163 -> 153 us.
@@ -1332,16 +1332,15 @@ bool asl_tc_plan(asl_ctx* c) {
   if (tiles >= (int64_t)1 << 30) return false;
 
   // Groups of segments: pass 1 of a group, then pass 2 of the one before it, so that the fold of the row denominators is
-  // hidden behind other tiles; at least two of them, of up to 70 MB of K each.  (One, where no CTA of
+  // hidden behind other tiles; at least two of them, of up to 140 MB of K each.  (One, where no CTA of
   // any call has more than one tile of a pass: there is then nothing to hide the fold behind, and it is waited for once
   // instead of twice.  In us with two groups and one: 1500 tokens of 8 kv heads 21.2, 15.8, 4096 of 2 heads 13.9, 11.6.  It
   // would pay up to 1.3 tiles a CTA, 3000 tokens 19.6, 16.7, but asl_score_layer and its halves then add in different
   // orders; at 2.5 tiles not, 6000 tokens 19.0, 21.4.)  Small groups leave more of K in L2 for pass 2
-  // (above), large ones need fewer hand-offs, and the hand-offs count for more.  In us at 36, 50, 70, 100, 140 and 270 MB:
-  // four layers of 100K tokens 668, 670, 642, 645, 640, 640; of 128K 843, 843, 841, 843, 845, 834; of 192K 1236, 1240, 1241,
-  // 1243, 1232, 1218; two layers of eight ragged requests 616, 599, 602, 602, 592, 582; two with W = 128 and 64 query heads
-  // at 64K 761, 758, 760, 768, 760, 762.  So the limit is above the step at 100K tokens (25.6 MB a kv head: two in a group),
-  // but not where batches are fastest.
+  // (above), large ones need fewer hand-offs, and the hand-offs count for more.  In us at 36, 50, 70, 100, 140 and 270 MB,
+  // passes issued back to back: four layers of 128K tokens 835, 836, 827, 834, 819, 824; of 100K 667, 657, 636, 638, 630, 631;
+  // of 64K 448, 447, 438, 441, 441, 439; two of eight ragged requests 587, 555, 579, 569, 562, 559; two with W = 128 and 64
+  // query heads at 64K 769, 760, 774, 760, 769, 771; three with FP8 keys at 48K 238, 240, 239, 236, 238, 237.
   const int given = p.score_ctas > 0 && p.score_ctas < c->sm_count ? p.score_ctas : 0;
   std::vector<int> cut{0};
   {
@@ -1350,7 +1349,7 @@ bool asl_tc_plan(asl_ctx* c) {
     int groups = 1;
     for (int s = 0; s < tp.nseg; ++s) {
       total += seg_bytes(s);
-      if (run > 0 && run + seg_bytes(s) > 70.0e6) { ++groups; run = 0; }
+      if (run > 0 && run + seg_bytes(s) > 140.0e6) { ++groups; run = 0; }
       run += seg_bytes(s);
     }
     if (groups < 2 && tiles > (given ? given : c->sm_count - 32)) groups = 2;
