@@ -63,3 +63,24 @@ def test_many_requests_in_several_groups(ctas):
     assert_scores_close(path.scores_kv.cpu().numpy(), P_ref, "scores_kv")
     assert B.asl_device_status(path.ctx) == (B.ASL_OK, 0)
     path.close()
+
+
+@pytest.mark.parametrize("ctas,n", [(8, 512), (8, 513), (0, 7424), (0, 7425), (0, 33)])
+def test_one_group_of_segments_where_a_cta_has_one_tile(ctas, n):
+    """The last length with a single group and the first with two (two kv heads: 8 tiles for 8 CTAs, 116 for the smallest
+    grid of a B200).  Other inputs in every call: an offset of the call before last, in whose set a call counts, shows."""
+    wl = I.workload("C1", seqlens=(n,), budgets=(32,), layers=1, l_min=1, l_obs=2)
+    path = make_path(wl, score_ctas=ctas)
+    for seed in range(5):
+        x = I.layer_inputs(wl, 0, seed=seed)
+        q, k = to_dev(x["q_obs"]), to_dev(x["k"])
+        if seed & 1:
+            B.asl_score_columns(path.ctx, q, k, None, path.workspace, path.ws_bytes, 0)
+            B.asl_pool_scores(path.ctx, path.workspace, path.ws_bytes, 0, path.scores_kv, path.scores_agg)
+        else:
+            B.asl_score_layer(path.ctx, q, k, path.scores_kv, path.scores_agg, path.workspace, path.ws_bytes)
+        torch.cuda.synchronize()
+        P_ref, _ = oracle_layer(wl, x)
+        assert_scores_close(path.scores_kv.cpu().numpy(), P_ref, f"scores_kv, inputs {seed}")
+    assert B.asl_device_status(path.ctx) == (B.ASL_OK, 0)
+    path.close()
