@@ -176,7 +176,10 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
   __shared__ int digit_off[256];
   pdl_release_successor();
   const int b = blockIdx.y, blk = blockIdx.x;
-  if (latch && latch[b].selected) return;
+  if (latch && latch[b].selected) {                    // (waits, as every request may be final: the tables are still being cleared)
+    pdl_wait_predecessor();
+    return;
+  }
   const AslReq rq = req[b];
   const int start = blk * TILE;
   if (start >= rq.T) return;
