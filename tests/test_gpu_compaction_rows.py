@@ -1,4 +1,4 @@
-"""GPU parity of K/V compaction at row counts around a block's 64, bf16 and FP8 keys."""
+"""GPU parity of K/V compaction at row counts around a block's 64, bf16 and FP8 keys, and of the row gather."""
 import numpy as np
 import pytest
 import torch
@@ -34,4 +34,21 @@ def test_compaction_of_any_number_of_rows(fp8):
             rows = cu[b] + idx[h, at:at + m]
             assert (k_out[h, at:at + m] == x["k"][rows, h]).all() and (v_out[h, at:at + m] == x["v"][rows, h]).all(), (b, h)
         at += m
+    path.close()
+
+
+@pytest.mark.parametrize("row_bytes", [16, 512, 528, 4080, 4096, 4112, 4608, 7168, 8192])
+def test_row_gather_of_rows_around_a_warps_loads(row_bytes):
+    """A warp has eight loads of 512 bytes in flight: rows below, at and above one and eight of them."""
+    w, seqlens, kept = 32, (40, 700, 90), (33, 321, 90)
+    wl = I.workload("C1", window=w, seqlens=seqlens, budgets=kept, layers=1, l_min=1, l_obs=2)
+    path = make_path(wl)
+    rng, cu = np.random.default_rng(row_bytes), wl.cu_seqlens()
+    x = rng.integers(-2**31, 2**31, (wl.total_tokens, row_bytes // 4), dtype=np.int64).astype(np.int32)
+    ids = [np.sort(rng.permutation(n)[:wl.kept(b)]) for b, n in enumerate(seqlens)]
+    out = torch.full((path.sum_kept + 1, row_bytes // 4), 7, dtype=torch.int32, device="cuda")
+    B.asl_compact_rows(path.ctx, torch.from_numpy(x).cuda(), torch.from_numpy(np.concatenate(ids).astype(np.int32)).cuda(), out, row_bytes)
+    got = out.cpu().numpy()
+    assert (got[:-1] == np.concatenate([x[int(cu[b]) + i] for b, i in enumerate(ids)])).all()
+    assert (got[-1] == 7).all()
     path.close()
