@@ -45,6 +45,16 @@ __device__ __forceinline__ uint32_t same_digit(uint32_t* lanes, uint32_t d, bool
   return peers;
 }
 
+// Adds the digits of a warp's valid lanes to the counts of a shared table.
+__device__ __forceinline__ void count_digit(int* counts, uint32_t d, bool valid, int lane) {
+  if (__all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {         // one digit: the adds would serialise
+    const int n = __popc(__ballot_sync(0xffffffffu, valid));
+    if (lane == 0) atomicAdd(counts + d, n);
+  } else if (valid) {
+    atomicAdd(counts + d, 1);
+  }
+}
+
 // The first pass reads the fp32 scores and forms keys on the fly (token index =
 // position); later passes read the (key, index) pairs of the previous pass.
 template <bool FIRST>
@@ -88,16 +98,7 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_hist_first(const float* __r
   load_tile<true>(agg, nullptr, nullptr, rq, start + wid * PER_WARP, lane, key, id);
   __syncthreads();
 #pragma unroll
-  for (int r = 0; r < ROUNDS; ++r) {
-    const bool valid = start + wid * PER_WARP + r * 32 + lane < rq.T;
-    const uint32_t d = key[r] & 255u;
-    if (__all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {       // one digit: the adds would serialise
-      const int n = __popc(__ballot_sync(0xffffffffu, valid));
-      if (lane == 0) atomicAdd(&cnt[d], n);
-    } else if (valid) {
-      atomicAdd(&cnt[d], 1);
-    }
-  }
+  for (int r = 0; r < ROUNDS; ++r) count_digit(cnt, key[r] & 255u, start + wid * PER_WARP + r * 32 + lane < rq.T, lane);
   __syncthreads();
   if (threadIdx.x < 256) hist[row] = cnt[threadIdx.x];
 }
@@ -515,7 +516,8 @@ __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
 //                       bucket in the sorted sample, writes the tile's pairs bucket after bucket, and where each begins
 //   rank_place_kernel   a block takes a few buckets: the pairs that go before them are the sum of their first places over
 //                       the tiles; its own are dealt to bins (two to four of them a pair on average) by where they lie
-//                       between their bucket's splitters, and a pair is compared with those of its bin only
+//                       between their bucket's splitters, and a pair is compared with those of its bin only; where
+//                       pairs crowd into a bucket or a bin, the block sorts them digit by digit (place_by_digits)
 //
 // Neither waits for another block, and the row does not depend on the order in which pairs arrive.  Bound by latency: the
 // first takes 4 to 6 us (the sample's round trip, its sort, 8 to 10 steps of search), the second 7 (three round trips).
@@ -635,7 +637,108 @@ struct PlaceSmem {
   int bin[BINS + 4];
   int first_of[SPLIT_MAX_TILES + 1], from[SPLIT_MAX_TILES];       // the tiles' parts in the buckets, and in their tiles
   int warp_tot[PLACE_THREADS / 32], base;
+  __device__ __forceinline__ int slot_of(int e) const {           // the block's e-th pair, tile after tile
+    int t = 0;
+#pragma unroll
+    for (int h = SPLIT_MAX_TILES / 2; h; h >>= 1) t += first_of[t + h] <= e ? h : 0;
+    return from[t] + (e - first_of[t]);
+  }
 };
+
+// The block's m pairs sorted, whatever they are: stable passes over the 8-bit digits in which they differ, lowest first, to and
+// fro between the pairs' own slots in the tiles and the list; the last one writes the ranks.  For blocks that have no room for
+// their pairs (some row in a thousand), and for bins of more than BIN_MAX pairs (a bucket's ends far apart and the rest nearly
+// alike: the border of two long runs of equal scores, scores on both sides of zero), whose compares grow with their square.
+// One SM's seven passes, 9 to 13 ns a pair, are what a row costs whose tokens, but for the sampled ones, lie in one bucket:
+// 131072 tokens of one value 1.6 s -> 1.3 ms, of random values 5.6 -> 1.7 ms, 5000 of one value 870 -> 66 us.  Rows that the
+// sample stands for do not get here, or with few pairs: 131072 tokens in runs of a dozen values 42 -> 30 us.  (512: with 256
+// the passes take over from compares that are still faster, 65536 tokens in runs 17.8 -> 22.1 us; with 1024 too late, 131072 tokens 50 us.)
+constexpr int BIN_MAX = 512;
+template <int S>
+__device__ __noinline__ void place_by_digits(PlaceSmem<S>& sm, unsigned long long* pairs, unsigned long long* list,
+                                             int32_t* rank_row, int m, int base) {
+  constexpr int THREADS = PLACE_THREADS, W = THREADS / 32, STEPS = 4;
+  uint32_t* const lanes = reinterpret_cast<uint32_t*>(sm.held);             // [W][256], see same_digit
+  uint16_t* const cnt = reinterpret_cast<uint16_t*>(lanes + W * 256);       // [W][256]
+  static_assert(sizeof(sm.held) >= W * 256 * 6 && PlaceSmem<S>::BINS == 8 * 256 && W * 256 == 8 * THREADS, "eight tables of digits, two of warps");
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const uint32_t lt = (1u << lane) - 1u;
+  *reinterpret_cast<int4*>(sm.bin + 4 * tid) = make_int4(0, 0, 0, 0);
+  for (int i = tid; i < W * 256; i += THREADS) lanes[i] = 0;
+  __syncthreads();
+  for (int e0 = 0; e0 < m; e0 += THREADS) {             // every digit's counts: no pass changes them
+    const bool valid = e0 + tid < m;
+    const unsigned long long p = valid ? __ldcg(pairs + sm.slot_of(e0 + tid)) : 0ull;
+#pragma unroll
+    for (int d = 0; d < 8; ++d) count_digit(sm.bin + 256 * d, (uint32_t)(p >> 8 * d) & 255u, valid, lane);
+  }
+  __syncthreads();
+  uint32_t differ = 0;                                  // (pairs are all different: not zero)
+  for (int d = 0; d < 8; ++d)
+    if (!__syncthreads_or(tid < 256 && sm.bin[256 * d + tid] == m)) differ |= 1u << d;
+  bool in_list = false;
+  for (; differ; differ &= differ - 1) {
+    const int d = __ffs(differ) - 1;
+    const bool last = (differ & (differ - 1)) == 0;
+    int* const start = sm.bin + 256 * d;
+    const int c = tid < 256 ? start[tid] : 0;
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) sm.warp_tot[wid] = incl;
+    __syncthreads();
+    const int before = __reduce_add_sync(0xffffffffu, lane < wid ? sm.warp_tot[lane] : 0);
+    if (tid < 256) start[tid] = before + incl - c;
+    for (int c0 = 0; c0 < m; c0 += STEPS * THREADS) {
+      const int w0 = c0 + wid * STEPS * 32 + lane;
+      unsigned long long p[STEPS];
+      uint32_t peers[STEPS];
+#pragma unroll
+      for (int r = 0; r < STEPS; ++r) {
+        const int e = w0 + 32 * r;
+        p[r] = e < m ? __ldcg(in_list ? list + e : pairs + sm.slot_of(e)) : 0ull;
+      }
+      *reinterpret_cast<uint4*>(cnt + 8 * tid) = make_uint4(0u, 0u, 0u, 0u);
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < STEPS; ++r) {
+        const bool valid = w0 + 32 * r < m;
+        const uint32_t v = (uint32_t)(p[r] >> 8 * d) & 255u;
+        peers[r] = same_digit(lanes + 256 * wid, v, valid, lane);
+        if (valid && (peers[r] & lt) == 0) cnt[256 * wid + v] += (uint16_t)__popc(peers[r]);
+        __syncwarp();
+      }
+      __syncthreads();
+      int total = 0;
+      if (tid < 256) {
+        uint16_t of[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) of[w] = cnt[256 * w + tid];
+#pragma unroll
+        for (int w = 0; w < W; ++w) { cnt[256 * w + tid] = (uint16_t)total; total += of[w]; }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < STEPS; ++r) {
+        const bool valid = w0 + 32 * r < m;
+        const uint32_t v = (uint32_t)(p[r] >> 8 * d) & 255u;
+        const int pos = start[v] + cnt[256 * wid + v] + __popc(peers[r] & lt);
+        __syncwarp();
+        if (valid && (peers[r] & lt) == 0) cnt[256 * wid + v] += (uint16_t)__popc(peers[r]);
+        __syncwarp();
+        if (valid && last) rank_row[(int)(uint32_t)p[r]] = base + pos;
+        else if (valid) *(in_list ? pairs + sm.slot_of(pos) : list + pos) = p[r];
+      }
+      __syncthreads();
+      if (tid < 256) start[tid] += total;
+    }
+    in_list = !in_list;
+    __syncthreads();
+  }
+}
 
 template <int S>
 __global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_kernel(RowArgs a) {
@@ -692,12 +795,6 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_k
   const int m = sm.first_of[SPLIT_MAX_TILES], base = sm.base;
   if (m == 0) return;
   const unsigned long long* const pairs = a.pairs + rq.u_off;
-  auto pair_at = [&](int e) {                          // the block's e-th pair, tile after tile
-    int t = 0;
-#pragma unroll
-    for (int h = SPLIT_MAX_TILES / 2; h; h >>= 1) t += sm.first_of[t + h] <= e ? h : 0;
-    return __ldcg(pairs + sm.from[t] + (e - sm.first_of[t]));
-  };
   auto bucket_of = [&](unsigned long long pair) {
     int g = 0;
     for (int h = group / 2; h; h >>= 1) g += pair >= sm.split[g + h] ? h : 0;
@@ -708,15 +805,14 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_k
     const unsigned long long least = sm.least[g];
     return g * own + (pair > least ? min(own - 1, (int)(__ull2float_rz(pair - least) * sm.scale[g])) : 0);
   };
-  auto put = [&](unsigned long long pair, int rank) { a.rank_row[rq.t_off + (int)(uint32_t)pair] = rank; };
-  const bool fits = m <= HELD;
   unsigned long long pair[PER];
   // a pair's place among those of its bin, in the order of arrival; then where the bins begin
   uint32_t at[PER];                              // bin << 16 | place
-  if (fits) {
+  bool sort = m > HELD;
+  if (!sort) {
 #pragma unroll
     for (int r = 0; r < PER; ++r)
-      if (r * THREADS < m) pair[r] = pair_at(min(r * THREADS + tid, m - 1));
+      if (r * THREADS < m) pair[r] = __ldcg(pairs + sm.slot_of(min(r * THREADS + tid, m - 1)));
     if (b0 == 0 || b0 + group == S) {                  // the segment's first pair, or its last one, is the bound that lacks
       unsigned long long end = pair[0];
 #pragma unroll
@@ -741,27 +837,15 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_k
 #pragma unroll
     for (int r = 0; r < PER; ++r)
       if (r * THREADS + tid < m) {
-        const int q = bin_of(pair[r]);
-        at[r] = (uint32_t)q << 16 | (uint32_t)atomicAdd(&sm.bin[q], 1);
+        const int q = bin_of(pair[r]), place = atomicAdd(&sm.bin[q], 1);
+        at[r] = (uint32_t)q << 16 | (uint32_t)place;
+        sort |= place >= BIN_MAX;
       }
-  } else {
-    // buckets that do not fit (some row in ten thousand has such, or one whose sampled scores are unlike the others): the
-    // same through global memory, the bins between the smallest and the largest pair that each bucket really has
-    __syncthreads();
-    if (tid < group) { sm.least[tid] = ~0ull; sm.most[tid] = 0ull; }
-    __syncthreads();
-    for (int e = tid; e < m; e += THREADS) {
-      const unsigned long long p = pair_at(e);
-      const int g = bucket_of(p);
-      if (p < *(volatile unsigned long long*)&sm.least[g]) atomicMin(&sm.least[g], p);
-      if (p > *(volatile unsigned long long*)&sm.most[g]) atomicMax(&sm.most[g], p);
-    }
-    __syncthreads();
-    if (tid < group) sm.scale[tid] = (float)own / __ull2float_rz(max(1ull, sm.most[tid] - sm.least[tid]));     // (an empty bucket's is not used)
-    __syncthreads();
-    for (int e = tid; e < m; e += THREADS) atomicAdd(&sm.bin[bin_of(pair_at(e))], 1);
   }
-  __syncthreads();
+  if (__syncthreads_or(sort)) {
+    place_by_digits(sm, a.pairs + rq.u_off, a.list + rq.u_off + base, a.rank_row + rq.t_off, m, base);
+    return;
+  }
   {
     const int4 c = *reinterpret_cast<int4*>(sm.bin + 4 * tid);
     const int mine = c.x + c.y + c.z + c.w;
@@ -780,37 +864,19 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_k
     if (tid == THREADS - 1) sm.bin[BINS] = m;
   }
   __syncthreads();
-  if (fits) {
 #pragma unroll
-    for (int r = 0; r < PER; ++r)
-      if (r * THREADS + tid < m) sm.held[sm.bin[at[r] >> 16] + (int)(at[r] & 0xffffu)] = pair[r];
-    __syncthreads();
+  for (int r = 0; r < PER; ++r)
+    if (r * THREADS + tid < m) sm.held[sm.bin[at[r] >> 16] + (int)(at[r] & 0xffffu)] = pair[r];
+  __syncthreads();
 #pragma unroll
-    for (int r = 0; r < PER; ++r)
-      if (r * THREADS + tid < m) {
-        const int q = (int)(at[r] >> 16), begin = sm.bin[q], end = sm.bin[q + 1];
-        int rank = base + begin;
-#pragma unroll 4
-        for (int i = begin; i < end; ++i) rank += sm.held[i] < pair[r] ? 1 : 0;
-        put(pair[r], rank);
-      }
-  } else {
-    // `bin` becomes the bins' ends as the pairs arrive
-    unsigned long long* const list = a.list + rq.u_off + base;
-    for (int e = tid; e < m; e += THREADS) {
-      const unsigned long long p = pair_at(e);
-      list[atomicAdd(&sm.bin[bin_of(p)], 1)] = p;
-    }
-    __syncthreads();
-    for (int e = tid; e < m; e += THREADS) {
-      const unsigned long long p = list[e];
-      const int q = bin_of(p), begin = q ? sm.bin[q - 1] : 0, end = sm.bin[q];
+  for (int r = 0; r < PER; ++r)
+    if (r * THREADS + tid < m) {
+      const int q = (int)(at[r] >> 16), begin = sm.bin[q], end = sm.bin[q + 1];
       int rank = base + begin;
 #pragma unroll 4
-      for (int i = begin; i < end; ++i) rank += list[i] < p ? 1 : 0;
-      put(p, rank);
+      for (int i = begin; i < end; ++i) rank += sm.held[i] < pair[r] ? 1 : 0;
+      a.rank_row[rq.t_off + (int)(uint32_t)pair[r]] = rank;
     }
-  }
 }
 
 template <int S>

@@ -69,3 +69,48 @@ def test_row_and_statistic_of_a_plan(lengths):
                 num, m, _ = O.rank_statistic(np.stack([r[b] for r in ranks[-min(layer + 1, rows):]]), T // 9)
                 assert (stat[b]["num"], stat[b]["m"]) == (num, m)
     path.close()
+
+
+@pytest.mark.parametrize("kind", ["one bucket", "one bucket, equal", "across zero"])
+def test_blocks_whose_pairs_crowd_into_one_bin(kind):
+    """Requests whose tokens, but for the 512 sampled ones, fall into one bucket: around the most pairs that a bin compares
+    with one another (512), the pairs of a step of the passes that sort longer ones (2048) and those that a block holds (4096)."""
+    lengths = (960, 1023, 1024, 1025, 1087, 2495, 2496, 2559, 2560, 2561, 4544, 4607, 4608, 4609, 4700, 40000)
+    w, S, rng = 32, 512, np.random.default_rng(5)
+    wl = I.workload("C1", seqlens=tuple(T + w for T in lengths), budgets=tuple(w + T // 9 for T in lengths), l_min=1, l_obs=2)
+    path = make_path(wl)
+    scores = []
+    for T in lengths:
+        i = np.arange(S, dtype=np.int64)
+        lo, hi = i * T // S, (i + 1) * T // S
+        at = np.minimum(T - 1, lo + ((i * 2654435761) % 2**32 >> 8) % np.maximum(1, hi - lo))
+        s = {"one bucket": rng.random(T), "one bucket, equal": np.full(T, 0.5), "across zero": 1e-30 * rng.standard_normal(T)}[kind]
+        s[at] = np.where(rng.random(S) < 0.5, 2.0, -2.0 if kind == "across zero" else 2.0) * (1 + rng.random(S))
+        scores.append(s.astype(np.float32))
+    path.scores_agg.copy_(torch.from_numpy(np.concatenate(scores)))
+    for layer in range(2):
+        B.asl_rank_stat(path.ctx, path.scores_agg, layer, layer + 1, path.rank_ring, path.stat, path.workspace, path.ws_bytes)
+    got, at, stat = path.rank_ring.cpu().numpy(), 0, path.read_stat()
+    for b, T in enumerate(lengths):
+        row = O.rank_desc(scores[b].astype(np.float64))
+        assert (got[:, at:at + T] == row).all(), b
+        num, m, _ = O.rank_statistic(np.stack([row, row]), T // 9)
+        assert (stat[b]["num"], stat[b]["m"]) == (num, m)
+        at += T
+    path.close()
+
+
+@pytest.mark.parametrize("T", [5119, 32768, 131072, 262144])
+def test_time_of_a_row_in_one_bucket_grows_with_its_length(T):
+    """At most 300 us and 30 ns a token, two to three times what one block's passes take (9 to 13 ns a token); comparing a
+    bucket's pairs with one another took 0.9 ms at 5000 tokens of one value and 1.6 s at 131072, 5.6 ms of random ones."""
+    rng = np.random.default_rng(T)
+    for kind in ("one bucket", "one bucket, equal"):
+        s, out = torch.from_numpy(_scores(T, kind, rng)).cuda(), torch.empty(T, dtype=torch.int32, device="cuda")
+        B.asl_rank_desc_static(s, T, out)
+        begin, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        begin.record()
+        B.asl_rank_desc_static(s, T, out)
+        end.record()
+        torch.cuda.synchronize()
+        assert begin.elapsed_time(end) < 0.3 + 30e-6 * T, kind
