@@ -637,6 +637,14 @@ struct PlaceSmem {
   int bin[BINS + 4];
   int first_of[SPLIT_MAX_TILES + 1], from[SPLIT_MAX_TILES];       // the tiles' parts in the buckets, and in their tiles
   int warp_tot[PLACE_THREADS / 32], base;
+  // buckets of a block: as many (a power of two) as give a block a sixth of the pairs that it can hold, so that nearly every
+  // block has room for its own (eight ragged requests, blocks of four buckets whatever their lengths: 39 us, not 31); fewer
+  // of a longer request, so that the longest one says how many blocks a request may need
+  __host__ __device__ static int group_of(int T) {
+    int group = MIN_GROUP;
+    while (group < MAX_GROUP && (long long)T * group * 2 <= (long long)S * (HELD / 6)) group *= 2;
+    return group;
+  }
   __device__ __forceinline__ int slot_of(int e) const {           // the block's e-th pair, tile after tile
     int t = 0;
 #pragma unroll
@@ -752,10 +760,7 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_k
   pdl_wait_predecessor();
   if (row_is_final(a, b)) return;
   const int tiles = (rq.T + TILE_N - 1) / TILE_N;
-  // buckets of a block: as many (a power of two) as give a block a sixth of the pairs that it can hold, so that nearly every
-  // block has room for its own (eight ragged requests, blocks of four buckets whatever their lengths: 39 us, not 31)
-  int group = M::MIN_GROUP;
-  while (group < M::MAX_GROUP && (long long)rq.T * group * 2 <= (long long)S * (HELD / 6)) group *= 2;
+  const int group = M::group_of(rq.T);
   const int b0 = blockIdx.x * group, own = BINS / group;
   if (b0 >= S) return;
   *reinterpret_cast<int4*>(sm.bin + 4 * tid) = make_int4(0, 0, 0, 0);
@@ -889,7 +894,7 @@ void launch_split_of(RowArgs r, int max_T, int batch, cudaStream_t st) {
   r.max_tiles = (max_T + 4 * S - 1) / (4 * S);
   r.table = reinterpret_cast<uint16_t*>(r.splitters + (size_t)batch * S);
   launch_after_smem(rank_split_kernel<S>, dim3(r.max_tiles, batch), dim3(S), split_smem_bytes<S>(), st, r);
-  launch_after_smem(rank_place_kernel<S>, dim3(S / PlaceSmem<S>::MIN_GROUP, batch), dim3(PLACE_THREADS), sizeof(PlaceSmem<S>), st, r);
+  launch_after_smem(rank_place_kernel<S>, dim3(S / PlaceSmem<S>::group_of(max_T), batch), dim3(PLACE_THREADS), sizeof(PlaceSmem<S>), st, r);
 }
 
 // Buckets of up to 128 pairs on average to 32K tokens, 256 above.  (A block of one bucket each, bins between its smallest and
