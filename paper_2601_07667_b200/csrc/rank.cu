@@ -3,7 +3,7 @@
 //
 // RankDesc: position of every (key, token index) pair in sorted order per request, key = bit pattern that ascends as the
 // score descends; equal scores keep ascending index order, so the position is the token's 0-based rank with ties to the
-// lower index.  Single segments of up to 4096 tokens: every token counts those before it.  Up to 256K tokens: split at
+// lower index.  Segments of up to 4096 tokens, single ones or few: every token counts those before it.  Up to 256K tokens: split at
 // sampled pairs, then placed bucket by bucket (below).  Longer ones: a stable least-significant-digit radix sort (8-bit
 // digits, one kernel per digit after a first histogram); the last pass scatters positions straight into the ring row.
 //
@@ -425,33 +425,42 @@ __device__ __forceinline__ AslReq row_request(const RowArgs& a, int b) {
 __device__ __forceinline__ bool row_is_final(const RowArgs& a, int b) { return a.req && a.stat.latch && a.stat.stat[b].selected; }
 
 // ---------------------------------------------------------------------------
-// One segment of up to COUNT_MAX_T tokens: a token's rank is the number of tokens that go before it, counted outright.
-// A block takes 32 tokens, one per lane; its warps share the others, which lie in shared memory (a broadcast load per
+// Segments of up to COUNT_MAX_T tokens: a token's rank is the number of tokens that go before it, counted outright.  A block
+// takes 32 tokens a group, one per lane; a group's warps share the others, which lie in shared memory (a broadcast load per
 // four).  The statistic of the block's tokens goes with them: one launch.  T^2 compares are 2 us of the whole GPU at 4096
 // tokens; bound by the launch and three round trips.  4096 scores: 14.3 us by one block's radix sort, a chain of shared-
-// memory passes, -> 7.4 us.  Not for batches, whose compares add up, and not above: at 8192 tokens the compares alone are
-// 8 us, and eight times that beside a scorer.
+// memory passes, -> 4.7 us.  Not above: at 8192 tokens the compares alone are 8 us, and eight times that beside a scorer.
+// Batches as long as their squares are few (count_takes): blocks of four groups, since a block's fixed costs count where
+// many requests share the GPU, and more so on the SMs that a scorer leaves.  Rank statistic in us, counted / split:
+// 2 of 500 tokens 5.9 / 9.7, 8 of 500 6.6 / 10.8, 16 of 500 6.6 / 10.9, 4 of 1000 7.7 / 10.7; a layer of them (32q/8kv)
+// 2 of 500 28.3 / 28.5, 4 of 1000 35.4 / 36.9; past the line 8 of 1000 7.8 / 11.1 but the layer 48.6 / 45.9, 8 of 2000 57.5 / 53.7.
 // ---------------------------------------------------------------------------
 constexpr int COUNT_MAX_T = 4096;
+constexpr int64_t COUNT_BATCH_PAIRS = 1 << 22;
 constexpr int COUNT_THREADS = 1024;
 constexpr int COUNT_WARPS = COUNT_THREADS / 32;
 
+template <int GROUPS>
 __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
   __shared__ __align__(16) uint32_t keys[COUNT_MAX_T];
   __shared__ int part[COUNT_WARPS][32];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  __shared__ unsigned long long s_num[GROUPS];
+  __shared__ int s_m[GROUPS];
+  constexpr int SHARE = COUNT_WARPS / GROUPS;
+  const int b = GROUPS > 1 ? blockIdx.y : 0, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;     // (one group: one segment)
   pdl_wait_predecessor();
-  const bool open = !row_is_final(a, 0);
-  const AslReq rq = row_request(a, 0);
+  const bool open = !row_is_final(a, b);
+  const AslReq rq = row_request(a, b);
   const int T = rq.T, padded = (T + 127) & ~127;                     // padding goes before nothing
   unsigned long long num = 0;
   int m = 0;
-  if (open) {
-    const int i0 = blockIdx.x * 32, i = i0 + lane;
+  const int group = wid / SHARE, first = blockIdx.x * 32 * GROUPS, i0 = first + 32 * group, i = i0 + lane;
+  const bool leads = wid % SHARE == 0;                               // its group's warp that closes the tokens
+  if (open && (GROUPS == 1 || first < T)) {
     // the earlier rows' ranks of the block's tokens, on their way while it counts
     long long s1 = 0, s2 = 0;
     int mn = 0x7fffffff;
-    if (wid == 0 && a.evaluate) {
+    if (leads && a.evaluate) {
       for (int r0 = 0; r0 < a.stat.n_rows - 1; r0 += 8) {
         int v[8];
 #pragma unroll
@@ -471,7 +480,7 @@ __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
     }
     __syncthreads();
     const uint32_t key = keys[min(i, padded - 1)];
-    const int per = padded / COUNT_WARPS, j0 = wid * per, j1 = j0 + per;        // (a multiple of four)
+    const int per = padded / SHARE, j0 = wid % SHARE * per, j1 = j0 + per;        // (a multiple of four)
     int before = 0;
     for (int j = j0; j < min(j1, i0); j += 4) {                       // earlier tokens go first among equals
       const uint4 k = *reinterpret_cast<const uint4*>(keys + j);
@@ -484,10 +493,10 @@ __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
     }
     part[wid][lane] = before;
     __syncthreads();
-    if (wid == 0) {
+    if (leads) {
       int rank = 0;
 #pragma unroll
-      for (int w = 0; w < COUNT_WARPS; ++w) rank += part[w][lane];
+      for (int w = 0; w < SHARE; ++w) rank += part[wid + w][lane];
       if (i < T) {
         a.rank_row[rq.t_off + i] = rank;
         mn = min(mn, rank);
@@ -504,8 +513,14 @@ __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
         m += __shfl_down_sync(0xffffffffu, m, o);
       }
     }
+    if (GROUPS > 1) {
+      if (leads && lane == 0) { s_num[group] = num; s_m[group] = m; }
+      __syncthreads();
+      if (tid == 0)
+        for (int g = 1; g < GROUPS; ++g) { num += s_num[g]; m += s_m[g]; }
+    }
   }
-  if (a.req) stat_close(a.stat, 0, num, m, a.evaluate);
+  if (a.req) stat_close(a.stat, b, num, m, a.evaluate);
 }
 
 // ---------------------------------------------------------------------------
@@ -887,7 +902,15 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_k
 template <int S>
 constexpr int split_smem_bytes() { return (int)(5 * S * sizeof(unsigned long long) + S * sizeof(int)); }
 
-void launch_count(const RowArgs& r, int T, cudaStream_t st) { launch_after(rank_count_kernel, dim3((T + 31) / 32), dim3(COUNT_THREADS), st, r); }
+template <int GROUPS>
+void launch_count_of(const RowArgs& r, int max_T, int batch, cudaStream_t st) {
+  launch_after(rank_count_kernel<GROUPS>, dim3((max_T + 32 * GROUPS - 1) / (32 * GROUPS), batch), dim3(COUNT_THREADS), st, r);
+}
+bool count_takes(int max_T, int batch) { return max_T <= COUNT_MAX_T && (batch == 1 || (int64_t)batch * max_T * max_T <= COUNT_BATCH_PAIRS); }
+void launch_count(const RowArgs& r, int max_T, int batch, cudaStream_t st) {
+  if (batch == 1) launch_count_of<1>(r, max_T, batch, st);
+  else launch_count_of<4>(r, max_T, batch, st);
+}
 
 template <int S>
 void launch_split_of(RowArgs r, int max_T, int batch, cudaStream_t st) {
@@ -931,8 +954,8 @@ asl_status asl_launch_rank(asl_ctx* c, const float* agg, int32_t layer_idx, int3
                    latch ? 1 : 0, p.tau};
   RowArgs r{agg, row, c->d_req, 0, reinterpret_cast<unsigned long long*>(keys[0]), reinterpret_cast<unsigned long long*>(idx[0]),
             reinterpret_cast<unsigned long long*>(hist), nullptr, 0, a, evaluate};
-  if (p.batch == 1 && c->max_T <= COUNT_MAX_T) {         // the statistic goes with the row
-    launch_count(r, c->max_T, st);
+  if (count_takes(c->max_T, p.batch)) {         // the statistic goes with the row
+    launch_count(r, c->max_T, p.batch, st);
     c->launches += 1;
     ASL_CUDA(cudaGetLastError());
     return ASL_OK;
@@ -1024,7 +1047,7 @@ extern "C" asl_status asl_rank_desc_static(const float* scores, int32_t T, int32
   if (ready != ASL_OK) return ready;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const RowArgs r{scores, rank_out, nullptr, T, s->pairs, s->list, s->table, nullptr, 0, StatArgs{}, 0};
-  if (T <= COUNT_MAX_T) launch_count(r, T, st);
+  if (count_takes(T, 1)) launch_count(r, T, 1, st);
   else launch_split(r, T, 1, st);
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;

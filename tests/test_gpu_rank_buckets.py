@@ -114,3 +114,37 @@ def test_time_of_a_row_in_one_bucket_grows_with_its_length(T):
         end.record()
         torch.cuda.synchronize()
         assert begin.elapsed_time(end) < 0.3 + 30e-6 * T, kind
+
+
+@pytest.mark.parametrize("lengths", [(1, 33), (500, 97) * 4, (129, 1, 128, 127, 900), (1448, 1447), (1449, 1448), (32,) * 9])
+def test_short_requests_of_a_batch_take_one_launch(lengths):
+    """Counted rows with their statistic up to 2^22 compares by the longest request's square, split ones above; a request
+    whose selection is final keeps its rank row and its record."""
+    w, rows, n = 32, 3, len(lengths)
+    wl = I.workload("C1", seqlens=tuple(T + w for T in lengths), budgets=tuple(w + T // 9 for T in lengths), l_min=1, l_obs=rows)
+    path = make_path(wl)
+    path.set_controller(B.ASL_CONTROLLER_LATCH)
+    rng, ranks = np.random.default_rng(sum(lengths)), []
+    selected_word = B.STAT_DTYPE.fields["selected"][1] // 4
+    for layer in range(rows + 1):
+        per = [_scores(T, KINDS[layer % 4], rng) for T in lengths]
+        path.scores_agg.copy_(torch.from_numpy(np.concatenate(per)))
+        if layer == rows:
+            path.stat.view(torch.int32)[n - 1, selected_word] = 1
+        before, ring, launches = path.read_stat().copy(), path.rank_ring[layer % rows].cpu().numpy(), B.asl_launch_count(path.ctx)
+        B.asl_rank_stat(path.ctx, path.scores_agg, layer, min(layer + 1, rows), path.rank_ring, path.stat, path.workspace, path.ws_bytes)
+        assert B.asl_launch_count(path.ctx) - launches == (1 if n * max(lengths) ** 2 <= 2**22 else 3)
+        ranks.append([O.rank_desc(s.astype(np.float64)) for s in per])
+        got, at, stat = path.rank_ring[layer % rows].cpu().numpy(), 0, path.read_stat()
+        for b, T in enumerate(lengths):
+            here = slice(at, at + T)
+            at += T
+            if before[b]["selected"]:
+                ranks[-1][b] = ring[here]
+                assert (got[here] == ring[here]).all() and stat[b].tobytes() == before[b].tobytes()
+                continue
+            assert (got[here] == ranks[-1][b]).all(), (layer, b)
+            if layer >= 1:
+                num, m, _ = O.rank_statistic(np.stack([r[b] for r in ranks[-min(layer + 1, rows):]]), T // 9)
+                assert (stat[b]["num"], stat[b]["m"], stat[b]["layer_idx"]) == (num, m, layer)
+    path.close()
