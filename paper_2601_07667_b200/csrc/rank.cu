@@ -56,7 +56,8 @@ __device__ __forceinline__ void count_digit(int* counts, uint32_t d, bool valid,
 }
 
 // The first pass reads the fp32 scores and forms keys on the fly (token index =
-// position); later passes read the (key, index) pairs of the previous pass.
+// position); later passes read the (key, index) pairs of the previous pass, which may
+// still be running when their blocks become resident: coherent loads, behind the wait.
 template <bool FIRST>
 __device__ __forceinline__ void load_tile(const float* __restrict__ agg, const uint32_t* __restrict__ keys_in,
                                           const int32_t* __restrict__ idx_in, const AslReq& rq, int wstart, int lane,
@@ -68,7 +69,7 @@ __device__ __forceinline__ void load_tile(const float* __restrict__ agg, const u
     id[r] = i;
     if (i < rq.T) {
       if (FIRST) key[r] = desc_key(agg[rq.t_off + i]);
-      else { key[r] = keys_in[rq.t_off + i]; id[r] = idx_in[rq.t_off + i]; }
+      else { key[r] = __ldcg(keys_in + rq.t_off + i); id[r] = __ldcg(idx_in + rq.t_off + i); }
     }
   }
 }
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(SORT_THREADS) rank_scatter(const float* __rest
   if (!FIRST) pdl_wait_predecessor();
   load_tile<FIRST>(agg, keys_in, idx_in, rq, wstart, lane, key, id);
   if (FIRST) pdl_wait_predecessor();
-  digit_off[threadIdx.x] = counts[((int64_t)b * nblk + blk) * 256 + threadIdx.x];
+  digit_off[threadIdx.x] = __ldcg(counts + ((int64_t)b * nblk + blk) * 256 + threadIdx.x);
   for (int i = threadIdx.x; i < WARPS * 256; i += SORT_THREADS) { (&cnt[0][0])[i] = 0; (&lanes[0][0])[i] = 0; }
   __syncthreads();
   // per-warp digit counts; the peer masks are kept for the second walk

@@ -79,3 +79,37 @@ def test_select_compact_and_rank_chains(T, how):
     stat = path.read_stat()[0]
     assert (stat["num"], stat["m"]) == (num, m)
     path.close()
+
+
+@pytest.mark.parametrize("how", ["calls", "graph"])
+@pytest.mark.parametrize("lengths", [(300,), (500, 33, 499), (40000, 700), (262145, 5000), (300000, 262200)])
+def test_rank_rows_with_nothing_in_between(lengths, how):
+    """Rank rows of several layers issued back to back over scores that lie ready, so that every kernel of the row follows
+    another of the library's: counted, split and radix rows (whose passes read what the kernel just before has written)."""
+    w, rounds = 32, 5
+    wl = I.workload("C1", seqlens=tuple(T + w for T in lengths), budgets=tuple(w + T // 9 for T in lengths), l_min=0, l_obs=rounds)
+    path = make_path(wl)
+    g = torch.Generator(device="cuda").manual_seed(len(lengths) + lengths[0])
+    scores = torch.randn((rounds, path.sum_T), generator=g, device="cuda")
+
+    def chain():
+        for r in range(rounds):
+            B.asl_rank_stat(path.ctx, scores[r], r, r + 1, path.rank_ring, path.stat, path.workspace, path.ws_bytes)
+
+    chain()
+    if how == "graph":
+        torch.cuda.synchronize()
+        path.rank_ring.fill_(-1)
+        path.stat.zero_()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            chain()
+        graph.replay()
+    got, s, stat, at = path.rank_ring.cpu().numpy(), scores.cpu().numpy().astype(np.float64), path.read_stat(), 0
+    for b, T in enumerate(lengths):
+        ranks = np.stack([O.rank_desc(s[r, at:at + T]) for r in range(rounds)])
+        assert (got[:, at:at + T] == ranks).all(), b
+        num, m, _ = O.rank_statistic(ranks, T // 9)
+        assert (stat[b]["num"], stat[b]["m"]) == (num, m)
+        at += T
+    path.close()
