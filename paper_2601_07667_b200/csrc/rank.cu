@@ -3,9 +3,10 @@
 //
 // RankDesc: position of every (key, token index) pair in sorted order per request, key = bit pattern that ascends as the
 // score descends; equal scores keep ascending index order, so the position is the token's 0-based rank with ties to the
-// lower index.  Segments of up to 4096 tokens, single ones or few: every token counts those before it.  Up to 256K tokens: split at
-// sampled pairs, then placed bucket by bucket (below).  Longer ones: a stable least-significant-digit radix sort (8-bit
-// digits, one kernel per digit after a first histogram); the last pass scatters positions straight into the ring row.
+// lower index.  One segment of up to 4096 tokens: every token counts those before it.  Batches of short ones: a block sorts
+// a segment (sort_takes).  Up to 256K tokens: split at sampled pairs, then placed bucket by bucket.  Longer ones: a stable
+// least-significant-digit radix sort (8-bit digits, one kernel per digit after a first histogram); the last pass scatters
+// positions straight into the ring row.
 //
 // Statistic: a token is in the union iff its smallest rank over the rows is < k
 // (the k smallest ranks of a row are exactly ranks 0..k-1).  The numerator
@@ -426,42 +427,33 @@ __device__ __forceinline__ AslReq row_request(const RowArgs& a, int b) {
 __device__ __forceinline__ bool row_is_final(const RowArgs& a, int b) { return a.req && a.stat.latch && a.stat.stat[b].selected; }
 
 // ---------------------------------------------------------------------------
-// Segments of up to COUNT_MAX_T tokens: a token's rank is the number of tokens that go before it, counted outright.  A block
-// takes 32 tokens a group, one per lane; a group's warps share the others, which lie in shared memory (a broadcast load per
+// One segment of up to COUNT_MAX_T tokens: a token's rank is the number of tokens that go before it, counted outright.
+// A block takes 32 tokens, one per lane; its warps share the others, which lie in shared memory (a broadcast load per
 // four).  The statistic of the block's tokens goes with them: one launch.  T^2 compares are 2 us of the whole GPU at 4096
 // tokens; bound by the launch and three round trips.  4096 scores: 14.3 us by one block's radix sort, a chain of shared-
-// memory passes, -> 4.7 us.  Not above: at 8192 tokens the compares alone are 8 us, and eight times that beside a scorer.
-// Batches as long as their squares are few (count_takes): blocks of four groups, since a block's fixed costs count where
-// many requests share the GPU, and more so on the SMs that a scorer leaves.  Rank statistic in us, counted / split:
-// 2 of 500 tokens 5.9 / 9.7, 8 of 500 6.6 / 10.8, 16 of 500 6.6 / 10.9, 4 of 1000 7.7 / 10.7; a layer of them (32q/8kv)
-// 2 of 500 28.3 / 28.5, 4 of 1000 35.4 / 36.9; past the line 8 of 1000 7.8 / 11.1 but the layer 48.6 / 45.9, 8 of 2000 57.5 / 53.7.
+// memory passes, -> 4.7 us.  Not for batches, whose compares add up, and not above: at 8192 tokens the compares alone are
+// 8 us, and eight times that beside a scorer.
 // ---------------------------------------------------------------------------
 constexpr int COUNT_MAX_T = 4096;
-constexpr int64_t COUNT_BATCH_PAIRS = 1 << 22;
 constexpr int COUNT_THREADS = 1024;
 constexpr int COUNT_WARPS = COUNT_THREADS / 32;
 
-template <int GROUPS>
 __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
   __shared__ __align__(16) uint32_t keys[COUNT_MAX_T];
   __shared__ int part[COUNT_WARPS][32];
-  __shared__ unsigned long long s_num[GROUPS];
-  __shared__ int s_m[GROUPS];
-  constexpr int SHARE = COUNT_WARPS / GROUPS;
-  const int b = GROUPS > 1 ? blockIdx.y : 0, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;     // (one group: one segment)
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   pdl_wait_predecessor();
-  const bool open = !row_is_final(a, b);
-  const AslReq rq = row_request(a, b);
+  const bool open = !row_is_final(a, 0);
+  const AslReq rq = row_request(a, 0);
   const int T = rq.T, padded = (T + 127) & ~127;                     // padding goes before nothing
   unsigned long long num = 0;
   int m = 0;
-  const int group = wid / SHARE, first = blockIdx.x * 32 * GROUPS, i0 = first + 32 * group, i = i0 + lane;
-  const bool leads = wid % SHARE == 0;                               // its group's warp that closes the tokens
-  if (open && (GROUPS == 1 || first < T)) {
+  if (open) {
+    const int i0 = blockIdx.x * 32, i = i0 + lane;
     // the earlier rows' ranks of the block's tokens, on their way while it counts
     long long s1 = 0, s2 = 0;
     int mn = 0x7fffffff;
-    if (leads && a.evaluate) {
+    if (wid == 0 && a.evaluate) {
       for (int r0 = 0; r0 < a.stat.n_rows - 1; r0 += 8) {
         int v[8];
 #pragma unroll
@@ -481,7 +473,7 @@ __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
     }
     __syncthreads();
     const uint32_t key = keys[min(i, padded - 1)];
-    const int per = padded / SHARE, j0 = wid % SHARE * per, j1 = j0 + per;        // (a multiple of four)
+    const int per = padded / COUNT_WARPS, j0 = wid * per, j1 = j0 + per;        // (a multiple of four)
     int before = 0;
     for (int j = j0; j < min(j1, i0); j += 4) {                       // earlier tokens go first among equals
       const uint4 k = *reinterpret_cast<const uint4*>(keys + j);
@@ -494,10 +486,10 @@ __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
     }
     part[wid][lane] = before;
     __syncthreads();
-    if (leads) {
+    if (wid == 0) {
       int rank = 0;
 #pragma unroll
-      for (int w = 0; w < SHARE; ++w) rank += part[wid + w][lane];
+      for (int w = 0; w < COUNT_WARPS; ++w) rank += part[w][lane];
       if (i < T) {
         a.rank_row[rq.t_off + i] = rank;
         mn = min(mn, rank);
@@ -514,14 +506,163 @@ __global__ void __launch_bounds__(COUNT_THREADS) rank_count_kernel(RowArgs a) {
         m += __shfl_down_sync(0xffffffffu, m, o);
       }
     }
-    if (GROUPS > 1) {
-      if (leads && lane == 0) { s_num[group] = num; s_m[group] = m; }
+  }
+  if (a.req) stat_close(a.stat, 0, num, m, a.evaluate);
+}
+
+// ---------------------------------------------------------------------------
+// Batches of short segments: a block a request sorts the whole segment in shared memory (four stable passes of 8-bit digits),
+// writes the row and takes the statistic: one launch, which takes as long as one request does while there is an SM for each.
+// Bound by what its rounds issue to shared memory and by five block barriers a pass.
+//
+// The split row (below) ranks a segment sooner, but in three launches, and its blocks add up over a batch: always slower up
+// to 1024 tokens, and above where the requests are many (sort_takes; the fit is within 1 us of the figures up to a wave of
+// requests).  Rank statistic in us, here / split: 8 of 500 tokens 7.9 / 10.8, 128 of 500 8.0 / 16.0, 1000 of 100 45 / 60,
+// 32 of 1000 9.3 / 11.6, 32 of 1500 11.8 / 11.5, 64 of 1500 11.8 / 12.7, 32 of 2000 13.3 / 12.2, 64 of 2000 13.3 / 13.7, 8 of
+// 4096 21.3 / 11.5, 64 of 4096 21.4 / 18.1, 96 of 4096 21.4 / 22.0, 200 of 4096 41.9 / 39.3.  (Counted rows for batches of few
+// compares: 8 of 500 tokens 6.9, but 128 of 500 22, and in a layer, on the SMs that a scorer leaves, never faster: four
+// layers (32q/8kv) of 8 requests of 500 tokens 129 us, here 117, of 4 of 1000 106, here 91.)
+// ---------------------------------------------------------------------------
+constexpr int SORT_MAX_T = 4096;
+constexpr int ROW_THREADS = 1024;
+constexpr int ROW_WARPS = ROW_THREADS / 32;
+
+__host__ __device__ constexpr int sort_smem_bytes(int rounds) {     // per warp: lanes per digit, digit counts; keys, token numbers
+  return rounds * ROW_THREADS * (int)(sizeof(uint32_t) + sizeof(uint16_t)) + ROW_WARPS * 256 * (int)(sizeof(uint16_t) + sizeof(uint32_t));
+}
+bool sort_takes(int max_T, int64_t sum_T, int batch, int sms) {
+  if (batch == 1 || max_T > SORT_MAX_T) return false;
+  const int waves = (batch + sms - 1) / sms;
+  return max_T <= 1024 || waves * (6.7 + 3.5e-3 * max_T) <= 10.3 + 0.028e-3 * (double)sum_T;
+}
+
+template <int R>
+__global__ void __launch_bounds__(ROW_THREADS, 1) rank_sort_kernel(RowArgs a) {
+  constexpr int N = R * ROW_THREADS;
+  extern __shared__ __align__(16) uint8_t sort_raw[];
+  uint32_t (*lanes)[256] = reinterpret_cast<uint32_t (*)[256]>(sort_raw);
+  uint32_t (*cnt2)[128] = reinterpret_cast<uint32_t (*)[128]>(lanes + ROW_WARPS);       // two digits' counts per word
+  uint32_t* s_key = reinterpret_cast<uint32_t*>(cnt2 + ROW_WARPS);
+  uint16_t* s_id = reinterpret_cast<uint16_t*>(s_key + N);
+  __shared__ uint32_t part_sum[8][128];
+  __shared__ int warp_tot[4];
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  uint16_t* const cnt = reinterpret_cast<uint16_t*>(cnt2[wid]);
+  pdl_wait_predecessor();
+  if (row_is_final(a, b)) return;
+  const AslReq rq = row_request(a, b);
+  const uint32_t lt = (1u << lane) - 1u;
+  const int w0 = wid * R * 32;                                        // a warp owns consecutive keys
+  uint32_t key[R];
+  uint32_t id[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int i = w0 + r * 32 + lane;
+    id[r] = i;
+    key[r] = i < rq.T ? desc_key(__ldcg(a.agg + rq.t_off + i)) : 0xffffffffu;   // padding sorts last (and stays behind equal keys)
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) lanes[wid][i * 32 + lane] = 0;
+#pragma unroll 1
+  for (int pass = 0; pass < 4; ++pass) {
+    const int shift = 8 * pass;
+    uint32_t before[R];                                               // keys of the warp with the same digit and a lower place
+#pragma unroll
+    for (int i = 0; i < 4; ++i) cnt2[wid][i * 32 + lane] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const uint32_t d = (key[r] >> shift) & 255u;
+      const uint32_t peers = same_digit(lanes[wid], d, true, lane);
+      const uint32_t c = cnt[d];
+      __syncwarp();
+      if ((peers & lt) == 0) cnt[d] = (uint16_t)(c + __popc(peers));
+      before[r] = c + __popc(peers & lt);
+      __syncwarp();
+    }
+    __syncthreads();
+    {  // the counts become positions, in (digit, warp) order: thread (part, word) has two digits of four warps
+      const int w = tid & 127, part = tid >> 7;
+      uint32_t v[4], total = 0, mine = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { v[i] = cnt2[part * 4 + i][w]; mine += v[i]; }
+      part_sum[part][w] = mine;
       __syncthreads();
-      if (tid == 0)
-        for (int g = 1; g < GROUPS; ++g) { num += s_num[g]; m += s_m[g]; }
+      mine = 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) { const uint32_t s = part_sum[q][w]; total += s; mine += q < part ? s : 0u; }
+      const int both = (int)((total & 0xffffu) + (total >> 16));
+      int incl = both;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+      }
+      if (part == 0 && lane == 31) warp_tot[wid] = incl;
+      __syncthreads();
+      uint32_t off = (uint32_t)(incl - both);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) off += q < (w >> 5) ? (uint32_t)warp_tot[q] : 0u;
+      uint32_t run = mine + (off | (off + (total & 0xffffu)) << 16);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { cnt2[part * 4 + i][w] = run; run += v[i]; }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const uint32_t pos = cnt[(key[r] >> shift) & 255u] + before[r];
+      if (pass == 3) { s_key[id[r]] = pos; continue; }      // the rank row, in token order
+      s_key[pos] = key[r];
+      s_id[pos] = (uint16_t)id[r];
+    }
+    __syncthreads();
+    if (pass == 3) break;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      key[r] = s_key[w0 + r * 32 + lane];
+      id[r] = s_id[w0 + r * 32 + lane];
     }
   }
-  if (a.req) stat_close(a.stat, b, num, m, a.evaluate);
+  // ---- the row, and the statistic over it and the earlier rows
+  __shared__ unsigned long long s_num[ROW_WARPS];
+  __shared__ int s_m[ROW_WARPS];
+  unsigned long long num = 0;
+  int m = 0;
+#pragma unroll 1
+  for (int i = tid; i < rq.T; i += ROW_THREADS) {
+    const int mine = (int)s_key[i];
+    a.rank_row[rq.t_off + i] = mine;
+    if (a.evaluate) {
+      long long s1 = mine, s2 = (long long)mine * mine;
+      int mn = mine;
+      for (int r0 = 0; r0 < a.stat.n_rows - 1; r0 += 8) {
+        int v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int slot = (a.stat.first_layer + r0 + q) % a.stat.l_obs;
+          v[q] = r0 + q < a.stat.n_rows - 1 ? __ldcg(a.stat.ring + (int64_t)slot * a.stat.sum_T + rq.t_off + i) : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (v[q] >= 0) { mn = min(mn, v[q]); s1 += v[q]; s2 += (long long)v[q] * v[q]; }
+      }
+      if (mn < rq.k) {
+        m += 1;
+        num += (unsigned long long)((long long)a.stat.n_rows * s2 - s1 * s1);
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    num += __shfl_down_sync(0xffffffffu, num, o);
+    m += __shfl_down_sync(0xffffffffu, m, o);
+  }
+  if (lane == 0) { s_num[wid] = num; s_m[wid] = m; }
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < ROW_WARPS; ++w) { num += s_num[w]; m += s_m[w]; }
+    stat_finalize_one(num, (unsigned long long)m, a.req, a.stat.stat, b, a.stat.layer_idx, a.stat.n_rows, a.evaluate, a.stat.tau, a.stat.latch);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -903,14 +1044,12 @@ __global__ void __launch_bounds__(PLACE_THREADS, S == 1024 ? 2 : 3) rank_place_k
 template <int S>
 constexpr int split_smem_bytes() { return (int)(5 * S * sizeof(unsigned long long) + S * sizeof(int)); }
 
-template <int GROUPS>
-void launch_count_of(const RowArgs& r, int max_T, int batch, cudaStream_t st) {
-  launch_after(rank_count_kernel<GROUPS>, dim3((max_T + 32 * GROUPS - 1) / (32 * GROUPS), batch), dim3(COUNT_THREADS), st, r);
-}
-bool count_takes(int max_T, int batch) { return max_T <= COUNT_MAX_T && (batch == 1 || (int64_t)batch * max_T * max_T <= COUNT_BATCH_PAIRS); }
-void launch_count(const RowArgs& r, int max_T, int batch, cudaStream_t st) {
-  if (batch == 1) launch_count_of<1>(r, max_T, batch, st);
-  else launch_count_of<4>(r, max_T, batch, st);
+void launch_count(const RowArgs& r, int T, cudaStream_t st) { launch_after(rank_count_kernel, dim3((T + 31) / 32), dim3(COUNT_THREADS), st, r); }
+
+void launch_row_sort(const RowArgs& r, int max_T, int batch, cudaStream_t st) {
+  const int rounds = max_T <= 1024 ? 1 : max_T <= 2048 ? 2 : 4;
+  const auto kernel = rounds == 1 ? rank_sort_kernel<1> : rounds == 2 ? rank_sort_kernel<2> : rank_sort_kernel<4>;
+  launch_after_smem(kernel, dim3(batch), dim3(ROW_THREADS), sort_smem_bytes(rounds), st, r);
 }
 
 template <int S>
@@ -934,6 +1073,9 @@ int launch_split(const RowArgs& r, int max_T, int batch, cudaStream_t st) {
 
 // once per device, with that device current
 asl_status asl_rank_ready() {
+  ASL_CUDA(cudaFuncSetAttribute(rank_sort_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sort_smem_bytes(1)));
+  ASL_CUDA(cudaFuncSetAttribute(rank_sort_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sort_smem_bytes(2)));
+  ASL_CUDA(cudaFuncSetAttribute(rank_sort_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sort_smem_bytes(4)));
   ASL_CUDA(cudaFuncSetAttribute(rank_split_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, split_smem_bytes<1024>()));
   ASL_CUDA(cudaFuncSetAttribute(rank_place_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlaceSmem<512>)));
   ASL_CUDA(cudaFuncSetAttribute(rank_place_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlaceSmem<1024>)));
@@ -955,8 +1097,10 @@ asl_status asl_launch_rank(asl_ctx* c, const float* agg, int32_t layer_idx, int3
                    latch ? 1 : 0, p.tau};
   RowArgs r{agg, row, c->d_req, 0, reinterpret_cast<unsigned long long*>(keys[0]), reinterpret_cast<unsigned long long*>(idx[0]),
             reinterpret_cast<unsigned long long*>(hist), nullptr, 0, a, evaluate};
-  if (count_takes(c->max_T, p.batch)) {         // the statistic goes with the row
-    launch_count(r, c->max_T, p.batch, st);
+  const bool counted = p.batch == 1 && c->max_T <= COUNT_MAX_T;
+  if (counted || sort_takes(c->max_T, c->sum_T, p.batch, c->sm_count)) {         // the statistic goes with the row
+    if (counted) launch_count(r, c->max_T, st);
+    else launch_row_sort(r, c->max_T, p.batch, st);
     c->launches += 1;
     ASL_CUDA(cudaGetLastError());
     return ASL_OK;
@@ -1048,7 +1192,7 @@ extern "C" asl_status asl_rank_desc_static(const float* scores, int32_t T, int32
   if (ready != ASL_OK) return ready;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const RowArgs r{scores, rank_out, nullptr, T, s->pairs, s->list, s->table, nullptr, 0, StatArgs{}, 0};
-  if (count_takes(T, 1)) launch_count(r, T, 1, st);
+  if (T <= COUNT_MAX_T) launch_count(r, T, st);
   else launch_split(r, T, 1, st);
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;

@@ -116,10 +116,12 @@ def test_time_of_a_row_in_one_bucket_grows_with_its_length(T):
         assert begin.elapsed_time(end) < 0.3 + 30e-6 * T, kind
 
 
-@pytest.mark.parametrize("lengths", [(1, 33), (500, 97) * 4, (129, 1, 128, 127, 900), (1448, 1447), (1449, 1448), (32,) * 9])
-def test_short_requests_of_a_batch_take_one_launch(lengths):
-    """Counted rows with their statistic up to 2^22 compares by the longest request's square, split ones above; a request
-    whose selection is final keeps its rank row and its record."""
+@pytest.mark.parametrize("lengths,launches", [
+    ((1, 33), 1), ((500, 97) * 4, 1), ((129, 1, 128, 127, 900), 1), ((1023, 1024), 1), ((32,) * 300, 1), ((1100, 1024), 3),
+    ((1025,) * 63, 1), ((2048, 2047) * 30, 3), ((2048, 2047) * 33, 1), ((4096, 2049) * 48, 3), ((4096, 4095) * 48, 1)])
+def test_short_requests_of_a_batch(lengths, launches):
+    """Up to 1024 tokens, and for many requests up to 4096, a block sorts a request and takes its statistic: one launch; three
+    for the split row.  Infinities and zeros of both signs; a request whose selection is final keeps its rank row and record."""
     w, rows, n = 32, 3, len(lengths)
     wl = I.workload("C1", seqlens=tuple(T + w for T in lengths), budgets=tuple(w + T // 9 for T in lengths), l_min=1, l_obs=rows)
     path = make_path(wl)
@@ -128,12 +130,14 @@ def test_short_requests_of_a_batch_take_one_launch(lengths):
     selected_word = B.STAT_DTYPE.fields["selected"][1] // 4
     for layer in range(rows + 1):
         per = [_scores(T, KINDS[layer % 4], rng) for T in lengths]
+        for s in per[:2]:
+            s[::5], s[1::7], s[2::9], s[3::9] = np.inf, -np.inf, 0.0, -0.0
         path.scores_agg.copy_(torch.from_numpy(np.concatenate(per)))
         if layer == rows:
             path.stat.view(torch.int32)[n - 1, selected_word] = 1
-        before, ring, launches = path.read_stat().copy(), path.rank_ring[layer % rows].cpu().numpy(), B.asl_launch_count(path.ctx)
+        before, ring, count = path.read_stat().copy(), path.rank_ring[layer % rows].cpu().numpy(), B.asl_launch_count(path.ctx)
         B.asl_rank_stat(path.ctx, path.scores_agg, layer, min(layer + 1, rows), path.rank_ring, path.stat, path.workspace, path.ws_bytes)
-        assert B.asl_launch_count(path.ctx) - launches == (1 if n * max(lengths) ** 2 <= 2**22 else 3)
+        assert B.asl_launch_count(path.ctx) - count == launches
         ranks.append([O.rank_desc(s.astype(np.float64)) for s in per])
         got, at, stat = path.rank_ring[layer % rows].cpu().numpy(), 0, path.read_stat()
         for b, T in enumerate(lengths):
