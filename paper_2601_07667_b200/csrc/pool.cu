@@ -14,7 +14,7 @@ namespace {
 constexpr int PT = 256;          // threads of a block / tokens per block of the general kernel
 constexpr int MAX_HALO = 16;     // pooling kernels up to 33 taps
 constexpr int HB = 8;            // general kernel: staged units per round
-constexpr int PV_ROWS = 8;       // vector kernel: partial rows in flight per lane
+constexpr int PV_ROWS = 8;       // vector kernel: partial rows in flight per lane, where a head has few
 constexpr int PV_THREADS = 128;
 
 struct PoolArgs {
@@ -29,15 +29,19 @@ struct PoolArgs {
 };
 
 // Windows of up to 9 taps, units of 1, 2, 4, 8 or 16 partial rows.  A lane owns 4 consecutive tokens: one 16-byte load per
-// partial row, eight in flight, the rows of a unit added in order, the neighbours' sums fetched by warp shuffles; the
+// partial row, the rows of a unit added in order, the neighbours' sums fetched by warp shuffles; the
 // first and the last lane of a warp only supply the halo, so a warp pools 120 tokens.  No shared memory and no
-// block-wide barrier.  Bound by the round trips for the rows (one per eight; with sixteen in flight the registers leave room
-// for half as many warps on the SMs that a scorer leaves free: eight layers of 32K tokens 434.3 -> 431.7 us): max pooling of 64 query
-// heads at 64K tokens 43 -> 10 us, eight ragged requests of 8 heads 25 -> 6.5 us against one thread per token with rows
-// staged in shared memory; 128K tokens of 8 heads, two partial rows each, 6.1 -> 4.4 us.
+// block-wide barrier.  Bound by the round trips for the rows.  In flight at a time: eight rows where a kv head has few (with
+// sixteen the registers leave room for half as many warps on the SMs that a scorer leaves: eight layers of 32K tokens
+// 434.3 -> 431.7 us), sixteen or two units where there are many.  The loads of a single unit in flight the compiler spreads
+// among its adds, those ahead of the test for a second unit it issues together.  Us at 8 / 16 / 32 in flight: 65536 tokens,
+// average of 8 kv heads with 8 rows each 7.8 / 4.2 (16 before), of 4 with 16 rows - / 10.0 / 3.5 (7.3 before), max of 64
+// query heads with 4 rows each 18.7 / 15.2, with 2 9.5 / 8.7, with one 7.4 / 8.8; average of 8 with 4 rows 3.4 / 4.7.
+// 128K tokens of 8 heads, two rows each, 3.3.
 template <bool MAX, int R, int NR>
 __global__ void __launch_bounds__(PV_THREADS) pool_vec4_kernel(PoolArgs a) {
-  constexpr int IN_FLIGHT = NR > PV_ROWS ? NR : PV_ROWS;
+  constexpr int IN_FLIGHT = NR >= 8 ? 2 * NR : MAX && NR >= 2 ? 16 : PV_ROWS;
+  constexpr bool ALL_LANES = !MAX && NR >= 8;                          // lanes outside load too, from the segment's first tokens
   pdl_wait_predecessor();
   const int b = blockIdx.y;
   if (a.latch && asl_finished(a.latch + b, a.cur_layer)) return;       // the request's scores stay as its selection layer left them
@@ -51,7 +55,7 @@ __global__ void __launch_bounds__(PV_THREADS) pool_vec4_kernel(PoolArgs a) {
   const int live = rq.T - j0;                                          // tokens from j0 on (4 or more: all of the lane's)
   const float outside = MAX ? -INFINITY : 0.f;
   const float inv = 1.0f / (float)a.S;
-  const float* base = a.u + rq.u_off + j0;
+  const float* base = a.u + rq.u_off + (ALL_LANES && !inside ? 0 : j0);
   const int per_head = MAX ? a.G : 1, units = a.Hk * per_head, rows = units * NR;
   auto store = [&](float* dst, const float (&p)[4]) {
     if (a.vec_out && live >= 4) *reinterpret_cast<float4*>(dst) = make_float4(p[0], p[1], p[2], p[3]);
@@ -66,7 +70,7 @@ __global__ void __launch_bounds__(PV_THREADS) pool_vec4_kernel(PoolArgs a) {
     float4 x[IN_FLIGHT];
 #pragma unroll
     for (int e = 0; e < IN_FLIGHT; ++e)
-      x[e] = (inside && r0 + e < rows) ? __ldcg(reinterpret_cast<const float4*>(base + (int64_t)(r0 + e) * a.u_stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      x[e] = ((ALL_LANES || inside) && r0 + e < rows) ? __ldcg(reinterpret_cast<const float4*>(base + (int64_t)(r0 + e) * a.u_stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int q = 0; q < IN_FLIGHT / NR; ++q) {
       if (r0 + q * NR >= rows) break;

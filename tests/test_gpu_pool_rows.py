@@ -17,6 +17,9 @@ pytestmark = pytest.mark.gpu
     (I.POOL_AVG, 9, 32, 1, 128), (I.POOL_AVG, 11, 4, 2, 32), (I.POOL_AVG, 33, 4, 2, 32), (I.POOL_AVG, 7, 14, 2, 64),
     (I.POOL_MAX, 1, 2, 2, 32), (I.POOL_MAX, 5, 6, 2, 64), (I.POOL_MAX, 7, 4, 1, 256), (I.POOL_MAX, 9, 8, 1, 128),
     (I.POOL_MAX, 15, 4, 2, 32),
+    # rows that are no multiple of those in flight: 3 kv heads of 8 and of 16, heads of 2, 4, 8 and 16
+    (I.POOL_AVG, 7, 24, 3, 128), (I.POOL_AVG, 5, 48, 3, 128), (I.POOL_AVG, 9, 8, 1, 128), (I.POOL_MAX, 5, 3, 3, 200),
+    (I.POOL_MAX, 7, 3, 1, 512), (I.POOL_MAX, 9, 3, 3, 1024), (I.POOL_MAX, 3, 3, 1, 2048),
 ])
 def test_pooling_of_ragged_segments(mode, S, Hq, Hk, w):
     seqlens = tuple(w + t for t in (1, 3, 121, 120, 479, 962))
