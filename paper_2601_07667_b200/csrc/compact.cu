@@ -8,7 +8,6 @@ namespace {
 
 constexpr int ROWS = 4;                   // rows per thread
 constexpr int BLOCK_ROWS = 16 * ROWS;     // rows per 256-thread block
-constexpr int GATHER_VECS = 8;            // row gather: vectors in flight per lane
 
 __global__ void __launch_bounds__(256) compact_kv_kernel(const uint8_t* __restrict__ k, const uint8_t* __restrict__ v,
                                                          const int32_t* __restrict__ idx, const AslReq* __restrict__ req,
@@ -42,9 +41,12 @@ __global__ void __launch_bounds__(256) compact_kv_kernel(const uint8_t* __restri
 }
 
 // Row gather of one tensor with rows of `row_bytes` (a multiple of 16): out[kept_off_b + r] = x[tok_off_b + idx[r]].
-// A warp moves one row, 16 bytes per lane, eight loads in flight (as written: a streaming load is not moved above the store
-// before it, and one at a time cost what the launch ahead of the top-k's end had gained).  Bound by HBM: 3.9K rows of 8 KB
-// (64 MB moved) behind their top-k 37.6 -> 32.0 us for both, 32.1 with four in flight.
+// A warp moves one row, 16 bytes per lane, up to eight loads in flight (as written: they are not moved above the stores before
+// them).  Bound by HBM where rows are long: 3.9K rows of 8 KB (64 MB moved) behind their top-k 37.6 -> 32.0 us for both.
+// Rows of up to 2 KB take as many loads as they have, the registers of eight cost short rows their warps, and no streaming
+// hint, which sends rows out of L2 that the next gather may find there.  30000 rows, us with eight / as many: of 64 bytes 5.5 /
+// 3.9, 400 6.7 / 4.4, 528 7.1 / 4.9, 1040 8.1 / 7.7; 20000 of 2 KB with the hint 9.4, without 8.8.
+template <int VECS>                       // vectors in flight per lane
 __global__ void __launch_bounds__(256) compact_rows_kernel(const uint4* __restrict__ x, const int32_t* __restrict__ idx,
                                                            const AslReq* __restrict__ req, int vec_per_row,
                                                            uint4* __restrict__ out) {
@@ -55,13 +57,13 @@ __global__ void __launch_bounds__(256) compact_rows_kernel(const uint4* __restri
   if (r >= rq.kept) return;
   const int64_t src = ((int64_t)rq.tok_off + __ldcg(idx + rq.kept_off + r)) * vec_per_row;
   const int64_t dst = ((int64_t)rq.kept_off + r) * vec_per_row;
-  for (int c0 = lane; c0 < vec_per_row; c0 += 32 * GATHER_VECS) {
-    uint4 v[GATHER_VECS];
+  for (int c0 = lane; c0 < vec_per_row; c0 += 32 * VECS) {
+    uint4 v[VECS];
 #pragma unroll
-    for (int q = 0; q < GATHER_VECS; ++q)
-      if (c0 + 32 * q < vec_per_row) v[q] = __ldcs(x + src + c0 + 32 * q);
+    for (int q = 0; q < VECS; ++q)
+      if (c0 + 32 * q < vec_per_row) v[q] = VECS == 8 ? __ldcs(x + src + c0 + 32 * q) : __ldcg(x + src + c0 + 32 * q);
 #pragma unroll
-    for (int q = 0; q < GATHER_VECS; ++q)
+    for (int q = 0; q < VECS; ++q)
       if (c0 + 32 * q < vec_per_row) out[dst + c0 + 32 * q] = v[q];
   }
 }
@@ -71,8 +73,10 @@ __global__ void __launch_bounds__(256) compact_rows_kernel(const uint4* __restri
 asl_status asl_launch_compact_rows(asl_ctx* c, const void* x, const int32_t* idx, void* out, int64_t row_bytes,
                                    cudaStream_t st) {
   dim3 grid((c->max_kept + 7) / 8, c->p.batch);
-  launch_after(compact_rows_kernel, grid, dim3(256), st, static_cast<const uint4*>(x), idx, c->d_req, (int)(row_bytes / 16),
-                                            static_cast<uint4*>(out));
+  const int vec_per_row = (int)(row_bytes / 16);
+  const auto kernel = vec_per_row > 128 ? compact_rows_kernel<8> : vec_per_row > 64 ? compact_rows_kernel<4>
+                      : vec_per_row > 32 ? compact_rows_kernel<2> : compact_rows_kernel<1>;
+  launch_after(kernel, grid, dim3(256), st, static_cast<const uint4*>(x), idx, c->d_req, vec_per_row, static_cast<uint4*>(out));
   c->launches += 1;
   ASL_CUDA(cudaGetLastError());
   return ASL_OK;

@@ -37,9 +37,9 @@ def test_compaction_of_any_number_of_rows(fp8):
     path.close()
 
 
-@pytest.mark.parametrize("row_bytes", [16, 512, 528, 4080, 4096, 4112, 4608, 7168, 8192])
+@pytest.mark.parametrize("row_bytes", [16, 400, 496, 512, 528, 1008, 1024, 1040, 2032, 2048, 2064, 4080, 4096, 4112, 4608, 7168, 8192])
 def test_row_gather_of_rows_around_a_warps_loads(row_bytes):
-    """A warp has eight loads of 512 bytes in flight: rows below, at and above one and eight of them."""
+    """A warp has one, two, four or eight loads of 512 bytes in flight: rows below, at and above each of them."""
     w, seqlens, kept = 32, (40, 700, 90), (33, 321, 90)
     wl = I.workload("C1", window=w, seqlens=seqlens, budgets=kept, layers=1, l_min=1, l_obs=2)
     path = make_path(wl)
