@@ -1332,7 +1332,7 @@ bool asl_tc_plan(asl_ctx* c) {
   if (tiles >= (int64_t)1 << 30) return false;
 
   // Groups of segments: pass 1 of a group, then pass 2 of the one before it, so that the fold of the row denominators is
-  // hidden behind other tiles; at least two of them, of up to 140 MB of K each.  (One, where no CTA of
+  // hidden behind other tiles; at least two of them, of up to 140 MB of K each, 70 MB where a kv head has several chunks.  (One, where no CTA of
   // any call has more than one tile of a pass: there is then nothing to hide the fold behind, and it is waited for once
   // instead of twice.  In us with two groups and one: 1500 tokens of 8 kv heads 21.2, 15.8, 4096 of 2 heads 13.9, 11.6.  It
   // would pay up to 1.3 tiles a CTA, 3000 tokens 19.6, 16.7, but asl_score_layer and its halves then add in different
@@ -1340,16 +1340,20 @@ bool asl_tc_plan(asl_ctx* c) {
   // (above), large ones need fewer hand-offs, and the hand-offs count for more.  In us at 36, 50, 70, 100, 140 and 270 MB,
   // passes issued back to back: four layers of 128K tokens 835, 836, 827, 834, 819, 824; of 100K 667, 657, 636, 638, 630, 631;
   // of 64K 448, 447, 438, 441, 441, 439; two of eight ragged requests 587, 555, 579, 569, 562, 559; two with W = 128 and 64
-  // query heads at 64K 769, 760, 774, 760, 769, 771; three with FP8 keys at 48K 238, 240, 239, 236, 238, 237.
+  // query heads at 64K 769, 760, 774, 760, 769, 771; three with FP8 keys at 48K 238, 240, 239, 236, 238, 237.  Every chunk of a kv
+  // head reads its K again, in either pass: with several, what does not stay in L2 counts for more.  At 70, 100, 140 MB, four
+  // layers: 64 query heads, W = 128 (four chunks) 128K 2799, 2761, 2971, 96K 2092, 2090, 2213, eight ragged requests 6375,
+  // 6418, 6665; W = 64 (two) 128K 1466, 1502, 1558; 32 query heads, W = 128 (two) 100K 1124, 1136, 1184.
   const int given = p.score_ctas > 0 && p.score_ctas < c->sm_count ? p.score_ctas : 0;
   std::vector<int> cut{0};
   {
+    const double limit = tp.nchunk > 1 ? 70.0e6 : 140.0e6;
     auto seg_bytes = [&](int s) { return (double)c->req[segs[s].b].n * 128 * c->k_elem_bytes / tp.nchunk; };
     double total = 0, run = 0;
     int groups = 1;
     for (int s = 0; s < tp.nseg; ++s) {
       total += seg_bytes(s);
-      if (run > 0 && run + seg_bytes(s) > 140.0e6) { ++groups; run = 0; }
+      if (run > 0 && run + seg_bytes(s) > limit) { ++groups; run = 0; }
       run += seg_bytes(s);
     }
     if (groups < 2 && tiles > (given ? given : c->sm_count - 32)) groups = 2;
