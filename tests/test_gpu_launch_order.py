@@ -113,3 +113,85 @@ def test_rank_rows_with_nothing_in_between(lengths, how):
         assert (stat[b]["num"], stat[b]["m"]) == (num, m)
         at += T
     path.close()
+
+
+def _score(path, x, lse, out):
+    if lse is None:
+        B.asl_score_layer(path.ctx, x[0], x[1], *out, path.workspace, path.ws_bytes)
+    else:
+        B.asl_score_layer_lse(path.ctx, x[0], x[1], lse, *out, path.workspace, path.ws_bytes)
+
+
+@pytest.mark.parametrize("how", ["calls", "graph"])
+@pytest.mark.parametrize("mode,seqlens", [(I.POOL_AVG, (2900,)), (I.POOL_AVG, (40001, 3000)), (I.POOL_MAX, (9000, 20011))])
+def test_layers_on_one_stream_with_nothing_in_between(mode, seqlens, how):
+    """Scorer, pooling, rank row, top-k and both gathers, six layers of other inputs in a row, every call right behind the one
+    whose results it reads and into buffers of its own; one-pass scoring in turn with two-pass, whose offsets are kept in two
+    sets.  The same, bit for bit, as with a synchronize after every call."""
+    w, rounds = 32, 6
+    wl = I.workload("C3", n_q_heads=8, n_kv_heads=2, window=w, pool_mode=mode, pool_kernel=5, seqlens=seqlens,
+                    budgets=tuple(w + n // 6 for n in seqlens), layers=1, l_min=1, l_obs=rounds, distractors=0)
+    path = make_path(wl)
+    H, d, n = wl.n_kv_heads, wl.head_dim, path.sum_tokens
+    g = torch.Generator(device="cuda").manual_seed(n)
+    rand = lambda *shape: torch.randn(shape, generator=g, device="cuda").to(torch.bfloat16)
+    inputs = [(rand(len(seqlens), wl.n_q_heads, w, d), rand(n, H, d), rand(n, H, d), rand(n, 2112)) for _ in range(rounds)]
+    lses = [None] * rounds
+    for r in range(1, rounds, 2):                              # every second layer in one pass over K
+        _score(path, inputs[r], None, (path.scores_kv, path.scores_agg))
+        lses[r] = torch.empty((len(seqlens), wl.n_q_heads, w), device="cuda")
+        B.asl_window_lse(path.ctx, path.workspace, path.ws_bytes, lses[r])
+    torch.cuda.synchronize()
+
+    def buffers():
+        return [(torch.zeros((H, path.sum_T), device="cuda"), torch.zeros(path.sum_T, device="cuda"), torch.zeros_like(path.idx),
+                 torch.zeros_like(path.k_out), torch.zeros_like(path.v_out), torch.zeros((path.sum_kept,), dtype=torch.int32, device="cuda"),
+                 torch.zeros((path.sum_kept, 2112), dtype=torch.bfloat16, device="cuda")) for _ in range(rounds)]
+
+    def chain(outs, between=lambda: None):
+        for r, (x, (kv, agg, idx, k_out, v_out, one, rows)) in enumerate(zip(inputs, outs)):
+            for call in (lambda: _score(path, x, lses[r], (kv, agg)),
+                         lambda: B.asl_rank_stat(path.ctx, agg, r, r + 1, path.rank_ring, path.stat, path.workspace, path.ws_bytes),
+                         lambda: B.asl_select_topk(path.ctx, kv, H, idx, path.workspace, path.ws_bytes),
+                         lambda: B.asl_compact_kv(path.ctx, x[1], x[2], idx, k_out, v_out),
+                         lambda: B.asl_select_topk(path.ctx, agg, 1, one, path.workspace, path.ws_bytes),
+                         lambda: B.asl_compact_rows(path.ctx, x[3], one, rows, 4224)):
+                call()
+                between()
+
+    def state():
+        path.stat.zero_()
+        path.rank_ring.zero_()
+        torch.cuda.synchronize()
+
+    alone, outs = buffers(), buffers()
+    state()
+    chain(alone, torch.cuda.synchronize)
+    ring, stat = path.rank_ring.clone(), path.read_stat().copy()
+    state()
+    if how == "graph":
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            chain(outs)
+        for _ in range(2):                                     # replays follow one another as calls do
+            graph.replay()
+        path.stat.zero_()
+        graph.replay()
+    else:
+        chain(outs)
+    torch.cuda.synchronize()
+    for r, (a, o) in enumerate(zip(alone, outs)):
+        for i, (x, y) in enumerate(zip(a, o)):
+            assert torch.equal(x, y), (r, i)
+    assert torch.equal(ring, path.rank_ring) and path.read_stat().tobytes() == stat.tobytes()
+    assert B.asl_device_status(path.ctx)[0] == 0
+    at = 0
+    for b, n_b in enumerate(seqlens):                          # and right: lists, rows and ranks of the scores, by the oracle
+        T, kept, s = n_b - w, w + n_b // 6, alone[-1][1].cpu().numpy().astype(np.float64)
+        here, k0 = slice(int(path.t_off[b]), int(path.t_off[b]) + T), int(path.kept_off[b])
+        assert (ring[rounds - 1, here].cpu().numpy() == O.rank_desc(s[here])).all()
+        ref = O.select_topk(s[here], kept - w, n_b, w)
+        assert (alone[-1][5][k0:k0 + kept].cpu().numpy() == ref).all()
+        assert torch.equal(alone[-1][6][k0:k0 + kept], inputs[-1][3][at + torch.from_numpy(ref).cuda()])
+        at += n_b
+    path.close()

@@ -1,6 +1,6 @@
-"""The one-CTA top-k where the last digits of the k-th key are settled by comparing the few keys of one bin, where all keys
-equal to it are kept or some of them, and where the kept tokens come in passages (words of the bitmap that a whole warp
-writes: none, a few, all of a warp's)."""
+"""The one-CTA top-k where the last digits of the k-th key are settled by comparing the few keys of one bin (128 at most: bins
+of 127, 128 and 129 keys, and some that are split further), where all keys equal to it are kept or some of them, and where the
+kept tokens come in passages (words of the bitmap that a whole warp writes: none, a few, all of a warp's)."""
 import numpy as np
 import pytest
 
@@ -13,11 +13,14 @@ pytestmark = pytest.mark.gpu
 
 def _row(T, k, kind, rng):
     s = np.exp(rng.normal(-9.0, 1.5, size=T))
-    if kind[0] == "equal":                               # `more` + 1 tokens share the k-th score, one or all of them kept
+    if kind[0] in ("equal", "apart"):                    # `more` + 1 tokens share the k-th score, one or all of them kept
         more, one = kind[1:]
         order = np.argsort(-s, kind="stable")
         first = k - 1 if one else max(0, k - 1 - more)
         s[order[first:first + 1 + more]] = s[order[first]]
+        if kind[0] == "apart":                           # and have their bin to themselves
+            s[order[:first]] *= 1.25
+            s[order[first + 1 + more:]] /= 1.25
     elif kind[0] == "passages":                          # runs of `length` tokens far above the rest
         length = kind[1]
         for f in rng.permutation(T // length)[:max(1, k // length)]:
@@ -26,7 +29,8 @@ def _row(T, k, kind, rng):
 
 
 @pytest.mark.parametrize("kind", [("smooth",), ("equal", 5, True), ("equal", 5, False), ("equal", 511, True), ("equal", 511, False),
-                                  ("equal", 700, True), ("equal", 700, False), ("passages", 17), ("passages", 128), ("passages", 1500)])
+                                  ("equal", 700, True), ("equal", 700, False), ("apart", 126, True), ("apart", 127, True),
+                                  ("apart", 127, False), ("apart", 128, True), ("apart", 128, False), ("passages", 17), ("passages", 128), ("passages", 1500)])
 @pytest.mark.parametrize("T,k", [(900, 800), (4097, 1000), (12288, 3000), (12289, 3000), (33001, 4000), (66003, 9000)])
 def test_topk(T, k, kind):
     w, heads = 32, 3
