@@ -678,7 +678,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) rank_sort_kernel(RowArgs a) {
 //
 // Neither waits for another block, and the row does not depend on the order in which pairs arrive.  Bound by latency: the
 // first takes 4 to 6 us (the sample's round trip, its sort, 8 to 10 steps of search), the second 7 (three round trips).
-// 100003 tokens with the statistic: five radix passes 34.6 us -> 20.8.  32768 tokens beside a scorer that leaves 16 SMs:
+// 100003 tokens with the statistic: five radix passes 34.8 us -> 16.7.  32768 tokens beside a scorer that leaves 16 SMs:
 // sorted tiles of 4096 and their merge, whose searches grow with the square of the length, 35 us -> 23; eight layers
 // 471 -> 460 us.  Longer segments would need a larger sample, whose sort every block repeats.
 // ---------------------------------------------------------------------------
@@ -812,7 +812,7 @@ struct PlaceSmem {
 
 // The block's m pairs sorted, whatever they are: stable passes over the 8-bit digits in which they differ, lowest first, to and
 // fro between the pairs' own slots in the tiles and the list; the last one writes the ranks.  For blocks that have no room for
-// their pairs (some row in a thousand), and for bins of more than BIN_MAX pairs (a bucket's ends far apart and the rest nearly
+// their pairs, and for bins of more than BIN_MAX pairs (a bucket's ends far apart and the rest nearly
 // alike: the border of two long runs of equal scores, scores on both sides of zero), whose compares grow with their square.
 // One SM's seven passes, 9 to 13 ns a pair, are what a row costs whose tokens, but for the sampled ones, lie in one bucket:
 // 131072 tokens of one value 1.6 s -> 1.3 ms, of random values 5.6 -> 1.7 ms, 5000 of one value 870 -> 66 us.  Rows that the

@@ -20,8 +20,8 @@
 // a CTA does its runs of pass 1 of group i, then those of pass 2 of group i - 1: it
 // meets one or two segments at a time and keeps a Q chunk for a whole run, and the
 // offsets that pass 2 needs were folded while other tiles were worked on.  Between the two
-// reads of a tile lie up to two groups (up to 140 MB each), so that of more than 134 MB of K (64K
-// tokens, 8 kv heads) pass 2 finds less than half in L2.  Dealing every segment's tiles round-robin
+// reads of a tile lie up to two groups (up to 140 MB each): of 268 MB of K (128K
+// tokens, 8 kv heads) pass 2 finds a quarter in L2 (464 MB are read from DRAM; in groups of 70 MB 438).  Dealing every segment's tiles round-robin
 // to all CTAs cost 3 us per segment and pass (64 KB of Q reloaded per CTA, a hand-off each):
 // 32K tokens, 8 kv heads 64 -> 48 us, eight ragged requests with W = 32 350 -> 184 us,
 // W = 128 with 64 query heads at 64K 374 -> 288 us, 128K tokens 163 -> 153 us.

@@ -291,8 +291,7 @@ __global__ void __launch_bounds__(THREADS) topk_emit_kernel(TopkArgs a) {
 // 16-byte boundary before the row and the row, so that a vector is a nibble of a word.  (One score per lane and a ballot
 // per word takes six times the instructions: 40 us for the pass over 131008 scores instead of 8.)  Bound by what one SM
 // pulls from L2 and by the chain of passes:
-// one segment of 96K scores, k = 3.8K: 24.8 -> 22.0 us; 32 segments of 3 to 24 K scores, k half of them: 29 us (five
-// tiled kernels) -> 15 us.
+// one segment of 96K scores, k = 3.8K, 18.8 us; 32 segments of 24K scores, k half of them, 13.7 us (back to back).
 // ---------------------------------------------------------------------------
 constexpr int SEG_THREADS = 1024;
 constexpr int SEG_WARPS = SEG_THREADS / 32;
@@ -364,8 +363,9 @@ __device__ __forceinline__ void seg_pick(SegSmem& sm, int remaining, int par, ui
 
 // The `rank`-th largest of keys[0..n) in shared memory (all of them in [lo, hi]), how many equal to it are wanted and how
 // many there are.  Digits from the top of the range, until the bin that counts holds few keys: after one digit of 2048 bins
-// as a rule.  (Few: 128.  Comparing up to 512 with one another took several digits' time where scores are heavy tailed: 128K
-// tokens, eight heads, k = 4032, call by call 35.0 us, 30.5 now.)
+// as a rule.  (Few: 128.  Comparing up to 512 with one another took several digits' time where scores are heavy tailed.)  128K
+// tokens, eight heads, k = 4032, call by call: the benchmark's scores 28.7 us with all digits counted and now, behind a
+// scorer that has swept L2, 28.7 -> 26.6 where a top-k ran shortly before; log-normal ones 31.8 -> 27.1, smooth 30.7 -> 25.6.
 __device__ __forceinline__ void seg_select(SegSmem& sm, int n, uint32_t lo, uint32_t hi, int rank, uint32_t& thr, int& need, int& equal) {
   int shift = 32 - __clz((int)((hi - lo) | 1u));            // bits of the range still open
   uint32_t base = lo;                                        // keys in [base, base + 2^shift) are still candidates
@@ -743,13 +743,16 @@ bool asl_topk_plan(asl_ctx* c) {
   return true;
 }
 
-// The faster form, in us measured back to back on an idle GPU (1, 8, 32 and 64 segments of 16K to 256K scores, k of 2 to 60 %
-// of them; within 2 us of most measurements): one CTA takes as long as the longest segment and the largest k say, for any
+// The faster form, on an idle GPU: one CTA takes as long as the longest segment and the largest k say, for any
 // number of segments up to the SM count (172 KB of shared memory a CTA at 256K scores: one to an SM), and 6 us more where k
-// is too large for the ordered copy; the tiled kernels take as long as the scores of all segments say.  An estimate, no
+// is too large for the ordered copy; the tiled kernels take as long as the scores of all segments say.  The constants were
+// fitted before kernels were launched ahead of their predecessor's end; both forms have since become 2 to 4 us faster, and
+// the line between them holds: measured again on 1, 2, 8, 32 and 64 segments of 4K to 256K smooth and log-normal scores, k of 2 to
+// 60 % of them, it takes the faster form or one within 6 %, but for 8 segments of 64K, k = 20K (22.5 / 19.9 us; call by call
+// 26.6 both), 8 of 256K, k = 5K (31.4 / 28.7) and one of 64K, k = 6.5K (19.1 / 17.4).  One CTA / tiled, back to back: one segment of
+// 128K, k = 2.6K, 18.9 / 17.9 us; 8 of 128K, k = 13K, 28.8 / 22.4; 64 of 64K, k = 20K, 22.7 / 50.7.  An estimate, no
 // bound: it takes the longest segment and the largest k for one request's where they are two, and a layer issues the call
-// beside a scorer that leaves 16 SMs, where neither form has been measured against the other.  One segment of 96K, k = 4K: 20.8 and 21.6 us; 8 of 128K, k = 13K: 31 and 27 us;
-// 64 of 64K, k = 23K: 26 and 55 us.
+// beside a scorer that leaves 16 SMs, where neither form has been measured against the other.
 static bool one_cta_is_faster(const asl_ctx* c, int n_heads) {
   const double k = c->max_kept - c->p.window;
   const double one = 10.0 + 0.08e-3 * c->max_T + 0.75e-3 * fmin(k, 6500.0) + 0.3e-3 * c->max_T / 65536.0 * fmax(0.0, k - 6500.0) +
